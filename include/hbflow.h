@@ -155,11 +155,12 @@ int hbf_set_inner_drop(hbf_ctx* ctx, double drop);
  * layout.  HBF_ERR_ARG unless on is 0 or 1. */
 int hbf_set_split_layout(hbf_ctx* ctx, int on);
 /* The fused tail of the V-cycles (the multigrid scheme of Sec. III B): from
- * the first level with at most max_cells cells down to the exact bottom solve
- * and back runs as one launch of one thread block, with block barriers
- * between the colour sweeps; the arithmetic and its order are those of the
- * level-by-level launches.  0 disables it; default 512.  HBF_ERR_ARG for a
- * negative count. */
+ * the first level (below the finest) with at most max_cells cells down to the
+ * coarsest-level solve and back runs as one launch of one thread-block
+ * cluster, with barriers between the colour sweeps; the arithmetic and its
+ * order are those of the level-by-level launches.  0 disables it; without a
+ * call the library chooses the level by size, dimension and precision.
+ * HBF_ERR_ARG for a negative count. */
 int hbf_set_tail(hbf_ctx* ctx, int max_cells);
 /* The 3D FP32 finest-level viscous smoothing of HBF_MIXED contexts: 1 runs
  * each component's red-black Gauss-Seidel sweep (Sec. III A's tensor solve,
@@ -545,8 +546,8 @@ int hbf_batch_step(hbf_batch* b, hbf_step_stats* stats);
 int hbf_batch_set_tiling(hbf_batch* b, int tile, int blocks_per_sm);
 int hbf_batch_get_tiling(const hbf_batch* b, int* tile, int* blocks_per_sm, int64_t* tiles_level0);
 /* Multigrid levels on which every cavity has at most max_cells cells (and
- * all coarser levels) run as one launch per V-cycle, one thread block per
- * cavity, with block barriers between colour sweeps; the arithmetic and its
+ * all coarser levels) run as one launch per V-cycle, one thread-block cluster
+ * per cavity, with barriers between colour sweeps; the arithmetic and its
  * order are those of the level-by-level launches.  0 disables it; default
  * 4096. */
 int hbf_batch_set_tail(hbf_batch* b, int max_cells);

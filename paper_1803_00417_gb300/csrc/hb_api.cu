@@ -154,6 +154,7 @@ static int allocate(hbf_ctx* c) {
       A(L.fvx, (long long)D * gl.ncell);
       A(L.fvb, (long long)D * gl.ncell);
       A(L.fvr, (long long)D * gl.ncell);
+      A(L.fvinv, (long long)D * gl.ncell);
       A(L.fcx, gl.ncell);
       A(L.fcb, gl.ncell);
       A(L.fcr, gl.ncell);
@@ -166,6 +167,7 @@ static int allocate(hbf_ctx* c) {
     }
     A(L.vb, (long long)D * gl.ncell);
     A(L.vr, (long long)D * gl.ncell);
+    if (c->precision == HBF_FP64 || !can_coarsen(gl, D)) A(L.vinv, (long long)D * gl.ncell);
     A(L.cb, gl.ncell);
     A(L.cr, gl.ncell);
     A(L.nb, gl.nnode);
@@ -419,9 +421,7 @@ int hbf_set_periodic(hbf_ctx* c, const int periodic[3]) {
     for (int a = 0; a < 3; ++a) c->lv[l].g.per[a] = per[a];
   // operators changed: rebuild the exact bottom inverses and the tail records
   for (auto& d : c->dense) d.valid = false;
-  c->tail_lf = -1;
-  for (auto& k : c->tail_host)
-    for (auto& h : k) h.clear();
+  for (auto& k : c->tail) k.reset();
   ++c->walls_version;
   return HBF_OK;
 }
@@ -503,9 +503,7 @@ int hbf_set_tail(hbf_ctx* c, int max_cells) {
   if (max_cells < 0) return fail(c, HBF_ERR_ARG, "negative tail size");
   if (max_cells != c->tail_cells) {
     c->tail_cells = max_cells;
-    c->tail_lf = -1;  // recomputed, and the tail records rebuilt, at the next cycle
-    for (auto& k : c->tail_host)
-      for (auto& h : k) h.clear();
+    for (auto& k : c->tail) k.reset();  // planned again, and the records rebuilt, at the next cycle
   }
   return HBF_OK;
 }

@@ -26,7 +26,25 @@ template <int D, typename T, int C>
 struct OpViscSmooth {
   using Arg = ViscArg<T>;
   static __device__ void apply(const Arg& a, int t, int col) {
-    k_visc_smooth_c_at<D, T, C, false>(a.x, a.b, a.ef[0], a.ef[1], a.ef[2], a.g, col, a.beta, a.hom, t);
+    visc_smooth_hom_at<D, T, C, false>(a.x, a.b, a.inv, a.ef, a.g, col, rn_mul(a.beta, g_ihh<T>(a.g)), t);
+  }
+};
+
+// the V-cycle's residual b - (x - beta L x), homogeneous walls
+template <int D, typename T>
+struct OpViscRes {
+  using Arg = ViscArg<T>;
+  static __device__ void apply(const Arg& a, int t, int) {
+    visc_res_hom_at<D, T, false>(a.x, a.b, a.out, a.ef, a.g, a.beta, t);
+  }
+};
+
+// the sweeps' reciprocals of a level
+template <int D, typename T>
+struct OpViscInv {
+  using Arg = ViscArg<T>;
+  static __device__ void apply(const Arg& a, int t, int) {
+    visc_inv_at<D, T, false>(a.inv, a.ef, a.g, rn_mul(a.beta, g_ihh<T>(a.g)), t);
   }
 };
 
@@ -224,7 +242,7 @@ __global__ void __launch_bounds__(128) k_batch_bottom(const BottomArg<T>* __rest
   if (c >= ncav || (mask && !mask[c])) return;
   const BottomArg<T>& a = args[c];
   if (a.level >= below) return;
-  bottom_block<D, T>(a);
+  bottom_block<D, T>(a, a.b, a.x);
 }
 
 // dense bottom operator of the viscous problem (it changes with eta and dt
@@ -440,6 +458,7 @@ struct LvView<double> {
   static double* vx(Level& L) { return L.vx; }
   static double* vb(Level& L) { return L.vb; }
   static double* vr(Level& L) { return L.vr; }
+  static double* vinv(Level& L) { return L.vinv; }
   static const double* ef(Level& L, int a) { return L.ef[a]; }
   static double* cx(Level& L) { return L.cx; }
   static double* cb(Level& L) { return L.cb; }
@@ -453,6 +472,7 @@ struct LvView<float> {
   static float* vx(Level& L) { return L.fvx; }
   static float* vb(Level& L) { return L.fvb; }
   static float* vr(Level& L) { return L.fvr; }
+  static float* vinv(Level& L) { return L.fvinv; }
   static const float* ef(Level& L, int a) { return L.fef[a]; }
   static float* cx(Level& L) { return L.fcx; }
   static float* cb(Level& L) { return L.fcb; }
@@ -474,8 +494,45 @@ struct Inst {
   void* re[kMaxLev] = {};  // restriction l -> l+1
   void* pr[kMaxLev] = {};  // prolongation l+1 -> l
   void* bot = nullptr;     // bottom solve
+  int ls = 0, nblk = 1;    // the fused tail's first solo level and cluster size
+  size_t smem = 0;
   Graph g;
 };
+
+// Solo levels, cluster size and shared memory of an instance's tail: the
+// finest level that is solo for every cavity, and the largest need of any
+template <int D, typename T, int KIND>
+static void plan_tail_kind(hbf_batch* B, Inst& I) {
+  const Geom* gs[kMaxLev];
+  const int lf = B->tail_level;
+  I.ls = lf;
+  for (int c = 0; c < B->ncav; ++c) {
+    const int L = B->nlev[c] - 1;
+    if (L < lf) continue;
+    for (int l = 0; l <= L; ++l) gs[l] = &B->cav[c]->lv[l].g;
+    I.ls = std::max(I.ls, tail_solo_level<D, T, KIND>(gs, lf, L, false));
+  }
+  I.smem = 0;
+  bool wide = false;
+  for (int c = 0; c < B->ncav; ++c) {
+    const int L = B->nlev[c] - 1;
+    if (L < lf) continue;
+    for (int l = 0; l <= L; ++l) gs[l] = &B->cav[c]->lv[l].g;
+    I.smem = std::max(I.smem, tail_smem<D, T, KIND>(gs, std::min(I.ls, L), L, false));
+    wide = wide || std::min(I.ls, L) > lf;
+  }
+  I.nblk = wide ? tail_blocks<D, T, KIND, false>(B->ncav, I.smem) : 1;
+}
+
+template <int D, typename T>
+static void plan_tail(hbf_batch* B, Inst& I) {
+  if (I.kind == kVisc)
+    plan_tail_kind<D, T, kVisc>(B, I);
+  else if (I.kind == kMac)
+    plan_tail_kind<D, T, kMac>(B, I);
+  else
+    plan_tail_kind<D, T, kNodal>(B, I);
+}
 
 template <int D, typename T>
 static void build_inst(hbf_batch* B, Inst& I, int kind, bool hom0, T* (*x0)(hbf_ctx*), T* (*b0)(hbf_ctx*)) {
@@ -505,6 +562,7 @@ static void build_inst(hbf_batch* B, Inst& I, int kind, bool hom0, T* (*x0)(hbf_
         a.x = X(c, l);
         a.b = Bv(c, l);
         a.out = R(c, l);
+        a.inv = V::vinv(L);
         for (int d = 0; d < 3; ++d) a.ef[d] = d < D ? V::ef(L, d) : nullptr;
         a.g = L.g;
         a.beta = (T)visc_beta(B->dt[q], c->rho, c->theta);
@@ -554,6 +612,7 @@ static void build_inst(hbf_batch* B, Inst& I, int kind, bool hom0, T* (*x0)(hbf_
     const int l = B->nlev[q] - 1;
     const Geom& g = c->lv[l].g;
     BottomArg<T> a;
+    std::memset(&a, 0, sizeof a);
     a.n = kind == kVisc ? D * g.ncell : kind == kMac ? g.ncell : g.nnode;
     a.m = kind == kVisc ? a.n : a.n + 1;
     a.Minv = c->dense[kind].Minv;
@@ -564,12 +623,9 @@ static void build_inst(hbf_batch* B, Inst& I, int kind, bool hom0, T* (*x0)(hbf_
     a.level = l;
     return a;
   });
-  for (int l = 0; l < kMaxLev; ++l) {
-    I.tail.lv[l] = I.lv[l];
-    I.tail.re[l] = I.re[l];
-    I.tail.pr[l] = I.pr[l];
-  }
+  for (int l = 0; l < kMaxLev; ++l) I.tail.lv[l] = I.lv[l];
   I.tail.bot = I.bot;
+  plan_tail<D, T>(B, I);
 }
 
 template <int D, typename T>
@@ -598,7 +654,7 @@ static void vcycle(hbf_batch* B, Inst& I, const int* mask) {
   for (int l = 0; l < top; ++l) {
     for (int s = 0; s < cfg.nu1; ++s) smooth<D, T>(B, I, l, mask);
     if (I.kind == kVisc) {
-      run<OpViscOp<D, T>>(B, I.lv[l], B->A[l][kCells], mask);
+      run<OpViscRes<D, T>>(B, I.lv[l], B->A[l][kCells], mask);
       run<OpRestrictCells<D, T>>(B, I.re[l], B->H[l + 1][kCellsD], mask);
     } else if (I.kind == kMac) {
       run<OpCellResid<D, T>>(B, I.lv[l], B->A[l][kCells], mask);
@@ -612,12 +668,11 @@ static void vcycle(hbf_batch* B, Inst& I, const int* mask) {
   ++B->nlaunch;
   if (lf < B->maxlev) {
     if (I.kind == kVisc)
-      k_vcycle_tail<D, T, kVisc, false><<<B->ncav, 256, 0, B->stream>>>(I.tail, lf, B->ncav, mask, cfg.nu1, cfg.nu2);
+      tail_launch<D, T, kVisc, false>(B->stream, I.tail, lf, I.ls, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
     else if (I.kind == kMac)
-      k_vcycle_tail<D, T, kMac, false><<<B->ncav, 256, 0, B->stream>>>(I.tail, lf, B->ncav, mask, cfg.nu1, cfg.nu2);
+      tail_launch<D, T, kMac, false>(B->stream, I.tail, lf, I.ls, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
     else
-      k_vcycle_tail<D, T, kNodal, false><<<B->ncav, 256, 0, B->stream>>>(I.tail, lf, B->ncav, mask, cfg.nu1,
-                                                                         cfg.nu2);
+      tail_launch<D, T, kNodal, false>(B->stream, I.tail, lf, I.ls, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
     ++B->nlaunch;
   }
   for (int l = top - 1; l >= 0; --l) {
@@ -882,6 +937,7 @@ struct SolversT : Solvers {
       run<OpRestrictFaces<D>>(B, facesR[l], B->H[l + 1][kFaces], B->mask_all);
     if (kMixed)
       for (int l = 0; l < B->maxlev; ++l) run<OpFacesF32>(B, facesF[l], B->H[l][kFaces], B->mask_all);
+    for (int l = 0; l < B->maxlev; ++l) run<OpViscInv<D, T>>(B, vph.lv[l], B->A[l][kCells], B->mask_all);
     k_batch_dense_build<D><<<dim3(kDenseMax, B->ncav), 128, 0, B->stream>>>((const DenseArg*)dense, B->ncav);
     k_batch_gauss_jordan<<<B->ncav, 256, 0, B->stream>>>((const DenseArg*)dense, B->ncav);
     B->nlaunch += 2;

@@ -346,9 +346,7 @@ int hbf_set_walls(hbf_ctx* c, const double wall_u[18]) {
   // solve for homogeneous errors); the fused tail records are rebuilt in
   // case the tail starts on the finest level
   c->lv[0].g = c->g;
-  c->tail_lf = -1;
-  for (auto& k : c->tail_host)
-    for (auto& h : k) h.clear();
+  for (auto& k : c->tail) k.reset();
   ++c->walls_version;
   return HBF_OK;
 }

@@ -16,6 +16,7 @@ struct Level {
   double* vx = nullptr;
   double* vb = nullptr;
   double* vr = nullptr;
+  double* vinv = nullptr;  // 1 / (1 + bs diag): the Gauss-Seidel reciprocals (hb_visc_hom.cuh)
   double* ef[3] = {nullptr, nullptr, nullptr};  // face eta
   // cell Poisson (MAC)
   double* cx = nullptr;
@@ -29,6 +30,7 @@ struct Level {
   float* fvx = nullptr;
   float* fvb = nullptr;
   float* fvr = nullptr;
+  float* fvinv = nullptr;
   float* fef[3] = {nullptr, nullptr, nullptr};
   float* feta = nullptr;  // level 0: the cell viscosity, whose face means the FP32 kernels form
   float* fvx2 = nullptr;  // level 0 in 3D: the second array of the fused red-black sweeps
@@ -82,6 +84,21 @@ struct Dense {
   double* Minv = nullptr;  // (kDenseMax+1)^2
   int n = 0;               // matrix size (unknowns, +1 when bordered)
   bool valid = false;
+};
+
+// the fused V-cycle tail of one problem kind: levels from lf on in one launch
+// (those from ls on by one block), its device argument records and their
+// staging copy
+struct TailPlan {
+  bool set = false;       // the plan below is up to date
+  bool on = false;        // there is a tail
+  bool uploaded = false;  // dev holds the records for beta and sweeps
+  int lf = 0, ls = 0, nblk = 1, sweeps = 0;
+  size_t smem = 0;
+  double beta = 0.0;
+  void* dev = nullptr;
+  std::vector<unsigned char> host;
+  void reset() { set = on = uploaded = false; }
 };
 
 struct SolverCfg {
@@ -176,12 +193,9 @@ struct hbf_ctx {
   hb::Prof prof;
   long long nlaunch = 0;
   hb::Dense dense[3];  // viscous, MAC, nodal
-  // fused V-cycle tail of the solves: levels >= tail_lf run in one block
-  int tail_lf = -1;                         // -1: not set up; >= levels: none
-  int tail_cells = 512;                     // the tail starts at the first level with at most this many cells
-  void* tail_dev[3][2] = {};                // device argument records [kind][FP32?]
-  std::vector<unsigned char> tail_host[3][2];
-  double tail_beta[2] = {0.0, 0.0};         // beta of the uploaded viscous records
+  // fused V-cycle tail of the solves
+  int tail_cells = -1;  // it starts at the first level with at most this many cells (-1: the library's rule)
+  hb::TailPlan tail[3]; // by problem kind
   double *dX = nullptr, *dM = nullptr, *dA = nullptr;  // build scratch
 };
 

@@ -18,6 +18,7 @@
 #include "hb_internal.h"
 #include "hb_mg_kernels.cuh"
 #include "hb_vcycle_tail.cuh"
+#include "hb_visc_hom.cuh"
 #include "hb_visc_fused.cuh"
 #include "hb_visc_split.cuh"
 #include "hb_visc_tma.cuh"
@@ -748,6 +749,7 @@ struct View<double> {
   static double* vx(Level& L) { return L.vx; }
   static double* vb(Level& L) { return L.vb; }
   static double* vr(Level& L) { return L.vr; }
+  static double* vinv(Level& L) { return L.vinv; }
   static double* ef(Level& L, int a) { return L.ef[a]; }
   static double* cx(Level& L) { return L.cx; }
   static double* cb(Level& L) { return L.cb; }
@@ -761,6 +763,7 @@ struct View<float> {
   static float* vx(Level& L) { return L.fvx; }
   static float* vb(Level& L) { return L.fvb; }
   static float* vr(Level& L) { return L.fvr; }
+  static float* vinv(Level& L) { return L.fvinv; }
   static float* ef(Level& L, int a) { return L.fef[a]; }
   static float* cx(Level& L) { return L.fcx; }
   static float* cb(Level& L) { return L.fcb; }
@@ -849,108 +852,141 @@ static void bottom_fp64(Problem<T>& P, int l, double* xd, double* bd, void (*run
 // back in one launch of one block, instead of about twenty launches per level
 // ---------------------------------------------------------------------------
 
-static int tail_level(hbf_ctx* c) {
-  if (c->tail_lf >= 0) return c->tail_lf;
+// the exact bottom solve of problem kind: at most kDenseMax unknowns on the
+// coarsest level
+static bool dense_bottom(const hbf_ctx* c, int kind) {
+  const Geom& g = c->lv.back().g;
+  return (kind == 0 ? (long long)c->dim * g.ncell : (long long)(kind == 1 ? g.ncell : g.nnode)) <= kDenseMax;
+}
+
+// The first level of the fused tail: the first one from level 1 on with at
+// most max_cells cells (hbf_set_tail), or, by default, small enough that a
+// cluster of 16 blocks takes a phase of it in less time than a launch over the
+// whole GPU does.
+template <int D, typename T>
+static int tail_level(const hbf_ctx* c) {
   const int nl = (int)c->lv.size();
-  const Geom& gb = c->lv[nl - 1].g;
-  const bool dense = (long long)c->dim * gb.ncell <= kDenseMax && gb.nnode <= kDenseMax;
-  int lf = nl;
-  if (dense)
-    for (int l = 1; l < nl; ++l)
-      if (c->lv[l].g.ncell <= c->tail_cells) {
-        lf = l;
-        break;
-      }
-  c->tail_lf = lf;
-  return lf;
+  const long long most = c->tail_cells >= 0 ? c->tail_cells : batch::tail_wide_cells<D, T>();
+  for (int l = 1; l < nl; ++l)
+    if (c->lv[l].g.ncell <= most) return l;
+  return nl;
 }
 
 template <typename T, typename A>
 struct TailBlock {
   A lv[batch::kMaxLev];
-  batch::XferArg<T> re[batch::kMaxLev];
-  batch::XferArg<T> pr[batch::kMaxLev];
   batch::BottomArg<T> bot;
 };
+
+// Levels, cluster size and shared memory of problem KIND's tail, and its
+// device records; made at the first cycle after a change (c->tail[..].set)
+template <int D, typename T, int KIND>
+static const TailPlan& tail_plan(hbf_ctx* c) {
+  using namespace batch;
+  TailPlan& P = c->tail[KIND];
+  if (P.set) return P;
+  using A = typename std::conditional<KIND == kVisc, ViscArg<T>, PoisArg<T>>::type;
+  using TB = TailBlock<T, A>;
+  const int nl = (int)c->lv.size(), L = nl - 1;
+  P.set = true;
+  P.on = false;
+  P.lf = tail_level<D, T>(c);
+  if (P.lf >= nl || nl > kMaxLev) return P;
+  const Geom* gs[kMaxLev];
+  for (int l = 0; l < nl; ++l) gs[l] = &c->lv[l].g;
+  const bool sweeps = !dense_bottom(c, KIND);
+  P.ls = tail_solo_level<D, T, KIND>(gs, P.lf, L, sweeps);
+  if (P.ls < 0) return P;
+  P.smem = tail_smem<D, T, KIND>(gs, P.ls, L, sweeps);
+  P.nblk = 1;
+  if (P.ls > P.lf)
+    P.nblk = any_per(c->g) ? tail_blocks<D, T, KIND, true>(1, P.smem) : tail_blocks<D, T, KIND, false>(1, P.smem);
+  if (!P.dev) {
+    void* d = nullptr;
+    if (cudaMalloc(&d, sizeof(TB)) != cudaSuccess) {
+      cudaGetLastError();
+      return P;  // level by level
+    }
+    c->allocs.push_back(d);
+    P.dev = d;
+  }
+  P.on = true;
+  P.uploaded = false;
+  return P;
+}
+
+// the tail of problem KIND starts at level l
+template <int D, typename T, int KIND>
+static bool tail_at(hbf_ctx* c, int l) {
+  const TailPlan& P = tail_plan<D, T, KIND>(c);
+  return P.on && P.lf == l;
+}
 
 template <int D, typename T, int KIND>
 static bool run_tail(hbf_ctx* c, int l, double beta) {
   using namespace batch;
-  const int lf = tail_level(c);
+  if (!tail_at<D, T, KIND>(c, l)) return false;
+  TailPlan& P = c->tail[KIND];
   const int nl = (int)c->lv.size(), L = nl - 1;
-  if (l != lf || lf >= nl || nl > kMaxLev) return false;
-  const int pi = sizeof(T) == 4 ? 1 : 0;
   using A = typename std::conditional<KIND == kVisc, ViscArg<T>, PoisArg<T>>::type;
   using TB = TailBlock<T, A>;
-  std::vector<unsigned char>& host = c->tail_host[KIND][pi];
-  void*& dev = c->tail_dev[KIND][pi];
-  const bool fresh = host.empty();
-  if (fresh) {
-    void* d = nullptr;
-    if (cudaMalloc(&d, sizeof(TB)) != cudaSuccess) return false;  // fall back to level-by-level
-    c->allocs.push_back(d);
-    dev = d;
-    host.assign(sizeof(TB), 0);
-  }
-  if (fresh || (KIND == kVisc && c->tail_beta[pi] != beta)) {
-    TB* h = (TB*)host.data();
-    auto X = [&](Level& Lv) -> T* { return KIND == kVisc ? View<T>::vx(Lv) : KIND == kMac ? View<T>::cx(Lv) : View<T>::nx(Lv); };
-    auto Bv = [&](Level& Lv) -> T* { return KIND == kVisc ? View<T>::vb(Lv) : KIND == kMac ? View<T>::cb(Lv) : View<T>::nb(Lv); };
-    auto R = [&](Level& Lv) -> T* { return KIND == kVisc ? View<T>::vr(Lv) : KIND == kMac ? View<T>::cr(Lv) : View<T>::nr(Lv); };
-    const int ncomp = KIND == kVisc ? D : 1, sign = KIND == kVisc ? -1 : 1;
-    for (int q = lf; q <= L; ++q) {
+  if (!P.uploaded || P.sweeps != c->cfg.nu_bottom || (KIND == kVisc && P.beta != beta)) {
+    P.host.assign(sizeof(TB), 0);
+    TB* h = (TB*)P.host.data();
+    for (int q = P.lf; q <= L; ++q) {
       Level& Lv = c->lv[q];
       A a;
       std::memset(&a, 0, sizeof a);
-      a.x = X(Lv);
-      a.b = Bv(Lv);
+      a.x = KIND == kVisc ? View<T>::vx(Lv) : KIND == kMac ? View<T>::cx(Lv) : View<T>::nx(Lv);
+      a.b = KIND == kVisc ? View<T>::vb(Lv) : KIND == kMac ? View<T>::cb(Lv) : View<T>::nb(Lv);
       a.g = Lv.g;
       if constexpr (KIND == kVisc) {
-        a.out = R(Lv);
+        a.out = View<T>::vr(Lv);
+        a.inv = View<T>::vinv(Lv);
         for (int d = 0; d < D; ++d) a.ef[d] = View<T>::ef(Lv, d);
         a.beta = (T)beta;
         a.hom = 1;
       } else {
-        a.r = R(Lv);
+        a.r = KIND == kMac ? View<T>::cr(Lv) : View<T>::nr(Lv);
       }
       h->lv[q] = a;
-      if (q < L) {
-        Level& Cv = c->lv[q + 1];
-        h->re[q] = XferArg<T>{R(Lv), Bv(Cv), X(Cv), Lv.g, Cv.g, ncomp, sign};
-        h->pr[q] = XferArg<T>{X(Cv), X(Lv), nullptr, Lv.g, Cv.g, ncomp, sign};
-      }
     }
     BottomArg<T> bt;
     std::memset(&bt, 0, sizeof bt);
-    const Geom& gb = c->lv[L].g;
+    const Level& Lb = c->lv[L];
+    const Geom& gb = Lb.g;
     bt.n = KIND == kVisc ? D * gb.ncell : KIND == kMac ? gb.ncell : gb.nnode;
     bt.m = KIND == kVisc ? bt.n : bt.n + 1;
-    bt.Minv = c->dense[KIND].Minv;
-    bt.x = X(c->lv[L]);
-    bt.b = Bv(c->lv[L]);
+    bt.Minv = dense_bottom(c, KIND) ? c->dense[KIND].Minv : nullptr;
+    bt.x = h->lv[L].x;
+    bt.b = const_cast<T*>(h->lv[L].b);
     bt.g = gb;
     bt.kind = KIND;
     bt.level = L;
+    bt.sweeps = c->cfg.nu_bottom;
+    for (int d = 0; d < D; ++d) bt.ef[d] = Lb.ef[d];
+    bt.inv = Lb.vinv;
+    bt.beta = beta;
     h->bot = bt;
     // pageable source: the call returns once the bytes are staged
-    if (cudaMemcpyAsync(dev, h, sizeof(TB), cudaMemcpyHostToDevice, c->stream) != cudaSuccess) return false;
-    if (KIND == kVisc) c->tail_beta[pi] = beta;
+    if (cudaMemcpyAsync(P.dev, h, sizeof(TB), cudaMemcpyHostToDevice, c->stream) != cudaSuccess) return false;
+    P.uploaded = true;
+    P.beta = beta;
+    P.sweeps = c->cfg.nu_bottom;
   }
-  ensure_dense(c, KIND, beta);  // the viscous inverse changes with eta and dt
-  TB* d = (TB*)dev;
+  if (dense_bottom(c, KIND)) ensure_dense(c, KIND, beta);  // the viscous inverse changes with eta and dt
+  TB* d = (TB*)P.dev;
   TailTabs tb;
-  for (int q = 0; q < kMaxLev; ++q) {
-    tb.lv[q] = &d->lv[q];
-    tb.re[q] = &d->re[q];
-    tb.pr[q] = &d->pr[q];
-  }
+  for (int q = 0; q < kMaxLev; ++q) tb.lv[q] = &d->lv[q];
   tb.bot = &d->bot;
+  const bool rec = prof_wants(c->prof, kSlotCoarse);
+  if (rec) prof_mark(c, kSlotCoarse, true);
   if (any_per(c->g))
-    launch(c, kSlotCoarse, k_vcycle_tail<D, T, KIND, true>, 1, kThreads, tb, lf, 1, (const int*)nullptr, c->cfg.nu1,
-           c->cfg.nu2);
+    tail_launch<D, T, KIND, true>(c->stream, tb, P.lf, P.ls, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
   else
-    launch(c, kSlotCoarse, k_vcycle_tail<D, T, KIND, false>, 1, kThreads, tb, lf, 1, (const int*)nullptr, c->cfg.nu1,
-           c->cfg.nu2);
+    tail_launch<D, T, KIND, false>(c->stream, tb, P.lf, P.ls, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
+  if (rec) prof_mark(c, kSlotCoarse, false);
+  ++c->nlaunch;
   return true;
 }
 
@@ -1025,27 +1061,33 @@ struct ViscProblem : Problem<T> {
                   (T)beta, hm);
       return;
     }
-    const T* e0 = View<T>::ef(L, 0);
-    const T* e1 = View<T>::ef(L, 1);
-    const T* e2 = View<T>::ef(L, 2);
+    any_per(c->g) ? smooth_hom<true>(l) : smooth_hom<false>(l);
+  }
+  // stored face viscosities: the branch-free sweep of hb_visc_hom.cuh (the
+  // V-cycles solve for errors, so the walls are homogeneous on every level)
+  template <bool PER>
+  void smooth_hom(int l) {
+    Level& L = c->lv[l];
+    const int slot = l == 0 ? kSlotViscSmooth : kSlotCoarse;
+    const int nt = rb_count<D>(L.g), th = spread_threads(nt), nb = (nt + th - 1) / th;
+    const T* ef[3] = {View<T>::ef(L, 0), View<T>::ef(L, 1), View<T>::ef(L, 2)};
+    const T bs = T(beta) * g_ihh<T>(L.g);
+    T* u = x(l);
+    const T *bb = b(l), *inv = View<T>::vinv(L);
     for (int col = 0; col < 2; ++col)
-      if (any_per(c->g))
-        launch3(c, slot, k_visc_smooth_c<D, T, 0, false, true>, grd, blk, x(l), (const T*)b(l), e0, e1, e2, L.g, col, (T)beta, hm);
-      else
-        launch3(c, slot, k_visc_smooth_c<D, T, 0, false, false>, grd, blk, x(l), (const T*)b(l), e0, e1, e2, L.g, col, (T)beta, hm);
+      launch(c, slot, k_visc_smooth_hom<D, T, 0, PER>, nb, th, u, bb, inv, ef[0], ef[1], ef[2], L.g, col, bs);
     for (int col = 0; col < 2; ++col)
-      if (any_per(c->g))
-        launch3(c, slot, k_visc_smooth_c<D, T, 1, false, true>, grd, blk, x(l), (const T*)b(l), e0, e1, e2, L.g, col, (T)beta, hm);
-      else
-        launch3(c, slot, k_visc_smooth_c<D, T, 1, false, false>, grd, blk, x(l), (const T*)b(l), e0, e1, e2, L.g, col, (T)beta, hm);
-    if (D == 3)
+      launch(c, slot, k_visc_smooth_hom<D, T, 1, PER>, nb, th, u, bb, inv, ef[0], ef[1], ef[2], L.g, col, bs);
+    if constexpr (D == 3)
       for (int col = 0; col < 2; ++col)
-        if (any_per(c->g))
-          launch3(c, slot, k_visc_smooth_c<D, T, 2, false, true>, grd, blk, x(l), (const T*)b(l), e0, e1, e2, L.g, col, (T)beta,
-                hm);
-        else
-          launch3(c, slot, k_visc_smooth_c<D, T, 2, false, false>, grd, blk, x(l), (const T*)b(l), e0, e1, e2, L.g, col, (T)beta,
-                hm);
+        launch(c, slot, k_visc_smooth_hom<D, T, 2, PER>, nb, th, u, bb, inv, ef[0], ef[1], ef[2], L.g, col, bs);
+  }
+  template <bool PER>
+  void resid_hom(int l) {
+    Level& L = c->lv[l];
+    const int th = spread_threads(L.g.ncell), nb = (L.g.ncell + th - 1) / th;
+    launch(c, l == 0 ? kSlotViscResid : kSlotCoarse, k_visc_res_hom<D, T, PER>, nb, th, (const T*)x(l), (const T*)b(l),
+           r(l), (const T*)View<T>::ef(L, 0), (const T*)View<T>::ef(L, 1), (const T*)View<T>::ef(L, 2), L.g, (T)beta);
   }
   // the FP32 finest level forms its face viscosities from the cell viscosity
   bool cell_eta(int l) const { return l == 0 && sizeof(T) == 4 && c->lv[0].feta != nullptr; }
@@ -1087,6 +1129,10 @@ struct ViscProblem : Problem<T> {
               L.g, (T)beta, (int)this->hom(l));
       return;
     }
+    if (this->hom(l)) {
+      any_per(c->g) ? resid_hom<true>(l) : resid_hom<false>(l);
+      return;
+    }
     if (any_per(c->g))
       launch3(c, l == 0 ? kSlotViscResid : kSlotCoarse, k_visc_op3<D, T, false, true>, grd, blk, (const T*)x(l), (const T*)b(l), r(l),
             (const T*)View<T>::ef(L, 0), (const T*)View<T>::ef(L, 1), (const T*)View<T>::ef(L, 2), L.g, (T)beta,
@@ -1103,7 +1149,8 @@ struct ViscProblem : Problem<T> {
       launch(c, kSlotTransfer, k_restrict_cells<D, T, true>, grid_for(n), kThreads, r(l), b(l + 1), F.g, C.g, D);
     else
       launch(c, kSlotTransfer, k_restrict_cells<D, T>, grid_for(n), kThreads, r(l), b(l + 1), F.g, C.g, D);
-    launch(c, kSlotTransfer, k_zero<T>, grid_for(n), kThreads, x(l + 1), n);
+    if (!tail_at<D, T, batch::kVisc>(c, l + 1))  // the tail zeroes its iterate itself
+      launch(c, kSlotTransfer, k_zero<T>, grid_for(n), kThreads, x(l + 1), n);
   }
   void prolong_add(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -1330,7 +1377,8 @@ struct MacProblem : Problem<T> {
   void restrict_to(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
     launch(c, kSlotTransfer, k_restrict_cells<D, T>, grid_for(C.g.ncell), kThreads, r(l), b(l + 1), F.g, C.g, 1);
-    launch(c, kSlotTransfer, k_zero<T>, grid_for(C.g.ncell), kThreads, x(l + 1), (long long)C.g.ncell);
+    if (!tail_at<D, T, batch::kMac>(c, l + 1))
+      launch(c, kSlotTransfer, k_zero<T>, grid_for(C.g.ncell), kThreads, x(l + 1), (long long)C.g.ncell);
   }
   void prolong_add(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -1405,7 +1453,8 @@ struct NodalProblem : Problem<T> {
       else
         launch(c, kSlotTransfer, k_restrict_nodes<D, T, false>, grid_for(C.g.nnode), kThreads, r(l), b(l + 1), F.g, C.g);
     }
-    launch(c, kSlotTransfer, k_zero<T>, grid_for(C.g.nnode), kThreads, x(l + 1), (long long)C.g.nnode);
+    if (!tail_at<D, T, batch::kNodal>(c, l + 1))
+      launch(c, kSlotTransfer, k_zero<T>, grid_for(C.g.nnode), kThreads, x(l + 1), (long long)C.g.nnode);
   }
   void prolong_add(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -1791,9 +1840,29 @@ static int solve_viscous_mixed(hbf_ctx* c, double beta, const double* b_in, doub
   return st;
 }
 
+// the Gauss-Seidel reciprocals of the V-cycles' levels (every level of the
+// FP64 cycles; the coarse levels of the FP32 ones, whose finest level reads
+// the cell viscosity; the coarsest level in FP64 too when it is swept)
+template <int D>
+static void build_inv_levels(hbf_ctx* c, double beta) {
+  const bool mixed = c->precision == HBF_MIXED;
+  const size_t nl = c->lv.size();
+  for (size_t l = mixed ? 1 : 0; l < nl; ++l) {
+    Level& L = c->lv[l];
+    const int th = spread_threads(L.g.ncell), nb = (L.g.ncell + th - 1) / th;
+    if (mixed)
+      launch(c, kSlotTransfer, k_visc_inv<D, float>, nb, th, L.fvinv, (const float*)L.fef[0], (const float*)L.fef[1],
+             (const float*)L.fef[2], L.g, (float)beta * L.g.fihh);
+    if (!mixed || (l + 1 == nl && !dense_bottom(c, 0)))
+      launch(c, kSlotTransfer, k_visc_inv<D, double>, nb, th, L.vinv, (const double*)L.ef[0], (const double*)L.ef[1],
+             (const double*)L.ef[2], L.g, beta * L.g.ihh);
+  }
+}
+
 template <int D>
 static int solve_viscous_d(hbf_ctx* c, double beta, const double* b_in, double* x, hbf_solve_stats* out) {
   build_eta_levels<D>(c);
+  build_inv_levels<D>(c, beta);
   c->dense[0].valid = false;  // new viscosity and dt: rebuild the bottom inverse
   if (c->precision == HBF_MIXED) return solve_viscous_mixed<D>(c, beta, b_in, x, out);
   const SolverCfg& cfg = c->cfg;
