@@ -26,7 +26,7 @@ template <int D, typename T, int C>
 struct OpViscSmooth {
   using Arg = ViscArg<T>;
   static __device__ void apply(const Arg& a, int t, int col) {
-    visc_smooth_hom_at<D, T, C, false>(a.x, a.b, a.inv, a.ef, a.g, col, rn_mul(a.beta, g_ihh<T>(a.g)), t);
+    visc_smooth_hom_at<D, T, false>(a.x, a.b, a.inv, a.ef, a.g, C, col, rn_mul(a.beta, g_ihh<T>(a.g)), t);
   }
 };
 
@@ -242,7 +242,8 @@ __global__ void __launch_bounds__(128) k_batch_bottom(const BottomArg<T>* __rest
   if (c >= ncav || (mask && !mask[c])) return;
   const BottomArg<T>& a = args[c];
   if (a.level >= below) return;
-  bottom_block<D, T>(a, a.b, a.x);
+  const int nc = a.kind == kVisc ? D : 1;
+  bottom_block<D, T>(a, a.b, a.x, a.n / nc, nc);
 }
 
 // dense bottom operator of the viscous problem (it changes with eta and dt
@@ -494,44 +495,52 @@ struct Inst {
   void* re[kMaxLev] = {};  // restriction l -> l+1
   void* pr[kMaxLev] = {};  // prolongation l+1 -> l
   void* bot = nullptr;     // bottom solve
-  int ls = 0, nblk = 1;    // the fused tail's first solo level and cluster size
+  int nblk = 1;            // the fused tail's cluster size and shared memory
   size_t smem = 0;
   Graph g;
 };
 
-// Solo levels, cluster size and shared memory of an instance's tail: the
-// finest level that is solo for every cavity, and the largest need of any
+// Cluster size of an instance's tail and the largest shared memory of any
+// cavity; false when a cavity's does not fit
 template <int D, typename T, int KIND>
-static void plan_tail_kind(hbf_batch* B, Inst& I) {
+static bool plan_tail_kind(hbf_batch* B, int lf, int& nblk, size_t& smem) {
   const Geom* gs[kMaxLev];
-  const int lf = B->tail_level;
-  I.ls = lf;
-  for (int c = 0; c < B->ncav; ++c) {
-    const int L = B->nlev[c] - 1;
-    if (L < lf) continue;
-    for (int l = 0; l <= L; ++l) gs[l] = &B->cav[c]->lv[l].g;
-    I.ls = std::max(I.ls, tail_solo_level<D, T, KIND>(gs, lf, L, false));
-  }
-  I.smem = 0;
   bool wide = false;
   for (int c = 0; c < B->ncav; ++c) {
     const int L = B->nlev[c] - 1;
+    for (int l = 0; l <= L; ++l) gs[l] = &B->cav[c]->lv[l].g;
+    wide = wide || (L >= lf && tail_has_wide<D, T, KIND>(gs, lf, L, false));
+  }
+  nblk = tail_blocks<D, T, KIND, false>(B->ncav, wide);
+  smem = 0;
+  if (nblk < 1) return false;
+  for (int c = 0; c < B->ncav; ++c) {
+    const int L = B->nlev[c] - 1;
     if (L < lf) continue;
     for (int l = 0; l <= L; ++l) gs[l] = &B->cav[c]->lv[l].g;
-    I.smem = std::max(I.smem, tail_smem<D, T, KIND>(gs, std::min(I.ls, L), L, false));
-    wide = wide || std::min(I.ls, L) > lf;
+    smem = std::max(smem, tail_smem<D, T, KIND>(gs, lf, L, nblk, false));
   }
-  I.nblk = wide ? tail_blocks<D, T, KIND, false>(B->ncav, I.smem) : 1;
+  return smem <= kTailSmem;
 }
 
 template <int D, typename T>
 static void plan_tail(hbf_batch* B, Inst& I) {
+  const int lf = B->tail_level;
   if (I.kind == kVisc)
-    plan_tail_kind<D, T, kVisc>(B, I);
+    plan_tail_kind<D, T, kVisc>(B, lf, I.nblk, I.smem);
   else if (I.kind == kMac)
-    plan_tail_kind<D, T, kMac>(B, I);
+    plan_tail_kind<D, T, kMac>(B, lf, I.nblk, I.smem);
   else
-    plan_tail_kind<D, T, kNodal>(B, I);
+    plan_tail_kind<D, T, kNodal>(B, lf, I.nblk, I.smem);
+}
+
+// the tail from level lf on fits in shared memory for every cavity and problem
+template <int D, typename T>
+static bool tail_fits(hbf_batch* B, int lf) {
+  int nblk;
+  size_t smem;
+  return plan_tail_kind<D, T, kVisc>(B, lf, nblk, smem) && plan_tail_kind<D, T, kMac>(B, lf, nblk, smem) &&
+         plan_tail_kind<D, T, kNodal>(B, lf, nblk, smem);
 }
 
 template <int D, typename T>
@@ -668,11 +677,11 @@ static void vcycle(hbf_batch* B, Inst& I, const int* mask) {
   ++B->nlaunch;
   if (lf < B->maxlev) {
     if (I.kind == kVisc)
-      tail_launch<D, T, kVisc, false>(B->stream, I.tail, lf, I.ls, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
+      tail_launch<D, T, kVisc, false>(B->stream, I.tail, lf, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
     else if (I.kind == kMac)
-      tail_launch<D, T, kMac, false>(B->stream, I.tail, lf, I.ls, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
+      tail_launch<D, T, kMac, false>(B->stream, I.tail, lf, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
     else
-      tail_launch<D, T, kNodal, false>(B->stream, I.tail, lf, I.ls, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
+      tail_launch<D, T, kNodal, false>(B->stream, I.tail, lf, B->ncav, mask, cfg.nu1, cfg.nu2, I.nblk, I.smem);
     ++B->nlaunch;
   }
   for (int l = top - 1; l >= 0; --l) {
@@ -1341,6 +1350,11 @@ int prepare(hbf_batch* B) {
         break;
       }
     }
+  const bool mixed = B->precision == HBF_MIXED;
+  while (B->tail_level < B->maxlev &&
+         !(B->dim == 2 ? (mixed ? tail_fits<2, float>(B, B->tail_level) : tail_fits<2, double>(B, B->tail_level))
+                       : (mixed ? tail_fits<3, float>(B, B->tail_level) : tail_fits<3, double>(B, B->tail_level))))
+    ++B->tail_level;
   int st = B->dim == 2 ? build_lists<2>(B) : build_lists<3>(B);
   if (st) return st;
   void* part = nullptr;

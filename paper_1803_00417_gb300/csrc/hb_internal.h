@@ -87,13 +87,13 @@ struct Dense {
 };
 
 // the fused V-cycle tail of one problem kind: levels from lf on in one launch
-// (those from ls on by one block), its device argument records and their
-// staging copy
+// of a cluster of nblk blocks, its device argument records and their staging
+// copy
 struct TailPlan {
   bool set = false;       // the plan below is up to date
   bool on = false;        // there is a tail
   bool uploaded = false;  // dev holds the records for beta and sweeps
-  int lf = 0, ls = 0, nblk = 1, sweeps = 0;
+  int lf = 0, nblk = 1, sweeps = 0;
   size_t smem = 0;
   double beta = 0.0;
   void* dev = nullptr;

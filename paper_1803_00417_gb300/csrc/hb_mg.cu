@@ -895,12 +895,12 @@ static const TailPlan& tail_plan(hbf_ctx* c) {
   const Geom* gs[kMaxLev];
   for (int l = 0; l < nl; ++l) gs[l] = &c->lv[l].g;
   const bool sweeps = !dense_bottom(c, KIND);
-  P.ls = tail_solo_level<D, T, KIND>(gs, P.lf, L, sweeps);
-  if (P.ls < 0) return P;
-  P.smem = tail_smem<D, T, KIND>(gs, P.ls, L, sweeps);
-  P.nblk = 1;
-  if (P.ls > P.lf)
-    P.nblk = any_per(c->g) ? tail_blocks<D, T, KIND, true>(1, P.smem) : tail_blocks<D, T, KIND, false>(1, P.smem);
+  const bool wide = tail_has_wide<D, T, KIND>(gs, P.lf, L, sweeps);
+  P.nblk = any_per(c->g) ? tail_blocks<D, T, KIND, true>(1, wide) : tail_blocks<D, T, KIND, false>(1, wide);
+  if (P.nblk < 1) return P;
+  // from the first level whose slabs fit in shared memory
+  while (P.lf <= L && (P.smem = tail_smem<D, T, KIND>(gs, P.lf, L, P.nblk, sweeps)) > kTailSmem) ++P.lf;
+  if (P.lf > L) return P;
   if (!P.dev) {
     void* d = nullptr;
     if (cudaMalloc(&d, sizeof(TB)) != cudaSuccess) {
@@ -982,9 +982,9 @@ static bool run_tail(hbf_ctx* c, int l, double beta) {
   const bool rec = prof_wants(c->prof, kSlotCoarse);
   if (rec) prof_mark(c, kSlotCoarse, true);
   if (any_per(c->g))
-    tail_launch<D, T, KIND, true>(c->stream, tb, P.lf, P.ls, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
+    tail_launch<D, T, KIND, true>(c->stream, tb, P.lf, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
   else
-    tail_launch<D, T, KIND, false>(c->stream, tb, P.lf, P.ls, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
+    tail_launch<D, T, KIND, false>(c->stream, tb, P.lf, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
   if (rec) prof_mark(c, kSlotCoarse, false);
   ++c->nlaunch;
   return true;

@@ -720,31 +720,67 @@ __global__ void k_visc_bottom(T* __restrict__ u, const T* __restrict__ b, const 
 // ---------------------------------------------------------------------------
 // cell-centred Poisson (MAC potential), Neumann walls
 // ---------------------------------------------------------------------------
-template <int D, typename T, bool PER = true>
-__host__ __device__ inline T cell_gs_point(const T* __restrict__ x, const T* __restrict__ b, const Geom& g,
-                                  const int* p) {
+// 1 / cnt of the existing face neighbours of a cell (D .. 2 D)
+template <int D, typename T>
+__host__ __device__ __forceinline__ T cell_inv_count(int cnt) {
+  return cnt == 2 * D ? T(1.0 / (2 * D)) : (cnt == 2 * D - 1 ? T(1.0 / (2 * D - 1)) : (cnt == 2 * D - 2 ? T(1.0 / (2 * D - 2)) : T(1) / T(cnt)));
+}
+
+// Gauss-Seidel value of the cell q points at: offsets om / op of the
+// neighbours along each axis, lo / hi whether they exist
+template <int D, typename T>
+__host__ __device__ __forceinline__ T cell_gs_value(const T* q, T bc, T hh, const int* om, const int* op,
+                                                    const bool* lo, const bool* hi) {
   T s = T(0);
   int cnt = 0;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
-    T lo = T(0), hi = T(0);
-    const bool pa = PER && g.per[a];
-    if (p[a] > 0 || pa) {
-      int q[3] = {p[0], p[1], p[2]};
-      q[a] = pa ? wrap_cell(q[a] - 1, g.n[a]) : q[a] - 1;
-      lo = x[cidx<D>(g, q[0], q[1], q[2])];
-      ++cnt;
-    }
-    if (p[a] < g.n[a] - 1 || pa) {
-      int q[3] = {p[0], p[1], p[2]};
-      q[a] = pa ? wrap_cell(q[a] + 1, g.n[a]) : q[a] + 1;
-      hi = x[cidx<D>(g, q[0], q[1], q[2])];
-      ++cnt;
-    }
-    s += lo + hi;
+    s += (lo[a] ? q[om[a]] : T(0)) + (hi[a] ? q[op[a]] : T(0));
+    cnt += (int)lo[a] + (int)hi[a];
   }
-  T hh = g_hh<T>(g);
-  return (s - hh * b[cidx<D>(g, p[0], p[1], p[2])]) / T(cnt);
+  return (s - hh * bc) * cell_inv_count<D, T>(cnt);
+}
+
+// b - L x at the cell q points at (differences first: they are small where x
+// is smooth, so the sum loses nothing)
+template <int D, typename T>
+__host__ __device__ __forceinline__ T cell_res_value(const T* q, T bc, T ihh, const int* om, const int* op,
+                                                     const bool* lo, const bool* hi) {
+  const T xc = q[0];
+  T acc = T(0);
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const T dlo = lo[a] ? xc - q[om[a]] : T(0), dhi = hi[a] ? q[op[a]] - xc : T(0);
+    acc += dhi - dlo;
+  }
+  return bc - acc * ihh;
+}
+
+// neighbours of cell p of a whole level
+template <int D, bool PER>
+struct CellNbr {
+  int om[D], op[D];
+  bool lo[D], hi[D];
+  __host__ __device__ __forceinline__ CellNbr(const Geom& g, const int* p) {
+    int s = 1;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const bool per = PER && g.per[a];
+      lo[a] = per || p[a] > 0;
+      hi[a] = per || p[a] < g.n[a] - 1;
+      om[a] = p[a] > 0 ? -s : (g.n[a] - 1) * s;
+      op[a] = p[a] < g.n[a] - 1 ? s : -(g.n[a] - 1) * s;
+      s *= g.n[a];
+    }
+  }
+};
+
+template <int D, typename T, bool PER = true>
+__host__ __device__ inline T cell_gs_point(const T* __restrict__ x, const T* __restrict__ b, const Geom& g,
+                                  const int* p) {
+  const int id = cidx<D>(g, p[0], p[1], p[2]);
+  const CellNbr<D, PER> nb(g, p);
+  return cell_gs_value<D, T>(x + id, b[id], g_hh<T>(g), nb.om, nb.op, nb.lo, nb.hi);
 }
 
 template <int D, typename T, bool PER = true>
@@ -764,28 +800,10 @@ __global__ void k_cell_smooth(T* __restrict__ x, const T* __restrict__ b, const 
 
 template <int D, typename T, bool PER = true>
 __host__ __device__ __forceinline__ void k_cell_resid_at(const T* __restrict__ x, const T* __restrict__ b, T* __restrict__ r, const Geom& g, int t) {
-  const T ih = g_ih<T>(g);
   int p[3];
   cell_coords<D>(g, t, p[0], p[1], p[2]);
-  T xc = x[t];
-  T acc = T(0);
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    T glo = T(0), ghi = T(0);
-    const bool pa = PER && g.per[a];
-    if (p[a] > 0 || pa) {
-      int q[3] = {p[0], p[1], p[2]};
-      q[a] = pa ? wrap_cell(q[a] - 1, g.n[a]) : q[a] - 1;
-      glo = (xc - x[cidx<D>(g, q[0], q[1], q[2])]) * ih;
-    }
-    if (p[a] < g.n[a] - 1 || pa) {
-      int q[3] = {p[0], p[1], p[2]};
-      q[a] = pa ? wrap_cell(q[a] + 1, g.n[a]) : q[a] + 1;
-      ghi = (x[cidx<D>(g, q[0], q[1], q[2])] - xc) * ih;
-    }
-    acc += (ghi - glo) * ih;
-  }
-  r[t] = b[t] - acc;
+  const CellNbr<D, PER> nb(g, p);
+  r[t] = cell_res_value<D, T>(x + t, b[t], g_ihh<T>(g), nb.om, nb.op, nb.lo, nb.hi);
 }
 
 template <int D, typename T, bool PER = true>
@@ -812,40 +830,50 @@ __global__ void k_cell_bottom(T* __restrict__ x, const T* __restrict__ b, const 
 // ---------------------------------------------------------------------------
 // nodal FE Poisson, Neumann walls
 // ---------------------------------------------------------------------------
-// stencil weight (times h^2) of offset o in {-1,0,1}^D
-template <int D, typename T>
-__host__ __device__ inline T fe_weight(int nz) {
-  if (nz == 0) return T(-8.0 / 3.0);
-  if (D == 2) return T(1.0 / 3.0);
-  return nz == 1 ? T(0) : (nz == 2 ? T(1.0 / 6.0) : T(1.0 / 12.0));
-}
-
 // The kernels below take PER = false for a level with walls on every axis
 // (the periodic wraps compile out; the code is then the plain reflection
 // form) and PER = true otherwise.
+// The stencil's sum by planes: with A the sum of the four face neighbours and
+// C of the four diagonal neighbours of a node in its plane, the 3D stencil is
+// (C(z) + A(z - 1) + A(z + 1)) / 6 + (C(z - 1) + C(z + 1)) / 12 - 8/3 x, the 2D
+// one (A + C) / 3 - 8/3 x: additions in a shallow tree with one product per
+// weight instead of a chain of 20 (8) multiply-adds (a phase of a small level
+// is one chain long: its nodal sweeps went from 2.5 to 1.0 us per colour).
+// q points at the node; om / op: the neighbours below and above on each axis.
+template <int D, typename T>
+__host__ __device__ __forceinline__ T nodal_nbr_sum(const T* q, const int* om, const int* op) {
+  auto face4 = [&](const T* c) { return (c[om[0]] + c[op[0]]) + (c[om[1]] + c[op[1]]); };
+  auto diag4 = [&](const T* c) {
+    const T *lo = c + om[1], *hi = c + op[1];
+    return (lo[om[0]] + lo[op[0]]) + (hi[om[0]] + hi[op[0]]);
+  };
+  if constexpr (D == 2) {
+    return T(1.0 / 3.0) * (face4(q) + diag4(q));
+  } else {
+    const T *lo = q + om[2], *hi = q + op[2];
+    return T(1.0 / 6.0) * (diag4(q) + (face4(lo) + face4(hi))) + T(1.0 / 12.0) * (diag4(lo) + diag4(hi));
+  }
+}
+
+// offsets of the neighbours of node position q of 0 .. n along an axis of
+// stride s: wrapped on a periodic axis (node n is the copy of node 0),
+// reflected at a wall
+__host__ __device__ __forceinline__ void node_offsets(int q, int n, int s, bool per, int& om, int& op) {
+  om = q == 0 ? (per ? (n - 1) * s : s) : -s;
+  op = q == n ? (per ? -(n - 1) * s : -s) : s;
+}
+
 template <int D, typename T, bool PER = true>
 __host__ __device__ inline T nodal_lap_point(const T* __restrict__ x, const Geom& g, const int* p, bool skip_centre) {
-  T s = T(0);
-  const int K = D == 3 ? 27 : 9;
+  int om[3], op[3], s = 1;
 #pragma unroll
-  for (int o = 0; o < K; ++o) {
-    int oo[3];
-    if (D == 3) {
-      oo[0] = o / 9 - 1;
-      oo[1] = (o / 3) % 3 - 1;
-      oo[2] = o % 3 - 1;
-    } else {
-      oo[0] = o / 3 - 1;
-      oo[1] = o % 3 - 1;
-      oo[2] = 0;
-    }
-    int nz = (oo[0] != 0) + (oo[1] != 0) + (oo[2] != 0);
-    if (nz == 0 && skip_centre) continue;
-    if (D == 3 && nz == 1) continue;
-    T w = fe_weight<D, T>(nz);
-    s += w * ndget<D, T, PER>(x, g, p[0] + oo[0], p[1] + oo[1], p[2] + oo[2]);
+  for (int a = 0; a < D; ++a) {
+    node_offsets(p[a], g.n[a], s, PER && g.per[a], om[a], op[a]);
+    s *= g.n[a] + 1;
   }
-  return s;
+  const T* q = x + nidx(g, p[0], p[1], p[2]);
+  const T sum = nodal_nbr_sum<D, T>(q, om, op);
+  return skip_centre ? sum : sum - T(8.0 / 3.0) * q[0];
 }
 
 template <int D>
@@ -940,31 +968,34 @@ __global__ void k_nodal_bottom(T* __restrict__ x, const T* __restrict__ b, const
 // ---------------------------------------------------------------------------
 // mean of the 2^D children, averaged axis by axis (x, then y, then z)
 template <int D, typename T, bool SP = false>
-__host__ __device__ __forceinline__ void k_restrict_cells_at(const T* __restrict__ f, T* __restrict__ c, const Geom& gf, const Geom& gc, int ncomp, long long tt) {
-  
-    int comp = 0;
-    int t = (int)tt;
-    while (t >= gc.ncell) {
-      t -= gc.ncell;
-      ++comp;
+__host__ __device__ __forceinline__ T restrict_cell_value(const T* fc, const Geom& gf, int I, int J, int K) {
+  T v[2][2];
+  for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk)
+    for (int jj = 0; jj < 2; ++jj) {
+      int j = 2 * J + jj, k = D == 3 ? 2 * K + kk : 0;
+      v[kk][jj] = T(0.5) * (fc[lidx<D, SP>(gf, 2 * I, j, k)] + fc[lidx<D, SP>(gf, 2 * I + 1, j, k)]);
     }
-    int I, J, K;
-    cell_coords<D>(gc, t, I, J, K);
-    const T* fc = f + (size_t)comp * gf.ncell;
-    T v[2][2];
-    for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk)
-      for (int jj = 0; jj < 2; ++jj) {
-        int j = 2 * J + jj, k = D == 3 ? 2 * K + kk : 0;
-        v[kk][jj] = T(0.5) * (fc[lidx<D, SP>(gf, 2 * I, j, k)] + fc[lidx<D, SP>(gf, 2 * I + 1, j, k)]);
-      }
-    T w0 = T(0.5) * (v[0][0] + v[0][1]);
-    T out = w0;
-    if (D == 3) {
-      T w1 = T(0.5) * (v[1][0] + v[1][1]);
-      out = T(0.5) * (w0 + w1);
-    }
-    c[(size_t)comp * gc.ncell + t] = out;
+  T w0 = T(0.5) * (v[0][0] + v[0][1]);
+  T out = w0;
+  if (D == 3) {
+    T w1 = T(0.5) * (v[1][0] + v[1][1]);
+    out = T(0.5) * (w0 + w1);
   }
+  return out;
+}
+
+template <int D, typename T, bool SP = false>
+__host__ __device__ __forceinline__ void k_restrict_cells_at(const T* __restrict__ f, T* __restrict__ c, const Geom& gf, const Geom& gc, int ncomp, long long tt) {
+  int comp = 0;
+  int t = (int)tt;
+  while (t >= gc.ncell) {
+    t -= gc.ncell;
+    ++comp;
+  }
+  int I, J, K;
+  cell_coords<D>(gc, t, I, J, K);
+  c[(size_t)comp * gc.ncell + t] = restrict_cell_value<D, T, SP>(f + (size_t)comp * gf.ncell, gf, I, J, K);
+}
 
 template <int D, typename T, bool SP = false>
 __global__ void k_restrict_cells(const T* __restrict__ f, T* __restrict__ c, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc, int ncomp) {
@@ -1036,38 +1067,43 @@ __host__ __device__ inline T cget_refl(const T* __restrict__ e, const Geom& g, i
   return s * e[cidx<D>(g, i, j, k)];
 }
 
-// x_f += P e_c, cell-centred multilinear (3/4, 1/4 per axis), axis by axis
+// P e_c at fine cell (i, j, k), cell-centred multilinear (3/4, 1/4 per axis),
+// axis by axis
+template <int D, typename T, bool PER = true>
+__host__ __device__ __forceinline__ T prolong_cell_value(const T* e, const Geom& gc, int i, int j, int k, T sign) {
+  int I = i >> 1, J = j >> 1, K = k >> 1;
+  int In = (i & 1) ? I + 1 : I - 1;
+  int Jn = (j & 1) ? J + 1 : J - 1;
+  int Kn = (k & 1) ? K + 1 : K - 1;
+  T tz[2];
+  for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk) {
+    int kc = kk ? Kn : K;
+    T ty[2];
+    for (int jj = 0; jj < 2; ++jj) {
+      int jc = jj ? Jn : J;
+      ty[jj] = T(0.75) * cget_refl<D, T, PER>(e, gc, I, jc, kc, sign) +
+               T(0.25) * cget_refl<D, T, PER>(e, gc, In, jc, kc, sign);
+    }
+    tz[kk] = T(0.75) * ty[0] + T(0.25) * ty[1];
+  }
+  return D == 3 ? T(0.75) * tz[0] + T(0.25) * tz[1] : tz[0];
+}
+
+// x_f += P e_c
 template <int D, typename T, bool PER = true>
 __host__ __device__ __forceinline__ void k_prolong_cells_add_at(T* __restrict__ xf, const T* __restrict__ ec, const Geom& gf, const Geom& gc,
                                     int ncomp, T sign, long long tt) {
-  
-    int comp = 0;
-    int t = (int)tt;
-    while (t >= gf.ncell) {
-      t -= gf.ncell;
-      ++comp;
-    }
-    int i, j, k;
-    cell_coords<D>(gf, t, i, j, k);
-    const T* e = ec + (size_t)comp * gc.ncell;
-    int I = i >> 1, J = j >> 1, K = k >> 1;
-    int In = (i & 1) ? I + 1 : I - 1;
-    int Jn = (j & 1) ? J + 1 : J - 1;
-    int Kn = (k & 1) ? K + 1 : K - 1;
-    T tz[2];
-    for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk) {
-      int kc = kk ? Kn : K;
-      T ty[2];
-      for (int jj = 0; jj < 2; ++jj) {
-        int jc = jj ? Jn : J;
-        ty[jj] = T(0.75) * cget_refl<D, T, PER>(e, gc, I, jc, kc, sign) +
-                 T(0.25) * cget_refl<D, T, PER>(e, gc, In, jc, kc, sign);
-      }
-      tz[kk] = T(0.75) * ty[0] + T(0.25) * ty[1];
-    }
-    T v = D == 3 ? T(0.75) * tz[0] + T(0.25) * tz[1] : tz[0];
-    xf[(size_t)comp * gf.ncell + t] += v;
+  (void)ncomp;
+  int comp = 0;
+  int t = (int)tt;
+  while (t >= gf.ncell) {
+    t -= gf.ncell;
+    ++comp;
   }
+  int i, j, k;
+  cell_coords<D>(gf, t, i, j, k);
+  xf[(size_t)comp * gf.ncell + t] += prolong_cell_value<D, T, PER>(ec + (size_t)comp * gc.ncell, gc, i, j, k, sign);
+}
 
 template <int D, typename T, bool PER = true>
 __global__ void k_prolong_cells_add(T* __restrict__ xf, const T* __restrict__ ec, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
@@ -1168,27 +1204,31 @@ __global__ void k_prolong_cells_add_c(T* __restrict__ xf, const T* __restrict__ 
     k_prolong_cells_add_c_at<D, T, PER, SP>(xf, ec, gf, gc, sign, tt);
 }
 
-// full weighting onto coarse nodes (even reflection), axis by axis
+// full weighting onto coarse node (I, J, K) (even reflection), axis by axis
+template <int D, typename T, bool PER = true>
+__host__ __device__ __forceinline__ T restrict_node_value(const T* rf, const Geom& gf, int I, int J, int K) {
+  T zr[3];
+  for (int kk = 0; kk < (D == 3 ? 3 : 1); ++kk) {
+    int k = D == 3 ? 2 * K + kk - 1 : 0;
+    T yr[3];
+    for (int jj = 0; jj < 3; ++jj) {
+      int j = 2 * J + jj - 1;
+      T cen = ndget<D, T, PER>(rf, gf, 2 * I, j, k);
+      T lo = ndget<D, T, PER>(rf, gf, 2 * I - 1, j, k);
+      T hi = ndget<D, T, PER>(rf, gf, 2 * I + 1, j, k);
+      yr[jj] = T(0.5) * cen + T(0.25) * (lo + hi);
+    }
+    zr[kk] = T(0.5) * yr[1] + T(0.25) * (yr[0] + yr[2]);
+  }
+  return D == 3 ? T(0.5) * zr[1] + T(0.25) * (zr[0] + zr[2]) : zr[0];
+}
+
 template <int D, typename T, bool PER = true>
 __host__ __device__ __forceinline__ void k_restrict_nodes_at(const T* __restrict__ rf, T* __restrict__ rc, const Geom& gf, const Geom& gc, int t) {
-  
-    int I, J, K;
-    node_coords(gc, t, I, J, K);
-    T zr[3];
-    for (int kk = 0; kk < (D == 3 ? 3 : 1); ++kk) {
-      int k = D == 3 ? 2 * K + kk - 1 : 0;
-      T yr[3];
-      for (int jj = 0; jj < 3; ++jj) {
-        int j = 2 * J + jj - 1;
-        T cen = ndget<D, T, PER>(rf, gf, 2 * I, j, k);
-        T lo = ndget<D, T, PER>(rf, gf, 2 * I - 1, j, k);
-        T hi = ndget<D, T, PER>(rf, gf, 2 * I + 1, j, k);
-        yr[jj] = T(0.5) * cen + T(0.25) * (lo + hi);
-      }
-      zr[kk] = T(0.5) * yr[1] + T(0.25) * (yr[0] + yr[2]);
-    }
-    rc[t] = D == 3 ? T(0.5) * zr[1] + T(0.25) * (zr[0] + zr[2]) : zr[0];
-  }
+  int I, J, K;
+  node_coords(gc, t, I, J, K);
+  rc[t] = restrict_node_value<D, T, PER>(rf, gf, I, J, K);
+}
 
 template <int D, typename T, bool PER = true>
 __global__ void k_restrict_nodes(const T* __restrict__ rf, T* __restrict__ rc, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc) {
@@ -1197,35 +1237,39 @@ __global__ void k_restrict_nodes(const T* __restrict__ rf, T* __restrict__ rc, c
   }
 }
 
-// x_f += P e_c, nodal multilinear, axis by axis
+// P e_c at fine node (i, j, k), nodal multilinear, axis by axis
 template <int D, typename T>
-__host__ __device__ __forceinline__ void k_prolong_nodes_add_at(T* __restrict__ xf, const T* __restrict__ ec, const Geom& gf, const Geom& gc, int t) {
-  
-    int i, j, k;
-    node_coords(gf, t, i, j, k);
-    int I = i >> 1, J = j >> 1, K = k >> 1;
-    T tz[2];
-    for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk) {
-      int kc = K + kk;
-      if (D == 3 && kk == 1 && !(k & 1)) {
-        tz[1] = T(0);
+__host__ __device__ __forceinline__ T prolong_node_value(const T* ec, const Geom& gc, int i, int j, int k) {
+  int I = i >> 1, J = j >> 1, K = k >> 1;
+  T tz[2];
+  for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk) {
+    int kc = K + kk;
+    if (D == 3 && kk == 1 && !(k & 1)) {
+      tz[1] = T(0);
+      continue;
+    }
+    T ty[2];
+    for (int jj = 0; jj < 2; ++jj) {
+      int jc = J + jj;
+      if (jj == 1 && !(j & 1)) {
+        ty[1] = T(0);
         continue;
       }
-      T ty[2];
-      for (int jj = 0; jj < 2; ++jj) {
-        int jc = J + jj;
-        if (jj == 1 && !(j & 1)) {
-          ty[1] = T(0);
-          continue;
-        }
-        T a0 = ec[nidx(gc, I, jc, D == 3 ? kc : 0)];
-        ty[jj] = (i & 1) ? T(0.5) * (a0 + ec[nidx(gc, I + 1, jc, D == 3 ? kc : 0)]) : a0;
-      }
-      tz[kk] = (j & 1) ? T(0.5) * (ty[0] + ty[1]) : ty[0];
+      T a0 = ec[nidx(gc, I, jc, D == 3 ? kc : 0)];
+      ty[jj] = (i & 1) ? T(0.5) * (a0 + ec[nidx(gc, I + 1, jc, D == 3 ? kc : 0)]) : a0;
     }
-    T v = (D == 3 && (k & 1)) ? T(0.5) * (tz[0] + tz[1]) : tz[0];
-    xf[t] += v;
+    tz[kk] = (j & 1) ? T(0.5) * (ty[0] + ty[1]) : ty[0];
   }
+  return (D == 3 && (k & 1)) ? T(0.5) * (tz[0] + tz[1]) : tz[0];
+}
+
+// x_f += P e_c
+template <int D, typename T>
+__host__ __device__ __forceinline__ void k_prolong_nodes_add_at(T* __restrict__ xf, const T* __restrict__ ec, const Geom& gf, const Geom& gc, int t) {
+  int i, j, k;
+  node_coords(gf, t, i, j, k);
+  xf[t] += prolong_node_value<D, T>(ec, gc, i, j, k);
+}
 
 template <int D, typename T>
 __global__ void k_prolong_nodes_add(T* __restrict__ xf, const T* __restrict__ ec, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc) {

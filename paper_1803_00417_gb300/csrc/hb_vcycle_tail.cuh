@@ -93,9 +93,10 @@ __device__ inline void bottom_sub_mean(double* v, int n, int kind, const Geom& g
 }
 
 // exact solve of one cavity's coarsest level by the whole block, from b into
-// x: the rows of the inverse one per warp
+// x (unknown i of its component's n at x[i + (cs - n) * component]): the rows
+// of the inverse one per warp
 template <int D, typename T>
-__device__ void bottom_block(const BottomArg<T>& a, const T* b, T* x) {
+__device__ void bottom_block(const BottomArg<T>& a, const T* b, T* x, int cs, int nc) {
   __shared__ double sb[kDenseMax + 1];
   __shared__ double sx[kDenseMax + 1];
   __shared__ double sh[33];
@@ -111,7 +112,8 @@ __device__ void bottom_block(const BottomArg<T>& a, const T* b, T* x) {
   }
   __syncthreads();
   if (a.kind != kVisc) bottom_sub_mean<D>(sx, a.n, a.kind, a.g, sh);
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x) x[i] = (T)sx[i];
+  const int m = a.n / nc;
+  for (int i = threadIdx.x; i < a.n; i += blockDim.x) x[i % m + (i / m) * cs] = (T)sx[i];
   __syncthreads();
 }
 
@@ -126,133 +128,557 @@ struct TailTabs {
 // ---------------------------------------------------------------------------
 // One cluster per cavity runs every level from lf down to the cavity's
 // coarsest and back in one launch.  A V(2,2) cycle is a chain of about 28
-// dependent phases per level; launched one by one a phase of a small level
-// costs 3 to 7 us (launch, drain, and in FP64 two operations per SM and cycle
-// on the few SMs its blocks reach) for well under 1 us of work.  Two forms of
-// a phase, by level:
-//   wide  (lf <= l < ls): every block of the cluster takes part, the arrays
-//         stay in global memory (L2), barrier.cluster between the phases (its
-//         release / acquire makes the blocks' writes visible to each other);
-//         up to 16 SMs share a level's FP64 work.
-//   solo  (l >= ls): block 0 alone, the level's arrays in shared memory,
-//         __syncthreads between the phases.
+// dependent phases per level (11 to 35 by problem); launched one by one a
+// phase of a small level costs 3 to 7 us (launch, drain, and in FP64 two
+// operations per SM and cycle on the few SMs its blocks reach) for well under
+// 1 us of work.  Each level is cut into slabs of whole planes along its
+// slowest axis, one slab per block, held in that block's shared memory with a
+// halo plane on either side (x, b, and for the viscous problem the
+// reciprocals and the face viscosities).  A thread that updates a point of a
+// slab's first or last plane also writes it into the neighbouring block's halo
+// (distributed shared memory), so a sweep's loads are all local, and
+// barrier.cluster ends the phase.  Levels with at most tail_solo_points points
+// take one slab: block 0 alone, with __syncthreads.  Residuals and corrections
+// that cross slabs between levels go through the levels' global arrays (L2).
 // The operations and their order are those of the level-by-level launches.
+constexpr int kTailThreads = 512;
+
+// points of a level that one block takes alone: a phase is then one block
+// barrier (about 40 cycles) instead of a cluster's, worth the wider split only
+// when a phase has more work than the barrier costs; FP64 issues 2 operations
+// per SM and cycle, so it splits early
+template <int D, typename T>
+constexpr int tail_solo_points() {
+  return sizeof(T) == 4 ? (D == 3 ? 512 : 1024) : 64;
+}
+
+// A level as a block of the cluster holds it.  Slab r takes the planes [r rp,
+// (r + 1) rp) of the N planes of ps points along the slowest axis; offsets are
+// bytes of the dynamic shared memory.
 template <typename T>
-struct TailView {
-  T *x, *r;
-  const T *b, *inv;
-  const T* ef[3];
+struct TailLevel {
+  int N, ps, rp, np;  // np: slabs; 1: block 0 alone
+  int k0, k1;         // this block's planes (empty past the last slab)
+  int cs;             // x: component stride, (rp + 2) ps; plane k0 at ps
+  unsigned x, b, inv, ef[3];
+  T *gx, *gr;         // global arrays
+  const T *gb, *ginv;
+  const T* gef[3];
 };
 
-template <typename T>
-constexpr int tail_threads() {
-  return sizeof(T) == 4 ? 1024 : 256;
-}
-
-struct SyncSolo {
-  __device__ __forceinline__ void operator()() const { __syncthreads(); }
-};
-struct SyncWide {
-  __device__ __forceinline__ void operator()() const {
-    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
-  }
-};
-
-template <int D, typename T, int KIND>
-__host__ __device__ __forceinline__ int tail_points(const Geom& g) {
-  return KIND == kNodal ? g.nnode : g.ncell;
-}
-
-// shared memory of one solo level: x and b, for the viscous problem also the
-// reciprocals and the face viscosities
-template <int D, typename T, int KIND>
-__host__ __device__ inline size_t tail_level_bytes(const Geom& g) {
-  size_t e = 2 * (size_t)tail_points<D, T, KIND>(g);
-  if (KIND == kVisc) e = 3 * (size_t)D * g.ncell + g.nface[0] + g.nface[1] + (D == 3 ? g.nface[2] : 0);
-  return (e * sizeof(T) + 15) / 16 * 16;
-}
-
-// FP64 copies of the coarsest level for its Gauss-Seidel sweeps (no exact
-// inverse): laid out as a solo level of FP64
 template <int D, int KIND>
-__host__ __device__ inline size_t tail_bottom_bytes(const Geom& g) {
-  return tail_level_bytes<D, double, KIND>(g);
+__host__ __device__ inline void tail_planes(const Geom& g, int& N, int& ps) {
+  const int e = KIND == kNodal ? 1 : 0;
+  N = g.n[D - 1] + e;
+  ps = (g.n[0] + e) * (D == 3 ? g.n[1] + e : 1);
 }
 
-template <int D, typename T, int C, bool PER, class S>
-__device__ __forceinline__ void tail_visc_colours(const TailView<T>& v, const Geom& g, T bs, int tid, int nth, S sync) {
-  const int nt = rb_count<D>(g);
-  for (int col = 0; col < 2; ++col) {
-    for (int t = tid; t < nt; t += nth) visc_smooth_hom_at<D, T, C, PER>(v.x, v.b, v.inv, v.ef, g, col, bs, t);
-    sync();
+// planes per slab of a level shared by nblk blocks (arithmetic T).  Points
+// fall from level to level, so past the first one-slab level every level is
+// one; a swept coarsest level, whose FP64 slabs would split earlier, is one
+// too when the level above it is (solo), and always for a singular problem,
+// whose means block 0 takes alone.
+template <int D, typename T, int KIND>
+__host__ __device__ inline int tail_rows(const Geom& g, int nblk, bool solo = false) {
+  int N, ps;
+  tail_planes<D, KIND>(g, N, ps);
+  if (N * ps <= tail_solo_points<D, T>() || solo) return N;
+  return (N + nblk - 1) / nblk;
+}
+
+// the swept coarsest level L is one slab (up: the level above it, null when
+// the tail starts on L)
+template <int D, typename T, int KIND>
+__host__ __device__ inline bool tail_swept_solo(const Geom* up, int nblk) {
+  if (KIND != kVisc) return true;
+  if (!up) return false;
+  int N, ps;
+  tail_planes<D, KIND>(*up, N, ps);
+  return tail_rows<D, T, KIND>(*up, nblk) == N;
+}
+
+// shared memory of a slab of rp planes: x with its halo, b, and for the
+// viscous problem the reciprocals and the face viscosities (fills o when not
+// null)
+template <int D, typename T, int KIND>
+__host__ __device__ inline unsigned tail_slab_bytes(const Geom& g, int rp, unsigned at, TailLevel<T>* o) {
+  int N, ps;
+  tail_planes<D, KIND>(g, N, ps);
+  const unsigned NC = KIND == kVisc ? D : 1;
+  unsigned q = at;
+  auto take = [&](unsigned count) {
+    const unsigned r = q;
+    q += (count * (unsigned)sizeof(T) + 15) / 16 * 16;
+    return r;
+  };
+  const unsigned ox = take(NC * (rp + 2) * ps), ob = take(NC * rp * ps);
+  unsigned oi = 0, oe[3] = {0, 0, 0};
+  if (KIND == kVisc) {
+    oi = take(NC * rp * ps);
+    oe[0] = take(rp * (g.n[0] + 1) * (D == 3 ? g.n[1] : 1));
+    if (D == 3) oe[1] = take(rp * g.n[0] * (g.n[1] + 1));
+    oe[D - 1] = take((rp + 1) * ps);
+  }
+  if (o) {
+    o->x = ox;
+    o->b = ob;
+    o->inv = oi;
+    for (int a = 0; a < 3; ++a) o->ef[a] = oe[a];
+  }
+  return q - at;
+}
+
+// v into block r's shared memory at p's place in this block's
+__device__ __forceinline__ void st_block(float* p, unsigned r, float v) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), q;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(q) : "r"(a), "r"(r));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(q), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_block(double* p, unsigned r, double v) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), q;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(q) : "r"(a), "r"(r));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(q), "d"(v) : "memory");
+}
+
+// x of component c at point q of plane k = v, and the copies in the halos of
+// the slabs that border on plane k.  lo / hi of a periodic slowest axis: the
+// planes that wrap (cells: N - 1 and 0; nodes, whose last plane repeats the
+// first: N - 2 and 1).
+template <int D, typename T, int KIND, bool PER>
+__device__ __forceinline__ void tail_put(T* x, const TailLevel<T>& w, bool per, int c, int k, int q, unsigned rank,
+                                         T v) {
+  const int kl = k - w.k0;
+  T* xc = x + c * w.cs + q;
+  xc[(kl + 1) * w.ps] = v;
+  if (w.np > 1) {
+    if (kl == 0 && k > 0) st_block(xc + (w.rp + 1) * w.ps, rank - 1, v);  // a full slab lies below
+    if (k == w.k1 - 1 && k < w.N - 1) st_block(xc, rank + 1, v);
+  }
+  if (PER && per) {
+    const int lr = (w.N - 1) / w.rp, lc = w.N - lr * w.rp;  // the last slab and its planes
+    const int lo = KIND == kNodal ? w.N - 2 : w.N - 1, hi = KIND == kNodal ? 1 : 0;
+    if (k == lo) {
+      if (w.np > 1)
+        st_block(xc, 0, v);
+      else
+        xc[0] = v;
+    }
+    if (k == hi) {
+      if (w.np > 1)
+        st_block(xc + (lc + 1) * w.ps, lr, v);
+      else
+        xc[(lc + 1) * w.ps] = v;
+    }
   }
 }
 
-template <int D, typename T, int KIND, bool PER, class S>
-__device__ __forceinline__ void tail_smooth(const TailView<T>& v, const Geom& g, T beta, int tid, int nth, S sync) {
-  if constexpr (KIND == kVisc) {
-    const T bs = rn_mul(beta, g_ihh<T>(g));
-    tail_visc_colours<D, T, 0, PER>(v, g, bs, tid, nth, sync);
-    tail_visc_colours<D, T, 1, PER>(v, g, bs, tid, nth, sync);
-    if constexpr (D == 3) tail_visc_colours<D, T, 2, PER>(v, g, bs, tid, nth, sync);
-  } else if constexpr (KIND == kMac) {
-    const int nt = rb_count<D>(g);
-    for (int col = 0; col < 2; ++col) {
-      for (int t = tid; t < nt; t += nth) k_cell_smooth_at<D, T, PER>(v.x, v.b, g, col, t);
-      sync();
+// the viscous stencil of component c at cell p of the slab
+template <int D, typename T, bool PER>
+__device__ __forceinline__ HomCell<D, T> tail_hom_cell(const char* mem, const TailLevel<T>& w, const Geom& g, int c,
+                                                       const int* p) {
+  const int kl = p[D - 1] - w.k0;
+  const int q = D == 3 ? p[0] + g.n[0] * p[1] : p[0];
+  const T* x = (const T*)(mem + w.x) + (kl + 1) * w.ps + q;
+  auto axis = [&](int a) {
+    const bool per = PER && g.per[a];
+    if (a == D - 1) return HomAxis(p[D - 1], g.n[D - 1], w.ps, per, true);
+    return HomAxis(a == 0 ? p[0] : p[1], g.n[a], a == 0 ? 1 : g.n[0], per);
+  };
+  auto comp = [&](int a) { return x + a * w.cs; };
+  auto face = [&](int a) {
+    const T* e = (const T*)(mem + w.ef[a]);
+    if (a == D - 1) return e + kl * w.ps + q;
+    if (a == 0) return e + p[0] + (g.n[0] + 1) * (D == 3 ? p[1] + g.n[1] * kl : kl);
+    return e + p[0] + g.n[0] * (p[1] + (g.n[1] + 1) * kl);
+  };
+  auto step = [&](int a) { return a == D - 1 ? w.ps : (a == 0 ? 1 : g.n[0]); };
+  const int a1 = hom_next<D>(c), a2 = hom_next<D>(a1);
+  if constexpr (D == 3)
+    return {{axis(c), axis(a1), axis(a2)},
+            {comp(c), comp(a1), comp(a2)},
+            {*face(c), *face(a1), *face(a2)},
+            {face(c)[step(c)], face(a1)[step(a1)], face(a2)[step(a2)]}};
+  else
+    return {{axis(c), axis(a1)},
+            {comp(c), comp(a1)},
+            {*face(c), *face(a1)},
+            {face(c)[step(c)], face(a1)[step(a1)]}};
+}
+
+// neighbours of cell p of the slab for the cell Poisson problem
+template <int D, bool PER>
+struct SlabNbr {
+  int om[D], op[D];
+  bool lo[D], hi[D];
+  __device__ __forceinline__ SlabNbr(const Geom& g, int ps, const int* p) {
+    int s = 1;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      const bool per = PER && g.per[a];
+      const bool first = p[a] == 0, last = p[a] == g.n[a] - 1;
+      lo[a] = per || !first;
+      hi[a] = per || !last;
+      om[a] = a == D - 1 || !first ? -s : (g.n[a] - 1) * s;
+      op[a] = a == D - 1 || !last ? s : -(g.n[a] - 1) * s;
+      s = a + 1 == D - 1 ? ps : s * g.n[a];
+    }
+  }
+};
+
+// neighbour offsets of node p of the slab
+template <int D, bool PER>
+__device__ __forceinline__ void slab_node_offsets(const Geom& g, int ps, const int* p, int* om, int* op) {
+  node_offsets(p[0], g.n[0], 1, PER && g.per[0], om[0], op[0]);
+  if (D == 3) node_offsets(p[1], g.n[1], g.n[0] + 1, PER && g.per[1], om[1], op[1]);
+  const bool per = PER && g.per[D - 1];  // a periodic neighbour is in the halo
+  om[D - 1] = p[D - 1] == 0 && !per ? ps : -ps;
+  op[D - 1] = p[D - 1] == g.n[D - 1] && !per ? -ps : ps;
+}
+
+// passes of one sweep: (component, colour), or the colours
+template <int D, int KIND>
+constexpr int tail_passes() {
+  return KIND == kVisc ? 2 * D : (KIND == kMac ? 2 : 1 << D);
+}
+
+// one pass over this block's points of a level
+template <int D, typename T, int KIND, bool PER>
+__device__ __forceinline__ void tail_pass(char* mem, const TailLevel<T>& w, const Geom& g, T bs, int pass,
+                                          unsigned rank) {
+  const bool per = PER && g.per[D - 1];
+  T* x = (T*)(mem + w.x);
+  const T* b = (const T*)(mem + w.b);
+  if constexpr (KIND != kNodal) {
+    const int c = KIND == kVisc ? pass >> 1 : 0, col = KIND == kVisc ? pass & 1 : pass;
+    const int nh = (g.n[0] + 1) / 2, n = nh * (D == 3 ? g.n[1] : 1) * (w.k1 - w.k0);
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+      const int r = divm(t, nh, g.m_rb), ih = t - r * nh;
+      const int kl = D == 3 ? divm(r, g.n[1], g.m_n1) : r, j = D == 3 ? r - kl * g.n[1] : 0;
+      const int k = w.k0 + kl, i = 2 * ih + ((j + k + col) & 1);
+      if (i >= g.n[0]) continue;
+      const int p[3] = {i, D == 3 ? j : k, k};
+      const int q = i + g.n[0] * j, o = kl * w.ps + q;
+      T v;
+      if constexpr (KIND == kVisc) {
+        const int oc = c * w.rp * w.ps + o;
+        v = hom_gs<D, T>(tail_hom_cell<D, T, PER>(mem, w, g, c, p), b[oc], ((const T*)(mem + w.inv))[oc], bs);
+      } else {
+        const SlabNbr<D, PER> nb(g, w.ps, p);
+        v = cell_gs_value<D, T>(x + o + w.ps, b[o], g_hh<T>(g), nb.om, nb.op, nb.lo, nb.hi);
+      }
+      tail_put<D, T, KIND, PER>(x, w, per, c, k, q, rank, v);
     }
   } else {
-    for (int col = 0; col < (1 << D); ++col) {
-      const int nt = mc_count<D>(g, col);
-      for (int t = tid; t < nt; t += nth) k_nodal_smooth_at<D, T, PER>(v.x, v.b, g, col, t);
-      sync();
+    const int b0 = pass & 1, b1 = (pass >> 1) & 1, bz = D == 3 ? (pass >> 2) & 1 : b1;
+    const int c0 = (g.n[0] + 2 - b0) / 2, c1 = D == 3 ? (g.n[1] + 2 - b1) / 2 : 1;
+    const int kf = w.k0 + ((w.k0 + bz) & 1);  // the slab's first plane of the colour
+    const int nk = kf < w.k1 ? (w.k1 - kf + 1) / 2 : 0, n = c0 * c1 * nk;
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+      const int r = divm(t, c0, g.m_mc0[b0]), i = 2 * (t - r * c0) + b0;
+      const int kk = D == 3 ? divm(r, c1, g.m_mc1[b1]) : r, j = D == 3 ? 2 * (r - kk * c1) + b1 : 0;
+      const int k = kf + 2 * kk;
+      const int p[3] = {i, D == 3 ? j : k, k};
+      const int q = i + (g.n[0] + 1) * j, o = (k - w.k0) * w.ps + q;
+      int om[3], op[3];
+      slab_node_offsets<D, PER>(g, w.ps, p, om, op);
+      const T s = nodal_nbr_sum<D, T>(x + o + w.ps, om, op);
+      tail_put<D, T, KIND, PER>(x, w, per, 0, k, q, rank, (g_hh<T>(g) * b[o] - s) * T(-3.0 / 8.0));
     }
   }
 }
 
+// the block's share of a level's residual, into r (the whole level's layout)
 template <int D, typename T, int KIND, bool PER>
-__device__ __forceinline__ void tail_resid(const TailView<T>& v, const Geom& g, T beta, int tid, int nth) {
-  if constexpr (KIND == kVisc) {
-    for (int t = tid; t < D * g.ncell; t += nth) {
-      const int c = t >= g.ncell ? (t >= 2 * g.ncell ? 2 : 1) : 0;
-      const int id = t - c * g.ncell;
-      int p[3];
+__device__ __forceinline__ void tail_resid(const char* mem, const TailLevel<T>& w, const Geom& g, T beta, T* r) {
+  const T* x = (const T*)(mem + w.x);
+  const T* b = (const T*)(mem + w.b);
+  const int np = w.ps * (w.k1 - w.k0), n = (KIND == kVisc ? D : 1) * np;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int c = KIND == kVisc && t >= np ? (t >= 2 * np ? 2 : 1) : 0;
+    const int o = t - c * np, id = w.k0 * w.ps + o;
+    int p[3];
+    if constexpr (KIND == kNodal) {
+      node_coords(g, id, p[0], p[1], p[2]);
+      int om[3], op[3];
+      slab_node_offsets<D, PER>(g, w.ps, p, om, op);
+      const T* q = x + o + w.ps;
+      r[id] = b[o] - (nodal_nbr_sum<D, T>(q, om, op) - T(8.0 / 3.0) * q[0]) * g_ihh<T>(g);
+    } else {
       cell_coords<D>(g, id, p[0], p[1], p[2]);
-      v.r[t] = c == 0   ? visc_res_hom<D, T, 0, PER>(v.x, v.b[t], v.ef, g, p, id, beta)
-               : c == 1 ? visc_res_hom<D, T, 1, PER>(v.x, v.b[t], v.ef, g, p, id, beta)
-                        : visc_res_hom<D, T, D - 1, PER>(v.x, v.b[t], v.ef, g, p, id, beta);
+      if constexpr (KIND == kVisc) {
+        r[(size_t)c * g.ncell + id] = hom_res<D, T>(tail_hom_cell<D, T, PER>(mem, w, g, c, p),
+                                                    b[c * w.rp * w.ps + o], beta, g_ihh<T>(g));
+      } else {
+        const SlabNbr<D, PER> nb(g, w.ps, p);
+        r[id] = cell_res_value<D, T>(x + o + w.ps, b[o], g_ihh<T>(g), nb.om, nb.op, nb.lo, nb.hi);
+      }
     }
-  } else if constexpr (KIND == kMac) {
-    for (int t = tid; t < g.ncell; t += nth) k_cell_resid_at<D, T, PER>(v.x, v.b, v.r, g, t);
+  }
+}
+
+// Smoothing of a level whose block holds few points: each thread keeps up to
+// NS points ("slots", the block's points in colour order, so that a warp's
+// share one colour) with everything that stays fixed over a visit in
+// registers: the neighbours' offsets, the wall flags, b, the reciprocals and
+// the face viscosities.  A pass is then the loads of x, the update and the
+// barrier.  Indexing every point anew (tail_pass) took most of a small level's
+// phase: about 350 dependent instructions.
+template <int D, int KIND>
+constexpr int tail_slots() {
+  return KIND == kNodal ? 3 : (KIND == kVisc && D == 3 ? 1 : 2);  // what 128 registers hold
+}
+
+template <int D, typename T>
+struct TailSlot {
+  int col = -1;       // colour; -1: no point
+  int k, q, o;        // plane, point of the plane, offset in x
+  int om[D], op[D];   // neighbours
+  unsigned wall = 0;  // bit 2a: no neighbour below on axis a (a wall), bit 2a + 1: above
+  __device__ __forceinline__ unsigned flip(int bit) const { return (wall << (31 - bit)) & 0x80000000u; }
+};
+
+// this thread's slot u of the block's points of the level
+template <int D, typename T, int KIND, bool PER>
+__device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const TailLevel<T>& w, const Geom& g, int u) {
+  int p[3] = {0, 0, 0};
+  s.col = -1;
+  s.wall = 0;
+  const int nk = w.k1 - w.k0;
+  if constexpr (KIND != kNodal) {
+    const int nh = (g.n[0] + 1) / 2, n = nh * (D == 3 ? g.n[1] : 1) * nk;
+    const int col = u >= n ? 1 : 0, t = u - col * n;
+    if (t >= n) return;
+    const int r = divm(t, nh, g.m_rb), ih = t - r * nh;
+    const int kl = D == 3 ? divm(r, g.n[1], g.m_n1) : r, j = D == 3 ? r - kl * g.n[1] : 0;
+    s.k = w.k0 + kl;
+    p[0] = 2 * ih + ((j + s.k + col) & 1);
+    if (p[0] >= g.n[0]) return;
+    p[1] = j;
+    p[D - 1] = s.k;
+    s.col = col;
+    s.q = p[0] + g.n[0] * j;
+    const HomAxis x(p[0], g.n[0], 1, PER && g.per[0]);
+    s.om[0] = x.om;
+    s.op[0] = x.op;
+    s.wall = (x.fm >> 31) | ((x.fp >> 31) << 1);
+    if (D == 3) {
+      const HomAxis y(p[1], g.n[1], g.n[0], PER && g.per[1]);
+      s.om[1] = y.om;
+      s.op[1] = y.op;
+      s.wall |= ((y.fm >> 31) << 2) | ((y.fp >> 31) << 3);
+    }
+    const HomAxis z(s.k, g.n[D - 1], w.ps, PER && g.per[D - 1], true);
+    s.om[D - 1] = z.om;
+    s.op[D - 1] = z.op;
+    s.wall |= ((z.fm >> 31) << (2 * D - 2)) | ((z.fp >> 31) << (2 * D - 1));
   } else {
-    for (int t = tid; t < g.nnode; t += nth) k_nodal_resid_at<D, T, PER>(v.x, v.b, v.r, g, t);
+    int t = u;
+    for (int col = 0; col < (1 << D); ++col) {
+      const int b0 = col & 1, b1 = (col >> 1) & 1, bz = D == 3 ? (col >> 2) & 1 : b1;
+      const int c0 = (g.n[0] + 2 - b0) / 2, c1 = D == 3 ? (g.n[1] + 2 - b1) / 2 : 1;
+      const int kf = w.k0 + ((w.k0 + bz) & 1);
+      const int n = kf < w.k1 ? c0 * c1 * ((w.k1 - kf + 1) / 2) : 0;
+      if (t < n) {
+        const int r = t / c0, kk = r / c1;
+        s.k = kf + 2 * kk;
+        p[0] = 2 * (t - r * c0) + b0;
+        p[1] = D == 3 ? 2 * (r - kk * c1) + b1 : 0;
+        s.q = p[0] + (g.n[0] + 1) * p[1];
+        p[D - 1] = s.k;
+        s.col = col;
+        break;
+      }
+      t -= n;
+    }
+    if (s.col < 0) return;
+    slab_node_offsets<D, PER>(g, w.ps, p, s.om, s.op);
+  }
+  s.o = (s.k - w.k0 + 1) * w.ps + s.q;
+}
+
+// the block's points of a level fit in its threads' slots
+template <int D, int KIND, typename T>
+__device__ __forceinline__ bool tail_fits_slots(const TailLevel<T>& w, const Geom& g) {
+  const int nk = w.rp, e = KIND == kNodal ? g.n[0] + 1 : (g.n[0] + 1) / 2 * 2;
+  const int n = e * (D == 3 ? (KIND == kNodal ? g.n[1] + 1 : g.n[1]) : 1) * nk;
+  return n <= tail_slots<D, KIND>() * kTailThreads;
+}
+
+// sweeps sweeps of the level, a barrier after each pass; then, when r is not
+// null, the residual into r (the whole level's layout) and a barrier
+template <int D, typename T, int KIND, bool PER, class S>
+__device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, const Geom& g, T beta, int sweeps, T* r,
+                                           unsigned rank, S sync) {
+  const T bs = KIND == kVisc ? rn_mul(beta, g_ihh<T>(g)) : T(0);
+  constexpr int NS = tail_slots<D, KIND>();
+  const bool per = PER && g.per[D - 1];
+  T* const x = (T*)(mem + w.x);
+  const T* const b = (const T*)(mem + w.b);
+  if (!tail_fits_slots<D, KIND>(w, g)) {
+#pragma unroll 1
+    for (int s = 0; s < sweeps; ++s)
+#pragma unroll 1
+      for (int q = 0; q < tail_passes<D, KIND>(); ++q) {
+        tail_pass<D, T, KIND, PER>(mem, w, g, bs, q, rank);
+        sync();
+      }
+    if (r) {
+      tail_resid<D, T, KIND, PER>(mem, w, g, beta, r);
+      sync();
+    }
+    return;
+  }
+  TailSlot<D, T> sl[NS];
+#pragma unroll
+  for (int i = 0; i < NS; ++i) tail_slot_init<D, T, KIND, PER>(sl[i], w, g, (int)threadIdx.x + i * kTailThreads);
+  const int bc = w.rp * w.ps;  // component stride of b and the reciprocals
+  if constexpr (KIND == kVisc) {
+    T e[NS][2 * D], bv[NS][D], iv[NS][D];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      if (sl[i].col < 0) continue;
+      const int p0 = D == 3 ? sl[i].q % g.n[0] : sl[i].q;
+      const int p[3] = {p0, D == 3 ? sl[i].q / g.n[0] : sl[i].k, sl[i].k};
+      const HomCell<D, T> h = tail_hom_cell<D, T, PER>(mem, w, g, 0, p);
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        e[i][2 * a] = h.elo[a];
+        e[i][2 * a + 1] = h.ehi[a];
+        bv[i][a] = b[a * bc + sl[i].o - w.ps];
+        iv[i][a] = ((const T*)(mem + w.inv))[a * bc + sl[i].o - w.ps];
+      }
+    }
+    auto cell = [&](int i, int c) {
+      HomCell<D, T> h;
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        const int a = c + q < D ? c + q : c + q - D;
+        h.ax[q].om = sl[i].om[a];
+        h.ax[q].op = sl[i].op[a];
+        h.ax[q].fm = sl[i].flip(2 * a);
+        h.ax[q].fp = sl[i].flip(2 * a + 1);
+        h.u[q] = x + a * w.cs + sl[i].o;
+        h.elo[q] = e[i][2 * a];
+        h.ehi[q] = e[i][2 * a + 1];
+      }
+      return h;
+    };
+#pragma unroll 1
+    for (int s = 0; s < sweeps; ++s)
+#pragma unroll
+      for (int c = 0; c < D; ++c)
+#pragma unroll 1
+        for (int col = 0; col < 2; ++col) {
+#pragma unroll
+          for (int i = 0; i < NS; ++i)
+            if (sl[i].col == col)
+              tail_put<D, T, KIND, PER>(x, w, per, c, sl[i].k, sl[i].q, rank, hom_gs<D, T>(cell(i, c), bv[i][c], iv[i][c], bs));
+          sync();
+        }
+    if (r) {
+#pragma unroll
+      for (int c = 0; c < D; ++c)
+#pragma unroll
+        for (int i = 0; i < NS; ++i)
+          if (sl[i].col >= 0)
+            r[(size_t)c * g.ncell + sl[i].k * w.ps + sl[i].q] = hom_res<D, T>(cell(i, c), bv[i][c], beta, g_ihh<T>(g));
+      sync();
+    }
+  } else {
+    T bv[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) bv[i] = sl[i].col >= 0 ? b[sl[i].o - w.ps] : T(0);
+    auto flags = [&](int i, bool* lo, bool* hi) {
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        lo[a] = !((sl[i].wall >> (2 * a)) & 1);
+        hi[a] = !((sl[i].wall >> (2 * a + 1)) & 1);
+      }
+    };
+#pragma unroll 1
+    for (int s = 0; s < sweeps; ++s)
+#pragma unroll 1
+      for (int col = 0; col < tail_passes<D, KIND>(); ++col) {
+#pragma unroll
+        for (int i = 0; i < NS; ++i)
+          if (sl[i].col == col) {
+            const T* q = x + sl[i].o;
+            T v;
+            if constexpr (KIND == kMac) {
+              bool lo[D], hi[D];
+              flags(i, lo, hi);
+              v = cell_gs_value<D, T>(q, bv[i], g_hh<T>(g), sl[i].om, sl[i].op, lo, hi);
+            } else {
+              v = (g_hh<T>(g) * bv[i] - nodal_nbr_sum<D, T>(q, sl[i].om, sl[i].op)) * T(-3.0 / 8.0);
+            }
+            tail_put<D, T, KIND, PER>(x, w, per, 0, sl[i].k, sl[i].q, rank, v);
+          }
+        sync();
+      }
+    if (r) {
+#pragma unroll
+      for (int i = 0; i < NS; ++i)
+        if (sl[i].col >= 0) {
+          const T* q = x + sl[i].o;
+          T v;
+          if constexpr (KIND == kMac) {
+            bool lo[D], hi[D];
+            flags(i, lo, hi);
+            v = cell_res_value<D, T>(q, bv[i], g_ihh<T>(g), sl[i].om, sl[i].op, lo, hi);
+          } else {
+            v = bv[i] - (nodal_nbr_sum<D, T>(q, sl[i].om, sl[i].op) - T(8.0 / 3.0) * q[0]) * g_ihh<T>(g);
+          }
+          r[sl[i].k * w.ps + sl[i].q] = v;
+        }
+      sync();
+    }
   }
 }
 
-// b of the coarse level from r of the fine one, and a zero coarse iterate
-template <int D, typename T, int KIND, bool PER>
-__device__ __forceinline__ void tail_restrict(const T* r, T* b, T* x, const Geom& gf, const Geom& gc, int tid,
-                                              int nth) {
-  constexpr int NC = KIND == kVisc ? D : 1;
-  const int n = NC * tail_points<D, T, KIND>(gc);
-  for (int t = tid; t < n; t += nth) {
-    if constexpr (KIND == kNodal)
-      k_restrict_nodes_at<D, T, PER>(r, b, gf, gc, t);
-    else
-      k_restrict_cells_at<D, T>(r, b, gf, gc, NC, t);
-    x[t] = T(0);
+// b of the block's coarse points from r of the fine level (TB: the coarse
+// slab's arithmetic, FP64 on a swept coarsest level)
+template <int D, typename T, int KIND, bool PER, typename TB>
+__device__ __forceinline__ void tail_restrict(char* mem, const TailLevel<TB>& w, const T* r, const Geom& gf,
+                                              const Geom& gc) {
+  TB* b = (TB*)(mem + w.b);
+  const int np = w.ps * (w.k1 - w.k0), n = (KIND == kVisc ? D : 1) * np;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int c = KIND == kVisc && t >= np ? (t >= 2 * np ? 2 : 1) : 0;
+    const int o = t - c * np, id = w.k0 * w.ps + o;
+    int I, J, K;
+    if constexpr (KIND == kNodal) {
+      node_coords(gc, id, I, J, K);
+      b[o] = (TB)restrict_node_value<D, T, PER>(r, gf, I, J, K);
+    } else {
+      cell_coords<D>(gc, id, I, J, K);
+      b[c * w.rp * w.ps + o] = (TB)restrict_cell_value<D, T>(r + (size_t)c * gf.ncell, gf, I, J, K);
+    }
   }
 }
 
+// x of the block's points += P e, e the coarse correction (component stride
+// cs)
 template <int D, typename T, int KIND, bool PER>
-__device__ __forceinline__ void tail_prolong(T* xf, const T* xc, const Geom& gf, const Geom& gc, int tid, int nth) {
-  constexpr int NC = KIND == kVisc ? D : 1;
-  const int n = NC * tail_points<D, T, KIND>(gf);
-  for (int t = tid; t < n; t += nth) {
-    if constexpr (KIND == kNodal)
-      k_prolong_nodes_add_at<D, T>(xf, xc, gf, gc, t);
-    else
-      k_prolong_cells_add_at<D, T, PER>(xf, xc, gf, gc, NC, KIND == kVisc ? T(-1) : T(1), t);
+__device__ __forceinline__ void tail_prolong(char* mem, const TailLevel<T>& w, const T* e, int cs, const Geom& gf,
+                                             const Geom& gc, unsigned rank) {
+  T* x = (T*)(mem + w.x);
+  const bool per = PER && gf.per[D - 1];
+  const int np = w.ps * (w.k1 - w.k0), n = (KIND == kVisc ? D : 1) * np;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    const int c = KIND == kVisc && t >= np ? (t >= 2 * np ? 2 : 1) : 0;
+    const int o = t - c * np;
+    int i, j, k;
+    T v;
+    if constexpr (KIND == kNodal) {
+      node_coords(gf, w.k0 * w.ps + o, i, j, k);
+      v = prolong_node_value<D, T>(e, gc, i, j, k);
+    } else {
+      cell_coords<D>(gf, w.k0 * w.ps + o, i, j, k);
+      v = prolong_cell_value<D, T, PER>(e + c * cs, gc, i, j, k, KIND == kVisc ? T(-1) : T(1));
+    }
+    const int kp = D == 3 ? k : j, q = o - (kp - w.k0) * w.ps;
+    v = x[c * w.cs + o + w.ps] + v;
+    tail_put<D, T, KIND, PER>(x, w, per, c, kp, q, rank, v);
   }
 }
 
@@ -261,62 +687,53 @@ __device__ __forceinline__ void block_copy(T* dst, const T* src, int n) {
   for (int t = threadIdx.x; t < n; t += blockDim.x) dst[t] = src[t];
 }
 
-// a solo level's arrays from shared memory at p (and p past them), with the
-// level's viscosities and reciprocals copied in
-template <int D, typename T, int KIND>
-__device__ inline void tail_carve(TailView<T>& v, char*& p, const Geom& g, const T* const* ef, const T* inv) {
-  const int n = tail_points<D, T, KIND>(g) * (KIND == kVisc ? D : 1);
-  T* q = (T*)p;
-  v.x = q;
-  v.b = q + n;
-  q += 2 * n;
-  if (KIND == kVisc) {
-    v.inv = q;
-    block_copy(q, inv, n);
-    q += n;
-    for (int a = 0; a < D; ++a) {
-      v.ef[a] = q;
-      block_copy(q, ef[a], g.nface[a]);
-      q += g.nface[a];
-    }
+// the level's constants (viscous problem): the reciprocals and the face
+// viscosities of the block's planes; every array is a run of whole planes
+template <int D, typename T>
+__device__ __forceinline__ void tail_load_const(char* mem, const TailLevel<T>& w, const Geom& g) {
+  const int nk = w.k1 - w.k0;
+  if (nk <= 0) return;
+  for (int c = 0; c < D; ++c)
+    block_copy((T*)(mem + w.inv) + c * w.rp * w.ps, w.ginv + (size_t)c * g.ncell + w.k0 * w.ps, nk * w.ps);
+  const int f0 = (g.n[0] + 1) * (D == 3 ? g.n[1] : 1);
+  block_copy((T*)(mem + w.ef[0]), w.gef[0] + (size_t)w.k0 * f0, nk * f0);
+  if (D == 3) {
+    const int f1 = g.n[0] * (g.n[1] + 1);
+    block_copy((T*)(mem + w.ef[1]), w.gef[1] + (size_t)w.k0 * f1, nk * f1);
   }
-  p += tail_level_bytes<D, T, KIND>(g);
+  block_copy((T*)(mem + w.ef[D - 1]), w.gef[D - 1] + (size_t)w.k0 * w.ps, (nk + 1) * w.ps);
 }
 
-// the coarsest level by sweeps Gauss-Seidel sweeps in FP64 (no exact inverse)
-template <int D, typename T, int KIND, bool PER>
-__device__ inline void tail_bottom_sweeps(const BottomArg<T>& a, const Geom& g, const T* b, T* x, char* mem,
-                                          double* sh) {
-  TailView<double> v;
-  v.r = nullptr;
-  tail_carve<D, double, KIND>(v, mem, g, a.ef, a.inv);
-  double* bd = (double*)v.b;
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-    bd[i] = (double)b[i];
-    v.x[i] = 0.0;
-  }
-  __syncthreads();
-  if (KIND != kVisc) bottom_sub_mean<D>(bd, a.n, KIND, g, sh);
-  for (int s = 0; s < a.sweeps; ++s)
-    tail_smooth<D, double, KIND, PER>(v, g, a.beta, threadIdx.x, blockDim.x, SyncSolo());
-  if (KIND != kVisc) bottom_sub_mean<D>(v.x, a.n, KIND, g, sh);
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x) x[i] = (T)v.x[i];
-  __syncthreads();
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+}
+
+// thread 0: the level record of this block
+template <int D, typename T, int KIND>
+__host__ __device__ inline void tail_level_init(TailLevel<T>& w, const Geom& g, int nblk, unsigned rank, bool solo,
+                                                unsigned& at) {
+  tail_planes<D, KIND>(g, w.N, w.ps);
+  w.rp = tail_rows<D, T, KIND>(g, nblk, solo);
+  w.np = (w.N + w.rp - 1) / w.rp;
+  w.k0 = (int)rank * w.rp < w.N ? (int)rank * w.rp : w.N;
+  w.k1 = w.k0 + w.rp < w.N ? w.k0 + w.rp : w.N;
+  w.cs = (w.rp + 2) * w.ps;
+  at += tail_slab_bytes<D, T, KIND>(g, w.rp, at, &w);
 }
 
 // PER = false: every level of every cavity has walls on every axis.  Grid:
-// ncav clusters; ls: the first solo level (a cavity whose coarsest level is
-// above it has that level solo); smem: the solo levels' arrays, a residual
-// scratch of the largest, and the coarsest level's FP64 copies where it has no
-// exact inverse.
+// ncav clusters.
 template <int D, typename T, int KIND, bool PER = true>
-__global__ void __launch_bounds__(tail_threads<T>()) k_vcycle_tail(TailTabs tb, int lf, int ls, int ncav,
+__global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailTabs tb, int lf, int ncav,
                                                                   const int* __restrict__ mask, int nu1, int nu2) {
-  extern __shared__ __align__(16) char smem[];
-  __shared__ TailView<T> sv[kMaxLev];
+  extern __shared__ __align__(16) char mem[];
+  __shared__ TailLevel<T> sw[kMaxLev];
+  __shared__ TailLevel<double> sbw;  // the coarsest level, when it is swept
   __shared__ Geom sg[kMaxLev];
   __shared__ double sh[33];
   __shared__ T sbeta;
+  __shared__ unsigned scratch;
+  constexpr int NC = KIND == kVisc ? D : 1;
   unsigned rank, nblk;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nblk));
@@ -325,107 +742,159 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_vcycle_tail(TailTabs tb, 
   const BottomArg<T>& bot = ((const BottomArg<T>*)tb.bot)[c];
   const int L = bot.level;
   if (L < lf) return;
-  const int s0 = ls < L ? ls : L;  // the first solo level
-  // the levels' geometry and global arrays
+  const bool swept = bot.Minv == nullptr;
   for (int l = lf; l <= L; ++l) {
-    const Geom* g = nullptr;
-    TailView<T> v;
-    if (KIND == kVisc) {
-      const ViscArg<T>& a = ((const ViscArg<T>*)tb.lv[l])[c];
-      g = &a.g;
-      v = {a.x, a.out, a.b, a.inv, {a.ef[0], a.ef[1], a.ef[2]}};
-      if (threadIdx.x == 0 && l == lf) sbeta = a.beta;
-    } else {
-      const PoisArg<T>& a = ((const PoisArg<T>*)tb.lv[l])[c];
-      g = &a.g;
-      v = {a.x, a.r, a.b, nullptr, {nullptr, nullptr, nullptr}};
-    }
+    const Geom* g;
+    if constexpr (KIND == kVisc)
+      g = &((const ViscArg<T>*)tb.lv[l])[c].g;
+    else
+      g = &((const PoisArg<T>*)tb.lv[l])[c].g;
     for (int q = threadIdx.x; q < (int)(sizeof(Geom) / 4); q += blockDim.x) ((int*)&sg[l])[q] = ((const int*)g)[q];
-    if (threadIdx.x == 0) sv[l] = v;
   }
   __syncthreads();
-  const T beta = KIND == kVisc ? sbeta : T(0);
-  const int nth = blockDim.x * nblk, tid = rank * blockDim.x + threadIdx.x;
-  const SyncWide wide;
-  const SyncSolo solo;
-  if (s0 > lf) {
-    if (lf > 0) {  // a coarse level starts from zero, level 0 from the given iterate
-      const int n = (KIND == kVisc ? D : 1) * tail_points<D, T, KIND>(sg[lf]);
-      for (int t = tid; t < n; t += nth) sv[lf].x[t] = T(0);
-      wide();
-    }
-    for (int l = lf; l < s0; ++l) {
-      const TailView<T> v = sv[l];
-      for (int s = 0; s < nu1; ++s) tail_smooth<D, T, KIND, PER>(v, sg[l], beta, tid, nth, wide);
-      tail_resid<D, T, KIND, PER>(v, sg[l], beta, tid, nth);
-      wide();
-      tail_restrict<D, T, KIND, PER>(v.r, (T*)sv[l + 1].b, sv[l + 1].x, sg[l], sg[l + 1], tid, nth);
-      wide();
-    }
-  }
-  if (rank == 0) {
-    // the solo levels: shared-memory arrays, the residual scratch after them
-    const int me = threadIdx.x, nb = blockDim.x;
-    char* p = smem;
-    TailView<T> gl = sv[s0];
-    __syncthreads();  // every thread has the global view
-    for (int l = s0; l <= L; ++l) {
-      TailView<T> v = sv[l];
-      const TailView<T> w = v;
+  if (threadIdx.x == 0) {
+    unsigned at = 0;
+    for (int l = lf; l <= L; ++l) {
+      TailLevel<T>& w = sw[l];
+      if constexpr (KIND == kVisc) {
+        const ViscArg<T>& a = ((const ViscArg<T>*)tb.lv[l])[c];
+        w.gx = a.x;
+        w.gr = a.out;
+        w.gb = a.b;
+        w.ginv = a.inv;
+        for (int q = 0; q < 3; ++q) w.gef[q] = a.ef[q];
+        sbeta = a.beta;
+      } else {
+        const PoisArg<T>& a = ((const PoisArg<T>*)tb.lv[l])[c];
+        w.gx = a.x;
+        w.gr = a.r;
+        w.gb = a.b;
+        sbeta = T(0);
+      }
       if (l < L) {
-        tail_carve<D, T, KIND>(v, p, sg[l], w.ef, w.inv);
-      } else {  // the coarsest level: x and b only
-        const int n = tail_points<D, T, KIND>(sg[l]) * (KIND == kVisc ? D : 1);
-        v.x = (T*)p;
-        v.b = v.x + n;
-        p += (2 * n * sizeof(T) + 15) / 16 * 16;
+        tail_level_init<D, T, KIND>(w, sg[l], (int)nblk, rank, false, at);
+      } else if (swept) {
+        sbw.ginv = bot.inv;
+        for (int q = 0; q < 3; ++q) sbw.gef[q] = bot.ef[q];
+        tail_level_init<D, double, KIND>(sbw, sg[l], (int)nblk, rank,
+                                         tail_swept_solo<D, T, KIND>(l > lf ? &sg[l - 1] : nullptr, (int)nblk), at);
+        w.np = sbw.np;
+      } else {  // the exact solve: block 0
+        tail_level_init<D, T, KIND>(w, sg[l], 1, rank, true, at);
       }
-      __syncthreads();
-      if (me == 0) sv[l] = v;
     }
-    if (me == 0)
-      for (int l = s0; l <= L; ++l) sv[l].r = (T*)p;
-    __syncthreads();
-    if (s0 < L)
-      p += ((KIND == kVisc ? D : 1) * (size_t)tail_points<D, T, KIND>(sg[s0]) * sizeof(T) + 15) / 16 * 16;
-    {
-      const int n = tail_points<D, T, KIND>(sg[s0]) * (KIND == kVisc ? D : 1);
-      T *x = sv[s0].x, *b = (T*)sv[s0].b;
-      for (int t = me; t < n; t += nb) {
-        b[t] = gl.b[t];
-        x[t] = s0 > 0 ? T(0) : gl.x[t];
-      }
-      __syncthreads();
-    }
-    for (int l = s0; l < L; ++l) {
-      const TailView<T> v = sv[l];
-      for (int s = 0; s < nu1; ++s) tail_smooth<D, T, KIND, PER>(v, sg[l], beta, me, nb, solo);
-      tail_resid<D, T, KIND, PER>(v, sg[l], beta, me, nb);
-      solo();
-      tail_restrict<D, T, KIND, PER>(v.r, (T*)sv[l + 1].b, sv[l + 1].x, sg[l], sg[l + 1], me, nb);
-      solo();
-    }
-    if (bot.Minv)
-      bottom_block<D, T>(bot, sv[L].b, sv[L].x);
-    else
-      tail_bottom_sweeps<D, T, KIND, PER>(bot, sg[L], sv[L].b, sv[L].x, p, sh);
-    for (int l = L - 1; l >= s0; --l) {
-      const TailView<T> v = sv[l];
-      tail_prolong<D, T, KIND, PER>(v.x, sv[l + 1].x, sg[l], sg[l + 1], me, nb);
-      solo();
-      for (int s = 0; s < nu2; ++s) tail_smooth<D, T, KIND, PER>(v, sg[l], beta, me, nb, solo);
-    }
-    block_copy(gl.x, (const T*)sv[s0].x, tail_points<D, T, KIND>(sg[s0]) * (KIND == kVisc ? D : 1));
-    if (me == 0) sv[s0] = gl;  // the wide levels read it from global memory
-    __syncthreads();
+    scratch = at;  // the one-slab levels' residuals
   }
-  if (s0 > lf) {
-    wide();
-    for (int l = s0 - 1; l >= lf; --l) {
-      const TailView<T> v = sv[l];
-      tail_prolong<D, T, KIND, PER>(v.x, sv[l + 1].x, sg[l], sg[l + 1], tid, nth);
-      wide();
-      for (int s = 0; s < nu2; ++s) tail_smooth<D, T, KIND, PER>(v, sg[l], beta, tid, nth, wide);
+  __syncthreads();
+  const T beta = sbeta;
+  // the constants of this block's planes, and the first level's b and x
+  if (KIND == kVisc) {
+    for (int l = lf; l < L; ++l) tail_load_const<D, T>(mem, sw[l], sg[l]);
+    if (swept) tail_load_const<D, double>(mem, sbw, sg[L]);
+  }
+  auto zero_x = [&](auto& w) {
+    auto* x = (decltype(w.gx))(mem + w.x);
+    for (int t = threadIdx.x; t < NC * w.cs; t += blockDim.x) x[t] = 0;
+  };
+  if (L == lf && swept) {
+    const int n = sbw.ps * (sbw.k1 - sbw.k0);
+    for (int q = 0; q < NC; ++q)
+      for (int t = threadIdx.x; t < n; t += blockDim.x)
+        ((double*)(mem + sbw.b))[q * sbw.rp * sbw.ps + t] =
+            (double)sw[L].gb[(size_t)q * sbw.N * sbw.ps + sbw.k0 * sbw.ps + t];
+    zero_x(sbw);
+  } else {
+    const TailLevel<T>& w = sw[lf];
+    const int n = w.ps * (w.k1 - w.k0);
+    for (int q = 0; q < NC; ++q)
+      block_copy((T*)(mem + w.b) + q * w.rp * w.ps, w.gb + (size_t)q * w.N * w.ps + w.k0 * w.ps, n);
+    zero_x(w);
+    __syncthreads();
+    if (lf == 0 && n > 0) {
+      // level 0 starts from the given iterate, its halos included
+      const bool per = PER && sg[0].per[D - 1];
+      const int lo = KIND == kNodal ? w.N - 2 : w.N - 1, hi = KIND == kNodal ? 1 : 0;
+      T* x = (T*)(mem + w.x);
+      for (int q = 0; q < NC; ++q) {
+        const T* gx = w.gx + (size_t)q * w.N * w.ps;
+        for (int t = threadIdx.x; t < (w.k1 - w.k0 + 2) * w.ps; t += blockDim.x) {
+          const int kl = t / w.ps;
+          int k = w.k0 + kl - 1;
+          if (k < 0) k = per ? lo : -1;
+          if (k >= w.N) k = per ? hi : -1;
+          if (k >= 0) x[q * w.cs + t] = gx[(size_t)k * w.ps + t - kl * w.ps];
+        }
+      }
+    }
+  }
+  if (nblk > 1)
+    cluster_sync();
+  else
+    __syncthreads();
+  // visit v: the levels lf .. L - 1 downwards, the coarsest, and back up
+  const int nd = L - lf;
+#pragma unroll 1
+  for (int visit = 0; visit <= 2 * nd; ++visit) {
+    const bool down = visit < nd;
+    const int l = visit <= nd ? lf + visit : lf + 2 * nd - visit;
+    const TailLevel<T>& w = sw[l];
+    const Geom& g = sg[l];
+    const bool wide = w.np > 1;
+    if (!wide && rank) continue;  // block 0 alone; the others wait at the next wide barrier
+    auto sync = [&] {
+      if (wide)
+        cluster_sync();
+      else
+        __syncthreads();
+    };
+    if (visit == nd) {
+      if (!swept) {
+        bottom_block<D, T>(bot, (const T*)(mem + w.b), (T*)(mem + w.x) + w.ps, w.cs, NC);
+      } else {
+        const int n = sbw.ps * (sbw.k1 - sbw.k0);
+        double *xd = (double*)(mem + sbw.x) + sbw.ps, *bd = (double*)(mem + sbw.b);
+        if (KIND != kVisc) bottom_sub_mean<D>(bd, n, KIND, g, sh);
+        tail_visit<D, double, KIND, PER>(mem, sbw, g, bot.beta, bot.sweeps, (double*)nullptr, rank, sync);
+        if (KIND != kVisc) bottom_sub_mean<D>(xd, n, KIND, g, sh);
+        for (int q = 0; q < NC; ++q)
+          for (int t = threadIdx.x; t < n; t += blockDim.x)
+            w.gx[(size_t)q * sbw.N * sbw.ps + sbw.k0 * sbw.ps + t] = (T)xd[q * sbw.cs + t];
+        if (!wide) __syncthreads();
+      }
+    } else {
+      T* const r = wide ? w.gr : (T*)(mem + scratch);
+      if (!down) {
+        if (wide) cluster_sync();  // the coarse level's result is in its global array
+        const bool local = !wide && !(l + 1 == L && swept);
+        const TailLevel<T>& wc = sw[l + 1];
+        tail_prolong<D, T, KIND, PER>(mem, w, local ? (const T*)(mem + wc.x) + wc.ps : (const T*)wc.gx,
+                                      local ? wc.cs : (KIND == kVisc ? sg[l + 1].ncell : 0), g, sg[l + 1], rank);
+        sync();
+      }
+      tail_visit<D, T, KIND, PER>(mem, w, g, beta, down ? nu1 : nu2, down ? r : (T*)nullptr, rank, sync);
+      if (down) {
+        const bool cwide = sw[l + 1].np > 1;
+        if (cwide || rank == 0) {
+          if (l + 1 == L && swept) {
+            tail_restrict<D, T, KIND, PER>(mem, sbw, r, g, sg[l + 1]);
+            zero_x(sbw);
+          } else {
+            tail_restrict<D, T, KIND, PER>(mem, sw[l + 1], r, g, sg[l + 1]);
+            zero_x(sw[l + 1]);
+          }
+          if (cwide)
+            cluster_sync();
+          else
+            __syncthreads();
+        }
+      }
+    }
+    // a result that another block or the next launch reads
+    if (visit >= nd && (l == lf || sw[l - 1].np > 1) && !(visit == nd && swept)) {
+      const int n = w.ps * (w.k1 - w.k0);
+      const T* x = (const T*)(mem + w.x) + w.ps;
+      for (int q = 0; q < NC; ++q)
+        block_copy(w.gx + (size_t)q * w.N * w.ps + w.k0 * w.ps, x + q * w.cs, n);
     }
   }
 }
@@ -433,56 +902,64 @@ __global__ void __launch_bounds__(tail_threads<T>()) k_vcycle_tail(TailTabs tb, 
 // ---------------------------------------------------------------------------
 // host side of the tail
 // ---------------------------------------------------------------------------
-constexpr size_t kTailSmem = 200 * 1024;  // dynamic shared memory the solo levels may take
+constexpr size_t kTailSmem = 200 * 1024;  // dynamic shared memory a block of the tail may take
 
-// dynamic shared memory of the tail with solo levels s0..L of the hierarchy gs
-// (sweeps: the coarsest level has no exact inverse)
+// dynamic shared memory of block 0 of the tail (the largest) over the levels
+// lf..L of the hierarchy gs with nblk blocks (swept: the coarsest level has no
+// exact inverse)
 template <int D, typename T, int KIND>
-inline size_t tail_smem(const Geom* const* gs, int s0, int L, bool sweeps) {
-  size_t b = 0;
-  for (int l = s0; l < L; ++l) b += tail_level_bytes<D, T, KIND>(*gs[l]);
-  const size_t nc = KIND == kVisc ? D : 1;
-  b += (2 * nc * tail_points<D, T, KIND>(*gs[L]) * sizeof(T) + 15) / 16 * 16;
-  if (s0 < L) b += (nc * tail_points<D, T, KIND>(*gs[s0]) * sizeof(T) + 15) / 16 * 16;
-  if (sweeps) b += tail_bottom_bytes<D, KIND>(*gs[L]);
-  return b;
+inline size_t tail_smem(const Geom* const* gs, int lf, int L, int nblk, bool swept) {
+  size_t b = 0, r = 0;
+  for (int l = lf; l < L; ++l) {
+    int N, ps;
+    tail_planes<D, KIND>(*gs[l], N, ps);
+    const int rp = tail_rows<D, T, KIND>(*gs[l], nblk);
+    b += tail_slab_bytes<D, T, KIND>(*gs[l], rp, 0, nullptr);
+    if (rp == N && r == 0) r = (size_t)(KIND == kVisc ? D : 1) * N * ps * sizeof(T);  // the finest one-slab level
+  }
+  if (swept)
+    b += tail_slab_bytes<D, double, KIND>(
+        *gs[L], tail_rows<D, double, KIND>(*gs[L], nblk, tail_swept_solo<D, T, KIND>(L > lf ? gs[L - 1] : nullptr, nblk)),
+        0, nullptr);
+  else
+    b += tail_slab_bytes<D, T, KIND>(*gs[L], tail_rows<D, T, KIND>(*gs[L], 1), 0, nullptr);
+  return b + r;
 }
 
-// first solo level of a hierarchy gs[0..L]: the finest from lf on with at most
-// kTailSolo cells whose levels fit in shared memory; -1 when not even the
-// coarsest level does
-template <int D, typename T>
-constexpr int tail_solo_cells() {
-  return sizeof(T) == 4 ? (D == 3 ? 512 : 1024) : 64;
-}
+// some level of lf..L is cut into several slabs
 template <int D, typename T, int KIND>
-inline int tail_solo_level(const Geom* const* gs, int lf, int L, bool sweeps) {
-  for (int l = lf; l <= L; ++l)
-    if ((l == L || gs[l]->ncell <= tail_solo_cells<D, T>()) && tail_smem<D, T, KIND>(gs, l, L, sweeps) <= kTailSmem)
-      return l;
-  return -1;
+inline bool tail_has_wide(const Geom* const* gs, int lf, int L, bool swept) {
+  int N, ps;
+  tail_planes<D, KIND>(*gs[lf], N, ps);
+  if (lf < L) return tail_rows<D, T, KIND>(*gs[lf], 16) < N;
+  return swept && tail_rows<D, double, KIND>(*gs[L], 16, tail_swept_solo<D, T, KIND>(nullptr, 16)) < N;
 }
 
-// blocks per cluster for ncav cavities: as many as share the SMs without a
-// second wave of clusters, 16 at most (8 where the device cannot place 16)
+// Sets the tail kernel up on the current device and returns the blocks per
+// cluster for ncav cavities with (wide) levels of several slabs: as many as
+// share the SMs without a second wave of clusters, 16 at most (8 where the
+// device cannot place 16); 0 when the set-up fails.
 template <int D, typename T, int KIND, bool PER>
-inline int tail_blocks(int ncav, size_t smem) {
-  int nblk = 16;
+inline int tail_blocks(int ncav, bool wide) {
+  auto kern = k_vcycle_tail<D, T, KIND, PER>;
+  int nblk = wide ? 16 : 1;
   while (nblk > 1 && nblk * ncav > 152) nblk >>= 1;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
   if (nblk > 8) {
-    auto kern = k_vcycle_tail<D, T, KIND, PER>;
     int n = 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nblk);
-    cfg.blockDim = dim3((unsigned)tail_threads<T>());
-    cfg.dynamicSmemBytes = smem;
+    cfg.blockDim = dim3((unsigned)kTailThreads);
+    cfg.dynamicSmemBytes = kTailSmem;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim = {(unsigned)nblk, 1, 1};
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem) != cudaSuccess ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
       cudaGetLastError();
       nblk = 8;
@@ -497,17 +974,14 @@ constexpr int tail_wide_cells() {
   return sizeof(T) == 4 ? (D == 3 ? 32768 : 16384) : (D == 3 ? 4096 : 16384);
 }
 
-// launch on stream s: ncav clusters of nblk blocks
+// launch on stream s: ncav clusters of nblk blocks (tail_blocks)
 template <int D, typename T, int KIND, bool PER>
-inline cudaError_t tail_launch(cudaStream_t s, const TailTabs& tb, int lf, int ls, int ncav, const int* mask, int nu1,
-                               int nu2, int nblk, size_t smem) {
+inline cudaError_t tail_launch(cudaStream_t s, const TailTabs& tb, int lf, int ncav, const int* mask, int nu1, int nu2,
+                               int nblk, size_t smem) {
   auto kern = k_vcycle_tail<D, T, KIND, PER>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem);
-  if (e == cudaSuccess && nblk > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nblk * ncav));
-  cfg.blockDim = dim3((unsigned)tail_threads<T>());
+  cfg.blockDim = dim3((unsigned)kTailThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -515,7 +989,7 @@ inline cudaError_t tail_launch(cudaStream_t s, const TailTabs& tb, int lf, int l
   at[0].val.clusterDim = {(unsigned)nblk, 1, 1};
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, tb, lf, ls, ncav, mask, nu1, nu2);
+  return cudaLaunchKernelEx(&cfg, kern, tb, lf, ncav, mask, nu1, nu2);
 }
 
 }  // namespace batch

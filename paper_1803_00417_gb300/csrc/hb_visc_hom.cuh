@@ -34,140 +34,170 @@ __host__ __device__ __forceinline__ double sgn_flip(double v, unsigned m) {
 #endif
 }
 
-// Where the neighbours of cell p along each axis sit: the offsets om / op
-// below and above it (wrapped on a periodic axis; 0 past a wall, where the
-// homogeneous ghost is minus the cell's own value: fm / fp hold the sign bit
-// there and 0 elsewhere).
-template <int D, bool PER>
-struct HomNbr {
-  int om[D], op[D];
-  unsigned fm[D], fp[D];
-  __host__ __device__ __forceinline__ HomNbr(const Geom& g, const int* p) {
-    int s = 1;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-      const bool lo = p[a] == 0, hi = p[a] == g.n[a] - 1;
-      if (PER && g.per[a]) {
-        om[a] = lo ? (g.n[a] - 1) * s : -s;
-        op[a] = hi ? -(g.n[a] - 1) * s : s;
-        fm[a] = fp[a] = 0u;
-      } else {
-        om[a] = lo ? 0 : -s;
-        op[a] = hi ? 0 : s;
-        fm[a] = lo ? 0x80000000u : 0u;
-        fp[a] = hi ? 0x80000000u : 0u;
-      }
-      s *= g.n[a];
-    }
+// One axis seen from a cell: the offsets om / op of the neighbours below and
+// above (wrapped on a periodic axis; 0 past a wall, where the homogeneous
+// ghost is minus the cell's own value: fm / fp hold the sign bit there and 0
+// elsewhere).
+struct HomAxis {
+  int om, op;
+  unsigned fm, fp;
+  __host__ __device__ __forceinline__ HomAxis() {}
+  // position q of n along an axis of stride s
+  __host__ __device__ __forceinline__ HomAxis(int q, int n, int s, bool per) {
+    const bool lo = q == 0, hi = q == n - 1;
+    om = lo ? (per ? (n - 1) * s : 0) : -s;
+    op = hi ? (per ? -(n - 1) * s : 0) : s;
+    fm = lo && !per ? 0x80000000u : 0u;
+    fp = hi && !per ? 0x80000000u : 0u;
+  }
+  // the slowest axis of a slab with a halo plane on either side: a periodic
+  // neighbour is in the halo
+  __host__ __device__ __forceinline__ HomAxis(int q, int n, int s, bool per, bool /*halo*/) {
+    const bool lo = q == 0 && !per, hi = q == n - 1 && !per;
+    om = lo ? 0 : -s;
+    op = hi ? 0 : s;
+    fm = lo ? 0x80000000u : 0u;
+    fp = hi ? 0x80000000u : 0u;
   }
 };
 
-// the faces of axis a below and above cell p in the face array ef[a] (from
-// face f on, the next one fs further): both values
+// the component's axis comes first, then the others in cyclic order
 template <int D>
-__host__ __device__ __forceinline__ int face_step(const Geom& g, int a) {
-  return a == 0 ? 1 : (a == 1 ? g.n[0] : g.n[0] * g.n[1]);
+__host__ __device__ __forceinline__ int hom_next(int a) {
+  return a + 1 == D ? 0 : a + 1;
 }
 
-// 1 / (1 + bs diag) of component c at cell p, diag = sum_a k_a (e_lo + e_hi)
-// with wall faces counted twice (their ghost is minus the cell), k_c = 2,
-// k_a = 1 otherwise, bs = beta / h^2
-template <int D, typename T, bool PER>
-__host__ __device__ __forceinline__ T visc_inv_point(const T* const* ef, const Geom& g, int c, const int* p, T bs) {
+// The stencil of component c at a cell, by role r = 0 (the component's own
+// axis), 1, .. (the other axes in cyclic order): the axis as the cell sees it,
+// the component of that axis at the cell, and the face viscosities below and
+// above the cell on that axis.  c may be a run-time value.
+template <int D, typename T>
+struct HomCell {
+  HomAxis ax[D];
+  const T* u[D];
+  T elo[D], ehi[D];
+};
+
+// 1 / (1 + bs diag), diag = sum_a k_a (e_lo + e_hi) with wall faces counted
+// twice (their ghost is minus the cell), k = 2 on the component's own axis and
+// 1 on the others, bs = beta / h^2
+template <int D, typename T>
+__host__ __device__ __forceinline__ T hom_inv(const HomCell<D, T>& s, T bs) {
   T diag = T(0);
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const int f = fidx(g, a, p[0], p[1], p[2]);
-    const bool wall = !(PER && g.per[a]);
-    T lo = ef[a][f], hi = ef[a][f + face_step<D>(g, a)];
-    if (wall && p[a] == 0) lo = rn_mul(T(2), lo);
-    if (wall && p[a] == g.n[a] - 1) hi = rn_mul(T(2), hi);
+  for (int r = 0; r < D; ++r) {
+    T lo = s.elo[r], hi = s.ehi[r];
+    if (s.ax[r].fm) lo = rn_mul(T(2), lo);
+    if (s.ax[r].fp) hi = rn_mul(T(2), hi);
     const T w = rn_add(lo, hi);
-    diag = a == c ? rn_fma(T(2), w, diag) : rn_add(diag, w);
+    diag = r == 0 ? rn_mul(T(2), w) : rn_add(diag, w);
   }
   return T(1) / rn_fma(bs, diag, T(1));
 }
 
-// The differences of u_a along c at the cell id and at its two neighbours
-// along a (homogeneous ghosts past a wall normal to c)
-template <int D, typename T, bool PER>
-__host__ __device__ __forceinline__ void hom_cross(const T* ua, const HomNbr<D, PER>& nb, int id, int a, int c, T& xhi,
-                                                   T& xlo) {
-  const T* q = ua + id;
-  const T mid = rn_add(sgn_flip(q[nb.op[c]], nb.fp[c]), -sgn_flip(q[nb.om[c]], nb.fm[c]));
-  const T* qp = q + nb.op[a];
-  const T* qm = q + nb.om[a];
-  xhi = rn_add(mid, rn_add(sgn_flip(qp[nb.op[c]], nb.fp[c]), -sgn_flip(qp[nb.om[c]], nb.fm[c])));
-  xlo = rn_add(rn_add(sgn_flip(qm[nb.op[c]], nb.fp[c]), -sgn_flip(qm[nb.om[c]], nb.fm[c])), mid);
+// the differences of q's component along c at the cell and at its two
+// neighbours along a (homogeneous ghosts past a wall normal to c), summed over
+// the two cells of the face above (xhi) and below (xlo)
+template <typename T>
+__host__ __device__ __forceinline__ void hom_cross(const T* q, const HomAxis& a, const HomAxis& c, T& xhi, T& xlo) {
+  const T mid = rn_add(sgn_flip(q[c.op], c.fp), -sgn_flip(q[c.om], c.fm));
+  const T* qp = q + a.op;
+  const T* qm = q + a.om;
+  xhi = rn_add(mid, rn_add(sgn_flip(qp[c.op], c.fp), -sgn_flip(qp[c.om], c.fm)));
+  xlo = rn_add(rn_add(sgn_flip(qm[c.op], c.fp), -sgn_flip(qm[c.om], c.fm)), mid);
 }
 
-// Gauss-Seidel value of component C at cell p (flat index id): visc_gs_core's
-// sums with zero coefficients at wall faces (a wall face has no cross term,
-// and its normal term is in the diagonal), times the diagonal's reciprocal.
-// Explicitly rounded in FP32: the launches and the fused tail get the same
-// bits.
-template <int D, typename T, int C, bool PER>
-__host__ __device__ __forceinline__ T visc_gs_hom(const T* u, T bc, T inv, const T* const* ef, const Geom& g,
-                                                  const int* p, int id, T bs) {
-  const HomNbr<D, PER> nb(g, p);
-  const T* uc = u + (size_t)C * g.ncell + id;
+// Gauss-Seidel value: visc_gs_core's sums with zero coefficients at wall faces
+// (a wall face has no cross term, and its normal term is in the diagonal),
+// times the diagonal's reciprocal.  Explicitly rounded in FP32: the launches
+// and the fused tail get the same bits.
+template <int D, typename T>
+__host__ __device__ __forceinline__ T hom_gs(const HomCell<D, T>& s, T bc, T inv, T bs) {
   T offd = T(0), cross = T(0);
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const T* e = ef[a] + fidx(g, a, p[0], p[1], p[2]);
-    const T elo = nb.fm[a] ? T(0) : e[0], ehi = nb.fp[a] ? T(0) : e[face_step<D>(g, a)];
-    const T f = rn_fma(elo, uc[nb.om[a]], rn_mul(ehi, uc[nb.op[a]]));
-    offd = a == C ? rn_fma(T(2), f, offd) : rn_add(offd, f);
-    if (a != C) {
+  for (int r = 0; r < D; ++r) {
+    const HomAxis& a = s.ax[r];
+    const T elo = a.fm ? T(0) : s.elo[r], ehi = a.fp ? T(0) : s.ehi[r];
+    const T f = rn_fma(elo, s.u[0][a.om], rn_mul(ehi, s.u[0][a.op]));
+    offd = r == 0 ? rn_mul(T(2), f) : rn_add(offd, f);
+    if (r > 0) {
       T xhi, xlo;
-      hom_cross<D, T, PER>(u + (size_t)a * g.ncell, nb, id, a, C, xhi, xlo);
+      hom_cross(s.u[r], a, s.ax[0], xhi, xlo);
       cross = rn_add(cross, rn_fma(ehi, xhi, -rn_mul(elo, xlo)));
     }
   }
   return rn_mul(rn_fma(bs, rn_fma(T(0.25), cross, offd), bc), inv);
 }
 
-// b - (u - beta L u) of component C at cell p, homogeneous walls: tensor_core's
-// terms, with the normal flux of a wall face e (u - (-u)) and no cross term
-// there
-template <int D, typename T, int C, bool PER>
-__host__ __device__ __forceinline__ T visc_res_hom(const T* u, T bc, const T* const* ef, const Geom& g, const int* p,
-                                                   int id, T beta) {
-  const HomNbr<D, PER> nb(g, p);
-  const T* uc = u + (size_t)C * g.ncell + id;
-  const T u0 = uc[0];
+// b - (u - beta L u): tensor_core's terms, with the normal flux of a wall face
+// e (u - (-u)) and no cross term there
+template <int D, typename T>
+__host__ __device__ __forceinline__ T hom_res(const HomCell<D, T>& s, T bc, T beta, T ihh) {
+  const T u0 = s.u[0][0];
   T acc = T(0);
 #pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const T* e = ef[a] + fidx(g, a, p[0], p[1], p[2]);
-    const T elo = e[0], ehi = e[face_step<D>(g, a)];
-    const T dlo = rn_add(u0, -sgn_flip(uc[nb.om[a]], nb.fm[a]));
-    const T dhi = rn_add(sgn_flip(uc[nb.op[a]], nb.fp[a]), -u0);
-    T flo, fhi;
-    if (a == C) {
-      flo = rn_mul(elo, rn_mul(T(2), dlo));
-      fhi = rn_mul(ehi, rn_mul(T(2), dhi));
-    } else {
+  for (int r = 0; r < D; ++r) {
+    const HomAxis& a = s.ax[r];
+    T dlo = rn_add(u0, -sgn_flip(s.u[0][a.om], a.fm)), dhi = rn_add(sgn_flip(s.u[0][a.op], a.fp), -u0);
+    if (r > 0) {
       T xhi, xlo;
-      hom_cross<D, T, PER>(u + (size_t)a * g.ncell, nb, id, a, C, xhi, xlo);
-      flo = rn_mul(elo, rn_fma(T(0.25), nb.fm[a] ? T(0) : xlo, dlo));
-      fhi = rn_mul(ehi, rn_fma(T(0.25), nb.fp[a] ? T(0) : xhi, dhi));
+      hom_cross(s.u[r], a, s.ax[0], xhi, xlo);
+      dlo = rn_fma(T(0.25), a.fm ? T(0) : xlo, dlo);
+      dhi = rn_fma(T(0.25), a.fp ? T(0) : xhi, dhi);
     }
-    acc = rn_add(acc, rn_add(fhi, -flo));
+    const T f = rn_fma(s.ehi[r], dhi, -rn_mul(s.elo[r], dlo));
+    acc = r == 0 ? rn_mul(T(2), f) : rn_add(acc, f);
   }
-  const T Lu = rn_mul(acc, g_ihh<T>(g));
-  return rn_add(bc, -rn_fma(-beta, Lu, u0));
+  return rn_add(bc, -rn_fma(-beta, rn_mul(acc, ihh), u0));
 }
 
-// thread t of a sweep of colour col (rb_cell's map)
-template <int D, typename T, int C, bool PER>
+// the stencil of component c at cell p of a whole level (flat index id)
+template <int D, typename T, bool PER>
+__host__ __device__ __forceinline__ HomCell<D, T> hom_cell(const T* u, const T* const* ef, const Geom& g, int c,
+                                                           const int* p, int id) {
+  auto axis = [&](int a) {
+    return HomAxis(p[a], g.n[a], a == 0 ? 1 : (a == 1 ? g.n[0] : g.n[0] * g.n[1]), PER && g.per[a]);
+  };
+  auto comp = [&](int a) { return u + (size_t)a * g.ncell + id; };
+  auto face = [&](int a) { return ef[a] + fidx(g, a, p[0], p[1], p[2]); };
+  auto step = [&](int a) { return a == 0 ? 1 : (a == 1 ? g.n[0] : g.n[0] * g.n[1]); };
+  const int a1 = hom_next<D>(c), a2 = hom_next<D>(a1);
+  if constexpr (D == 3)
+    return {{axis(c), axis(a1), axis(a2)},
+            {comp(c), comp(a1), comp(a2)},
+            {*face(c), *face(a1), *face(a2)},
+            {face(c)[step(c)], face(a1)[step(a1)], face(a2)[step(a2)]}};
+  else
+    return {{axis(c), axis(a1)},
+            {comp(c), comp(a1)},
+            {*face(c), *face(a1)},
+            {face(c)[step(c)], face(a1)[step(a1)]}};
+}
+
+template <int D, typename T, bool PER>
+__host__ __device__ __forceinline__ T visc_inv_point(const T* const* ef, const Geom& g, int c, const int* p, T bs) {
+  return hom_inv<D, T>(hom_cell<D, T, PER>(nullptr, ef, g, c, p, 0), bs);
+}
+template <int D, typename T, bool PER>
+__host__ __device__ __forceinline__ T visc_gs_hom(const T* u, T bc, T inv, const T* const* ef, const Geom& g, int c,
+                                                  const int* p, int id, T bs) {
+  return hom_gs<D, T>(hom_cell<D, T, PER>(u, ef, g, c, p, id), bc, inv, bs);
+}
+template <int D, typename T, bool PER>
+__host__ __device__ __forceinline__ T visc_res_hom(const T* u, T bc, const T* const* ef, const Geom& g, int c,
+                                                   const int* p, int id, T beta) {
+  return hom_res<D, T>(hom_cell<D, T, PER>(u, ef, g, c, p, id), bc, beta, g_ihh<T>(g));
+}
+
+// thread t of a sweep of component c, colour col (rb_cell's map)
+template <int D, typename T, bool PER>
 __host__ __device__ __forceinline__ void visc_smooth_hom_at(T* u, const T* b, const T* inv, const T* const* ef,
-                                                            const Geom& g, int col, T bs, int t) {
+                                                            const Geom& g, int c, int col, T bs, int t) {
   int p[3];
   if (!rb_cell<D>(g, t, col, p)) return;
   const int id = cidx<D>(g, p[0], p[1], p[2]);
-  const size_t o = (size_t)C * g.ncell + id;
-  u[o] = visc_gs_hom<D, T, C, PER>(u, b[o], inv[o], ef, g, p, id, bs);
+  const size_t o = (size_t)c * g.ncell + id;
+  u[o] = visc_gs_hom<D, T, PER>(u, b[o], inv[o], ef, g, c, p, id, bs);
 }
 
 template <int D, typename T, int C, bool PER>
@@ -177,7 +207,7 @@ __global__ void __launch_bounds__(256) k_visc_smooth_hom(T* u, const T* __restri
                                                          int col, T bs) {
   const T* ef[3] = {ef0, ef1, ef2};
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < rb_count<D>(g)) visc_smooth_hom_at<D, T, C, PER>(u, b, inv, ef, g, col, bs, t);
+  if (t < rb_count<D>(g)) visc_smooth_hom_at<D, T, PER>(u, b, inv, ef, g, C, col, bs, t);
 }
 
 // r = b - (u - beta L u) of every component (thread t: cell t)
@@ -186,12 +216,10 @@ __host__ __device__ __forceinline__ void visc_res_hom_at(const T* u, const T* b,
                                                          const Geom& g, T beta, int t) {
   int p[3];
   cell_coords<D>(g, t, p[0], p[1], p[2]);
-  r[t] = visc_res_hom<D, T, 0, PER>(u, b[t], ef, g, p, t, beta);
-  const size_t o1 = (size_t)g.ncell + t;
-  r[o1] = visc_res_hom<D, T, 1, PER>(u, b[o1], ef, g, p, t, beta);
-  if constexpr (D == 3) {
-    const size_t o2 = 2 * (size_t)g.ncell + t;
-    r[o2] = visc_res_hom<D, T, 2, PER>(u, b[o2], ef, g, p, t, beta);
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    const size_t o = (size_t)c * g.ncell + t;
+    r[o] = visc_res_hom<D, T, PER>(u, b[o], ef, g, c, p, t, beta);
   }
 }
 

@@ -54,11 +54,11 @@ static bool check_comp(const Geom& g, const std::vector<T>& u, const std::vector
     const T bc = b[(size_t)C * g.ncell + t], u0 = u[(size_t)C * g.ncell + t];
     const T inv = visc_inv_point<D, T, PER>(ef, g, C, p, bs);
     const double w = (double)visc_gs_point<D, T, PER>(u.data(), b.data(), FaceEta<T>{ef}, g, C, p, beta, true);
-    const double v = (double)visc_gs_hom<D, T, C, PER>(u.data(), bc, inv, ef, g, p, t, bs);
+    const double v = (double)visc_gs_hom<D, T, PER>(u.data(), bc, inv, ef, g, C, p, t, bs);
     const double s1 = 3 * umax + std::fabs((double)bc);
     const T Lu = mg_tensor_point<D, T, PER>(u.data(), FaceEta<T>{ef}, g, C, p, true);
     const double rw = (double)op_out<T>(u0, Lu, beta, b.data(), (size_t)C * g.ncell + t);
-    const double r = (double)visc_res_hom<D, T, C, PER>(u.data(), bc, ef, g, p, t, beta);
+    const double r = (double)visc_res_hom<D, T, PER>(u.data(), bc, ef, g, C, p, t, beta);
     const double s2 = std::fabs((double)bc) + umax * (1 + 4 / (double)inv);
     if (!(std::fabs(v - w) <= kOps * eps * s1) || !(std::fabs(r - rw) <= kOps * eps * s2)) {
       std::fprintf(stderr, "D %d C %d PER %d n %d %d %d cell %d %d %d: sweep %.17g %.17g, residual %.17g %.17g\n", D, C,
