@@ -7,6 +7,7 @@
 // The network maps the normalised warm-start residual of the nodal projection
 // solve (Eq. 17) to a correction of its initial guess; the multigrid solve
 // remains the judge and runs to the same tolerance from that guess.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -65,25 +66,27 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int 
   }
 }
 
-// nearest upsampling of in (coarse, Cin channels) into channels [0, Cin) of out (stride Cs)
+// the decoder's input: nearest upsampling of up (coarse, Cup channels) and the
+// skip channels (Cs), concatenated; one thread per 8 channels (16 bytes; the
+// channel counts are multiples of 16)
 template <int D>
-__global__ void k_upsample(const bf16* __restrict__ in, int Cin, bf16* __restrict__ out, int Cs, Box fine) {
-  const Box c{fine.X / 2, fine.Y / 2, D == 3 ? fine.Z / 2 : 1};
-  const long long n = (long long)fine.X * fine.Y * fine.Z * Cin;
+__global__ void k_concat(const bf16* __restrict__ up, int Cup, const bf16* __restrict__ skip, int Cs,
+                         bf16* __restrict__ out, Box fine) {
+  const int cx = fine.X / 2, cy = fine.Y / 2, q8 = (Cup + Cs) / 8, u8 = Cup / 8;
+  const long long n = (long long)fine.X * fine.Y * fine.Z * q8;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(t % Cin);
-    long long p = t / Cin;
-    int i, j, k;
-    coords(fine, p, i, j, k);
-    long long P = (long long)(i / 2) + (long long)c.X * ((long long)(j / 2) + (long long)c.Y * (k / 2));
-    out[p * Cs + ch] = in[P * Cin + ch];
+    const long long p = t / q8;
+    const int ch = (int)(t - p * q8);
+    uint4 v;
+    if (ch < u8) {
+      const int pi = (int)p, r = pi / fine.X, i = pi - r * fine.X, k = r / fine.Y, j = r - k * fine.Y;
+      const long long P = (i >> 1) + (long long)cx * ((j >> 1) + (long long)cy * (k >> 1));
+      v = reinterpret_cast<const uint4*>(up + P * Cup)[ch];
+    } else {
+      v = reinterpret_cast<const uint4*>(skip + p * Cs)[ch - u8];
+    }
+    reinterpret_cast<uint4*>(out)[t] = v;
   }
-}
-
-// copy C channels of src (stride C) into channels [off, off+C) of dst (stride Cs)
-__global__ void k_copy_channels(const bf16* __restrict__ src, int C, bf16* __restrict__ dst, int Cs, int off, long long P) {
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < P * C; t += (long long)gridDim.x * blockDim.x)
-    dst[(t / C) * Cs + off + t % C] = src[t];
 }
 
 // head: y[p] = sum_c h[p, c] w[c] + b (FP32 output)
@@ -110,38 +113,53 @@ __global__ void k_head_bwd(const bf16* __restrict__ h, const float* __restrict__
       gh[p * 16 + c] = __float2bfloat16_rn(g * w[c]);
     }
   }
+  // one atomic per block and value: the sums end in 17 words
+  __shared__ float sh[8][17];
   for (int off = 16; off > 0; off >>= 1) {
     ab += __shfl_xor_sync(0xffffffffu, ab, off);
     for (int c = 0; c < 16; ++c) aw[c] += __shfl_xor_sync(0xffffffffu, aw[c], off);
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicAdd(gb, ab);
-    for (int c = 0; c < 16; ++c) atomicAdd(gw + c, aw[c]);
+    sh[threadIdx.x >> 5][16] = ab;
+    for (int c = 0; c < 16; ++c) sh[threadIdx.x >> 5][c] = aw[c];
+  }
+  __syncthreads();
+  if (threadIdx.x < 17) {
+    float s = 0.f;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w][threadIdx.x];
+    atomicAdd(threadIdx.x < 16 ? gw + threadIdx.x : gb, s);
   }
 }
 
-// ReLU backward in place: g *= (y > 0)
-__global__ void k_relu_bwd(bf16* __restrict__ g, const bf16* __restrict__ y, long long n) {
-  const bf16 z = __float2bfloat16_rn(0.f);
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
-    if (!(__bfloat162float(y[t]) > 0.f)) g[t] = z;
-}
-
-// bias gradient: gb[c] += sum_p g[p, c]
-__global__ void k_bias_grad(const bf16* __restrict__ g, int C, long long P, float* __restrict__ gb) {
+// ReLU backward in place, g *= (y > 0), and the bias gradient gb[c] += sum_p
+// g[p, c] of the result in the same pass: a thread keeps 8 channels (16 bytes)
+// of every (blockDim C / 8)-th point; blockDim a multiple of C / 8, dynamic
+// shared memory blockDim * 8 floats
+__global__ void k_relu_bias_bwd(bf16* __restrict__ g, const bf16* __restrict__ y, int C, long long P,
+                                float* __restrict__ gb) {
   extern __shared__ float sh[];
-  const int c = threadIdx.x % C;
-  const int rows = blockDim.x / C;
-  const int r = threadIdx.x / C;
-  float acc = 0.f;
-  if (r < rows)
-    for (long long p = (long long)blockIdx.x * rows + r; p < P; p += (long long)gridDim.x * rows)
-      acc += __bfloat162float(g[p * C + c]);
-  sh[threadIdx.x] = acc;
+  const int q8 = C / 8, ch = threadIdx.x % q8, rows = blockDim.x / q8, r = threadIdx.x / q8;
+  float acc[8] = {};
+  for (long long p = (long long)blockIdx.x * rows + r; p < P; p += (long long)gridDim.x * rows) {
+    uint4* gp = reinterpret_cast<uint4*>(g + p * C) + ch;
+    uint4 gv = *gp;
+    const uint4 yv = reinterpret_cast<const uint4*>(y + p * C)[ch];
+    bf16* ge = reinterpret_cast<bf16*>(&gv);
+    const bf16* ye = reinterpret_cast<const bf16*>(&yv);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (!(__bfloat162float(ye[i]) > 0.f)) ge[i] = __float2bfloat16_rn(0.f);
+      acc[i] += __bfloat162float(ge[i]);
+    }
+    *gp = gv;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sh[i * blockDim.x + threadIdx.x] = acc[i];
   __syncthreads();
   if (threadIdx.x < C) {
+    const int i = threadIdx.x % 8, c8 = threadIdx.x / 8;
     float s = 0.f;
-    for (int q = 0; q < rows; ++q) s += sh[q * C + threadIdx.x];
+    for (int q = 0; q < rows; ++q) s += sh[i * blockDim.x + q * q8 + c8];
     atomicAdd(gb + threadIdx.x, s);
   }
 }
@@ -312,26 +330,34 @@ void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const fl
           int ostride, int ooff, int relu) {
   if (N->tensor_path == 1 && cin % 16 == 0 && cout % 16 == 0 && cout >= 16 && cout <= 256 && N->tc_err) {
     const Box bx = N->box[lev];
-    const int hsmem = tc_halo_smem_bytes(N->d, cin, cout);
-    if (bx.X % 8 == 0 && hsmem <= kTcHaloMaxSmem) {
-      // every tap in shared memory: one MMA stream per CTA of 8 x 16 points
-      const int blocks = (bx.X / 8) * ((bx.Y + 15) / 16) * bx.Z;
+    const int nbuf = tc_halo_bufs(N->d, cin, cout);
+    if (bx.X % 8 == 0 && nbuf > 0) {
+      // every tap in shared memory: one MMA stream per tile of 8 x 16 points,
+      // as many CTAs as the SMs hold
+      const int hsmem = tc_halo_smem_bytes(N->d, cin, cout, nbuf);
+      const int tiles = (bx.X / 8) * ((bx.Y + 15) / 16) * bx.Z;
+      const int per_sm = std::min(227 * 1024 / (hsmem + 1024), 512 / tc_cols(cout));
+      const int blocks = std::min(tiles, 152 * std::max(1, per_sm));
       if (N->d == 3)
-        k_conv_fwd_tc_halo<3><<<blocks, kTcM, hsmem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu,
-                                                                  bx, tc_cols(cout), N->tc_err);
+        k_conv_fwd_tc_halo<3><<<blocks, kTcHaloThreads, hsmem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx,
+                                                                  nbuf, tc_cols(cout), N->tc_err);
       else
-        k_conv_fwd_tc_halo<2><<<blocks, kTcM, hsmem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu,
-                                                                  bx, tc_cols(cout), N->tc_err);
+        k_conv_fwd_tc_halo<2><<<blocks, kTcHaloThreads, hsmem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx,
+                                                                  nbuf, tc_cols(cout), N->tc_err);
       return;
     }
-    const int blocks = (int)((N->P[lev] + kTcM - 1) / kTcM);
-    const int smem = tc_smem_bytes(cin, cout);
-    if (N->d == 3)
-      k_conv_fwd_tc<3><<<blocks, kTcM, smem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx,
-                                                          tc_cols(cout), N->tc_err);
-    else
-      k_conv_fwd_tc<2><<<blocks, kTcM, smem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx,
-                                                          tc_cols(cout), N->tc_err);
+    const long long blocks = (N->P[lev] + kTcM - 1) / kTcM;
+    const int nt = tc_slice(blocks, cout), smem = tc_smem_bytes(cin, nt);
+    const dim3 g((unsigned)blocks, (unsigned)(cout / nt), 1);
+#define HB_TC(DD, SS) \
+  k_conv_fwd_tc<DD, SS><<<g, kTcThreads, smem, N->stream>>>(in, cin, W, b, cout, nt, out, ostride, ooff, relu, bx, tc_cols(nt), N->tc_err)
+    const int S = tc_stages(cin, nt);
+    if (N->d == 3) {
+      if (S == 4) HB_TC(3, 4); else if (S == 3) HB_TC(3, 3); else HB_TC(3, 2);
+    } else {
+      if (S == 4) HB_TC(2, 4); else if (S == 3) HB_TC(2, 3); else HB_TC(2, 2);
+    }
+#undef HB_TC
     return;
   }
   const int NT = cout / 8;
@@ -348,9 +374,11 @@ void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const fl
 }
 
 void wgrad(hbf_unet* N, int lev, const bf16* x, int cin, const bf16* gz, int cout, float* gW) {
-  const int chunk = 4096;
-  const int pairs = (cin / 8) * (cout / 16);
-  dim3 g((unsigned)((pairs + 3) / 4), (unsigned)taps(N->d), (unsigned)((N->P[lev] + chunk - 1) / chunk));
+  const int tiles = ((cin + kWgTile - 1) / kWgTile) * ((cout + kWgTile - 1) / kWgTile) * taps(N->d);
+  // chunks of whole stages, about eight blocks per SM in all
+  const long long want = std::max(1, 8 * 152 / tiles), stages = (N->P[lev] + kWgPts - 1) / kWgPts;
+  const int chunk = (int)((stages + want - 1) / want) * kWgPts;
+  dim3 g((unsigned)(tiles / taps(N->d)), (unsigned)taps(N->d), (unsigned)((N->P[lev] + chunk - 1) / chunk));
   if (N->d == 3)
     k_conv_wgrad<3><<<g, 128, 0, N->stream>>>(x, cin, gz, cout, gW, N->box[lev], chunk);
   else
@@ -362,9 +390,9 @@ void wgrad(hbf_unet* N, int lev, const bf16* x, int cin, const bf16* gz, int cou
 // (skipped when null)
 void layer_back(hbf_unet* N, int k, int lev, const bf16* in, const bf16* out, bf16* g_out, bf16* g_in) {
   auto& Ly = N->L[k];
-  const long long n = N->P[lev] * Ly.cout;
-  k_relu_bwd<<<grid(n), kThreads, 0, N->stream>>>(g_out, out, n);
-  k_bias_grad<<<grid(N->P[lev] / 8 + 1), 256, 256 * sizeof(float), N->stream>>>(g_out, Ly.cout, N->P[lev], Ly.gb);
+  const int rows = 256 / (Ly.cout / 8);  // points per block and step
+  const int rb = (int)std::min<long long>((N->P[lev] + 2 * rows - 1) / (2 * rows), 304);
+  k_relu_bias_bwd<<<rb, 256, 256 * 8 * sizeof(float), N->stream>>>(g_out, out, Ly.cout, N->P[lev], Ly.gb);
   wgrad(N, lev, in, Ly.cin, g_out, Ly.cout, Ly.gW);
   if (g_in) conv(N, lev, g_out, Ly.cout, Ly.Wt, nullptr, Ly.cin, g_in, Ly.cin, 0, 0);
 }
@@ -405,13 +433,11 @@ void forward(hbf_unet* N, const float* x) {
   const int cs[3] = {c0, c1, c2};
   for (int l = 2; l >= 0; --l) {
     const int Cs = cup + cs[l];
-    const long long n = N->P[l] * cup;
+    const long long n = N->P[l] * (Cs / 8);
     if (N->d == 3)
-      k_upsample<3><<<grid(n), kThreads, 0, N->stream>>>(up, cup, N->cat[l], Cs, N->box[l]);
+      k_concat<3><<<grid(n), kThreads, 0, N->stream>>>(up, cup, N->e[l][1], cs[l], N->cat[l], N->box[l]);
     else
-      k_upsample<2><<<grid(n), kThreads, 0, N->stream>>>(up, cup, N->cat[l], Cs, N->box[l]);
-    k_copy_channels<<<grid(N->P[l] * cs[l]), kThreads, 0, N->stream>>>(N->e[l][1], cs[l], N->cat[l], Cs, cup,
-                                                                        N->P[l]);
+      k_concat<2><<<grid(n), kThreads, 0, N->stream>>>(up, cup, N->e[l][1], cs[l], N->cat[l], N->box[l]);
     const int ka = 8 + 2 * (2 - l), kb = ka + 1;
     conv(N, l, N->cat[l], Cs, L[ka].Wb, L[ka].b, cs[l], N->dc[l][0], cs[l], 0, 1);
     conv(N, l, N->dc[l][0], cs[l], L[kb].Wb, L[kb].b, cs[l], N->dc[l][1], cs[l], 0, 1);
@@ -670,7 +696,7 @@ int hbf_unet_create(hbf_unet** out, int dim, const int64_t n[3], int train, uint
   if (!N) return HBF_ERR_OOM;
   N->d = dim;
   N->train = train != 0;
-  N->nlaunch_fwd = 25;  // pack, 14 convolutions, 3 pools, 3 upsamples, 3 copies, head
+  N->nlaunch_fwd = 22;  // pack, 14 convolutions, 3 pools, 3 concatenations, head
   N->stream = (cudaStream_t)stream;
   for (int l = 0; l < 4; ++l) {
     const int s = 1 << l;
@@ -813,14 +839,17 @@ int hbf_unet_get_grads(hbf_unet* N, float* dst) { return copy_params(N, dst, 1, 
 int hbf_unet_set_tensor_path(hbf_unet* N, int path) {
   if (!N || (path != 0 && path != 1)) return HBF_ERR_ARG;
   if (path == 1) {
-    // the largest tile: 128 points plus 256 output channels, of 256 input channels
-    const int bytes = tc_smem_bytes(256, 256);
-    if (cudaFuncSetAttribute(k_conv_fwd_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-        cudaFuncSetAttribute(k_conv_fwd_tc<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess ||
-        cudaFuncSetAttribute(k_conv_fwd_tc_halo<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcHaloMaxSmem) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(k_conv_fwd_tc_halo<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcHaloMaxSmem) !=
-            cudaSuccess) {
+    void (*const kern[])(const bf16*, int, const bf16*, const float*, int, int, bf16*, int, int, int, Box, int,
+                         int*) = {k_conv_fwd_tc<2, 2>, k_conv_fwd_tc<2, 3>, k_conv_fwd_tc<2, 4>,
+                                  k_conv_fwd_tc<3, 2>, k_conv_fwd_tc<3, 3>, k_conv_fwd_tc<3, 4>};
+    cudaError_t e = cudaSuccess;
+    for (auto k : kern)
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_conv_fwd_tc_halo<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_conv_fwd_tc_halo<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);
+    if (e != cudaSuccess) {
       cudaGetLastError();
       N->err = "tcgen05 convolution: shared-memory attribute";
       return HBF_ERR_CUDA;
