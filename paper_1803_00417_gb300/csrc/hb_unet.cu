@@ -328,7 +328,7 @@ int taps(int d) { return d == 3 ? 27 : 9; }
 
 void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const float* b, int cout, bf16* out,
           int ostride, int ooff, int relu) {
-  if (N->tensor_path == 1 && cin % 16 == 0 && cout % 16 == 0 && cout >= 16 && cout <= 256 && N->tc_err) {
+  if (N->tensor_path == 1 && cin % 16 == 0 && cin <= 192 && cout % 16 == 0 && N->tc_err) {
     const Box bx = N->box[lev];
     const int nbuf = tc_halo_bufs(N->d, cin, cout);
     if (bx.X % 8 == 0 && nbuf > 0) {
@@ -349,13 +349,13 @@ void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const fl
     const long long blocks = (N->P[lev] + kTcM - 1) / kTcM;
     const int nt = tc_slice(blocks, cout), smem = tc_smem_bytes(cin, nt);
     const dim3 g((unsigned)blocks, (unsigned)(cout / nt), 1);
-#define HB_TC(DD, SS) \
-  k_conv_fwd_tc<DD, SS><<<g, kTcThreads, smem, N->stream>>>(in, cin, W, b, cout, nt, out, ostride, ooff, relu, bx, tc_cols(nt), N->tc_err)
-    const int S = tc_stages(cin, nt);
+#define HB_TC(DD, KQ) \
+  k_conv_fwd_tc<DD, KQ><<<g, kTcThreads, smem, N->stream>>>(in, cin, W, b, cout, nt, out, ostride, ooff, relu, bx, tc_cols(nt), N->tc_err)
+    const int kq = (cin + 31) / 32;
     if (N->d == 3) {
-      if (S == 4) HB_TC(3, 4); else if (S == 3) HB_TC(3, 3); else HB_TC(3, 2);
+      if (kq == 1) HB_TC(3, 1); else if (kq == 2) HB_TC(3, 2); else if (kq == 3) HB_TC(3, 3); else if (kq == 4) HB_TC(3, 4); else HB_TC(3, 6);
     } else {
-      if (S == 4) HB_TC(2, 4); else if (S == 3) HB_TC(2, 3); else HB_TC(2, 2);
+      if (kq == 1) HB_TC(2, 1); else if (kq == 2) HB_TC(2, 2); else if (kq == 3) HB_TC(2, 3); else if (kq == 4) HB_TC(2, 4); else HB_TC(2, 6);
     }
 #undef HB_TC
     return;
@@ -840,8 +840,9 @@ int hbf_unet_set_tensor_path(hbf_unet* N, int path) {
   if (!N || (path != 0 && path != 1)) return HBF_ERR_ARG;
   if (path == 1) {
     void (*const kern[])(const bf16*, int, const bf16*, const float*, int, int, bf16*, int, int, int, Box, int,
-                         int*) = {k_conv_fwd_tc<2, 2>, k_conv_fwd_tc<2, 3>, k_conv_fwd_tc<2, 4>,
-                                  k_conv_fwd_tc<3, 2>, k_conv_fwd_tc<3, 3>, k_conv_fwd_tc<3, 4>};
+                         int*) = {k_conv_fwd_tc<2, 1>, k_conv_fwd_tc<2, 2>, k_conv_fwd_tc<2, 3>, k_conv_fwd_tc<2, 4>,
+                                  k_conv_fwd_tc<2, 6>, k_conv_fwd_tc<3, 1>, k_conv_fwd_tc<3, 2>, k_conv_fwd_tc<3, 3>,
+                                  k_conv_fwd_tc<3, 4>, k_conv_fwd_tc<3, 6>};
     cudaError_t e = cudaSuccess;
     for (auto k : kern)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem);

@@ -1,8 +1,8 @@
 // The U-Net convolution on the 5th-generation tensor cores (tcgen05): an
 // implicit GEMM D[p, co] = sum_tap sum_ci X[p + o_tap, ci] W[tap, co, ci]
 // with M = 128 points per CTA, N = a slice of Cout, K = Cin per tap.  The
-// operands are staged in shared memory by cp.async (K-major, no swizzle: core
-// matrices of 8 rows x 16 bytes), one thread issues the tcgen05.mma (BF16 in,
+// operands are staged in shared memory (K-major, no swizzle: core matrices of
+// 8 rows x 16 bytes), one thread issues the tcgen05.mma (BF16 in,
 // FP32 accumulate in TMEM), tcgen05.commit arrives on an mbarrier that the CTA
 // waits on (bounded); the epilogue reads the accumulators with tcgen05.ld
 // (warp w owns TMEM lanes 32w .. 32w+31, i.e. its 32 points), adds the bias,
@@ -160,63 +160,55 @@ constexpr int kTcMaxSmem = 200 * 1024;  // dynamic shared memory a convolution m
 
 // ---------------------------------------------------------------------------
 // General variant: any box, any layer.  The CTA takes 128 points and nt output
-// channels; tap t's operands (the 128 shifted input rows and the nt x Cin
-// weights) go to stage t mod S of a ring of S stages, S - 1 taps ahead of the
-// MMAs, so that the taps' global latencies overlap: staged one at a time a tap
-// took 2.4 us, of which the MMAs are a few tens of ns.  16 warps stage (with
-// one per scheduler the staging's own instructions took 1.2 us a tap).  nt is
-// a slice of Cout where the points alone leave SMs without a CTA (the coarse
-// levels: 1 to 46 CTAs of 128 points), and each slice then stages fewer
-// weights.
+// channels.  Per tap its 16 warps bring the 128 shifted input rows and the nt x
+// Cin weights to one of two shared-memory stages, through registers: the loads
+// of the next two taps are in flight while the current tap's MMAs run.  (By
+// cp.async a tap took 1.15 us whatever its size and the ring's depth: the
+// proxy fence that makes the stage visible to the tensor cores also waits for
+// the copies still in flight.  Staged by four warps one tap at a time it took
+// 2.4 us.)  nt is a slice of Cout where the points alone leave SMs without a
+// CTA (the coarse levels: 1 to 46 CTAs of 128 points), and each slice then
+// stages fewer weights.
 // ---------------------------------------------------------------------------
 constexpr int kTcThreads = 512;
 __host__ __device__ constexpr int tc_stage_bytes(int cin, int nt) { return (kTcM + nt) * cin * 2; }
-// stages of the ring: 4 while two CTAs share an SM, else 3, else 2
-__host__ __device__ constexpr int tc_stages(int cin, int nt) {
-  const int st = tc_stage_bytes(cin, nt);
-  return 4 * st + kTcSlack <= 110 * 1024 ? 4 : (3 * st + kTcSlack <= kTcMaxSmem ? 3 : 2);
-}
-__host__ __device__ constexpr int tc_smem_bytes(int cin, int nt) {
-  return tc_stages(cin, nt) * tc_stage_bytes(cin, nt) + kTcSlack;
-}
+__host__ __device__ constexpr int tc_smem_bytes(int cin, int nt) { return 2 * tc_stage_bytes(cin, nt) + kTcSlack; }
 // output channels per CTA: all of them, or the largest slice (16 at least)
 // that gives every SM a CTA
 __host__ __device__ constexpr int tc_slice(long long blocks, int cout) {
   int nt = cout;
-  while (nt % 32 == 0 && blocks * (cout / nt) < 152) nt /= 2;
+  while (nt % 32 == 0 && (nt > kTcM || blocks * (cout / nt) < 152)) nt /= 2;
   return nt;
 }
 
 // out[p, out_off + co] = act(bias[co] + sum_tap sum_ci in[p + o_tap, ci] W[tap, co, ci])
-// for co in slice blockIdx.y of nt channels.  Requires Cin % 16 == 0, nt % 16
-// == 0, 16 <= nt <= 256; tcols = tc_cols(nt), S = tc_stages(Cin, nt).  *err is
-// set when a wait on the tensor cores gives up (the outputs of that CTA are
-// then not written).
-template <int D, int S>
+// for co in slice blockIdx.y of nt channels.  Requires Cin % 16 == 0, Cin <=
+// 32 KQ, nt % 16 == 0, 16 <= nt <= 128; tcols = tc_cols(nt).  *err is set when
+// a wait on the tensor cores gives up (the outputs of that CTA are then not
+// written).
+template <int D, int KQ>
 __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const bf16* __restrict__ in, int Cin,
-                                                      const bf16* __restrict__ W, const float* __restrict__ bias,
-                                                      int Cout, int nt, bf16* __restrict__ out, int out_stride,
-                                                      int out_off, int relu, Box box, int tcols,
-                                                      int* __restrict__ err) {
+                                                            const bf16* __restrict__ W,
+                                                            const float* __restrict__ bias, int Cout, int nt,
+                                                            bf16* __restrict__ out, int out_stride, int out_off,
+                                                            int relu, Box box, int tcols, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bars[S + 1];  // one per stage, and one for the last MMA
+  __shared__ __align__(8) uint64_t bars[3];  // one per stage, and one for the last MMA
   __shared__ uint32_t tmem_slot;
+  constexpr int T = D == 3 ? 27 : 9;
   const int tid = threadIdx.x;
   const int KC = Cin / 8;  // 16-byte chunks per row
   const int co0 = blockIdx.y * nt;
   const long long P = (long long)box.X * box.Y * box.Z;
-  const long long p = (long long)blockIdx.x * kTcM + (tid & (kTcM - 1));
-  const bool valid = p < P;
-  const uint32_t tmem = tc_setup(&tmem_slot, bars, S + 1, tcols);
+  const uint32_t tmem = tc_setup(&tmem_slot, bars, 3, tcols);
   const uint32_t idesc = tc_idesc(kTcM, nt);
   const uint32_t base = smem_u32(smem), stage = (uint32_t)tc_stage_bytes(Cin, nt), boff = (uint32_t)kTcM * Cin * 2;
   const uint32_t dlo = tc_desc_lo(base, 128u), dhi = tc_desc_hi((uint32_t)KC * 128u);  // next 8-row group: KC chunks on
-  constexpr int T = D == 3 ? 27 : 9;
   // Staging: warp w copies rows 8 w .. 8 w + 7, 4 chunks at a time (lane: row
   // l % 8, chunk l / 8), so that it touches 8 lines of global memory at a time
-  // (one row per lane touched 32) and writes shared memory without conflicts.
-  // Bit t of vm tells that tap t of the lane's row of A lies in the box (taps
-  // run over (x, y(, z)) offsets, x slowest: three bits per axis).
+  // and writes shared memory without conflicts.  Bit t of vm tells that tap t
+  // of the lane's row of A lies in the box (taps run over (x, y(, z)) offsets,
+  // x slowest: three bits per axis).
   const int lane = tid & 31, c4 = lane >> 3, row = (tid >> 5) * 8 + (lane & 7);
   const long long pr = (long long)blockIdx.x * kTcM + row;
   uint32_t vm = 0u;
@@ -229,40 +221,46 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const bf16* __restri
     };
     vm = D == 3 ? spread(bx, spread(by, bz, 3), 9) : spread(bx, by, 3);
   }
-  const uint32_t arow = base + (uint32_t)((row >> 3) * KC + c4) * 128u + (uint32_t)(row & 7) * 16u;
+  const size_t place = (size_t)((row >> 3) * KC + c4) * 128u + (size_t)(row & 7) * 16u;
   const bf16* const wrow = W + ((size_t)co0 + row) * Cin + 8 * c4;
-  auto load = [&](int tap) {
-    const uint32_t so = (uint32_t)(tap % S) * stage;
+  uint4 ra[2][KQ], rb[2][KQ];
+  auto fetch = [&](int tap, uint4* a, uint4* b) {
     int o[3];
     tap_offset<D>(tap, o);
     const long long sh = (long long)o[0] + (long long)box.X * ((long long)o[1] + (long long)box.Y * o[2]);
     const bool in_box = (vm >> tap) & 1u;  // zeros outside
-    const bf16* src = in_box ? in + (pr + sh) * Cin + 8 * c4 : in;
-    for (int k = 0; k + c4 < KC; k += 4) cp_async16(arow + so + (uint32_t)k * 128u, src + 8 * k, in_box);
-    if (row < nt) {
-      const bf16* wt = wrow + (size_t)tap * Cout * Cin;
-      for (int k = 0; k + c4 < KC; k += 4) cp_async16(arow + so + boff + (uint32_t)k * 128u, wt + 8 * k, true);
-    }
-    for (int r = row + kTcM; r < nt; r += kTcM)  // more than 128 output channels
-      for (int k = c4; k < KC; k += 4)
-        cp_async16(base + so + boff + (uint32_t)((r >> 3) * KC + k) * 128u + (uint32_t)(r & 7) * 16u,
-                   W + ((size_t)tap * Cout + co0 + r) * Cin + 8 * k, true);
-  };
+    const bf16* src = in + (pr + sh) * Cin + 8 * c4;
+    const bf16* wt = wrow + (size_t)tap * Cout * Cin;
 #pragma unroll
-  for (int t = 0; t < S - 1; ++t) {
-    load(t);
-    cp_async_commit();
-  }
+    for (int k = 0; k < KQ; ++k) {
+      a[k] = b[k] = make_uint4(0u, 0u, 0u, 0u);
+      if (4 * k + c4 < KC) {
+        if (in_box) a[k] = *reinterpret_cast<const uint4*>(src + 32 * k);
+        if (row < nt) b[k] = *reinterpret_cast<const uint4*>(wt + 32 * k);
+      }
+    }
+  };
   bool ok = true;  // false once a wait gave up: nothing is staged any more
-  for (int tap = 0; tap < T; ++tap) {
-    cp_async_wait<S - 2>();
-    // make the staged operands visible to the tensor cores
+  auto step = [&](int tap, uint4* a, uint4* b) {
+    const int s = tap & 1;
+    // the stage's previous MMAs, two taps back
+    if (tap >= 2 && ok) ok = mbar_wait_parity(smem_u32(bars + s), (uint32_t)((tap >> 1) - 1) & 1u);
+    if (ok) {
+      unsigned char* dst = smem + (size_t)s * stage + place;
+#pragma unroll
+      for (int k = 0; k < KQ; ++k)
+        if (4 * k + c4 < KC) {
+          *reinterpret_cast<uint4*>(dst + (size_t)k * 512u) = a[k];
+          if (row < nt) *reinterpret_cast<uint4*>(dst + boff + (size_t)k * 512u) = b[k];
+        }
+    }
+    if (tap + 2 < T) fetch(tap + 2, a, b);
+    // make the stage visible to the tensor cores
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncthreads();
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      const uint32_t sa = (uint32_t)(tap % S) * (stage >> 4);
-      const uint32_t alo = dlo + sa, blo = dlo + sa + (boff >> 4);
+      const uint32_t alo = dlo + (uint32_t)s * (stage >> 4), blo = alo + (boff >> 4);
       if (tap == 0)
         tc_mma<true>(tmem, alo, dhi, blo, dhi, idesc);
       else
@@ -270,25 +268,26 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const bf16* __restri
 #pragma unroll 4
       for (int kc = 1; kc < KC / 2; ++kc)  // K = 16: two chunks of 128 bytes per core-matrix row group
         tc_mma<false>(tmem, alo + 16u * kc, dhi, blo + 16u * kc, dhi, idesc);
-      tc_commit(smem_u32(bars + tap % S));
-      if (tap == T - 1) tc_commit(smem_u32(bars + S));
+      tc_commit(smem_u32(bars + s));
+      if (tap == T - 1) tc_commit(smem_u32(bars + 2));
     }
-    if (tap + S - 1 < T) {
-      // the next load takes the previous tap's stage
-      if (tap > 0 && ok) ok = mbar_wait_parity(smem_u32(bars + (tap - 1) % S), (uint32_t)((tap - 1) / S) & 1u);
-      if (ok) load(tap + S - 1);
-    }
-    cp_async_commit();
+  };
+  fetch(0, ra[0], rb[0]);
+  fetch(1, ra[1], rb[1]);
+#pragma unroll 1
+  for (int tap = 0; tap < T; tap += 2) {
+    step(tap, ra[0], rb[0]);
+    if (tap + 1 < T) step(tap + 1, ra[1], rb[1]);
   }
-  cp_async_wait<0>();
-  if (ok) ok = mbar_wait_parity(smem_u32(bars + S), 0u);
+  if (ok) ok = mbar_wait_parity(smem_u32(bars + 2), 0u);
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   if (ok) {
-    tc_epilogue(tmem, nt, bias ? bias + co0 : nullptr, relu, out + p * out_stride + out_off + co0, valid);
+    const long long p = (long long)blockIdx.x * kTcM + (tid & (kTcM - 1));
+    tc_epilogue(tmem, nt, bias ? bias + co0 : nullptr, relu, out + p * out_stride + out_off + co0, p < P);
   } else {
     if (tid == 0) atomicExch(err, 1);
-    mbar_wait_parity(smem_u32(bars + S), 0u, kTcDrainLimit);  // drain before TMEM is freed
+    mbar_wait_parity(smem_u32(bars + 2), 0u, kTcDrainLimit);  // drain before TMEM is freed
   }
   tc_release(tmem, tcols);
 }
