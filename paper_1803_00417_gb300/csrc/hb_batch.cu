@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(128) k_batch_bottom(const BottomArg<T>* __rest
 // dense bottom operator of the viscous problem (it changes with eta and dt
 // every step) and its inverse, for every cavity in one launch each
 struct DenseArg {
-  double *X, *M, *A, *Minv;
+  double *X, *M, *Minv;
   int n, m;
   const double* ef[3];
   Geom g;
@@ -269,7 +269,7 @@ __global__ void k_batch_gauss_jordan(const DenseArg* __restrict__ args, int ncav
   const int c = blockIdx.x;
   if (c >= ncav) return;
   const DenseArg& a = args[c];
-  gauss_jordan_block(a.M, a.m, a.A, a.Minv);
+  gauss_jordan_block(a.M, a.m, a.Minv);
 }
 
 }  // namespace batch
@@ -835,7 +835,6 @@ struct SolversT : Solvers {
       std::memset(&a, 0, sizeof a);
       a.X = c->dX;
       a.M = c->dM;
-      a.A = c->dA;
       a.Minv = c->dense[0].Minv;
       a.n = a.m = D * L.g.ncell;
       for (int d = 0; d < D; ++d) a.ef[d] = L.ef[d];
@@ -948,7 +947,11 @@ struct SolversT : Solvers {
       for (int l = 0; l < B->maxlev; ++l) run<OpFacesF32>(B, facesF[l], B->H[l][kFaces], B->mask_all);
     for (int l = 0; l < B->maxlev; ++l) run<OpViscInv<D, T>>(B, vph.lv[l], B->A[l][kCells], B->mask_all);
     k_batch_dense_build<D><<<dim3(kDenseMax, B->ncav), 128, 0, B->stream>>>((const DenseArg*)dense, B->ncav);
-    k_batch_gauss_jordan<<<B->ncav, 256, 0, B->stream>>>((const DenseArg*)dense, B->ncav);
+    int m = 1;
+    for (int c = 0; c < B->ncav; ++c) m = std::max(m, D * B->cav[c]->lv.back().g.ncell);
+    cudaFuncSetAttribute(k_batch_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)gauss_jordan_smem(kDenseMax + 1));
+    k_batch_gauss_jordan<<<B->ncav, 256, gauss_jordan_smem(m), B->stream>>>((const DenseArg*)dense, B->ncav);
     B->nlaunch += 2;
   }
 

@@ -186,6 +186,7 @@ struct hbf_ctx {
         *fkph = nullptr, *fksh = nullptr, *fke = nullptr;
   // reductions
   double* partial = nullptr;  // 2 kRedBlocks doubles
+  unsigned* ticket = nullptr; // finished blocks of the running reduction
   double* dres = nullptr;     // device result slot(s)
   double* hres = nullptr;     // pinned host result
   std::vector<hb::Level> lv;
@@ -196,7 +197,7 @@ struct hbf_ctx {
   // fused V-cycle tail of the solves
   int tail_cells = -1;  // it starts at the first level with at most this many cells (-1: the library's rule)
   hb::TailPlan tail[3]; // by problem kind
-  double *dX = nullptr, *dM = nullptr, *dA = nullptr;  // build scratch
+  double *dX = nullptr, *dM = nullptr;  // build scratch
 };
 
 namespace hb {

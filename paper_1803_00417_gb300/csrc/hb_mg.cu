@@ -28,68 +28,108 @@
 namespace hb {
 
 // ---------------------------------------------------------------------------
-// deterministic reductions: fixed grid, per-block partials, one final block
+// deterministic reductions: a grid fixed by the length, per-block partials,
+// combined in a fixed order by the last block to finish
 // ---------------------------------------------------------------------------
+// MODE 0: max |x| (non-finite -> +inf), 1: sum
+template <int MODE>
+__device__ __forceinline__ double red_combine(double a, double b) {
+  return MODE == 0 ? fmax(a, b) : a + b;
+}
+
+// the block's value of acc (thread 0 returns it)
+template <int MODE>
+__device__ __forceinline__ double block_reduce(double acc) {
+  __shared__ double sh[kThreads / 32];
+  for (int off = 16; off > 0; off >>= 1) acc = red_combine<MODE>(acc, __shfl_xor_sync(0xffffffffu, acc, off));
+  __syncthreads();  // sh may still be read from an earlier call
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  double v = 0.0;
+  if (threadIdx.x < 32) {
+    v = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
+    for (int off = 16; off > 0; off >>= 1) v = red_combine<MODE>(v, __shfl_xor_sync(0xffffffffu, v, off));
+  }
+  return v;
+}
+
+// Where a reduction's results go: part holds the blocks' partials (two runs of
+// gridDim for a two-result kernel), ticket counts finished blocks (atomicInc
+// wraps it back to 0), dev and host (pinned, or null) take the results.  A
+// second launch for the combination and a copy for the host took 4 us and 3 us
+// per reduction, and a step of a small grid makes 60 of them.
+struct RedOut {
+  double* part;
+  unsigned* ticket;
+  double* dev;
+  double* host;
+};
+
+// Ends a reduction kernel: v0 (and v1 when M1 >= 0) are the block's values in
+// thread 0.  The last block combines all partials: thread t takes t, t + 256,
+// ..., then the block's tree.
+template <int M0, int M1 = -1>
+__device__ __forceinline__ void red_finish(const RedOut& o, double v0, double v1 = 0.0) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    o.part[blockIdx.x] = v0;
+    if (M1 >= 0) o.part[gridDim.x + blockIdx.x] = v1;
+    __threadfence();
+    last = atomicInc(o.ticket, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double a0 = 0.0, a1 = 0.0;
+  for (int t = threadIdx.x; t < (int)gridDim.x; t += kThreads) {
+    a0 = red_combine<M0>(a0, __ldcg(o.part + t));
+    if (M1 >= 0) a1 = red_combine<M1 >= 0 ? M1 : 0>(a1, __ldcg(o.part + gridDim.x + t));
+  }
+  a0 = block_reduce<M0>(a0);
+  if (M1 >= 0) a1 = block_reduce<M1 >= 0 ? M1 : 0>(a1);
+  if (threadIdx.x == 0) {
+    o.dev[0] = a0;
+    if (M1 >= 0) o.dev[1] = a1;
+    if (o.host) {
+      o.host[0] = a0;
+      if (M1 >= 0) o.host[1] = a1;
+      __threadfence_system();
+    }
+  }
+}
+
+// max |v| on the bit pattern: magnitudes compare as integers, so the FP64 pipe
+// (two operations per SM and cycle) stays out of the loop; a non-finite value
+// (exponent all ones) sorts above every finite one and becomes +inf
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+  return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+__device__ __forceinline__ double bits_max(unsigned long long m) {
+  return m >= 0x7ff0000000000000ull ? (double)INFINITY : __longlong_as_double((long long)m);
+}
+
+// unaligned arrays, and the weighted nodal sum (MODE 2)
 template <int MODE>  // 0: max |x| (non-finite -> +inf), 1: sum x, 2: weighted nodal sum
-__global__ void k_reduce_partial(const double* __restrict__ x, long long n, double* __restrict__ part,
-                                 const __grid_constant__ Geom g, int dim) {
+__global__ void k_reduce_partial(const double* __restrict__ x, long long n, RedOut out, const __grid_constant__ Geom g,
+                                 int dim) {
   double acc = 0.0;
+  unsigned long long m = 0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
     double v = x[t];
     if (MODE == 0) {
-      double a = fabs(v);
-      if (!isfinite(a)) a = INFINITY;
-      acc = fmax(acc, a);
+      const unsigned long long a = abs_bits(v);
+      m = a > m ? a : m;
     } else if (MODE == 1) {
       acc += v;
     } else {
-      int e0 = g.n[0] + 1, e1 = g.n[1] + 1;
-      int i = (int)(t % e0);
-      int q = (int)(t / e0);
-      int j = q % e1;
-      int k = q / e1;
-      double w = 1.0;
-      w = node_weight(g, i, j, k, dim);
-      acc += w * v;
+      int i, j, k;
+      node_coords(g, (int)t, i, j, k);
+      acc += node_weight(g, i, j, k, dim) * v;
     }
   }
-  __shared__ double sh[kThreads / 32];
-  for (int off = 16; off > 0; off >>= 1) {
-    double o = __shfl_xor_sync(0xffffffffu, acc, off);
-    acc = MODE == 0 ? fmax(acc, o) : acc + o;
-  }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) {
-      double o = __shfl_xor_sync(0xffffffffu, v, off);
-      v = MODE == 0 ? fmax(v, o) : v + o;
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = v;
-  }
-}
-
-template <int MODE>
-__global__ void k_reduce_final(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  __shared__ double sh[32];
-  double acc = 0.0;
-  for (int t = threadIdx.x; t < nb; t += blockDim.x) acc = MODE == 0 ? fmax(acc, part[t]) : acc + part[t];
-  for (int off = 16; off > 0; off >>= 1) {
-    double o = __shfl_xor_sync(0xffffffffu, acc, off);
-    acc = MODE == 0 ? fmax(acc, o) : acc + o;
-  }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (int)(blockDim.x / 32) ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) {
-      double o = __shfl_xor_sync(0xffffffffu, v, off);
-      v = MODE == 0 ? fmax(v, o) : v + o;
-    }
-    if (threadIdx.x == 0) *out = v;
-  }
+  if (MODE == 0) acc = bits_max(m);
+  red_finish<MODE == 0 ? 0 : 1>(out, block_reduce<MODE == 0 ? 0 : 1>(acc));
 }
 
 // x -= (*sum) * inv_count  (mean removal without a host round trip)
@@ -152,75 +192,47 @@ __global__ void k_zero(T* __restrict__ x, long long n) {
       [&](long long e) { x[e] = T(0); });
 }
 
-__global__ void k_dot_partial(const double* __restrict__ a, const double* __restrict__ b, long long n,
-                              double* __restrict__ part) {
+__global__ void k_dot_partial(const double* __restrict__ a, const double* __restrict__ b, long long n, RedOut out) {
   double acc = 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     acc += a[t] * b[t];
-  __shared__ double sh[kThreads / 32];
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (threadIdx.x == 0) part[blockIdx.x] = v;
-  }
+  red_finish<1>(out, block_reduce<1>(acc));
 }
 
-// Vectorised partials of the frequent reductions: 16-byte loads, four
-// iterations unrolled so that each thread keeps several loads in flight.
-// Thread t takes the vectors t, t + T, t + 2T, ... (T threads in the grid) in
-// that order, the tail past the last whole vector goes to thread 0, and the
-// block and final sums run in a fixed order: the result is the same on every
-// run.  MODE 0: max |x| (non-finite -> +inf); 1: sum x.  x 16-byte aligned.
+// The frequent reductions with 16-byte loads, four iterations unrolled so that
+// each thread keeps several loads in flight.  Thread t takes the vectors t, t +
+// T, t + 2T, ... (T threads in the grid) in that order, the tail past the last
+// whole vector goes to thread 0, and the block and final sums run in a fixed
+// order: the result is the same on every run.  MODE 0: max |x| (non-finite ->
+// +inf); 1: sum x.  x 16-byte aligned.
 template <int MODE>
-__device__ __forceinline__ double red_op(double acc, double v) {
-  if (MODE == 0) {
-    double a = fabs(v);
-    if (!isfinite(a)) a = INFINITY;
-    return fmax(acc, a);
-  }
-  return acc + v;
-}
-
-template <int MODE>
-__device__ __forceinline__ void block_partial(double acc, double* part) {
-  __shared__ double sh[kThreads / 32];
-  for (int off = 16; off > 0; off >>= 1) {
-    double o = __shfl_xor_sync(0xffffffffu, acc, off);
-    acc = MODE == 0 ? fmax(acc, o) : acc + o;
-  }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) {
-      double o = __shfl_xor_sync(0xffffffffu, v, off);
-      v = MODE == 0 ? fmax(v, o) : v + o;
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = v;
-  }
-}
-
-template <int MODE>
-__global__ void k_reduce_partial_v(const double* __restrict__ x, long long n, double* __restrict__ part) {
+__global__ void k_reduce_partial_v(const double* __restrict__ x, long long n, RedOut out) {
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n2 = n >> 1;
   const double2* x2 = reinterpret_cast<const double2*>(x);
   double acc = 0.0;
+  unsigned long long m = 0;
+  auto take = [&](double v) {
+    if (MODE == 0) {
+      const unsigned long long a = abs_bits(v);
+      m = a > m ? a : m;
+    } else {
+      acc += v;
+    }
+  };
 #pragma unroll 4
   for (long long q = tid; q < n2; q += T) {
     const double2 v = x2[q];
-    acc = red_op<MODE>(red_op<MODE>(acc, v.x), v.y);
+    take(v.x);
+    take(v.y);
   }
-  if (tid == 0 && (n & 1)) acc = red_op<MODE>(acc, x[n - 1]);
-  block_partial<MODE>(acc, part);
+  if (tid == 0 && (n & 1)) take(x[n - 1]);
+  if (MODE == 0) acc = bits_max(m);
+  red_finish<MODE>(out, block_reduce<MODE>(acc));
 }
 
-__global__ void k_dot_partial_v(const double* __restrict__ a, const double* __restrict__ b, long long n,
-                                double* __restrict__ part) {
+__global__ void k_dot_partial_v(const double* __restrict__ a, const double* __restrict__ b, long long n, RedOut out) {
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n2 = n >> 1;
   const double2* a2 = reinterpret_cast<const double2*>(a);
@@ -232,7 +244,7 @@ __global__ void k_dot_partial_v(const double* __restrict__ a, const double* __re
     acc += u.x * v.x + u.y * v.y;
   }
   if (tid == 0 && (n & 1)) acc += a[n - 1] * b[n - 1];
-  block_partial<1>(acc, part);
+  red_finish<1>(out, block_reduce<1>(acc));
 }
 
 static inline bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
@@ -255,47 +267,53 @@ static bool split0(const hbf_ctx* c) {
          !c->staged_tx && !c->staged_op_rows && !c->fused_sweep && !(c->vnet && c->vnet_level == 0);
 }
 
+// blocks of a reduction over n elements: 2048 elements each (8 per thread),
+// kRedBlocks at most
+static inline int red_grid(long long n) {
+  const long long b = (n + 2047) / 2048;
+  return (int)(b < 1 ? 1 : (b > kRedBlocks ? kRedBlocks : b));
+}
+static inline RedOut red_out(hbf_ctx* c, double* dev, double* host) { return {c->partial, c->ticket, dev, host}; }
+
 template <int MODE>
-static int reduce_to_device(hbf_ctx* c, const double* x, long long n, double* out) {
+static int reduce_to_device(hbf_ctx* c, const double* x, long long n, double* out, double* host = nullptr) {
   if (MODE < 2 && aligned16(x))
-    launch(c, kSlotReduce, k_reduce_partial_v<MODE < 2 ? MODE : 0>, kRedBlocks, kThreads, x, n, c->partial);
+    launch(c, kSlotReduce, k_reduce_partial_v<MODE < 2 ? MODE : 0>, red_grid(n), kThreads, x, n, red_out(c, out, host));
   else
-    launch(c, kSlotReduce, k_reduce_partial<MODE>, kRedBlocks, kThreads, x, n, c->partial, c->g, c->dim);
-  launch(c, kSlotReduce, k_reduce_final<MODE>, 1, 1024, c->partial, kRedBlocks, out);
+    launch(c, kSlotReduce, k_reduce_partial<MODE>, red_grid(n), kThreads, x, n, red_out(c, out, host), c->g, c->dim);
   return cuda_check(c, cudaGetLastError(), "reduction");
 }
 
-static double read_result(hbf_ctx* c, const double* dev, int* st) {
-  cudaError_t e = cudaMemcpyAsync(c->hres, dev, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) {
-    *st = cuda_check(c, e, "reading a reduction");
-    return NAN;
-  }
-  return *c->hres;
+// waits for the stream: the kernel's results are in c->hres
+static int wait_results(hbf_ctx* c) {
+  return cuda_check(c, cudaStreamSynchronize(c->stream), "reading a reduction");
+}
+static double read_result(hbf_ctx* c, int* st) {
+  *st = wait_results(c);
+  return *st ? NAN : *c->hres;
 }
 
 double reduce_max_abs(hbf_ctx* c, const double* x, long long n, int* st) {
-  *st = reduce_to_device<0>(c, x, n, c->dres);
+  *st = reduce_to_device<0>(c, x, n, c->dres, c->hres);
   if (*st) return NAN;
-  return read_result(c, c->dres, st);
+  return read_result(c, st);
 }
 
 double reduce_dot(hbf_ctx* c, const double* a, const double* b, long long n, int* st) {
+  const RedOut o = red_out(c, c->dres, c->hres);
   if (aligned16(a) && aligned16(b))
-    launch(c, kSlotReduce, k_dot_partial_v, kRedBlocks, kThreads, a, b, n, c->partial);
+    launch(c, kSlotReduce, k_dot_partial_v, red_grid(n), kThreads, a, b, n, o);
   else
-    launch(c, kSlotReduce, k_dot_partial, kRedBlocks, kThreads, a, b, n, c->partial);
-  launch(c, kSlotReduce, k_reduce_final<1>, 1, 1024, (const double*)c->partial, kRedBlocks, c->dres);
+    launch(c, kSlotReduce, k_dot_partial, red_grid(n), kThreads, a, b, n, o);
   *st = cuda_check(c, cudaGetLastError(), "dot");
   if (*st) return NAN;
-  return read_result(c, c->dres, st);
+  return read_result(c, st);
 }
 
 double reduce_sum(hbf_ctx* c, const double* x, long long n, int* st) {
-  *st = reduce_to_device<1>(c, x, n, c->dres);
+  *st = reduce_to_device<1>(c, x, n, c->dres, c->hres);
   if (*st) return NAN;
-  return read_result(c, c->dres, st);
+  return read_result(c, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -399,6 +417,22 @@ __global__ void k_convert(TO* __restrict__ out, const TI* __restrict__ in, long 
       [&](long long e) { out[e] = TO(in[e]); });
 }
 
+// b = (float) r and x = 0: the right-hand side and the iterate of an FP32
+// correction
+__global__ void k_convert_zero(float* __restrict__ b, float* __restrict__ x, const double* __restrict__ r, long long n) {
+  for_each4(
+      n, aligned16_all(b, x, r),
+      [&](long long q) {
+        const V4<double> a = ld4(r, q);
+        st4(b, q, V4<float>{{(float)a.v[0], (float)a.v[1], (float)a.v[2], (float)a.v[3]}});
+        st4(x, q, V4<float>{{0.f, 0.f, 0.f, 0.f}});
+      },
+      [&](long long e) {
+        b[e] = (float)r[e];
+        x[e] = 0.f;
+      });
+}
+
 // x (FP64) += e (FP32): the defect-correction update
 __global__ void k_add_f32(double* __restrict__ x, const float* __restrict__ e, long long n) {
   for_each4(
@@ -413,35 +447,45 @@ __global__ void k_add_f32(double* __restrict__ x, const float* __restrict__ e, l
       [&](long long i) { x[i] += (double)e[i]; });
 }
 
-// p = r + beta (p - omega v)
+// p = r + beta (p - omega v), and z = 0 (the iterate of the preconditioner's
+// V-cycle that follows)
 template <typename T>
 __global__ void k_bicg_p(T* __restrict__ p, const T* __restrict__ r, const T* __restrict__ v, T beta, T omega,
-                         long long n) {
+                         T* __restrict__ z, long long n) {
   for_each4(
-      n, aligned16_all(p, r, v),
+      n, aligned16_all(p, r, v, z),
       [&](long long q) {
         V4<T> a = ld4(p, q);
         const V4<T> b = ld4(r, q), c = ld4(v, q);
 #pragma unroll
         for (int i = 0; i < 4; ++i) a.v[i] = b.v[i] + beta * (a.v[i] - omega * c.v[i]);
         st4(p, q, a);
+        st4(z, q, V4<T>{{T(0), T(0), T(0), T(0)}});
       },
-      [&](long long e) { p[e] = r[e] + beta * (p[e] - omega * v[e]); });
+      [&](long long e) {
+        p[e] = r[e] + beta * (p[e] - omega * v[e]);
+        z[e] = T(0);
+      });
 }
 
-// out = x - a y
+// out = x - a y, and z = 0 where z is not null
 template <typename T>
-__global__ void k_axmy(T* __restrict__ out, const T* __restrict__ x, T a, const T* __restrict__ y, long long n) {
+__global__ void k_axmy(T* __restrict__ out, const T* __restrict__ x, T a, const T* __restrict__ y, T* __restrict__ z,
+                       long long n) {
   for_each4(
-      n, aligned16_all(out, x, y),
+      n, aligned16_all(out, x, y, z),
       [&](long long q) {
         const V4<T> b = ld4(x, q), c = ld4(y, q);
         V4<T> o;
 #pragma unroll
         for (int i = 0; i < 4; ++i) o.v[i] = b.v[i] - a * c.v[i];
         st4(out, q, o);
+        if (z) st4(z, q, V4<T>{{T(0), T(0), T(0), T(0)}});
       },
-      [&](long long e) { out[e] = x[e] - a * y[e]; });
+      [&](long long e) {
+        out[e] = x[e] - a * y[e];
+        if (z) z[e] = T(0);
+      });
 }
 
 // x = x + alpha ph + omega sh
@@ -465,8 +509,7 @@ __global__ void k_bicg_x(T* __restrict__ x, const T* __restrict__ ph, const T* _
 // small fraction of its FP32 rate, so a per-element FP64 product is the
 // bottleneck of this reduction)
 constexpr int kDotRun = 64;
-__global__ void k_dot_partial_f(const float* __restrict__ a, const float* __restrict__ b, long long n,
-                                double* __restrict__ part) {
+__global__ void k_dot_partial_f(const float* __restrict__ a, const float* __restrict__ b, long long n, RedOut out) {
   double acc = 0.0;
   float run = 0.f;
   int k = 0;
@@ -480,19 +523,11 @@ __global__ void k_dot_partial_f(const float* __restrict__ a, const float* __rest
     }
   }
   acc += (double)run;
-  __shared__ double sh[kThreads / 32];
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    if (threadIdx.x == 0) part[blockIdx.x] = v;
-  }
+  red_finish<1>(out, block_reduce<1>(acc));
 }
 
 // max |x| over a float array (non-finite -> +inf)
-__global__ void k_maxabs_partial_f(const float* __restrict__ x, long long n, double* __restrict__ part) {
+__global__ void k_maxabs_partial_f(const float* __restrict__ x, long long n, RedOut out) {
   float m = 0.f;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
@@ -500,16 +535,7 @@ __global__ void k_maxabs_partial_f(const float* __restrict__ x, long long n, dou
     if (!isfinite(a)) a = INFINITY;
     m = fmaxf(m, a);
   }
-  double acc = (double)m;
-  __shared__ double sh[kThreads / 32];
-  for (int off = 16; off > 0; off >>= 1) acc = fmax(acc, __shfl_xor_sync(0xffffffffu, acc, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-    if (threadIdx.x == 0) part[blockIdx.x] = v;
-  }
+  red_finish<0>(out, block_reduce<0>((double)m));
 }
 
 // the FP32 partials with 16-byte loads: products summed in FP32 over runs of
@@ -550,8 +576,7 @@ __device__ __forceinline__ void max_abs(float& m, float v) {
   m = fmaxf(m, a);
 }
 
-__global__ void k_dot_partial_f4(const float* __restrict__ a, const float* __restrict__ b, long long n,
-                                 double* __restrict__ part) {
+__global__ void k_dot_partial_f4(const float* __restrict__ a, const float* __restrict__ b, long long n, RedOut out) {
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* a4 = reinterpret_cast<const float4*>(a);
@@ -562,13 +587,11 @@ __global__ void k_dot_partial_f4(const float* __restrict__ a, const float* __res
   if (tid == 0)
     for (long long e = n4 << 2; e < n; ++e) run = fmaf(a[e], b[e], run);
   acc += (double)run;
-  block_partial<1>(acc, part);
+  red_finish<1>(out, block_reduce<1>(acc));
 }
 
-// x.x and x.y in one pass over x (BiCGStab's t.t and t.s): partials of the
-// first in part[0, gridDim), of the second in part[gridDim, 2 gridDim)
-__global__ void k_dot2_partial_f4(const float* __restrict__ x, const float* __restrict__ y, long long n,
-                                  double* __restrict__ part) {
+// x.x and x.y in one pass over x (BiCGStab's t.t and t.s)
+__global__ void k_dot2_partial_f4(const float* __restrict__ x, const float* __restrict__ y, long long n, RedOut out) {
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -596,17 +619,14 @@ __global__ void k_dot2_partial_f4(const float* __restrict__ x, const float* __re
       rxx = fmaf(x[e], x[e], rxx);
       rxy = fmaf(x[e], y[e], rxy);
     }
-  block_partial<1>(axx + (double)rxx, part);
-  __syncthreads();
-  block_partial<1>(axy + (double)rxy, part + gridDim.x);
+  const double bxx = block_reduce<1>(axx + (double)rxx), bxy = block_reduce<1>(axy + (double)rxy);
+  red_finish<1, 1>(out, bxx, bxy);
 }
 
 // out = x - a y (BiCGStab's r = s - omega t) with max |out| (non-finite ->
-// +inf) and w.out (the next iteration's r^.r) in the same pass: partials of
-// the max in part[0, gridDim), of the dot in part[gridDim, 2 gridDim)
+// +inf) and w.out (the next iteration's r^.r) in the same pass
 __global__ void k_axmy_red_f4(float* __restrict__ out, const float* __restrict__ x, float a,
-                              const float* __restrict__ y, const float* __restrict__ w, long long n,
-                              double* __restrict__ part) {
+                              const float* __restrict__ y, const float* __restrict__ w, long long n, RedOut red) {
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -636,12 +656,11 @@ __global__ void k_axmy_red_f4(float* __restrict__ out, const float* __restrict__
       max_abs(m, o);
       run = fmaf(w[e], o, run);
     }
-  block_partial<0>((double)m, part);
-  __syncthreads();
-  block_partial<1>(acc + (double)run, part + gridDim.x);
+  const double bm = block_reduce<0>((double)m), bd = block_reduce<1>(acc + (double)run);
+  red_finish<0, 1>(red, bm, bd);
 }
 
-__global__ void k_maxabs_partial_f4(const float* __restrict__ x, long long n, double* __restrict__ part) {
+__global__ void k_maxabs_partial_f4(const float* __restrict__ x, long long n, RedOut out) {
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -656,80 +675,39 @@ __global__ void k_maxabs_partial_f4(const float* __restrict__ x, long long n, do
   }
   if (tid == 0)
     for (long long e = n4 << 2; e < n; ++e) max_abs(m, x[e]);
-  block_partial<0>((double)m, part);
-}
-
-// the two finals of a two-result partial kernel: block 0 reduces
-// part[0, nb) with MODE0 into out[0], block 1 part[nb, 2 nb) with MODE1 into
-// out[1]
-template <int MODE0, int MODE1>
-__global__ void k_reduce_final2(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  __shared__ double sh[32];
-  const int mode = blockIdx.x == 0 ? MODE0 : MODE1;
-  const double* p = part + (size_t)blockIdx.x * nb;
-  double acc = 0.0;
-  for (int t = threadIdx.x; t < nb; t += blockDim.x) acc = mode == 0 ? fmax(acc, p[t]) : acc + p[t];
-  for (int off = 16; off > 0; off >>= 1) {
-    double o = __shfl_xor_sync(0xffffffffu, acc, off);
-    acc = mode == 0 ? fmax(acc, o) : acc + o;
-  }
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double v = threadIdx.x < (int)(blockDim.x / 32) ? sh[threadIdx.x] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) {
-      double o = __shfl_xor_sync(0xffffffffu, v, off);
-      v = mode == 0 ? fmax(v, o) : v + o;
-    }
-    if (threadIdx.x == 0) out[blockIdx.x] = v;
-  }
+  red_finish<0>(out, block_reduce<0>((double)m));
 }
 
 static double reduce_dot_f(hbf_ctx* c, const float* a, const float* b, long long n, int* st) {
+  const RedOut o = red_out(c, c->dres, c->hres);
   if (aligned16(a) && aligned16(b))
-    launch(c, kSlotReduce, k_dot_partial_f4, kRedBlocks, kThreads, a, b, n, c->partial);
+    launch(c, kSlotReduce, k_dot_partial_f4, red_grid(n), kThreads, a, b, n, o);
   else
-    launch(c, kSlotReduce, k_dot_partial_f, kRedBlocks, kThreads, a, b, n, c->partial);
-  launch(c, kSlotReduce, k_reduce_final<1>, 1, 1024, (const double*)c->partial, kRedBlocks, c->dres);
+    launch(c, kSlotReduce, k_dot_partial_f, red_grid(n), kThreads, a, b, n, o);
   *st = cuda_check(c, cudaGetLastError(), "dot");
   if (*st) return NAN;
-  return read_result(c, c->dres, st);
+  return read_result(c, st);
 }
 
-// both results of a two-result partial kernel (out[0], out[1]), one read
-static int read_results2(hbf_ctx* c, double* r0, double* r1) {
-  launch(c, kSlotReduce, k_reduce_final2<0, 1>, 2, 1024, (const double*)c->partial, kRedBlocks, c->dres);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->hres, c->dres, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return cuda_check(c, e, "reading a reduction");
-  *r0 = c->hres[0];
-  *r1 = c->hres[1];
-  return HBF_OK;
-}
-
-// (x.x, x.y) in one pass; sum-sum finals
+// (x.x, x.y) in one pass
 static int reduce_dot2_f(hbf_ctx* c, const float* x, const float* y, long long n, double* xx, double* xy) {
-  launch(c, kSlotReduce, k_dot2_partial_f4, kRedBlocks, kThreads, x, y, n, c->partial);
-  launch(c, kSlotReduce, k_reduce_final2<1, 1>, 2, 1024, (const double*)c->partial, kRedBlocks, c->dres);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->hres, c->dres, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  if (e != cudaSuccess) return cuda_check(c, e, "reading a reduction");
+  launch(c, kSlotReduce, k_dot2_partial_f4, red_grid(n), kThreads, x, y, n, red_out(c, c->dres, c->hres));
+  int st = cuda_check(c, cudaGetLastError(), "dot");
+  if (st || (st = wait_results(c))) return st;
   *xx = c->hres[0];
   *xy = c->hres[1];
   return HBF_OK;
 }
 
 static double reduce_max_abs_f(hbf_ctx* c, const float* x, long long n, int* st) {
+  const RedOut o = red_out(c, c->dres, c->hres);
   if (aligned16(x))
-    launch(c, kSlotReduce, k_maxabs_partial_f4, kRedBlocks, kThreads, x, n, c->partial);
+    launch(c, kSlotReduce, k_maxabs_partial_f4, red_grid(n), kThreads, x, n, o);
   else
-    launch(c, kSlotReduce, k_maxabs_partial_f, kRedBlocks, kThreads, x, n, c->partial);
-  launch(c, kSlotReduce, k_reduce_final<0>, 1, 1024, (const double*)c->partial, kRedBlocks, c->dres);
+    launch(c, kSlotReduce, k_maxabs_partial_f, red_grid(n), kThreads, x, n, o);
   *st = cuda_check(c, cudaGetLastError(), "max");
   if (*st) return NAN;
-  return read_result(c, c->dres, st);
+  return read_result(c, st);
 }
 
 // threads of the single-block coarsest-level solver: enough for the largest
@@ -817,7 +795,10 @@ static void build_dense(hbf_ctx* c, int kind, int l, long long n, double beta) {
   const int m = kind == 0 ? (int)n : (int)n + 1;
   launch(c, kSlotBottom, k_dense_build<D>, (int)n, 128, kind, c->dX, c->dM, (int)n, m, (const double*)L.ef[0],
          (const double*)L.ef[1], (const double*)L.ef[2], L.g, beta);
-  launch(c, kSlotBottom, k_gauss_jordan, 1, 256, (const double*)c->dM, m, c->dA, Dn.Minv);
+  cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)gauss_jordan_smem(kDenseMax + 1));
+  launch_smem(c, kSlotBottom, k_gauss_jordan, dim3(1), dim3(256), gauss_jordan_smem(m), (const double*)c->dM, m,
+              Dn.Minv);
   Dn.n = m;
   Dn.valid = true;
 }
@@ -998,6 +979,7 @@ struct ViscProblem : Problem<T> {
   using Problem<T>::c;
   T* x0;
   const T* b0 = nullptr;  // level-0 right-hand side in place of the level's own array (read only)
+  T* r0 = nullptr;        // level-0 residual in place of the level's own array
   double beta;
   const bool sp;  // level 0 in the colour-split layout (FP32 only)
   ViscProblem(hbf_ctx* ctx, T* x_in, double bt, bool h0)
@@ -1007,7 +989,7 @@ struct ViscProblem : Problem<T> {
   bool tail(int l) override { return run_tail<D, T, batch::kVisc>(c, l, beta); }
   T* x(int l) override { return l == 0 ? x0 : View<T>::vx(c->lv[l]); }
   T* b(int l) override { return (l == 0 && b0) ? const_cast<T*>(b0) : View<T>::vb(c->lv[l]); }
-  T* r(int l) override { return View<T>::vr(c->lv[l]); }
+  T* r(int l) override { return l == 0 && r0 ? r0 : View<T>::vr(c->lv[l]); }
   long long count(int l) override { return (long long)D * c->lv[l].g.ncell; }
   void smooth(int l) override {
     Level& L = c->lv[l];
@@ -1145,12 +1127,11 @@ struct ViscProblem : Problem<T> {
   void restrict_to(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
     long long n = (long long)D * C.g.ncell;
+    T* zero = tail_at<D, T, batch::kVisc>(c, l + 1) ? nullptr : x(l + 1);  // the tail zeroes its iterate itself
     if (l == 0 && sp)
-      launch(c, kSlotTransfer, k_restrict_cells<D, T, true>, grid_for(n), kThreads, r(l), b(l + 1), F.g, C.g, D);
+      launch(c, kSlotTransfer, k_restrict_cells<D, T, true>, grid_for(n), kThreads, r(l), b(l + 1), F.g, C.g, D, zero);
     else
-      launch(c, kSlotTransfer, k_restrict_cells<D, T>, grid_for(n), kThreads, r(l), b(l + 1), F.g, C.g, D);
-    if (!tail_at<D, T, batch::kVisc>(c, l + 1))  // the tail zeroes its iterate itself
-      launch(c, kSlotTransfer, k_zero<T>, grid_for(n), kThreads, x(l + 1), n);
+      launch(c, kSlotTransfer, k_restrict_cells<D, T>, grid_for(n), kThreads, r(l), b(l + 1), F.g, C.g, D, zero);
   }
   void prolong_add(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -1376,9 +1357,8 @@ struct MacProblem : Problem<T> {
   }
   void restrict_to(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
-    launch(c, kSlotTransfer, k_restrict_cells<D, T>, grid_for(C.g.ncell), kThreads, r(l), b(l + 1), F.g, C.g, 1);
-    if (!tail_at<D, T, batch::kMac>(c, l + 1))
-      launch(c, kSlotTransfer, k_zero<T>, grid_for(C.g.ncell), kThreads, x(l + 1), (long long)C.g.ncell);
+    launch(c, kSlotTransfer, k_restrict_cells<D, T>, grid_for(C.g.ncell), kThreads, r(l), b(l + 1), F.g, C.g, 1,
+           tail_at<D, T, batch::kMac>(c, l + 1) ? (T*)nullptr : x(l + 1));
   }
   void prolong_add(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -1447,14 +1427,11 @@ struct NodalProblem : Problem<T> {
   }
   void restrict_to(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
-    {
-      if (any_per(c->g))
-        launch(c, kSlotTransfer, k_restrict_nodes<D, T, true>, grid_for(C.g.nnode), kThreads, r(l), b(l + 1), F.g, C.g);
-      else
-        launch(c, kSlotTransfer, k_restrict_nodes<D, T, false>, grid_for(C.g.nnode), kThreads, r(l), b(l + 1), F.g, C.g);
-    }
-    if (!tail_at<D, T, batch::kNodal>(c, l + 1))
-      launch(c, kSlotTransfer, k_zero<T>, grid_for(C.g.nnode), kThreads, x(l + 1), (long long)C.g.nnode);
+    T* zero = tail_at<D, T, batch::kNodal>(c, l + 1) ? nullptr : x(l + 1);
+    if (any_per(c->g))
+      launch(c, kSlotTransfer, k_restrict_nodes<D, T, true>, grid_for(C.g.nnode), kThreads, r(l), b(l + 1), F.g, C.g, zero);
+    else
+      launch(c, kSlotTransfer, k_restrict_nodes<D, T, false>, grid_for(C.g.nnode), kThreads, r(l), b(l + 1), F.g, C.g, zero);
   }
   void prolong_add(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -1544,8 +1521,7 @@ static int mg_solve(Problem<double>& P, Problem<float>* P32, const double* b_in,
   int cycles = 0;
   while (rn > tol && cycles < cfg.max_cycles && std::isfinite(rn)) {
     if (P32) {
-      launch(c, kSlotTransfer, k_convert<float, double>, grid_for(n0), kThreads, P32->b(0), (const double*)P.r(0), n0);
-      launch(c, kSlotTransfer, k_zero<float>, grid_for(n0), kThreads, P32->x(0), n0);
+      launch(c, kSlotTransfer, k_convert_zero, grid_for(n0), kThreads, P32->b(0), P32->x(0), (const double*)P.r(0), n0);
       vcycle(*P32, 0, cfg);
       launch(c, kSlotTransfer, k_add_f32, grid_for(n0), kThreads, P.x(0), (const float*)P32->x(0), n0);
     } else {
@@ -1673,7 +1649,7 @@ static int visc_guess(hbf_ctx* c, double beta, double* x, double* r, double* rn,
     if (st) return st;
     if (!(ww > 0.0) || !std::isfinite(rw)) return HBF_OK;
     const double a = rw / ww;
-    launch(c, kSlotVector, k_axmy<float>, nb, kThreads, tmp, (const float*)cur, (float)a, (const float*)w, n);
+    launch(c, kSlotVector, k_axmy<float>, nb, kThreads, tmp, (const float*)cur, (float)a, (const float*)w, (float*)nullptr, n);
     const double m1 = reduce_max_abs_f(c, tmp, n, &st);
     if (st) return st;
     if (m1 < m) {
@@ -1718,19 +1694,18 @@ static int solve_viscous_mixed(hbf_ctx* c, double beta, const double* b_in, doub
   if (c->split_last != (int)sp) c->vprev_ok = false;  // the kept increment is in the other layout
   c->split_last = (int)sp;
   int st = 0;
+  P.b0 = kb;
+  P.r0 = r;
   auto true_residual = [&]() -> double {
-    cudaMemcpyAsync(L0.vb, kb, bytes, cudaMemcpyDeviceToDevice, c->stream);
     P.resid(0);
-    cudaMemcpyAsync(r, L0.vr, bytes, cudaMemcpyDeviceToDevice, c->stream);
     return reduce_max_abs(c, r, n, &st);
   };
   // the V-cycle reads q as its level-0 right-hand side in place (the fused
   // tail starts on level 1 or below, so its argument records never hold level
   // 0's array)
   auto precond = [&](const float* q, float* z) {
-    ViscProblem<D, float> Pz(c, z, beta, true);
+    ViscProblem<D, float> Pz(c, z, beta, true);  // z is 0
     Pz.b0 = q;
-    launch(c, kSlotTransfer, k_zero<float>, nb, kThreads, z, n);
     vcycle(Pz, 0, cfg);
   };
   const dim3 blk(256, 1, 1);
@@ -1790,14 +1765,14 @@ static int solve_viscous_mixed(hbf_ctx* c, double beta, const double* b_in, doub
       if (rho1 == 0.0 || !std::isfinite(rho1)) break;
       double bt = (rho1 / rho) * (alpha / omega);
       launch(c, kSlotVector, k_bicg_p<float>, nb, kThreads, fp, (const float*)fr, (const float*)fv, (float)bt,
-             (float)omega, n);
+             (float)omega, fph, n);
       precond(fp, fph);
       apply0(fph, fv);
       double den = reduce_dot_f(c, frh, fv, n, &st);
       if (st) return st;
       if (den == 0.0 || !std::isfinite(den)) break;
       alpha = rho1 / den;
-      launch(c, kSlotVector, k_axmy<float>, nb, kThreads, fs, (const float*)fr, (float)alpha, (const float*)fv, n);
+      launch(c, kSlotVector, k_axmy<float>, nb, kThreads, fs, (const float*)fr, (float)alpha, (const float*)fv, fsh, n);
       precond(fs, fsh);
       apply0(fsh, ft);
       double tt, ts;
@@ -1815,11 +1790,13 @@ static int solve_viscous_mixed(hbf_ctx* c, double beta, const double* b_in, doub
       double rr;
       if (fused) {
         // r = s - omega t with max |r| and r^.r of the new r in one pass
-        launch(c, kSlotVector, k_axmy_red_f4, kRedBlocks, kThreads, fr, (const float*)fs, (float)omega,
-               (const float*)ft, (const float*)frh, n, c->partial);
-        if ((st = read_results2(c, &rr, &rho_next))) return st;
+        launch(c, kSlotVector, k_axmy_red_f4, red_grid(n), kThreads, fr, (const float*)fs, (float)omega,
+               (const float*)ft, (const float*)frh, n, red_out(c, c->dres, c->hres));
+        if ((st = cuda_check(c, cudaGetLastError(), "reduction")) || (st = wait_results(c))) return st;
+        rr = c->hres[0];
+        rho_next = c->hres[1];
       } else {
-        launch(c, kSlotVector, k_axmy<float>, nb, kThreads, fr, (const float*)fs, (float)omega, (const float*)ft, n);
+        launch(c, kSlotVector, k_axmy<float>, nb, kThreads, fr, (const float*)fs, (float)omega, (const float*)ft, (float*)nullptr, n);
         rr = reduce_max_abs_f(c, fr, n, &st);
         if (st) return st;
       }
@@ -1873,28 +1850,18 @@ static int solve_viscous_d(hbf_ctx* c, double beta, const double* b_in, double* 
   double *kb = c->kb, *r = c->kr, *rh = c->krh, *p = c->kp, *v = c->kv, *s = c->ks, *t = c->kt, *ph = c->kph,
          *sh = c->ksh;
   ViscProblem<D, double> P(c, x, beta, false);
-  ViscProblem<D, float> Pre32(c, L0.fvx, beta, true);
-  const bool mixed = c->precision == HBF_MIXED;
   int st;
+  P.b0 = kb;
+  P.r0 = r;
   auto true_residual = [&]() -> double {
-    cudaMemcpyAsync(L0.vb, kb, bytes, cudaMemcpyDeviceToDevice, c->stream);
     P.resid(0);
-    cudaMemcpyAsync(r, L0.vr, bytes, cudaMemcpyDeviceToDevice, c->stream);
     return reduce_max_abs(c, r, n, &st);
   };
-  // z = M^{-1} q
+  // z = M^{-1} q, from z = 0
   auto precond = [&](const double* q, double* z) {
-    if (mixed) {
-      launch(c, kSlotTransfer, k_convert<float, double>, nb, kThreads, L0.fvb, q, n);
-      launch(c, kSlotTransfer, k_zero<float>, nb, kThreads, L0.fvx, n);
-      vcycle(Pre32, 0, cfg);
-      launch(c, kSlotTransfer, k_convert<double, float>, nb, kThreads, z, (const float*)L0.fvx, n);
-    } else {
-      ViscProblem<D, double> Pz(c, z, beta, true);
-      Pz.b0 = q;  // read in place, as in the mixed solve
-      launch(c, kSlotTransfer, k_zero<double>, nb, kThreads, z, n);
-      vcycle(Pz, 0, cfg);
-    }
+    ViscProblem<D, double> Pz(c, z, beta, true);
+    Pz.b0 = q;  // read in place, as in the mixed solve
+    vcycle(Pz, 0, cfg);
   };
   auto apply0 = [&](const double* q, double* out_) {
     const dim3 blk(256, 1, 1);
@@ -1926,14 +1893,14 @@ static int solve_viscous_d(hbf_ctx* c, double beta, const double* b_in, double* 
       if (st) return st;
       if (rho1 == 0.0 || !std::isfinite(rho1)) break;
       double bt = (rho1 / rho) * (alpha / omega);
-      launch(c, kSlotVector, k_bicg_p<double>, nb, kThreads, p, (const double*)r, (const double*)v, bt, omega, n);
+      launch(c, kSlotVector, k_bicg_p<double>, nb, kThreads, p, (const double*)r, (const double*)v, bt, omega, ph, n);
       precond(p, ph);
       apply0(ph, v);
       double den = reduce_dot(c, rh, v, n, &st);
       if (st) return st;
       if (den == 0.0 || !std::isfinite(den)) break;
       alpha = rho1 / den;
-      launch(c, kSlotVector, k_axmy<double>, nb, kThreads, s, (const double*)r, alpha, (const double*)v, n);
+      launch(c, kSlotVector, k_axmy<double>, nb, kThreads, s, (const double*)r, alpha, (const double*)v, sh, n);
       precond(s, sh);
       apply0(sh, t);
       double tt = reduce_dot(c, t, t, n, &st);
@@ -1942,7 +1909,7 @@ static int solve_viscous_d(hbf_ctx* c, double beta, const double* b_in, double* 
       if (st) return st;
       omega = tt > 0.0 ? ts / tt : 0.0;
       launch(c, kSlotVector, k_bicg_x<double>, nb, kThreads, x, (const double*)ph, (const double*)sh, alpha, omega, n);
-      launch(c, kSlotVector, k_axmy<double>, nb, kThreads, r, (const double*)s, omega, (const double*)t, n);
+      launch(c, kSlotVector, k_axmy<double>, nb, kThreads, r, (const double*)s, omega, (const double*)t, (double*)nullptr, n);
       rho = rho1;
       ++it;
       double rr = reduce_max_abs(c, r, n, &st);
@@ -2011,14 +1978,14 @@ void nodal_restrict(hbf_ctx* c, int l, const double* fine, double* coarse) {
   const Level &F = c->lv[l], &C = c->lv[l + 1];
   if (c->dim == 2) {
     if (any_per(c->g))
-      launch(c, kSlotTransfer, k_restrict_nodes<2, double, true>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g);
+      launch(c, kSlotTransfer, k_restrict_nodes<2, double, true>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g, (double*)nullptr);
     else
-      launch(c, kSlotTransfer, k_restrict_nodes<2, double, false>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g);
+      launch(c, kSlotTransfer, k_restrict_nodes<2, double, false>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g, (double*)nullptr);
   } else {
     if (any_per(c->g))
-      launch(c, kSlotTransfer, k_restrict_nodes<3, double, true>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g);
+      launch(c, kSlotTransfer, k_restrict_nodes<3, double, true>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g, (double*)nullptr);
     else
-      launch(c, kSlotTransfer, k_restrict_nodes<3, double, false>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g);
+      launch(c, kSlotTransfer, k_restrict_nodes<3, double, false>, grid_for(C.g.nnode), kThreads, fine, coarse, F.g, C.g, (double*)nullptr);
   }
 }
 
@@ -2034,20 +2001,20 @@ void cell_restrict_f(hbf_ctx* c, int l, const float* fine, float* coarse) {
   const Level &F = c->lv[l], &C = c->lv[l + 1];
   const long long n = (long long)c->dim * C.g.ncell;
   if (c->dim == 2)
-    launch(c, kSlotTransfer, k_restrict_cells<2, float>, grid_for(n), kThreads, fine, coarse, F.g, C.g, 2);
+    launch(c, kSlotTransfer, k_restrict_cells<2, float>, grid_for(n), kThreads, fine, coarse, F.g, C.g, 2, (float*)nullptr);
   else if (l == 0 && split0(c))  // the FP32 level-0 vectors of the mixed viscous solve
-    launch(c, kSlotTransfer, k_restrict_cells<3, float, true>, grid_for(n), kThreads, fine, coarse, F.g, C.g, 3);
+    launch(c, kSlotTransfer, k_restrict_cells<3, float, true>, grid_for(n), kThreads, fine, coarse, F.g, C.g, 3, (float*)nullptr);
   else
-    launch(c, kSlotTransfer, k_restrict_cells<3, float>, grid_for(n), kThreads, fine, coarse, F.g, C.g, 3);
+    launch(c, kSlotTransfer, k_restrict_cells<3, float>, grid_for(n), kThreads, fine, coarse, F.g, C.g, 3, (float*)nullptr);
 }
 
 void cell_restrict_d(hbf_ctx* c, int l, const double* fine, double* coarse, int ncomp) {
   const Level &F = c->lv[l], &C = c->lv[l + 1];
   const long long n = (long long)ncomp * C.g.ncell;
   if (c->dim == 2)
-    launch(c, kSlotTransfer, k_restrict_cells<2, double>, grid_for(n), kThreads, fine, coarse, F.g, C.g, ncomp);
+    launch(c, kSlotTransfer, k_restrict_cells<2, double>, grid_for(n), kThreads, fine, coarse, F.g, C.g, ncomp, (double*)nullptr);
   else
-    launch(c, kSlotTransfer, k_restrict_cells<3, double>, grid_for(n), kThreads, fine, coarse, F.g, C.g, ncomp);
+    launch(c, kSlotTransfer, k_restrict_cells<3, double>, grid_for(n), kThreads, fine, coarse, F.g, C.g, ncomp, (double*)nullptr);
 }
 
 void cell_prolong_add_f(hbf_ctx* c, int l, float* fine, const float* coarse) {
@@ -2084,7 +2051,7 @@ int visc_after_solve(hbf_ctx* c, const double* ustar, const double* u) {
 }
 
 void axmy(hbf_ctx* c, double* out, const double* x, double a, const double* y, long long n) {
-  launch(c, kSlotVector, k_axmy<double>, grid_for(n), kThreads, out, x, a, y, n);
+  launch(c, kSlotVector, k_axmy<double>, grid_for(n), kThreads, out, x, a, y, (double*)nullptr, n);
 }
 
 int tensor_lu(hbf_ctx* c, const double* u, double* out) {

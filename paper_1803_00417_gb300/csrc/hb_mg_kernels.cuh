@@ -76,6 +76,22 @@ __host__ __device__ __forceinline__ double rn_fma<double>(double a, double b, do
 #endif
 }
 
+// v, or -v when m has the sign bit set (on the integer pipe)
+__host__ __device__ __forceinline__ float sgn_flip(float v, unsigned m) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(__float_as_uint(v) ^ m);
+#else
+  return m ? -v : v;
+#endif
+}
+__host__ __device__ __forceinline__ double sgn_flip(double v, unsigned m) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
+#else
+  return m ? -v : v;
+#endif
+}
+
 struct Strides;
 
 // The face viscosities of a level, stored per face (FaceEta), or, on the
@@ -998,11 +1014,13 @@ __host__ __device__ __forceinline__ void k_restrict_cells_at(const T* __restrict
 }
 
 template <int D, typename T, bool SP = false>
-__global__ void k_restrict_cells(const T* __restrict__ f, T* __restrict__ c, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc, int ncomp) {
+__global__ void k_restrict_cells(const T* __restrict__ f, T* __restrict__ c, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc, int ncomp,
+                                 T* __restrict__ zero) {  // zero (or null): the coarse iterate, set to 0
   long long tot = (long long)gc.ncell * ncomp;
   for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt < tot;
        tt += (long long)gridDim.x * blockDim.x) {
     k_restrict_cells_at<D, T, SP>(f, c, gf, gc, ncomp, tt);
+    if (zero) zero[tt] = T(0);
   }
 }
 
@@ -1134,40 +1152,52 @@ __host__ __device__ __forceinline__ void k_prolong_cells_add_c_at(T* __restrict_
   int P[3];
   cell_coords<D>(gc, t, P[0], P[1], P[2]);
   const T* e = ec + (size_t)comp * gc.ncell;
-  // per axis: coarse index and sign of the offsets -1, 0, +1
+  // per axis: coarse index of the offsets -1, 0, +1, and the sign bit of those
+  // reflected (sign -1): signs cost no FP64 multiplication
+  const unsigned neg = sign < T(0) ? 0x80000000u : 0u;
   int ix[3][3];
-  T sg[3][3];
+  unsigned sg[3][3];
 #pragma unroll
   for (int a = 0; a < 3; ++a)
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       int q = (a < D) ? P[a] + d - 1 : 0;
-      T s = T(1);
+      unsigned s = 0u;
       if (a < D) {
         if (PER && gc.per[a]) q = wrap_cell(q, gc.n[a]);
         if (q < 0) {
           q = 0;
-          s *= sign;
+          s = neg;
         }
         if (q >= gc.n[a]) {
           q = gc.n[a] - 1;
-          s *= sign;
+          s = neg;
         }
       }
       ix[a][d] = q;
       sg[a][d] = s;
     }
-  T v[D == 3 ? 3 : 1][3][3];
+  // axis by axis, each interpolated value once: X to the two children along x
+  // of every row of the neighbourhood, Y along y of every plane
+  T Y[D == 3 ? 3 : 1][2][2];
 #pragma unroll
-  for (int dz = 0; dz < (D == 3 ? 3 : 1); ++dz)
+  for (int dz = 0; dz < (D == 3 ? 3 : 1); ++dz) {
+    T X[3][2];
 #pragma unroll
-    for (int dy = 0; dy < 3; ++dy)
+    for (int dy = 0; dy < 3; ++dy) {
+      T v[3];
 #pragma unroll
-      for (int dx = 0; dx < 3; ++dx) {
-        const int kz = D == 3 ? dz : 0;
-        const T s = sg[0][dx] * sg[1][dy] * (D == 3 ? sg[2][kz] : T(1));
-        v[dz][dy][dx] = s * e[cidx<D>(gc, ix[0][dx], ix[1][dy], D == 3 ? ix[2][kz] : 0)];
-      }
+      for (int dx = 0; dx < 3; ++dx)
+        v[dx] = sgn_flip(e[cidx<D>(gc, ix[0][dx], ix[1][dy], D == 3 ? ix[2][dz] : 0)],
+                         sg[0][dx] ^ sg[1][dy] ^ (D == 3 ? sg[2][dz] : 0u));
+#pragma unroll
+      for (int ci = 0; ci < 2; ++ci) X[dy][ci] = T(0.75) * v[1] + T(0.25) * v[ci ? 2 : 0];
+    }
+#pragma unroll
+    for (int cj = 0; cj < 2; ++cj)
+#pragma unroll
+      for (int ci = 0; ci < 2; ++ci) Y[dz][cj][ci] = T(0.75) * X[1][ci] + T(0.25) * X[cj ? 2 : 0][ci];
+  }
   T* x = xf + (size_t)comp * gf.ncell;
 #pragma unroll
   for (int ck = 0; ck < (D == 3 ? 2 : 1); ++ck)
@@ -1177,20 +1207,8 @@ __host__ __device__ __forceinline__ void k_prolong_cells_add_c_at(T* __restrict_
       for (int ci = 0; ci < 2; ++ci) {
         // child (2I + ci, 2J + cj, 2K + ck): its own coarse cell (offset 1)
         // and the neighbour on the child's side (offset 2 or 0)
-        const int nx = ci ? 2 : 0, ny = cj ? 2 : 0, nz = D == 3 ? (ck ? 2 : 0) : 0;
-        T tz[2];
-#pragma unroll
-        for (int kk = 0; kk < (D == 3 ? 2 : 1); ++kk) {
-          const int kz = D == 3 ? (kk ? nz : 1) : 0;
-          T ty[2];
-#pragma unroll
-          for (int jj = 0; jj < 2; ++jj) {
-            const int jy = jj ? ny : 1;
-            ty[jj] = T(0.75) * v[kz][jy][1] + T(0.25) * v[kz][jy][nx];
-          }
-          tz[kk] = T(0.75) * ty[0] + T(0.25) * ty[1];
-        }
-        const T val = D == 3 ? T(0.75) * tz[0] + T(0.25) * tz[1] : tz[0];
+        const T val = D == 3 ? T(0.75) * Y[D == 3 ? 1 : 0][cj][ci] + T(0.25) * Y[D == 3 ? (ck ? 2 : 0) : 0][cj][ci]
+                             : Y[0][cj][ci];
         x[lidx<D, SP>(gf, 2 * P[0] + ci, 2 * P[1] + cj, D == 3 ? 2 * P[2] + ck : 0)] += val;
       }
 }
@@ -1231,9 +1249,11 @@ __host__ __device__ __forceinline__ void k_restrict_nodes_at(const T* __restrict
 }
 
 template <int D, typename T, bool PER = true>
-__global__ void k_restrict_nodes(const T* __restrict__ rf, T* __restrict__ rc, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc) {
+__global__ void k_restrict_nodes(const T* __restrict__ rf, T* __restrict__ rc, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
+                                 T* __restrict__ zero) {
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < gc.nnode; t += gridDim.x * blockDim.x) {
     k_restrict_nodes_at<D, T, PER>(rf, rc, gf, gc, t);
+    if (zero) zero[t] = T(0);
   }
 }
 
@@ -1356,69 +1376,87 @@ __global__ void k_dense_build(int kind, double* __restrict__ X, double* __restri
   dense_build_col<D>(kind, X, M, n, ld, ef0, ef1, ef2, g, beta, blockIdx.x);
 }
 
-// Gauss-Jordan with partial pivoting on [M | I] (m x 2m, A), one block;
-// writes the inverse to Minv (m x m).  Returns with Minv = 0 if singular.
-__device__ inline void gauss_jordan_block(const double* __restrict__ M, int m, double* __restrict__ A,
-                                          double* __restrict__ Minv) {
-  __shared__ double fcol[kDenseMax + 1];
-  __shared__ double sv[256];
-  __shared__ int si[256];
-  __shared__ int piv;
-  const int w2 = 2 * m;
-  for (int t = threadIdx.x; t < m * w2; t += blockDim.x) {
-    const int i = t / w2, j = t % w2;
-    A[t] = j < m ? M[(size_t)i * m + j] : (j - m == i ? 1.0 : 0.0);
-  }
+// Inverse of M (m x m, m <= kDenseMax + 1) by Gauss-Jordan with partial
+// pivoting, one block, in place in shared memory (gauss_jordan_smem(m) bytes
+// of it): per pivot one warp finds the row, the block swaps and scales it and
+// eliminates the column, three barriers in all.  The arithmetic is that on [M
+// | I] (the columns of I that are still unit vectors are not stored).  In
+// global memory, with 13 barriers and a serial pivot search per column, 24
+// unknowns took 337 us, and every viscous solve inverts its coarsest operator.
+__host__ __device__ inline size_t gauss_jordan_smem(int m) { return ((size_t)m * m + m) * sizeof(double); }
+
+__device__ inline void gauss_jordan_block(const double* __restrict__ M, int m, double* __restrict__ Minv) {
+  extern __shared__ __align__(16) double gj_mem[];
+  __shared__ int prow[kDenseMax + 1], src[kDenseMax + 1];
+  __shared__ double pval, kval;
+  double *A = gj_mem, *f = gj_mem + (size_t)m * m;
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) A[t] = M[t];
   __syncthreads();
   for (int k = 0; k < m; ++k) {
-    double best = -1.0;
-    int bi = k;
-    for (int i = k + threadIdx.x; i < m; i += blockDim.x) {
-      const double a = fabs(A[(size_t)i * w2 + k]);
-      if (a > best) {
-        best = a;
-        bi = i;
-      }
-    }
-    sv[threadIdx.x] = best;
-    si[threadIdx.x] = bi;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double b = -1.0;
-      int ib = k;
-      for (int q = 0; q < (int)blockDim.x; ++q)
-        if (sv[q] > b) {
-          b = sv[q];
-          ib = si[q];
+    if (threadIdx.x < 32) {
+      // the largest magnitude of the column at or below the diagonal, the
+      // first of equals
+      double best = -1.0;
+      int bi = k;
+      for (int i = k + (int)threadIdx.x; i < m; i += 32) {
+        const double a = fabs(A[i * m + k]);
+        if (a > best) {
+          best = a;
+          bi = i;
         }
-      piv = ib;
+      }
+      for (int off = 16; off > 0; off >>= 1) {
+        const double o = __shfl_xor_sync(0xffffffffu, best, off);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+        if (o > best || (o == best && oi < bi)) {
+          best = o;
+          bi = oi;
+        }
+      }
+      if (threadIdx.x == 0) {
+        prow[k] = bi;
+        pval = A[bi * m + k];
+        kval = A[k * m + k];
+      }
     }
     __syncthreads();
-    const int pr = piv;
-    if (pr != k)
-      for (int j = threadIdx.x; j < w2; j += blockDim.x) {
-        const double t0 = A[(size_t)k * w2 + j];
-        A[(size_t)k * w2 + j] = A[(size_t)pr * w2 + j];
-        A[(size_t)pr * w2 + j] = t0;
-      }
+    const int pr = prow[k];
+    const double d = pval;
+    // rows k and pr change places, row k is scaled; f: column k of the others
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+      f[j] = j == pr ? kval : A[j * m + k];  // entry k is not used
+    }
     __syncthreads();
-    const double d = A[(size_t)k * w2 + k];
+    for (int j = threadIdx.x; j < m; j += blockDim.x) {
+      const double t = j == k ? 1.0 : A[pr * m + j];
+      if (pr != k) A[pr * m + j] = A[k * m + j];
+      A[k * m + j] = t / d;
+    }
     __syncthreads();
-    for (int j = threadIdx.x; j < w2; j += blockDim.x) A[(size_t)k * w2 + j] /= d;
-    __syncthreads();
-    for (int i = threadIdx.x; i < m; i += blockDim.x) fcol[i] = A[(size_t)i * w2 + k];
-    __syncthreads();
-    for (int t = threadIdx.x; t < m * w2; t += blockDim.x) {
-      const int i = t / w2, j = t % w2;
-      if (i != k) A[t] -= fcol[i] * A[(size_t)k * w2 + j];
+    for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+      const int i = t / m, j = t - i * m;
+      if (i != k) A[t] = (j == k ? 0.0 : A[t]) - f[i] * A[k * m + j];
     }
     __syncthreads();
   }
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) Minv[t] = A[(size_t)(t / m) * w2 + m + t % m];
+  if (threadIdx.x == 0) {
+    // undo the row exchanges on the columns
+    for (int j = 0; j < m; ++j) src[j] = j;
+    for (int k = m - 1; k >= 0; --k) {
+      const int t = src[k];
+      src[k] = src[prow[k]];
+      src[prow[k]] = t;
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    const int i = t / m, j = t - i * m;
+    Minv[t] = A[i * m + src[j]];
+  }
 }
 
-static __global__ void k_gauss_jordan(const double* __restrict__ M, int m, double* __restrict__ A, double* __restrict__ Minv) {
-  gauss_jordan_block(M, m, A, Minv);
+static __global__ void k_gauss_jordan(const double* __restrict__ M, int m, double* __restrict__ Minv) {
+  gauss_jordan_block(M, m, Minv);
 }
 
 // x[i] = sum_j Minv[i][j] b[j] over the n unknowns (the bordered row/column,

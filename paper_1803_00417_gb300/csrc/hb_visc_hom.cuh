@@ -18,22 +18,6 @@
 
 namespace hb {
 
-// v, or -v when m has the sign bit set (on the integer pipe)
-__host__ __device__ __forceinline__ float sgn_flip(float v, unsigned m) {
-#ifdef __CUDA_ARCH__
-  return __uint_as_float(__float_as_uint(v) ^ m);
-#else
-  return m ? -v : v;
-#endif
-}
-__host__ __device__ __forceinline__ double sgn_flip(double v, unsigned m) {
-#ifdef __CUDA_ARCH__
-  return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
-#else
-  return m ? -v : v;
-#endif
-}
-
 // One axis seen from a cell: the offsets om / op of the neighbours below and
 // above (wrapped on a periodic axis; 0 past a wall, where the homogeneous
 // ghost is minus the cell's own value: fm / fp hold the sign bit there and 0
