@@ -398,6 +398,7 @@ int hbf_set_split_layout(hbf_ctx* c, int on) {
   if (!c) return HBF_ERR_ARG;
   if (on != 0 && on != 1) return fail(c, HBF_ERR_ARG, "split layout must be 0 or 1");
   c->split_layout = on;
+  for (auto& k : c->tail) k.reset();  // the finest level may enter or leave the tail
   return HBF_OK;
 }
 
@@ -477,6 +478,7 @@ int hbf_restrict(hbf_ctx* c, int kind, int level, const double* src, double* dst
 int hbf_set_fused_sweep(hbf_ctx* c, int on) {
   if (!c) return HBF_ERR_ARG;
   c->fused_sweep = on ? 1 : 0;
+  for (auto& k : c->tail) k.reset();
   return HBF_OK;
 }
 
@@ -485,6 +487,7 @@ int hbf_set_staged_sweep(hbf_ctx* c, int tile_x, int tile_z) {
   if ((tile_x != 0 && tile_x != 64 && tile_x != 128) || tile_z < 1 || tile_z > 4096)
     return fail(c, HBF_ERR_ARG, "staged sweep tile: width 0, 64 or 128, 1 <= planes <= 4096");
   c->staged_tx = tile_x;
+  for (auto& k : c->tail) k.reset();
   c->staged_tz = tile_z;
   return HBF_OK;
 }
@@ -494,6 +497,7 @@ int hbf_set_staged_op(hbf_ctx* c, int rows, int tile_z) {
   if ((rows != 0 && rows != 4 && rows != 8) || tile_z < 1 || tile_z > 4096)
     return fail(c, HBF_ERR_ARG, "staged operator tile: rows 0, 4 or 8, 1 <= planes <= 4096");
   c->staged_op_rows = rows;
+  for (auto& k : c->tail) k.reset();  // the finest level may enter or leave the tail
   c->staged_op_tz = tile_z;
   return HBF_OK;
 }

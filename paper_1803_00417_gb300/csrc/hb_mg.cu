@@ -260,9 +260,22 @@ static inline bool any_per(const Geom& g) { return g.per[0] || g.per[1] || g.per
 // (staged, fused) nor a network on level 0.  Every FP32 level-0 vector of the
 // solve (the BiCGStab vectors, the V-cycle's level-0 arrays, the cell
 // viscosity, the previous increment) is then split; FP64 arrays stay natural.
+// A small FP32 finest level of the mixed viscous solve (in the default layout,
+// no opt-in form) is handled like the coarse levels: natural layout, stored
+// face viscosities and reciprocals, the branch-free kernels of hb_visc_hom.cuh,
+// and the fused tail where it starts there.  It is bound by the latency of one
+// sweep's chain, not by bytes: 6 us per split sweep and 8 us per natural one at
+// 32^3 to 96 x 64 x 64, 3 us this way; the split layout, with half the bytes,
+// wins from about 80^3 on.
+constexpr int kFaces0Cells = 1 << 19;
+static bool faces0(const hbf_ctx* c) {
+  return c->precision == HBF_MIXED && c->split_layout && c->g.ncell <= kFaces0Cells && !c->staged_tx &&
+         !c->staged_op_rows && !c->fused_sweep;
+}
+
 static bool split0(const hbf_ctx* c) {
   const Geom& g = c->g;
-  return c->split_layout && c->dim == 3 && c->precision == HBF_MIXED && !any_per(g) && g.n[0] % 2 == 0 &&
+  return c->split_layout && !faces0(c) && c->dim == 3 && c->precision == HBF_MIXED && !any_per(g) && g.n[0] % 2 == 0 &&
          g.n[0] >= 4 && g.n[1] >= 3 && g.n[2] >= 3 && c->lv.size() >= 2 && c->lv[0].feta != nullptr &&
          !c->staged_tx && !c->staged_op_rows && !c->fused_sweep && !(c->vnet && c->vnet_level == 0);
 }
@@ -840,15 +853,17 @@ static bool dense_bottom(const hbf_ctx* c, int kind) {
   return (kind == 0 ? (long long)c->dim * g.ncell : (long long)(kind == 1 ? g.ncell : g.nnode)) <= kDenseMax;
 }
 
-// The first level of the fused tail: the first one from level 1 on with at
-// most max_cells cells (hbf_set_tail), or, by default, small enough that a
-// cluster of 16 blocks takes a phase of it in less time than a launch over the
-// whole GPU does.
-template <int D, typename T>
+// The first level of problem kind's fused tail: the first one with at most
+// max_cells cells (hbf_set_tail), or, by default, small enough that a cluster
+// of 16 blocks takes a phase of it in less time than a launch over the whole
+// GPU does.  The finest level too where the V-cycles run on it in the natural
+// layout with stored faces and there is a coarser one.
+template <int D, typename T, int KIND>
 static int tail_level(const hbf_ctx* c) {
   const int nl = (int)c->lv.size();
-  const long long most = c->tail_cells >= 0 ? c->tail_cells : batch::tail_wide_cells<D, T>();
-  for (int l = 1; l < nl; ++l)
+  const long long most = c->tail_cells >= 0 ? c->tail_cells : batch::tail_wide_cells<D, T, KIND>();
+  const bool finest = nl > 1 && (sizeof(T) == 8 || KIND != batch::kVisc || faces0(c));
+  for (int l = finest ? 0 : 1; l < nl; ++l)
     if (c->lv[l].g.ncell <= most) return l;
   return nl;
 }
@@ -871,7 +886,7 @@ static const TailPlan& tail_plan(hbf_ctx* c) {
   const int nl = (int)c->lv.size(), L = nl - 1;
   P.set = true;
   P.on = false;
-  P.lf = tail_level<D, T>(c);
+  P.lf = tail_level<D, T, KIND>(c);
   if (P.lf >= nl || nl > kMaxLev) return P;
   const Geom* gs[kMaxLev];
   for (int l = 0; l < nl; ++l) gs[l] = &c->lv[l].g;
@@ -904,7 +919,7 @@ static bool tail_at(hbf_ctx* c, int l) {
 }
 
 template <int D, typename T, int KIND>
-static bool run_tail(hbf_ctx* c, int l, double beta) {
+static bool run_tail(hbf_ctx* c, int l, double beta, T* x0, const T* b0) {
   using namespace batch;
   if (!tail_at<D, T, KIND>(c, l)) return false;
   TailPlan& P = c->tail[KIND];
@@ -963,9 +978,9 @@ static bool run_tail(hbf_ctx* c, int l, double beta) {
   const bool rec = prof_wants(c->prof, kSlotCoarse);
   if (rec) prof_mark(c, kSlotCoarse, true);
   if (any_per(c->g))
-    tail_launch<D, T, KIND, true>(c->stream, tb, P.lf, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
+    tail_launch<D, T, KIND, true>(c->stream, tb, P.lf, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem, x0, b0);
   else
-    tail_launch<D, T, KIND, false>(c->stream, tb, P.lf, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem);
+    tail_launch<D, T, KIND, false>(c->stream, tb, P.lf, 1, nullptr, c->cfg.nu1, c->cfg.nu2, P.nblk, P.smem, x0, b0);
   if (rec) prof_mark(c, kSlotCoarse, false);
   ++c->nlaunch;
   return true;
@@ -973,6 +988,18 @@ static bool run_tail(hbf_ctx* c, int l, double beta) {
 
 static bool staged_op(hbf_ctx* c, int slot, const float* u, const float* b, float* out, const float* eta,
                       const Geom& g, float beta, int hm);
+
+// u - beta L u of a small FP32 finest level (faces0)
+template <int D>
+static void faces0_op(hbf_ctx* c, int slot, const float* u, float* out, float beta) {
+  const Level& L = c->lv[0];
+  const int th = spread_threads(L.g.ncell), nb = (L.g.ncell + th - 1) / th;
+  const float *e0 = L.fef[0], *e1 = L.fef[1], *e2 = L.fef[2];
+  if (any_per(c->g))
+    launch(c, slot, k_visc_res_hom<D, float, true>, nb, th, u, (const float*)nullptr, out, e0, e1, e2, L.g, beta);
+  else
+    launch(c, slot, k_visc_res_hom<D, float, false>, nb, th, u, (const float*)nullptr, out, e0, e1, e2, L.g, beta);
+}
 
 template <int D, typename T>
 struct ViscProblem : Problem<T> {
@@ -986,7 +1013,7 @@ struct ViscProblem : Problem<T> {
       : Problem<T>(ctx, false, h0), x0(x_in), beta(bt), sp(sizeof(T) == 4 && D == 3 && split0(ctx)) {}
   int kind() const override { return 0; }
   double dense_beta() const override { return beta; }
-  bool tail(int l) override { return run_tail<D, T, batch::kVisc>(c, l, beta); }
+  bool tail(int l) override { return run_tail<D, T, batch::kVisc>(c, l, beta, x(l), b(l)); }
   T* x(int l) override { return l == 0 ? x0 : View<T>::vx(c->lv[l]); }
   T* b(int l) override { return (l == 0 && b0) ? const_cast<T*>(b0) : View<T>::vb(c->lv[l]); }
   T* r(int l) override { return l == 0 && r0 ? r0 : View<T>::vr(c->lv[l]); }
@@ -1072,7 +1099,7 @@ struct ViscProblem : Problem<T> {
            r(l), (const T*)View<T>::ef(L, 0), (const T*)View<T>::ef(L, 1), (const T*)View<T>::ef(L, 2), L.g, (T)beta);
   }
   // the FP32 finest level forms its face viscosities from the cell viscosity
-  bool cell_eta(int l) const { return l == 0 && sizeof(T) == 4 && c->lv[0].feta != nullptr; }
+  bool cell_eta(int l) const { return l == 0 && sizeof(T) == 4 && c->lv[0].feta != nullptr && !faces0(c); }
   // 3D FP32 finest level with walls on every axis: the sweeps of k_visc_smooth_c
   // with the planes staged in shared memory by TMA (hb_visc_tma.cuh); false
   // (nothing launched) when the staged sweep is off or the level does not
@@ -1328,7 +1355,7 @@ struct MacProblem : Problem<T> {
   T* x0;
   MacProblem(hbf_ctx* ctx, T* x_in) : Problem<T>(ctx, true, true), x0(x_in) {}
   int kind() const override { return 1; }
-  bool tail(int l) override { return run_tail<D, T, batch::kMac>(c, l, 0.0); }
+  bool tail(int l) override { return run_tail<D, T, batch::kMac>(c, l, 0.0, x(l), b(l)); }
   T* x(int l) override { return l == 0 ? x0 : View<T>::cx(c->lv[l]); }
   T* b(int l) override { return View<T>::cb(c->lv[l]); }
   T* r(int l) override { return View<T>::cr(c->lv[l]); }
@@ -1397,7 +1424,7 @@ struct NodalProblem : Problem<T> {
   T* x0;
   NodalProblem(hbf_ctx* ctx, T* x_in) : Problem<T>(ctx, true, true), x0(x_in) {}
   int kind() const override { return 2; }
-  bool tail(int l) override { return run_tail<D, T, batch::kNodal>(c, l, 0.0); }
+  bool tail(int l) override { return run_tail<D, T, batch::kNodal>(c, l, 0.0, x(l), b(l)); }
   T* x(int l) override { return l == 0 ? x0 : View<T>::nx(c->lv[l]); }
   T* b(int l) override { return View<T>::nb(c->lv[l]); }
   T* r(int l) override { return View<T>::nr(c->lv[l]); }
@@ -1547,7 +1574,7 @@ static void build_eta_levels(hbf_ctx* c) {
              C.ef[a], a, F.g, C.g);
   }
   if (c->precision == HBF_MIXED) {
-    for (size_t l = 1; l < c->lv.size(); ++l) {
+    for (size_t l = faces0(c) ? 0 : 1; l < c->lv.size(); ++l) {
       Level& L = c->lv[l];
       for (int a = 0; a < D; ++a)
         launch(c, kSlotTransfer, k_convert<float, double>, grid_for(L.g.nface[a]), kThreads, L.fef[a],
@@ -1556,6 +1583,7 @@ static void build_eta_levels(hbf_ctx* c) {
     // the finest level of the FP32 V-cycles reads the cell viscosity (the
     // level-0 faces are the means of its cells, wall faces the interior cell)
     Level& L0 = c->lv[0];
+    if (faces0(c)) return;
     if (split0(c))
       launch(c, kSlotTransfer, k_split_from, grid_for(L0.g.ncell / 2), kThreads, L0.feta, (const double*)c->eta,
              (const double*)nullptr, L0.g, 1);
@@ -1632,7 +1660,9 @@ static int visc_guess(hbf_ctx* c, double beta, double* x, double* r, double* rn,
   const dim3 grd(op3_blocks<D>(L0.g), 1, 1);
   auto step_along = [&](const float* d, int bit) -> int {
     const float* e0 = L0.feta;
-    if (sp)
+    if (faces0(c))
+      faces0_op<D>(c, kSlotVector, d, w, fbeta);
+    else if (sp)
       launch3(c, kSlotVector, k_visc_op_split, split_grid(L0.g), split_block_dim(L0.g, 2), d, (const float*)nullptr, w,
               e0, L0.g, fbeta, 1);
     else if (staged_op(c, kSlotVector, d, nullptr, w, e0, L0.g, fbeta, 1))
@@ -1712,6 +1742,10 @@ static int solve_viscous_mixed(hbf_ctx* c, double beta, const double* b_in, doub
   const dim3 grd(op3_blocks<D>(L0.g), 1, 1);
   auto apply0 = [&](const float* q, float* o) {
     const float* e0 = L0.feta;
+    if (faces0(c)) {
+      faces0_op<D>(c, kSlotViscResid, q, o, fbeta);
+      return;
+    }
     if (sp) {
       launch3(c, kSlotViscResid, k_visc_op_split, split_grid(L0.g), split_block_dim(L0.g, 2), q, (const float*)nullptr, o,
               e0, L0.g, fbeta, 1);
@@ -1824,7 +1858,7 @@ template <int D>
 static void build_inv_levels(hbf_ctx* c, double beta) {
   const bool mixed = c->precision == HBF_MIXED;
   const size_t nl = c->lv.size();
-  for (size_t l = mixed ? 1 : 0; l < nl; ++l) {
+  for (size_t l = mixed && !faces0(c) ? 1 : 0; l < nl; ++l) {
     Level& L = c->lv[l];
     const int th = spread_threads(L.g.ncell), nb = (L.g.ncell + th - 1) / th;
     if (mixed)

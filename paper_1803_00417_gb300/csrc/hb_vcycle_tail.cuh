@@ -722,10 +722,12 @@ __host__ __device__ inline void tail_level_init(TailLevel<T>& w, const Geom& g, 
 }
 
 // PER = false: every level of every cavity has walls on every axis.  Grid:
-// ncav clusters.
+// ncav clusters.  x_lf, b_lf: level lf's iterate and right-hand side in place
+// of the record's (null: the record's).
 template <int D, typename T, int KIND, bool PER = true>
 __global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailTabs tb, int lf, int ncav,
-                                                                  const int* __restrict__ mask, int nu1, int nu2) {
+                                                                  const int* __restrict__ mask, int nu1, int nu2,
+                                                                  T* x_lf, const T* b_lf) {
   extern __shared__ __align__(16) char mem[];
   __shared__ TailLevel<T> sw[kMaxLev];
   __shared__ TailLevel<double> sbw;  // the coarsest level, when it is swept
@@ -770,6 +772,10 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailTabs tb, in
         w.gr = a.r;
         w.gb = a.b;
         sbeta = T(0);
+      }
+      if (l == lf && x_lf) {
+        w.gx = x_lf;
+        w.gb = b_lf;
       }
       if (l < L) {
         tail_level_init<D, T, KIND>(w, sg[l], (int)nblk, rank, false, at);
@@ -968,16 +974,20 @@ inline int tail_blocks(int ncav, bool wide) {
   return nblk;
 }
 
-// the default first level of a single cavity's tail (see there): cells
-template <int D, typename T>
+// Cells of the default first level of a single cavity's tail.  Measured per
+// phase, a cluster of 16 against launches: FP32 128^2 1.2 against 2.9 us, 32^3
+// 3.7 against 3 to 6 us; FP64, which is bound by the operations of 16 SMs, 64^2
+// 1.4 against 3.1 us and 128^2 5.7 against 3.6 us (viscous; the cheaper MAC and
+// nodal phases 3 against 3 us), 16^3 2.3 against 3 us.
+template <int D, typename T, int KIND>
 constexpr int tail_wide_cells() {
-  return sizeof(T) == 4 ? (D == 3 ? 32768 : 16384) : (D == 3 ? 4096 : 16384);
+  return sizeof(T) == 4 ? (D == 3 ? 32768 : 16384) : (D == 3 || KIND == kVisc ? 4096 : 16384);
 }
 
 // launch on stream s: ncav clusters of nblk blocks (tail_blocks)
 template <int D, typename T, int KIND, bool PER>
 inline cudaError_t tail_launch(cudaStream_t s, const TailTabs& tb, int lf, int ncav, const int* mask, int nu1, int nu2,
-                               int nblk, size_t smem) {
+                               int nblk, size_t smem, T* x_lf = nullptr, const T* b_lf = nullptr) {
   auto kern = k_vcycle_tail<D, T, KIND, PER>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(nblk * ncav));
@@ -989,7 +999,7 @@ inline cudaError_t tail_launch(cudaStream_t s, const TailTabs& tb, int lf, int n
   at[0].val.clusterDim = {(unsigned)nblk, 1, 1};
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, tb, lf, ncav, mask, nu1, nu2);
+  return cudaLaunchKernelEx(&cfg, kern, tb, lf, ncav, mask, nu1, nu2, x_lf, b_lf);
 }
 
 }  // namespace batch

@@ -113,10 +113,10 @@ __host__ __device__ __forceinline__ T hom_gs(const HomCell<D, T>& s, T bc, T inv
   return rn_mul(rn_fma(bs, rn_fma(T(0.25), cross, offd), bc), inv);
 }
 
-// b - (u - beta L u): tensor_core's terms, with the normal flux of a wall face
+// u - beta L u: tensor_core's terms, with the normal flux of a wall face
 // e (u - (-u)) and no cross term there
 template <int D, typename T>
-__host__ __device__ __forceinline__ T hom_res(const HomCell<D, T>& s, T bc, T beta, T ihh) {
+__host__ __device__ __forceinline__ T hom_op(const HomCell<D, T>& s, T beta, T ihh) {
   const T u0 = s.u[0][0];
   T acc = T(0);
 #pragma unroll
@@ -132,7 +132,11 @@ __host__ __device__ __forceinline__ T hom_res(const HomCell<D, T>& s, T bc, T be
     const T f = rn_fma(s.ehi[r], dhi, -rn_mul(s.elo[r], dlo));
     acc = r == 0 ? rn_mul(T(2), f) : rn_add(acc, f);
   }
-  return rn_add(bc, -rn_fma(-beta, rn_mul(acc, ihh), u0));
+  return rn_fma(-beta, rn_mul(acc, ihh), u0);
+}
+template <int D, typename T>
+__host__ __device__ __forceinline__ T hom_res(const HomCell<D, T>& s, T bc, T beta, T ihh) {
+  return rn_add(bc, -hom_op<D, T>(s, beta, ihh));
 }
 
 // the stencil of component c at cell p of a whole level (flat index id)
@@ -194,7 +198,8 @@ __global__ void __launch_bounds__(256) k_visc_smooth_hom(T* u, const T* __restri
   if (t < rb_count<D>(g)) visc_smooth_hom_at<D, T, PER>(u, b, inv, ef, g, C, col, bs, t);
 }
 
-// r = b - (u - beta L u) of every component (thread t: cell t)
+// r = b - (u - beta L u) of every component, or u - beta L u when b is null
+// (thread t: cell t)
 template <int D, typename T, bool PER>
 __host__ __device__ __forceinline__ void visc_res_hom_at(const T* u, const T* b, T* r, const T* const* ef,
                                                          const Geom& g, T beta, int t) {
@@ -203,7 +208,8 @@ __host__ __device__ __forceinline__ void visc_res_hom_at(const T* u, const T* b,
 #pragma unroll
   for (int c = 0; c < D; ++c) {
     const size_t o = (size_t)c * g.ncell + t;
-    r[o] = visc_res_hom<D, T, PER>(u, b[o], ef, g, c, p, t, beta);
+    const T Au = hom_op<D, T>(hom_cell<D, T, PER>(u, ef, g, c, p, t), beta, g_ihh<T>(g));
+    r[o] = b ? rn_add(b[o], -Au) : Au;
   }
 }
 

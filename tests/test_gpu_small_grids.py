@@ -1,8 +1,12 @@
-"""Multigrid solves on grids that are their own coarsest level, with exact (at
-most 128 unknowns) and swept bottoms, against the oracle.
+"""Multigrid solves at the sizes where their paths change: grids that are their
+own coarsest level, with exact (at most 128 unknowns) and swept bottoms; small
+FP32 finest levels with stored faces that run wholly inside the V-cycle tail,
+against the same solves level by level and in the general layout; and the first
+grid above that range.
 
-Tolerance: the oracle's steps to 1e-10 (each side stops its solves at 1e-10 of
-the right-hand side and the steps scale that down)."""
+Tolerances: the oracle's steps to 1e-10 (each side stops its solves at 1e-10 of
+the right-hand side and the steps scale that down); solver routes of the mixed
+precision against each other to 1e-8, as the layouts' test."""
 
 import numpy as np
 import pytest
@@ -48,3 +52,28 @@ def test_coarsest_grids_match_oracle(n):
     got, want = np.array(sim.velocity()), np.array(ref.u)
     assert np.linalg.norm(got - want) <= 1e-10 * np.linalg.norm(want)
     sim.close()
+
+
+# 80^3 is the last cube whose finest level stores its faces; the grids with more cells end inside
+# the operator's 64-cell tile (48, 112 and 160 cells along x) and at its edge (128)
+@pytest.mark.parametrize("n", [(24, 20, 12), (12, 40, 28), (80, 80, 80), (112, 80, 64), (48, 128, 96), (160, 64, 56),
+                               (128, 64, 80), (72, 48)])
+def test_mixed_routes_agree(n):
+    cfg = cavity(n, Re=100.0, Bi=10.0, Pa=1e4, nexp=1.2)
+    u, p = random_state(cfg["n"], seed=sum(n))
+    outs = []
+    for tail, split in ((None, None), (0, None), (None, 0)):
+        sim = _sim(cfg, u, p, 1)
+        if tail is not None:
+            sim.set_tail(tail)
+        if split is not None:
+            sim.set_split_layout(split)
+        for _ in range(2):
+            st = sim.step(cfg["dt"])
+            for k in ("mac", "visc", "nodal"):
+                assert st[k]["converged"], (k, st[k])
+                assert st[k]["rnorm"] <= 1e-10 * st[k]["bnorm"]
+        outs.append(np.concatenate([sim.get_field("U"), sim.get_field("P")]))
+        sim.close()
+    for other in outs[1:]:
+        assert np.max(np.abs(other - outs[0])) <= 1e-8 * np.max(np.abs(outs[0]))
