@@ -7,6 +7,7 @@
 // decisions on the sign of computed values, and keeping every product rounded
 // separately keeps those decisions aligned with a plain FP64 evaluation.
 #include "hb_explicit.cuh"
+#include "hb_explicit_march.cuh"
 
 namespace hb {
 
@@ -39,10 +40,18 @@ int launch_predict(hbf_ctx* c, double dt) {
   int st = launch_eta_faces(c);
   if (st) return st;
   if ((st = tensor_lu(c, c->u, c->Lu))) return st;
-  HB_DISPATCH(c->dim, k_slopes, grid_for(g.ncell), c->u, c->slopes, g);
   const StepC k = step_consts(g, c->dim, dt, c->rho, c->theta);
-  HB_DISPATCH(c->dim, k_hats, grid_for(g.ncell), c->u, c->slopes, c->Gp, c->Lu, fo, c->predictor_visc, c->hats,
-              c->tcom, g, k);
+  if (c->dim == 3 && march_box(g)) {
+    const int chunk = march_chunk(g);
+    launch3(c, kSlotExplicit, k_slopes_x, slopes_x_grid(g), dim3(kRowX, kRowY), c->u, c->slopes, g);
+    launch3(c, kSlotExplicit, k_slopes_yz, slopes_yz_grid(g), dim3(kPredX, kPredY), c->u, c->slopes, g);
+    launch3(c, kSlotExplicit, k_hats_march, march_grid(g, chunk), dim3(kMarchThreads), c->u, c->slopes, c->Gp, c->Lu,
+            fo, c->predictor_visc, c->hats, c->tcom, g, k, chunk);
+  } else {
+    HB_DISPATCH(c->dim, k_slopes, grid_for(g.ncell), c->u, c->slopes, g);
+    HB_DISPATCH(c->dim, k_hats, grid_for(g.ncell), c->u, c->slopes, c->Gp, c->Lu, fo, c->predictor_visc, c->hats,
+                c->tcom, g, k);
+  }
   for (int a = 0; a < c->dim; ++a)
     HB_DISPATCH(c->dim, k_traces, grid_for(g.nface[a]), c->u, c->slopes, c->tcom, a, c->uL[a], c->uR[a],
                 c->uadv[a], g, k);
