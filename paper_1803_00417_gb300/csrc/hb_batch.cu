@@ -238,6 +238,7 @@ struct OpSubMean {
 template <int D, typename T>
 __global__ void __launch_bounds__(128) k_batch_bottom(const BottomArg<T>* __restrict__ args, int ncav,
                                                       const int* __restrict__ mask, int below) {
+  pdl_wait();
   const int c = blockIdx.x;
   if (c >= ncav || (mask && !mask[c])) return;
   const BottomArg<T>& a = args[c];
@@ -258,6 +259,7 @@ struct DenseArg {
 
 template <int D>
 __global__ void k_batch_dense_build(const DenseArg* __restrict__ args, int ncav) {
+  pdl_wait();
   const int c = blockIdx.y;
   if (c >= ncav) return;
   const DenseArg& a = args[c];
@@ -266,6 +268,7 @@ __global__ void k_batch_dense_build(const DenseArg* __restrict__ args, int ncav)
 }
 
 __global__ void k_batch_gauss_jordan(const DenseArg* __restrict__ args, int ncav) {
+  pdl_wait();
   const int c = blockIdx.x;
   if (c >= ncav) return;
   const DenseArg& a = args[c];
@@ -370,8 +373,8 @@ static void reduce(hbf_batch* B, const void* tab, const List& L, int mode, int s
   int grid = 152 * B->blocks_per_sm;
   if (grid > (L.n + wpb - 1) / wpb) grid = (L.n + wpb - 1) / wpb;
   if (grid < 1) grid = 1;
-  k_batch_reduce<T><<<grid, kThreads, 0, B->stream>>>((const RedArg<T>*)tab, L.d, L.n, mask, mode, B->part);
-  k_batch_combine<<<(B->ncav + wpb - 1) / wpb, kThreads, 0, B->stream>>>(B->part, L.dfirst, B->ncav, mode, scale,
+  launch_kernel(B->stream, dim3(grid), dim3(kThreads), 0, k_batch_reduce<T>, (const RedArg<T>*)tab, L.d, L.n, mask, mode, B->part);
+  launch_kernel(B->stream, dim3((B->ncav + wpb - 1) / wpb), dim3(kThreads), 0, k_batch_combine, B->part, L.dfirst, B->ncav, mode, scale,
                                                                          B->red + (size_t)slot * B->ncav);
   B->nlaunch += 2;
 }
@@ -673,7 +676,7 @@ static void vcycle(hbf_batch* B, Inst& I, const int* mask) {
       run<OpRestrictNodes<D, T>>(B, I.re[l], B->H[l + 1][kNodes], mask);
     }
   }
-  k_batch_bottom<D, T><<<B->ncav, 128, 0, B->stream>>>((const BottomArg<T>*)I.bot, B->ncav, mask, lf);
+  launch_kernel(B->stream, dim3(B->ncav), dim3(128), 0, k_batch_bottom<D, T>, (const BottomArg<T>*)I.bot, B->ncav, mask, lf);
   ++B->nlaunch;
   if (lf < B->maxlev) {
     if (I.kind == kVisc)

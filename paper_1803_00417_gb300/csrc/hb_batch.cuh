@@ -21,6 +21,7 @@ template <class Op>
 __global__ void __launch_bounds__(256) k_batch(const typename Op::Arg* __restrict__ args,
                                                const Tile* __restrict__ tiles, int ntiles,
                                                const int* __restrict__ mask, int extra) {
+  pdl_wait();
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
     const Tile T = tiles[ti];
     if (mask && !mask[T.cav]) continue;
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(256) k_batch_reduce(const RedArg<T>* __restric
                                                       const Tile* __restrict__ tiles, int ntiles,
                                                       const int* __restrict__ mask, int mode,
                                                       double* __restrict__ part) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
   for (int ti = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); ti < ntiles; ti += nwarps) {
@@ -109,6 +111,7 @@ static __global__ void __launch_bounds__(256) k_batch_combine(const double* __re
                                                               const int* __restrict__ first, int ncav, int mode,
                                                               const double* __restrict__ scale,
                                                               double* __restrict__ out) {
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
   for (int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); c < ncav; c += nwarps) {

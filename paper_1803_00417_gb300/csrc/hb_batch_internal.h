@@ -102,7 +102,8 @@ inline void run(hbf_batch* B, const void* tab, const List& L, const int* mask, i
   if (L.n == 0) return;
   int grid = 152 * B->blocks_per_sm;
   if (grid > L.n) grid = L.n;
-  k_batch<Op><<<grid, kThreads, 0, B->stream>>>((const typename Op::Arg*)tab, L.d, L.n, mask, extra);
+  launch_kernel(B->stream, dim3(grid), dim3(kThreads), 0, k_batch<Op>, (const typename Op::Arg*)tab, L.d, L.n, mask,
+                extra);
   ++B->nlaunch;
 }
 

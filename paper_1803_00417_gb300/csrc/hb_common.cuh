@@ -15,6 +15,41 @@ namespace hb {
 
 constexpr int kThreads = 256;
 
+// Programmatic dependent launch.  The solvers are chains of short kernels
+// (2 to 8 us on all levels but the finest of a large grid), and between two of
+// them the GPU stood idle for over a microsecond: draining the first, then
+// launching the second.  Each kernel of the library is therefore launched with
+// leave to start while the one before it in the stream drains (launch_kernel),
+// and begins with pdl_wait(): it waits there until every kernel before it has
+// completed and its writes are visible, and only then lets the next one start
+// launching.  So no kernel reads or writes anything before its predecessors
+// are through, and at most one launched kernel waits.  Every kernel that
+// launch_kernel launches begins with it, before any access to memory; work of
+// other kinds (copies, a caller's own kernels) is ordered as in any stream.
+__device__ __forceinline__ void pdl_wait() {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+
+// launches a kernel that begins with pdl_wait()
+template <typename... P, typename... Args>
+inline cudaError_t launch_kernel(cudaStream_t stream, dim3 grid, dim3 block, size_t smem, void (*kern)(P...),
+                                 Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 struct Geom {
   int n[3];          // cells per axis (n[2] == 1 in 2D)
   int per[3];        // 1: the axis is periodic (no walls normal to it), 0: walls

@@ -30,6 +30,7 @@ namespace {
 template <int D>
 __global__ void k_tau_norm(const double* __restrict__ u, double* __restrict__ out, const __grid_constant__ Geom g,
                            Rheo r) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     const double gn = strain_norm_at<D>(u, g, t);
     out[t] = 2.0 * viscosity(gn, r) * gn;
@@ -38,12 +39,14 @@ __global__ void k_tau_norm(const double* __restrict__ u, double* __restrict__ ou
 
 __global__ void k_absdiff(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,
                           long long n) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
     out[t] = fabs(a[t] - b[t]);
 }
 
 __global__ void k_zone_init(const double* __restrict__ tau, double tau_y, int* __restrict__ lab,
                             int* __restrict__ touch, int n) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
     lab[t] = tau[t] <= tau_y ? t : -1;
     touch[t] = 0;
@@ -54,6 +57,7 @@ __global__ void k_zone_init(const double* __restrict__ tau, double tau_y, int* _
 // pointer jump; *changed is set when any label decreased
 template <int D>
 __global__ void k_zone_step(int* __restrict__ lab, const __grid_constant__ Geom g, int* __restrict__ changed) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     const int l = lab[t];
     if (l < 0) continue;
@@ -87,6 +91,7 @@ __global__ void k_zone_step(int* __restrict__ lab, const __grid_constant__ Geom 
 // cells next to a wall
 template <int D>
 __global__ void k_zone_touch(const int* __restrict__ lab, int* __restrict__ touch, const __grid_constant__ Geom g) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     const int l = lab[t];
     if (l < 0) continue;
@@ -110,6 +115,7 @@ __global__ void k_zone_touch(const int* __restrict__ lab, int* __restrict__ touc
 // (roots) of kind 0 stagnant, 1 plug, 2 attached
 __global__ void k_zone_count(const int* __restrict__ lab, const int* __restrict__ touch,
                              unsigned long long* __restrict__ cnt, int n) {
+  pdl_wait();
   __shared__ unsigned long long sc[7];
   if (threadIdx.x < 7) sc[threadIdx.x] = 0ull;
   __syncthreads();
@@ -163,6 +169,7 @@ __device__ double centre_avg(const double* __restrict__ uc, const Geom& g, int i
 template <int D>
 __global__ void k_centreline(const double* __restrict__ uc, int along, double* __restrict__ out,
                              const __grid_constant__ Geom g) {
+  pdl_wait();
   const int mask = ((1 << D) - 1) & ~(1 << along);
   for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < g.n[along]; q += gridDim.x * blockDim.x) {
     int p[3] = {0, 0, 0};
@@ -175,6 +182,7 @@ __global__ void k_centreline(const double* __restrict__ uc, int along, double* _
 // column i sums h u_x over the cell rows
 template <int D>
 __global__ void k_psi(const double* __restrict__ ux, double* __restrict__ psi, const __grid_constant__ Geom g) {
+  pdl_wait();
   const int na = g.n[0], nb = D == 3 ? g.n[2] : g.n[1];
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= na; i += gridDim.x * blockDim.x) {
     double acc = 0.0;
@@ -196,6 +204,7 @@ __global__ void k_psi(const double* __restrict__ ux, double* __restrict__ psi, c
 // values at it and its four in-plane neighbours (NaN where outside):
 // res = {index, psi, psi(i-1), psi(i+1), psi(j-1), psi(j+1)}
 __global__ void k_psi_peak(const double* __restrict__ psi, int ea, int eb, double* __restrict__ res) {
+  pdl_wait();
   __shared__ double sv[1024];
   __shared__ int si[1024];
   const int n = ea * eb;

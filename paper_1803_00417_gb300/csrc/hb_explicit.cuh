@@ -115,6 +115,7 @@ __host__ __device__ __forceinline__ void k_eta_at(const double* __restrict__ u, 
 
 template <int D>
 __global__ void k_eta(const double* __restrict__ u, double* __restrict__ eta, const __grid_constant__ Geom g, Rheo r) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_eta_at<D>(u, eta, g, r, t);
   }
@@ -140,6 +141,7 @@ __host__ __device__ __forceinline__ void k_eta_faces_at(const double* __restrict
 
 template <int D>
 __global__ void k_eta_faces(const double* __restrict__ eta, double* __restrict__ ef, int a, const __grid_constant__ Geom g) {
+  pdl_wait();
   int ex[3] = {g.n[0] + (a == 0), g.n[1] + (a == 1), g.n[2] + (a == 2 && D == 3)};
   int nf = ex[0] * ex[1] * ex[2];
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nf; t += gridDim.x * blockDim.x) {
@@ -194,6 +196,7 @@ __host__ __device__ __forceinline__ void k_grad_p_at(const double* __restrict__ 
 
 template <int D>
 __global__ void k_grad_p(const double* __restrict__ p, double* __restrict__ Gp, const __grid_constant__ Geom g) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_grad_p_at<D>(p, Gp, g, t);
   }
@@ -250,6 +253,7 @@ __host__ __device__ __forceinline__ void k_slopes_at(const double* __restrict__ 
 
 template <int D>
 __global__ void k_slopes(const double* __restrict__ u, double* __restrict__ slopes, const __grid_constant__ Geom g) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_slopes_at<D>(u, slopes, g, t);
   }
@@ -366,6 +370,7 @@ __global__ void k_hats(const double* __restrict__ u, const double* __restrict__ 
                        const double* __restrict__ Gp, const double* __restrict__ Lu, Force fo, int pv,
                        double* __restrict__ hats, double* __restrict__ tcom, const __grid_constant__ Geom g,
                        const StepC k) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_hats_at<D>(u, slopes, Gp, Lu, fo, pv, hats, tcom, g, k, t);
   }
@@ -435,6 +440,7 @@ __global__ void k_traces(const double* __restrict__ u, const double* __restrict_
                          const double* __restrict__ tcom, int a,
                          double* __restrict__ uL, double* __restrict__ uR, double* __restrict__ uadv,
                          const __grid_constant__ Geom g, const StepC k) {
+  pdl_wait();
   int ex[3] = {g.n[0] + (a == 0), g.n[1] + (a == 1), g.n[2] + (a == 2 && D == 3)};
   int nf = ex[0] * ex[1] * ex[2];
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nf; t += gridDim.x * blockDim.x) {
@@ -467,6 +473,7 @@ __host__ __device__ __forceinline__ void k_mac_rhs_at(const double* ua0, const d
 template <int D>
 __global__ void k_mac_rhs(const double* ua0, const double* ua1, const double* ua2,
                           double* __restrict__ rhs, const __grid_constant__ Geom g) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_mac_rhs_at<D>(ua0, ua1, ua2, rhs, g, t);
   }
@@ -495,6 +502,7 @@ __host__ __device__ __forceinline__ void k_mac_correct_at(const double* __restri
 template <int D>
 __global__ void k_mac_correct(const double* __restrict__ uadv, const double* __restrict__ phi,
                               double* __restrict__ umac, int a, const __grid_constant__ Geom g) {
+  pdl_wait();
   int ex[3] = {g.n[0] + (a == 0), g.n[1] + (a == 1), g.n[2] + (a == 2 && D == 3)};
   int nf = ex[0] * ex[1] * ex[2];
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nf; t += gridDim.x * blockDim.x) {
@@ -550,6 +558,7 @@ __global__ void k_advect_rhs(const double* __restrict__ u, const double* uL0, co
                              const double* um2, const double* __restrict__ Gp,
                              const double* __restrict__ Lu, Force fo,
                              double* __restrict__ rhs, const __grid_constant__ Geom g, const StepC k) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_advect_rhs_at<D>(u, uL0, uL1, uL2, uR0, uR1, uR2, um0, um1, um2, Gp, Lu, fo, rhs, g, k, t);
   }
@@ -579,6 +588,7 @@ __host__ __device__ __forceinline__ void k_grad_p_w_at(const double* __restrict_
 template <int D>
 __global__ void k_grad_p_w(const double* __restrict__ p, const double* __restrict__ ustar, double* __restrict__ Gp,
                            double* __restrict__ w, const __grid_constant__ Geom g, const StepC k) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_grad_p_w_at<D>(p, ustar, Gp, w, g, k, t);
   }
@@ -631,6 +641,7 @@ __host__ __device__ __forceinline__ void k_nodal_rhs_at(const double* __restrict
 template <int D>
 __global__ void k_nodal_rhs(const double* __restrict__ w, double* __restrict__ out, const __grid_constant__ Geom g,
                             const StepC k) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.nnode; t += gridDim.x * blockDim.x) {
     k_nodal_rhs_at<D>(w, out, g, k, t);
   }
@@ -653,6 +664,7 @@ __host__ __device__ __forceinline__ void k_project_update_at(double* __restrict_
 template <int D>
 __global__ void k_project_update(double* __restrict__ u, const double* __restrict__ Gp,
                                  const double* __restrict__ phi, const __grid_constant__ Geom g, const StepC k) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_project_update_at<D>(u, Gp, phi, g, k, t);
   }

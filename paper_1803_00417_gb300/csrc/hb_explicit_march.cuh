@@ -82,6 +82,7 @@ __host__ __device__ __forceinline__ void slope_line(const double* __restrict__ u
 __global__ void __launch_bounds__(kPredX* kPredY) k_slopes_yz(const double* __restrict__ u,
                                                               double* __restrict__ slopes,
                                                               const __grid_constant__ Geom g) {
+  pdl_wait();
   const int nx = (g.n[0] + kPredX - 1) / kPredX, ny = (g.n[1] + kPredChunk - 1) / kPredChunk;
   const int c = blockIdx.x / nx;
   const int i = (blockIdx.x - c * nx) * kPredX + threadIdx.x;
@@ -106,6 +107,7 @@ inline dim3 slopes_yz_grid(const Geom& g) {
 // block's ends are formed by its first and last thread.
 __global__ void __launch_bounds__(kRowX* kRowY) k_slopes_x(const double* __restrict__ u, double* __restrict__ slopes,
                                                            const __grid_constant__ Geom g) {
+  pdl_wait();
   __shared__ double sdf[kRowY][3][kRowX + 2];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int i = blockIdx.y * kRowX + tx;
@@ -268,6 +270,7 @@ __global__ void __launch_bounds__(kMarchThreads, 2) k_hats_march(const double* _
                                                                  double* __restrict__ hats, double* __restrict__ tcom,
                                                                  const __grid_constant__ Geom g, const StepC k,
                                                                  int chunk) {
+  pdl_wait();
   __shared__ MarchShare sh;
   const MarchThread th(g, chunk);
   double v;

@@ -227,7 +227,7 @@ template <typename K, typename... Args>
 inline void launch(hbf_ctx* c, int slot, K kern, int grid, int block, Args... args) {
   const bool rec = prof_wants(c->prof, slot);
   if (rec) prof_mark(c, slot, true);
-  kern<<<grid, block, 0, c->stream>>>(args...);
+  launch_kernel(c->stream, dim3(grid), dim3(block), 0, kern, args...);
   if (rec) prof_mark(c, slot, false);
   ++c->nlaunch;
 }
@@ -236,7 +236,7 @@ template <typename K, typename... Args>
 inline void launch3(hbf_ctx* c, int slot, K kern, dim3 grid, dim3 block, Args... args) {
   const bool rec = prof_wants(c->prof, slot);
   if (rec) prof_mark(c, slot, true);
-  kern<<<grid, block, 0, c->stream>>>(args...);
+  launch_kernel(c->stream, dim3(grid), dim3(block), 0, kern, args...);
   if (rec) prof_mark(c, slot, false);
   ++c->nlaunch;
 }
@@ -245,7 +245,7 @@ template <typename K, typename... Args>
 inline void launch_smem(hbf_ctx* c, int slot, K kern, dim3 grid, dim3 block, size_t smem, Args... args) {
   const bool rec = prof_wants(c->prof, slot);
   if (rec) prof_mark(c, slot, true);
-  kern<<<grid, block, smem, c->stream>>>(args...);
+  launch_kernel(c->stream, grid, block, smem, kern, args...);
   if (rec) prof_mark(c, slot, false);
   ++c->nlaunch;
 }

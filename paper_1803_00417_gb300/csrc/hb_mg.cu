@@ -112,6 +112,7 @@ __device__ __forceinline__ double bits_max(unsigned long long m) {
 template <int MODE>  // 0: max |x| (non-finite -> +inf), 1: sum x, 2: weighted nodal sum
 __global__ void k_reduce_partial(const double* __restrict__ x, long long n, RedOut out, const __grid_constant__ Geom g,
                                  int dim) {
+  pdl_wait();
   double acc = 0.0;
   unsigned long long m = 0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
@@ -135,6 +136,7 @@ __global__ void k_reduce_partial(const double* __restrict__ x, long long n, RedO
 // x -= (*sum) * inv_count  (mean removal without a host round trip)
 template <typename T>
 __global__ void k_sub_mean(T* __restrict__ x, long long n, const double* __restrict__ sum, double inv_count) {
+  pdl_wait();
   T m = T(*sum * inv_count);
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
@@ -187,12 +189,14 @@ __device__ __forceinline__ void for_each4(long long n, bool vec, F4 f4, F1 f1) {
 
 template <typename T>
 __global__ void k_zero(T* __restrict__ x, long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(x), [&](long long q) { st4(x, q, V4<T>{{T(0), T(0), T(0), T(0)}}); },
       [&](long long e) { x[e] = T(0); });
 }
 
 __global__ void k_dot_partial(const double* __restrict__ a, const double* __restrict__ b, long long n, RedOut out) {
+  pdl_wait();
   double acc = 0.0;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
@@ -208,6 +212,7 @@ __global__ void k_dot_partial(const double* __restrict__ a, const double* __rest
 // +inf); 1: sum x.  x 16-byte aligned.
 template <int MODE>
 __global__ void k_reduce_partial_v(const double* __restrict__ x, long long n, RedOut out) {
+  pdl_wait();
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n2 = n >> 1;
   const double2* x2 = reinterpret_cast<const double2*>(x);
@@ -233,6 +238,7 @@ __global__ void k_reduce_partial_v(const double* __restrict__ x, long long n, Re
 }
 
 __global__ void k_dot_partial_v(const double* __restrict__ a, const double* __restrict__ b, long long n, RedOut out) {
+  pdl_wait();
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n2 = n >> 1;
   const double2* a2 = reinterpret_cast<const double2*>(a);
@@ -346,6 +352,7 @@ static __device__ __align__(256) double g_noalloc_partial[kNoAllocBlocks];
 
 // one block per kNoAllocPerBlock elements: max |x| of its chunk (non-finite -> +inf)
 __global__ void k_noalloc_maxabs_partial(const double* __restrict__ x, long long n, double* __restrict__ part) {
+  pdl_wait();
   long long base = (long long)blockIdx.x * kNoAllocPerBlock;
   double acc = 0.0;
   for (int q = 0; q < 8; ++q) {
@@ -370,6 +377,7 @@ __global__ void k_noalloc_maxabs_partial(const double* __restrict__ x, long long
 // reduce the nb partials written by this call and write dt
 __global__ void k_noalloc_cfl_final(const double* __restrict__ part, int nb, double h, double cfl,
                                     double* __restrict__ dt_out) {
+  pdl_wait();
   __shared__ double sh[32];
   double acc = 0.0;
   for (int t = threadIdx.x; t < nb; t += blockDim.x) acc = fmax(acc, part[t]);
@@ -421,6 +429,7 @@ static double* noalloc_scratch(int* st) {
 // ---------------------------------------------------------------------------
 template <typename TO, typename TI>
 __global__ void k_convert(TO* __restrict__ out, const TI* __restrict__ in, long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(out, in),
       [&](long long q) {
@@ -433,6 +442,7 @@ __global__ void k_convert(TO* __restrict__ out, const TI* __restrict__ in, long 
 // b = (float) r and x = 0: the right-hand side and the iterate of an FP32
 // correction
 __global__ void k_convert_zero(float* __restrict__ b, float* __restrict__ x, const double* __restrict__ r, long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(b, x, r),
       [&](long long q) {
@@ -448,6 +458,7 @@ __global__ void k_convert_zero(float* __restrict__ b, float* __restrict__ x, con
 
 // x (FP64) += e (FP32): the defect-correction update
 __global__ void k_add_f32(double* __restrict__ x, const float* __restrict__ e, long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(x, e),
       [&](long long q) {
@@ -465,6 +476,7 @@ __global__ void k_add_f32(double* __restrict__ x, const float* __restrict__ e, l
 template <typename T>
 __global__ void k_bicg_p(T* __restrict__ p, const T* __restrict__ r, const T* __restrict__ v, T beta, T omega,
                          T* __restrict__ z, long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(p, r, v, z),
       [&](long long q) {
@@ -485,6 +497,7 @@ __global__ void k_bicg_p(T* __restrict__ p, const T* __restrict__ r, const T* __
 template <typename T>
 __global__ void k_axmy(T* __restrict__ out, const T* __restrict__ x, T a, const T* __restrict__ y, T* __restrict__ z,
                        long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(out, x, y, z),
       [&](long long q) {
@@ -505,6 +518,7 @@ __global__ void k_axmy(T* __restrict__ out, const T* __restrict__ x, T a, const 
 template <typename T>
 __global__ void k_bicg_x(T* __restrict__ x, const T* __restrict__ ph, const T* __restrict__ sh, T alpha, T omega,
                          long long n) {
+  pdl_wait();
   for_each4(
       n, aligned16_all(x, ph, sh),
       [&](long long q) {
@@ -523,6 +537,7 @@ __global__ void k_bicg_x(T* __restrict__ x, const T* __restrict__ ph, const T* _
 // bottleneck of this reduction)
 constexpr int kDotRun = 64;
 __global__ void k_dot_partial_f(const float* __restrict__ a, const float* __restrict__ b, long long n, RedOut out) {
+  pdl_wait();
   double acc = 0.0;
   float run = 0.f;
   int k = 0;
@@ -541,6 +556,7 @@ __global__ void k_dot_partial_f(const float* __restrict__ a, const float* __rest
 
 // max |x| over a float array (non-finite -> +inf)
 __global__ void k_maxabs_partial_f(const float* __restrict__ x, long long n, RedOut out) {
+  pdl_wait();
   float m = 0.f;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x) {
@@ -590,6 +606,7 @@ __device__ __forceinline__ void max_abs(float& m, float v) {
 }
 
 __global__ void k_dot_partial_f4(const float* __restrict__ a, const float* __restrict__ b, long long n, RedOut out) {
+  pdl_wait();
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* a4 = reinterpret_cast<const float4*>(a);
@@ -605,6 +622,7 @@ __global__ void k_dot_partial_f4(const float* __restrict__ a, const float* __res
 
 // x.x and x.y in one pass over x (BiCGStab's t.t and t.s)
 __global__ void k_dot2_partial_f4(const float* __restrict__ x, const float* __restrict__ y, long long n, RedOut out) {
+  pdl_wait();
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -640,6 +658,7 @@ __global__ void k_dot2_partial_f4(const float* __restrict__ x, const float* __re
 // +inf) and w.out (the next iteration's r^.r) in the same pass
 __global__ void k_axmy_red_f4(float* __restrict__ out, const float* __restrict__ x, float a,
                               const float* __restrict__ y, const float* __restrict__ w, long long n, RedOut red) {
+  pdl_wait();
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -674,6 +693,7 @@ __global__ void k_axmy_red_f4(float* __restrict__ out, const float* __restrict__
 }
 
 __global__ void k_maxabs_partial_f4(const float* __restrict__ x, long long n, RedOut out) {
+  pdl_wait();
   const long long T = (long long)gridDim.x * blockDim.x, tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n4 = n >> 2;
   const float4* x4 = reinterpret_cast<const float4*>(x);
@@ -1048,25 +1068,25 @@ struct ViscProblem : Problem<T> {
       const T* e0 = (const T*)L.feta;
       for (int col = 0; col < 2; ++col)
         if (any_per(c->g))
-          launch3(c, slot, k_visc_smooth_c<D, T, 0, true, true>, grd, blk, x(l), (const T*)b(l), e0, e0, e0, L.g, col,
+          launch3(c, slot, k_visc_smooth_c<D, T, 0, true>, grd, blk, x(l), (const T*)b(l), e0, L.g, col,
                 (T)beta, hm);
         else
-          launch3(c, slot, k_visc_smooth_c<D, T, 0, true, false>, grd, blk, x(l), (const T*)b(l), e0, e0, e0, L.g, col,
+          launch3(c, slot, k_visc_smooth_c<D, T, 0, false>, grd, blk, x(l), (const T*)b(l), e0, L.g, col,
                 (T)beta, hm);
       for (int col = 0; col < 2; ++col)
         if (any_per(c->g))
-          launch3(c, slot, k_visc_smooth_c<D, T, 1, true, true>, grd, blk, x(l), (const T*)b(l), e0, e0, e0, L.g, col,
+          launch3(c, slot, k_visc_smooth_c<D, T, 1, true>, grd, blk, x(l), (const T*)b(l), e0, L.g, col,
                 (T)beta, hm);
         else
-          launch3(c, slot, k_visc_smooth_c<D, T, 1, true, false>, grd, blk, x(l), (const T*)b(l), e0, e0, e0, L.g, col,
+          launch3(c, slot, k_visc_smooth_c<D, T, 1, false>, grd, blk, x(l), (const T*)b(l), e0, L.g, col,
                 (T)beta, hm);
       if (D == 3)
         for (int col = 0; col < 2; ++col)
           if (any_per(c->g))
-            launch3(c, slot, k_visc_smooth_c<D, T, 2, true, true>, grd, blk, x(l), (const T*)b(l), e0, e0, e0, L.g, col,
+            launch3(c, slot, k_visc_smooth_c<D, T, 2, true>, grd, blk, x(l), (const T*)b(l), e0, L.g, col,
                   (T)beta, hm);
           else
-            launch3(c, slot, k_visc_smooth_c<D, T, 2, true, false>, grd, blk, x(l), (const T*)b(l), e0, e0, e0, L.g, col,
+            launch3(c, slot, k_visc_smooth_c<D, T, 2, false>, grd, blk, x(l), (const T*)b(l), e0, L.g, col,
                   (T)beta, hm);
       return;
     }
@@ -1607,6 +1627,7 @@ constexpr int kInnerMax = 40;  // the drop is c->inner_drop (hbf_set_inner_drop,
 
 // x (FP64) += a d (FP32);  r (FP64) -= a w (FP32)
 __global__ void k_add_scaled_f32(double* __restrict__ x, double a, const float* __restrict__ d, long long n) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     x[t] += a * (double)d[t];
@@ -1614,6 +1635,7 @@ __global__ void k_add_scaled_f32(double* __restrict__ x, double a, const float* 
 
 // y = x - y
 __global__ void k_rsub(const double* __restrict__ x, double* y, long long n) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     y[t] = x[t] - y[t];
@@ -1622,6 +1644,7 @@ __global__ void k_rsub(const double* __restrict__ x, double* y, long long n) {
 // out (FP32) = a - b (FP64)
 __global__ void k_diff_to_f32(float* __restrict__ out, const double* __restrict__ a, const double* __restrict__ b,
                               long long n) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
        t += (long long)gridDim.x * blockDim.x)
     out[t] = (float)(a[t] - b[t]);

@@ -601,20 +601,15 @@ __host__ __device__ inline bool rbx_cell(const Geom& g, int t, int col, int* p) 
 // Grid-stride over the cells of one colour (x-interior cells first); the
 // component is a template parameter so every a == C decision folds at compile
 // time.  (A grid-stride launch of about 24 blocks per SM measured faster than
-// one thread per cell.)  CE: ef0 is the cell viscosity (CellEta), else the
-// face arrays.
-template <int D, typename T, int C, bool CE = false, bool PER = true>
-__global__ void __launch_bounds__(256, CE ? 6 : 8) k_visc_smooth_c(T* __restrict__ u, const T* __restrict__ b, const T* ef0,
-                                                      const T* ef1, const T* ef2, const __grid_constant__ Geom g, int col, T beta, int hom) {
+// one thread per cell.)  eta: the cell viscosity (CellEta).
+template <int D, typename T, int C, bool PER>
+__global__ void __launch_bounds__(256, 6) k_visc_smooth_c(T* __restrict__ u, const T* __restrict__ b, const T* eta,
+                                                         const __grid_constant__ Geom g, int col, T beta, int hom) {
+  pdl_wait();
   const int nt = rbx_count<D>(g);
-  const T* ef[3] = {ef0, ef1, ef2};
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
     int p[3];
-    if (!rbx_cell<D>(g, t, col, p)) continue;
-    if (CE)
-      visc_smooth_cell<D, T, C, PER>(u, b, CellEta<T>{ef0}, g, beta, hom, p);
-    else
-      visc_smooth_cell<D, T, C, PER>(u, b, FaceEta<T>{ef}, g, beta, hom, p);
+    if (rbx_cell<D>(g, t, col, p)) visc_smooth_cell<D, T, C, PER>(u, b, CellEta<T>{eta}, g, beta, hom, p);
   }
 }
 
@@ -660,6 +655,7 @@ template <int D, typename T, bool CE = false, bool PER = true>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (CE ? 4 : 5) : 4) k_visc_op3(const T* __restrict__ u, const T* __restrict__ b,
                                                  T* __restrict__ out, const T* ef0, const T* ef1, const T* ef2,
                                                  const __grid_constant__ Geom g, T beta, int hom) {
+  pdl_wait();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   int p[3];
   if (t >= xi_count<D>(g) || !xi_cell<D>(g, t, p)) return;
@@ -707,6 +703,7 @@ __host__ __device__ __forceinline__ void k_tensor_lu_at(const T* __restrict__ u,
 template <int D, typename T>
 __global__ void __launch_bounds__(256) k_tensor_lu(const T* __restrict__ u, T* __restrict__ out, const T* ef0,
                                                   const T* ef1, const T* ef2, const __grid_constant__ Geom g, int hom) {
+  pdl_wait();
   const int nt = xi_count<D>(g);
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
     int p[3];
@@ -718,6 +715,7 @@ __global__ void __launch_bounds__(256) k_tensor_lu(const T* __restrict__ u, T* _
 template <int D, typename T>
 __global__ void k_visc_bottom(T* __restrict__ u, const T* __restrict__ b, const T* ef0, const T* ef1,
                               const T* ef2, const __grid_constant__ Geom g, T beta, int nsweep, int hom) {
+  pdl_wait();
   const T* ef[3] = {ef0, ef1, ef2};
   int nt = rb_count<D>(g);
   for (int sw = 0; sw < nsweep; ++sw)
@@ -808,6 +806,7 @@ __host__ __device__ __forceinline__ void k_cell_smooth_at(T* __restrict__ x, con
 
 template <int D, typename T, bool PER = true>
 __global__ void k_cell_smooth(T* __restrict__ x, const T* __restrict__ b, const __grid_constant__ Geom g, int col) {
+  pdl_wait();
   int nt = rb_count<D>(g);
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += gridDim.x * blockDim.x) {
     k_cell_smooth_at<D, T, PER>(x, b, g, col, t);
@@ -824,6 +823,7 @@ __host__ __device__ __forceinline__ void k_cell_resid_at(const T* __restrict__ x
 
 template <int D, typename T, bool PER = true>
 __global__ void k_cell_resid(const T* __restrict__ x, const T* __restrict__ b, T* __restrict__ r, const __grid_constant__ Geom g) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.ncell; t += gridDim.x * blockDim.x) {
     k_cell_resid_at<D, T, PER>(x, b, r, g, t);
   }
@@ -831,6 +831,7 @@ __global__ void k_cell_resid(const T* __restrict__ x, const T* __restrict__ b, T
 
 template <int D, typename T>
 __global__ void k_cell_bottom(T* __restrict__ x, const T* __restrict__ b, const __grid_constant__ Geom g, int nsweep) {
+  pdl_wait();
   int nt = rb_count<D>(g);
   for (int sw = 0; sw < nsweep; ++sw)
     for (int col = 0; col < 2; ++col) {
@@ -935,6 +936,7 @@ __host__ __device__ __forceinline__ void k_nodal_smooth_at(T* __restrict__ x, co
 
 template <int D, typename T, bool PER = true>
 __global__ void k_nodal_smooth(T* __restrict__ x, const T* __restrict__ b, const __grid_constant__ Geom g, int col) {
+  pdl_wait();
   int nt = mc_count<D>(g, col);
   const T hh = g_hh<T>(g);
   const T is0 = T(-3.0 / 8.0);  // 1 / centre weight
@@ -954,6 +956,7 @@ __host__ __device__ __forceinline__ void k_nodal_resid_at(const T* __restrict__ 
 
 template <int D, typename T, bool PER = true>
 __global__ void k_nodal_resid(const T* __restrict__ x, const T* __restrict__ b, T* __restrict__ r, const __grid_constant__ Geom g) {
+  pdl_wait();
   const T ihh = g_ihh<T>(g);
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < g.nnode; t += gridDim.x * blockDim.x) {
     k_nodal_resid_at<D, T, PER>(x, b, r, g, t);
@@ -962,6 +965,7 @@ __global__ void k_nodal_resid(const T* __restrict__ x, const T* __restrict__ b, 
 
 template <int D, typename T>
 __global__ void k_nodal_bottom(T* __restrict__ x, const T* __restrict__ b, const __grid_constant__ Geom g, int nsweep) {
+  pdl_wait();
   const T hh = g_hh<T>(g);
   const T is0 = T(-3.0 / 8.0);
   const int ncol = 1 << D;
@@ -1015,7 +1019,8 @@ __host__ __device__ __forceinline__ void k_restrict_cells_at(const T* __restrict
 
 template <int D, typename T, bool SP = false>
 __global__ void k_restrict_cells(const T* __restrict__ f, T* __restrict__ c, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc, int ncomp,
-                                 T* __restrict__ zero) {  // zero (or null): the coarse iterate, set to 0
+                                 T* __restrict__ zero) {
+  pdl_wait();  // zero (or null): the coarse iterate, set to 0
   long long tot = (long long)gc.ncell * ncomp;
   for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt < tot;
        tt += (long long)gridDim.x * blockDim.x) {
@@ -1058,6 +1063,7 @@ __host__ __device__ __forceinline__ void k_restrict_faces_at(const T* __restrict
 
 template <int D, typename T>
 __global__ void k_restrict_faces(const T* __restrict__ ff, T* __restrict__ fc, int a, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc) {
+  pdl_wait();
   int ex[3] = {gc.n[0] + (a == 0), gc.n[1] + (a == 1), gc.n[2] + (a == 2 && D == 3)};
   int nf = ex[0] * ex[1] * ex[2];
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nf; t += gridDim.x * blockDim.x) {
@@ -1121,16 +1127,6 @@ __host__ __device__ __forceinline__ void k_prolong_cells_add_at(T* __restrict__ 
   int i, j, k;
   cell_coords<D>(gf, t, i, j, k);
   xf[(size_t)comp * gf.ncell + t] += prolong_cell_value<D, T, PER>(ec + (size_t)comp * gc.ncell, gc, i, j, k, sign);
-}
-
-template <int D, typename T, bool PER = true>
-__global__ void k_prolong_cells_add(T* __restrict__ xf, const T* __restrict__ ec, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
-                                    int ncomp, T sign) {
-  long long tot = (long long)gf.ncell * ncomp;
-  for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt < tot;
-       tt += (long long)gridDim.x * blockDim.x) {
-    k_prolong_cells_add_at<D, T, PER>(xf, ec, gf, gc, ncomp, sign, tt);
-  }
 }
 
 // The same prolongation with one thread per (coarse cell, component): the
@@ -1216,6 +1212,7 @@ __host__ __device__ __forceinline__ void k_prolong_cells_add_c_at(T* __restrict_
 template <int D, typename T, bool PER = true, bool SP = false>
 __global__ void k_prolong_cells_add_c(T* __restrict__ xf, const T* __restrict__ ec, const __grid_constant__ Geom gf,
                                       const __grid_constant__ Geom gc, int ncomp, T sign) {
+  pdl_wait();
   const long long tot = (long long)gc.ncell * ncomp;
   for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt < tot;
        tt += (long long)gridDim.x * blockDim.x)
@@ -1251,6 +1248,7 @@ __host__ __device__ __forceinline__ void k_restrict_nodes_at(const T* __restrict
 template <int D, typename T, bool PER = true>
 __global__ void k_restrict_nodes(const T* __restrict__ rf, T* __restrict__ rc, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc,
                                  T* __restrict__ zero) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < gc.nnode; t += gridDim.x * blockDim.x) {
     k_restrict_nodes_at<D, T, PER>(rf, rc, gf, gc, t);
     if (zero) zero[t] = T(0);
@@ -1293,6 +1291,7 @@ __host__ __device__ __forceinline__ void k_prolong_nodes_add_at(T* __restrict__ 
 
 template <int D, typename T>
 __global__ void k_prolong_nodes_add(T* __restrict__ xf, const T* __restrict__ ec, const __grid_constant__ Geom gf, const __grid_constant__ Geom gc) {
+  pdl_wait();
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < gf.nnode; t += gridDim.x * blockDim.x) {
     k_prolong_nodes_add_at<D, T>(xf, ec, gf, gc, t);
   }
@@ -1373,6 +1372,7 @@ __device__ inline void dense_build_col(int kind, double* __restrict__ X, double*
 template <int D>
 __global__ void k_dense_build(int kind, double* __restrict__ X, double* __restrict__ M, int n, int ld,
                               const double* ef0, const double* ef1, const double* ef2, const __grid_constant__ Geom g, double beta) {
+  pdl_wait();
   dense_build_col<D>(kind, X, M, n, ld, ef0, ef1, ef2, g, beta, blockIdx.x);
 }
 
@@ -1456,6 +1456,7 @@ __device__ inline void gauss_jordan_block(const double* __restrict__ M, int m, d
 }
 
 static __global__ void k_gauss_jordan(const double* __restrict__ M, int m, double* __restrict__ Minv) {
+  pdl_wait();
   gauss_jordan_block(M, m, Minv);
 }
 
@@ -1463,6 +1464,7 @@ static __global__ void k_gauss_jordan(const double* __restrict__ M, int m, doubl
 // when present, multiplies a zero constraint value)
 static __global__ void k_dense_apply(const double* __restrict__ Minv, int m, const double* __restrict__ b, int n,
                               double* __restrict__ x) {
+  pdl_wait();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     double acc = 0.0;
     for (int j = 0; j < n; ++j) acc += Minv[(size_t)i * m + j] * b[j];

@@ -728,6 +728,7 @@ template <int D, typename T, int KIND, bool PER = true>
 __global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailTabs tb, int lf, int ncav,
                                                                   const int* __restrict__ mask, int nu1, int nu2,
                                                                   T* x_lf, const T* b_lf) {
+  pdl_wait();
   extern __shared__ __align__(16) char mem[];
   __shared__ TailLevel<T> sw[kMaxLev];
   __shared__ TailLevel<double> sbw;  // the coarsest level, when it is swept
@@ -994,11 +995,13 @@ inline cudaError_t tail_launch(cudaStream_t s, const TailTabs& tb, int lf, int n
   cfg.blockDim = dim3((unsigned)kTailThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim = {(unsigned)nblk, 1, 1};
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // it begins with pdl_wait()
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, tb, lf, ncav, mask, nu1, nu2, x_lf, b_lf);
 }
 

@@ -1,7 +1,7 @@
 // One red-black Gauss-Seidel sweep of one velocity component of the tensor
 // viscous operator (I - beta L_eta) u = b in a single launch, for the FP32
 // finest level of the viscous V-cycles in 3D (cell viscosity; the same
-// per-cell update as k_visc_smooth_c<3, float, C, true>: red cells, those with
+// per-cell update as k_visc_smooth_c<3, float, C>: red cells, those with
 // i + j + k even, from the old values, then black cells from the new red
 // ones).
 //
@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(NT, 4) k_visc_sweep_rb(const float* __restrict
                                                         const float* __restrict__ ub, const float* __restrict__ eta,
                                                         const float* __restrict__ bc, float* __restrict__ out,
                                                         const __grid_constant__ Geom g, float beta, int hom) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem& s = *reinterpret_cast<Smem*>(smem_raw);
   const int nx = g.n[0], ny = g.n[1], nz = g.n[2];

@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(256) k_visc_smooth_hom(T* u, const T* __restri
                                                          const T* __restrict__ ef0, const T* __restrict__ ef1,
                                                          const T* __restrict__ ef2, const __grid_constant__ Geom g,
                                                          int col, T bs) {
+  pdl_wait();
   const T* ef[3] = {ef0, ef1, ef2};
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < rb_count<D>(g)) visc_smooth_hom_at<D, T, PER>(u, b, inv, ef, g, C, col, bs, t);
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(256) k_visc_res_hom(const T* __restrict__ u, c
                                                       T* __restrict__ r, const T* __restrict__ ef0,
                                                       const T* __restrict__ ef1, const T* __restrict__ ef2,
                                                       const __grid_constant__ Geom g, T beta) {
+  pdl_wait();
   const T* ef[3] = {ef0, ef1, ef2};
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < g.ncell) visc_res_hom_at<D, T, PER>(u, b, r, ef, g, beta, t);
@@ -235,6 +237,7 @@ __host__ __device__ __forceinline__ void visc_inv_at(T* inv, const T* const* ef,
 template <int D, typename T>
 __global__ void __launch_bounds__(256) k_visc_inv(T* inv, const T* __restrict__ ef0, const T* __restrict__ ef1,
                                                   const T* __restrict__ ef2, const __grid_constant__ Geom g, T bs) {
+  pdl_wait();
   const T* ef[3] = {ef0, ef1, ef2};
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t < g.ncell) visc_inv_at<D, T, true>(inv, ef, g, bs, t);

@@ -507,6 +507,7 @@ __global__ void __launch_bounds__(256, VEC ? 4 : 6) k_visc_smooth_split(float* _
                                                                const float* __restrict__ eta,
                                                                const __grid_constant__ Geom g, int col, float beta,
                                                                int hom) {
+  pdl_wait();
   // the map's sizes are the launch's (split_sweep(g) on the host)
   const SplitSweep w{(int)blockDim.x, (int)blockDim.y, (int)gridDim.x, (int)gridDim.y - (g.n[1] + 31) / 32};
   split_smooth_thread<C, VEC>(u, b, eta, g, col, beta, hom, w, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x,
@@ -573,6 +574,7 @@ __global__ void __maxnreg__(64) k_visc_op_split(const float* __restrict__ u,
                                                                         const float* __restrict__ eta,
                                                                         const __grid_constant__ Geom g, float beta,
                                                                         int hom) {
+  pdl_wait();
   split_op_thread(u, b, out, eta, g, beta, hom, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x);
 }
 
@@ -625,6 +627,7 @@ __host__ __device__ __forceinline__ void split_add_pair(double* __restrict__ x, 
 // grid-stride over the ncomp ncell / 2 pairs
 __global__ void k_split_from(float* __restrict__ out, const double* __restrict__ a, const double* __restrict__ bsub,
                              const __grid_constant__ Geom g, int ncomp) {
+  pdl_wait();
   const long long tot = (long long)ncomp * (g.ncell >> 1);
   for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt < tot;
        tt += (long long)gridDim.x * blockDim.x)
@@ -633,6 +636,7 @@ __global__ void k_split_from(float* __restrict__ out, const double* __restrict__
 
 __global__ void k_split_add(double* __restrict__ x, double sc, const float* __restrict__ d,
                             const __grid_constant__ Geom g, int ncomp) {
+  pdl_wait();
   const long long tot = (long long)ncomp * (g.ncell >> 1);
   for (long long tt = blockIdx.x * (long long)blockDim.x + threadIdx.x; tt < tot;
        tt += (long long)gridDim.x * blockDim.x)

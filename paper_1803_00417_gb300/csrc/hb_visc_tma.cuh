@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(kThreads) k_visc_smooth_tma(const __grid_const
                                                               const float* __restrict__ eta,
                                                               const __grid_constant__ Geom g, const SweepGrid sg,
                                                               int col, float beta, int hom, int* __restrict__ err) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const CellEta<float> ce{eta};
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(kThreads) k_visc_op_tma(const __grid_constant_
                                                           float* __restrict__ out, const float* __restrict__ eta,
                                                           const __grid_constant__ Geom g, const SweepGrid sg,
                                                           float beta, int hom, int* __restrict__ err) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
   const CellEta<float> ce{eta};
