@@ -31,12 +31,14 @@ constexpr int kCh[4] = {16, 32, 64, 128};
 // elementwise kernels
 // ---------------------------------------------------------------------------
 __global__ void k_f32_to_bf16(bf16* __restrict__ o, const float* __restrict__ i, long long n) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
     o[t] = __float2bfloat16_rn(i[t]);
 }
 
 // input x (P points, one value) -> channel 0 of a 16-channel BF16 tensor (others 0)
 __global__ void k_pack_input(bf16* __restrict__ o, const float* __restrict__ x, long long P) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < P * 16; t += (long long)gridDim.x * blockDim.x)
     o[t] = __float2bfloat16_rn((t & 15) == 0 ? x[t >> 4] : 0.f);
 }
@@ -44,6 +46,7 @@ __global__ void k_pack_input(bf16* __restrict__ o, const float* __restrict__ x, 
 // 2^D average of children into the parent (channels-last)
 template <int D>
 __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int C, Box fine) {
+  pdl_wait();
   const Box c{fine.X / 2, fine.Y / 2, D == 3 ? fine.Z / 2 : 1};
   const long long n = (long long)c.X * c.Y * c.Z * C;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -72,6 +75,7 @@ __global__ void k_pool(const bf16* __restrict__ in, bf16* __restrict__ out, int 
 template <int D>
 __global__ void k_concat(const bf16* __restrict__ up, int Cup, const bf16* __restrict__ skip, int Cs,
                          bf16* __restrict__ out, Box fine) {
+  pdl_wait();
   const int cx = fine.X / 2, cy = fine.Y / 2, q8 = (Cup + Cs) / 8, u8 = Cup / 8;
   const long long n = (long long)fine.X * fine.Y * fine.Z * q8;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -92,6 +96,7 @@ __global__ void k_concat(const bf16* __restrict__ up, int Cup, const bf16* __res
 // head: y[p] = sum_c h[p, c] w[c] + b (FP32 output)
 __global__ void k_head_fwd(const bf16* __restrict__ h, const float* __restrict__ w, const float* __restrict__ b,
                            float* __restrict__ y, long long P) {
+  pdl_wait();
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
     float acc = b[0];
     for (int c = 0; c < 16; ++c) acc += __bfloat162float(h[p * 16 + c]) * w[c];
@@ -102,6 +107,7 @@ __global__ void k_head_fwd(const bf16* __restrict__ h, const float* __restrict__
 // head backward: gh[p, c] = gy[p] w[c] (BF16); gw[c] += sum gy h[:, c]; gb += sum gy
 __global__ void k_head_bwd(const bf16* __restrict__ h, const float* __restrict__ w, const float* __restrict__ gy,
                            bf16* __restrict__ gh, float* __restrict__ gw, float* __restrict__ gb, long long P) {
+  pdl_wait();
   float aw[16];
   float ab = 0.f;
   for (int c = 0; c < 16; ++c) aw[c] = 0.f;
@@ -137,6 +143,7 @@ __global__ void k_head_bwd(const bf16* __restrict__ h, const float* __restrict__
 // shared memory blockDim * 8 floats
 __global__ void k_relu_bias_bwd(bf16* __restrict__ g, const bf16* __restrict__ y, int C, long long P,
                                 float* __restrict__ gb) {
+  pdl_wait();
   extern __shared__ float sh[];
   const int q8 = C / 8, ch = threadIdx.x % q8, rows = blockDim.x / q8, r = threadIdx.x / q8;
   float acc[8] = {};
@@ -167,6 +174,7 @@ __global__ void k_relu_bias_bwd(bf16* __restrict__ g, const bf16* __restrict__ y
 // upsample backward: g_coarse[P, c] = sum over children of g_cat[child, c] (c < Cup)
 template <int D>
 __global__ void k_upsample_bwd(const bf16* __restrict__ gcat, int Cs, int Cup, bf16* __restrict__ gc, Box fine) {
+  pdl_wait();
   const Box c{fine.X / 2, fine.Y / 2, D == 3 ? fine.Z / 2 : 1};
   const long long n = (long long)c.X * c.Y * c.Z * Cup;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -192,6 +200,7 @@ __global__ void k_upsample_bwd(const bf16* __restrict__ gcat, int Cs, int Cup, b
 template <int D>
 __global__ void k_pool_bwd_add(const bf16* __restrict__ gnext, const bf16* __restrict__ gcat, int Cs, int off,
                                bf16* __restrict__ gout, int C, Box fine) {
+  pdl_wait();
   const Box c{fine.X / 2, fine.Y / 2, D == 3 ? fine.Z / 2 : 1};
   const float w = D == 3 ? 0.125f : 0.25f;
   const long long n = (long long)fine.X * fine.Y * fine.Z * C;
@@ -210,6 +219,7 @@ __global__ void k_pool_bwd_add(const bf16* __restrict__ gnext, const bf16* __res
 // Wt[tap', ci, co] = W[tap, co, ci], tap' = mirror of tap
 template <int D>
 __global__ void k_flip_transpose(const bf16* __restrict__ W, bf16* __restrict__ Wt, int Cout, int Cin) {
+  pdl_wait();
   const int T = D == 3 ? 27 : 9;
   const long long n = (long long)T * Cout * Cin;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
@@ -223,6 +233,7 @@ __global__ void k_flip_transpose(const bf16* __restrict__ W, bf16* __restrict__ 
 // MSE over masked points: gy = 2 mask (y - t) / nvalid; partial sums of the loss
 __global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, const float* __restrict__ mask,
                       float* __restrict__ gy, double* __restrict__ part, long long P, double inv_n) {
+  pdl_wait();
   double acc = 0.0;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
     const double r = (double)mask[p] * ((double)y[p] - (double)t[p]);
@@ -242,6 +253,7 @@ __global__ void k_mse(const float* __restrict__ y, const float* __restrict__ t, 
 
 // per-block sums of a 0/1 mask
 __global__ void k_mask_sum(const float* __restrict__ mask, double* __restrict__ part, long long P) {
+  pdl_wait();
   double acc = 0.0;
   for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x)
     acc += (double)mask[p];
@@ -260,6 +272,7 @@ __global__ void k_mask_sum(const float* __restrict__ mask, double* __restrict__ 
 __global__ void k_adam(float* __restrict__ w, float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                        bf16* __restrict__ wb, long long n, float lr, float b1, float b2, float eps, float c1,
                        float c2) {
+  pdl_wait();
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const float gg = g[t];
     const float mm = b1 * m[t] + (1.f - b1) * gg;
@@ -309,6 +322,7 @@ struct hbf_unet {
 namespace {
 
 using hb::kThreads;
+using hb::launch_kernel;
 using namespace hb::nn;
 
 template <typename T>
@@ -339,10 +353,10 @@ void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const fl
       const int per_sm = std::min(227 * 1024 / (hsmem + 1024), 512 / tc_cols(cout));
       const int blocks = std::min(tiles, 152 * std::max(1, per_sm));
       if (N->d == 3)
-        k_conv_fwd_tc_halo<3><<<blocks, kTcHaloThreads, hsmem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx,
+        launch_kernel(N->stream, dim3(blocks), dim3(kTcHaloThreads), hsmem, k_conv_fwd_tc_halo<3>, in, cin, W, b, cout, out, ostride, ooff, relu, bx,
                                                                   nbuf, tc_cols(cout), N->tc_err);
       else
-        k_conv_fwd_tc_halo<2><<<blocks, kTcHaloThreads, hsmem, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx,
+        launch_kernel(N->stream, dim3(blocks), dim3(kTcHaloThreads), hsmem, k_conv_fwd_tc_halo<2>, in, cin, W, b, cout, out, ostride, ooff, relu, bx,
                                                                   nbuf, tc_cols(cout), N->tc_err);
       return;
     }
@@ -350,7 +364,7 @@ void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const fl
     const int nt = tc_slice(blocks, cout), smem = tc_smem_bytes(cin, nt);
     const dim3 g((unsigned)blocks, (unsigned)(cout / nt), 1);
 #define HB_TC(DD, KQ) \
-  k_conv_fwd_tc<DD, KQ><<<g, kTcThreads, smem, N->stream>>>(in, cin, W, b, cout, nt, out, ostride, ooff, relu, bx, tc_cols(nt), N->tc_err)
+  launch_kernel(N->stream, dim3(g), dim3(kTcThreads), smem, k_conv_fwd_tc<DD, KQ>, in, cin, W, b, cout, nt, out, ostride, ooff, relu, bx, tc_cols(nt), N->tc_err)
     const int kq = (cin + 31) / 32;
     if (N->d == 3) {
       if (kq == 1) HB_TC(3, 1); else if (kq == 2) HB_TC(3, 2); else if (kq == 3) HB_TC(3, 3); else if (kq == 4) HB_TC(3, 4); else HB_TC(3, 6);
@@ -364,7 +378,7 @@ void conv(hbf_unet* N, int lev, const bf16* in, int cin, const bf16* W, const fl
   const int NTB = NT <= 8 ? NT : (NT % 8 == 0 ? 8 : (NT % 6 == 0 ? 6 : 4));
   dim3 g((unsigned)((N->P[lev] + 63) / 64), (unsigned)(NT / NTB), 1);
   const Box bx = N->box[lev];
-#define HB_CONV(DD, NN) k_conv_fwd<DD, NN><<<g, 128, 0, N->stream>>>(in, cin, W, b, cout, out, ostride, ooff, relu, bx)
+#define HB_CONV(DD, NN) launch_kernel(N->stream, dim3(g), dim3(128), 0, k_conv_fwd<DD, NN>, in, cin, W, b, cout, out, ostride, ooff, relu, bx)
   if (N->d == 3) {
     if (NTB == 2) HB_CONV(3, 2); else if (NTB == 4) HB_CONV(3, 4); else if (NTB == 6) HB_CONV(3, 6); else HB_CONV(3, 8);
   } else {
@@ -380,9 +394,9 @@ void wgrad(hbf_unet* N, int lev, const bf16* x, int cin, const bf16* gz, int cou
   const int chunk = (int)((stages + want - 1) / want) * kWgPts;
   dim3 g((unsigned)(tiles / taps(N->d)), (unsigned)taps(N->d), (unsigned)((N->P[lev] + chunk - 1) / chunk));
   if (N->d == 3)
-    k_conv_wgrad<3><<<g, 128, 0, N->stream>>>(x, cin, gz, cout, gW, N->box[lev], chunk);
+    launch_kernel(N->stream, dim3(g), dim3(128), 0, k_conv_wgrad<3>, x, cin, gz, cout, gW, N->box[lev], chunk);
   else
-    k_conv_wgrad<2><<<g, 128, 0, N->stream>>>(x, cin, gz, cout, gW, N->box[lev], chunk);
+    launch_kernel(N->stream, dim3(g), dim3(128), 0, k_conv_wgrad<2>, x, cin, gz, cout, gW, N->box[lev], chunk);
 }
 
 // backward of conv layer k (input `in` at level lev, output gradient g_out in
@@ -392,7 +406,7 @@ void layer_back(hbf_unet* N, int k, int lev, const bf16* in, const bf16* out, bf
   auto& Ly = N->L[k];
   const int rows = 256 / (Ly.cout / 8);  // points per block and step
   const int rb = (int)std::min<long long>((N->P[lev] + 2 * rows - 1) / (2 * rows), 304);
-  k_relu_bias_bwd<<<rb, 256, 256 * 8 * sizeof(float), N->stream>>>(g_out, out, Ly.cout, N->P[lev], Ly.gb);
+  launch_kernel(N->stream, dim3(rb), dim3(256), 256 * 8 * sizeof(float), k_relu_bias_bwd, g_out, out, Ly.cout, N->P[lev], Ly.gb);
   wgrad(N, lev, in, Ly.cin, g_out, Ly.cout, Ly.gW);
   if (g_in) conv(N, lev, g_out, Ly.cout, Ly.Wt, nullptr, Ly.cin, g_in, Ly.cin, 0, 0);
 }
@@ -401,18 +415,18 @@ void refresh_bf16(hbf_unet* N) {
   for (int k = 0; k < 14; ++k) {
     auto& Ly = N->L[k];
     const long long n = (long long)taps(N->d) * Ly.cout * Ly.cin;
-    k_f32_to_bf16<<<grid(n), kThreads, 0, N->stream>>>(Ly.Wb, Ly.W, n);
+    launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_f32_to_bf16, Ly.Wb, Ly.W, n);
     if (N->d == 3)
-      k_flip_transpose<3><<<grid(n), kThreads, 0, N->stream>>>(Ly.Wb, Ly.Wt, Ly.cout, Ly.cin);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_flip_transpose<3>, Ly.Wb, Ly.Wt, Ly.cout, Ly.cin);
     else
-      k_flip_transpose<2><<<grid(n), kThreads, 0, N->stream>>>(Ly.Wb, Ly.Wt, Ly.cout, Ly.cin);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_flip_transpose<2>, Ly.Wb, Ly.Wt, Ly.cout, Ly.cin);
   }
 }
 
 void forward(hbf_unet* N, const float* x) {
   const int c0 = kCh[0], c1 = kCh[1], c2 = kCh[2], c3 = kCh[3];
   auto* L = N->L;
-  k_pack_input<<<grid(N->P[0] * 16), kThreads, 0, N->stream>>>(N->x16, x, N->P[0]);
+  launch_kernel(N->stream, dim3(grid(N->P[0] * 16)), dim3(kThreads), 0, k_pack_input, N->x16, x, N->P[0]);
   const bf16* h = N->x16;
   for (int l = 0; l < 3; ++l) {
     conv(N, l, h, L[2 * l].cin, L[2 * l].Wb, L[2 * l].b, L[2 * l].cout, N->e[l][0], L[2 * l].cout, 0, 1);
@@ -421,9 +435,9 @@ void forward(hbf_unet* N, const float* x) {
     const int C = kCh[l];
     const long long n = N->P[l + 1] * C;
     if (N->d == 3)
-      k_pool<3><<<grid(n), kThreads, 0, N->stream>>>(N->e[l][1], N->pl[l], C, N->box[l]);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_pool<3>, N->e[l][1], N->pl[l], C, N->box[l]);
     else
-      k_pool<2><<<grid(n), kThreads, 0, N->stream>>>(N->e[l][1], N->pl[l], C, N->box[l]);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_pool<2>, N->e[l][1], N->pl[l], C, N->box[l]);
     h = N->pl[l];
   }
   conv(N, 3, N->pl[2], c2, L[6].Wb, L[6].b, c3, N->bt[0], c3, 0, 1);
@@ -435,22 +449,22 @@ void forward(hbf_unet* N, const float* x) {
     const int Cs = cup + cs[l];
     const long long n = N->P[l] * (Cs / 8);
     if (N->d == 3)
-      k_concat<3><<<grid(n), kThreads, 0, N->stream>>>(up, cup, N->e[l][1], cs[l], N->cat[l], N->box[l]);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_concat<3>, up, cup, N->e[l][1], cs[l], N->cat[l], N->box[l]);
     else
-      k_concat<2><<<grid(n), kThreads, 0, N->stream>>>(up, cup, N->e[l][1], cs[l], N->cat[l], N->box[l]);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_concat<2>, up, cup, N->e[l][1], cs[l], N->cat[l], N->box[l]);
     const int ka = 8 + 2 * (2 - l), kb = ka + 1;
     conv(N, l, N->cat[l], Cs, L[ka].Wb, L[ka].b, cs[l], N->dc[l][0], cs[l], 0, 1);
     conv(N, l, N->dc[l][0], cs[l], L[kb].Wb, L[kb].b, cs[l], N->dc[l][1], cs[l], 0, 1);
     up = N->dc[l][1];
     cup = cs[l];
   }
-  k_head_fwd<<<grid(N->P[0]), kThreads, 0, N->stream>>>(N->dc[0][1], L[14].W, L[14].b, N->y, N->P[0]);
+  launch_kernel(N->stream, dim3(grid(N->P[0])), dim3(kThreads), 0, k_head_fwd, N->dc[0][1], L[14].W, L[14].b, N->y, N->P[0]);
 }
 
 void backward(hbf_unet* N, const float* gy) {
   const int c3 = kCh[3];
   auto* L = N->L;
-  k_head_bwd<<<grid(N->P[0]), kThreads, 0, N->stream>>>(N->dc[0][1], L[14].W, gy, N->gdc[0][1], L[14].gW,
+  launch_kernel(N->stream, dim3(grid(N->P[0])), dim3(kThreads), 0, k_head_bwd, N->dc[0][1], L[14].W, gy, N->gdc[0][1], L[14].gW,
                                                          L[14].gb, N->P[0]);
   const int cs[3] = {kCh[0], kCh[1], kCh[2]};
   // decoder levels 0, 1, 2
@@ -463,9 +477,9 @@ void backward(hbf_unet* N, const float* gy) {
     bf16* gup = l == 2 ? N->gbt[1] : N->gdc[l + 1][1];
     const long long n = N->P[l + 1] * cup;
     if (N->d == 3)
-      k_upsample_bwd<3><<<grid(n), kThreads, 0, N->stream>>>(N->gcat[l], Cs, cup, gup, N->box[l]);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_upsample_bwd<3>, N->gcat[l], Cs, cup, gup, N->box[l]);
     else
-      k_upsample_bwd<2><<<grid(n), kThreads, 0, N->stream>>>(N->gcat[l], Cs, cup, gup, N->box[l]);
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_upsample_bwd<2>, N->gcat[l], Cs, cup, gup, N->box[l]);
   }
   // bottleneck
   layer_back(N, 7, 3, N->bt[0], N->bt[1], N->gbt[1], N->gbt[0]);
@@ -476,10 +490,10 @@ void backward(hbf_unet* N, const float* gy) {
     const int Cs = cup + cs[l];
     const long long n = N->P[l] * cs[l];
     if (N->d == 3)
-      k_pool_bwd_add<3><<<grid(n), kThreads, 0, N->stream>>>(N->gpl[l], N->gcat[l], Cs, cup, N->ge[l][1], cs[l],
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_pool_bwd_add<3>, N->gpl[l], N->gcat[l], Cs, cup, N->ge[l][1], cs[l],
                                                              N->box[l]);
     else
-      k_pool_bwd_add<2><<<grid(n), kThreads, 0, N->stream>>>(N->gpl[l], N->gcat[l], Cs, cup, N->ge[l][1], cs[l],
+      launch_kernel(N->stream, dim3(grid(n)), dim3(kThreads), 0, k_pool_bwd_add<2>, N->gpl[l], N->gcat[l], Cs, cup, N->ge[l][1], cs[l],
                                                              N->box[l]);
     layer_back(N, 2 * l + 1, l, N->e[l][0], N->e[l][1], N->ge[l][1], N->ge[l][0]);
     const bf16* in = l == 0 ? N->x16 : N->pl[l - 1];
@@ -505,6 +519,7 @@ namespace {
 // x[point] = r[node] * scale on the nodes, 0 in the padding
 __global__ void k_nodes_to_net(const double* __restrict__ r, double scale, int e0, int e1, int e2, Box box,
                                float* __restrict__ x) {
+  hb::pdl_wait();
   const long long P = (long long)box.X * box.Y * box.Z;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < P; t += (long long)gridDim.x * blockDim.x) {
     int i, j, k;
@@ -515,6 +530,7 @@ __global__ void k_nodes_to_net(const double* __restrict__ r, double scale, int e
 
 // delta[node] = y[point]
 __global__ void k_net_to_nodes(const float* __restrict__ y, int e0, int e1, int e2, Box box, double* __restrict__ out) {
+  hb::pdl_wait();
   const long long n = (long long)e0 * e1 * e2;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(t % e0);
@@ -543,6 +559,7 @@ int take_tc_err(hbf_unet* N, cudaStream_t s) {
 // x[point] = r[cell] * scale (FP32 cells), 0 in the padding
 __global__ void k_cells_to_net_f(const float* __restrict__ r, float scale, int e0, int e1, int e2, Box box,
                                  float* __restrict__ x) {
+  pdl_wait();
   const long long P = (long long)box.X * box.Y * box.Z;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < P; t += (long long)gridDim.x * blockDim.x) {
     int i, j, k;
@@ -552,6 +569,7 @@ __global__ void k_cells_to_net_f(const float* __restrict__ r, float scale, int e
 }
 
 __global__ void k_net_to_cells_f(const float* __restrict__ y, int e0, int e1, int e2, Box box, float* __restrict__ out) {
+  pdl_wait();
   const long long n = (long long)e0 * e1 * e2;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(t % e0);
@@ -581,10 +599,10 @@ bool visc_net_direction(hbf_ctx* c, const float* r32, double scale, float* d32) 
   cudaStream_t saved = N->stream;
   N->stream = c->stream;
   for (int q = 0; q < c->dim; ++q) {
-    k_cells_to_net_f<<<grid(N->P[0]), kThreads, 0, c->stream>>>(src + (size_t)q * gL.ncell, (float)scale, e0, e1, e2,
+    launch_kernel(c->stream, dim3(grid(N->P[0])), dim3(kThreads), 0, k_cells_to_net_f, src + (size_t)q * gL.ncell, (float)scale, e0, e1, e2,
                                                                  N->box[0], c->vnet_x);
     forward(N, c->vnet_x);
-    k_net_to_cells_f<<<grid((long long)gL.ncell), kThreads, 0, c->stream>>>(N->y, e0, e1, e2, N->box[0],
+    launch_kernel(c->stream, dim3(grid((long long)gL.ncell)), dim3(kThreads), 0, k_net_to_cells_f, N->y, e0, e1, e2, N->box[0],
                                                                            outL + (size_t)q * gL.ncell);
     c->nlaunch += N->nlaunch_fwd + 2;
   }
@@ -642,11 +660,11 @@ int apply_guess(hbf_ctx* c, const double* b, double* p, int* used) {
   const int e0 = gL.n[0] + 1, e1 = gL.n[1] + 1, e2 = c->dim == 3 ? gL.n[2] + 1 : 1;
   cudaStream_t saved = N->stream;
   N->stream = c->stream;
-  k_nodes_to_net<<<grid(N->P[0]), kThreads, 0, c->stream>>>(src, 1.0 / n0, e0, e1, e2, N->box[0], c->net_x);
+  launch_kernel(c->stream, dim3(grid(N->P[0])), dim3(kThreads), 0, k_nodes_to_net, src, 1.0 / n0, e0, e1, e2, N->box[0], c->net_x);
   forward(N, c->net_x);
   N->stream = saved;
   double* outL = L == 0 ? c->ntry : c->lv[L].nx;
-  k_net_to_nodes<<<grid((long long)gL.nnode), kThreads, 0, c->stream>>>(N->y, e0, e1, e2, N->box[0], outL);
+  launch_kernel(c->stream, dim3(grid((long long)gL.nnode)), dim3(kThreads), 0, k_net_to_nodes, N->y, e0, e1, e2, N->box[0], outL);
   c->nlaunch += N->nlaunch_fwd + 2;
   for (int l = L - 1; l >= 0; --l) {
     double* fine = l == 0 ? c->ntry : c->lv[l].nx;
@@ -894,14 +912,14 @@ int hbf_unet_loss(hbf_unet* N, const float* t_dev, const float* mask_dev, float*
   if (!N || !t_dev || !mask_dev || !gy_dev || !loss) return HBF_ERR_ARG;
   const int nb = 2432;
   // number of valid points: the mask's sum
-  k_mask_sum<<<nb, kThreads, 0, N->stream>>>(mask_dev, N->part, N->P[0]);
+  launch_kernel(N->stream, dim3(nb), dim3(kThreads), 0, k_mask_sum, mask_dev, N->part, N->P[0]);
   if (cudaMemcpyAsync(N->hpart, N->part, nb * sizeof(double), cudaMemcpyDeviceToHost, N->stream) != cudaSuccess ||
       cudaStreamSynchronize(N->stream) != cudaSuccess)
     return HBF_ERR_CUDA;
   double nvalid = 0.0;
   for (int q = 0; q < nb; ++q) nvalid += N->hpart[q];
   if (!(nvalid > 0.0)) return HBF_ERR_ARG;
-  k_mse<<<nb, kThreads, 0, N->stream>>>(N->y, t_dev, mask_dev, gy_dev, N->part, N->P[0], 1.0 / nvalid);
+  launch_kernel(N->stream, dim3(nb), dim3(kThreads), 0, k_mse, N->y, t_dev, mask_dev, gy_dev, N->part, N->P[0], 1.0 / nvalid);
   if (cudaMemcpyAsync(N->hpart, N->part, nb * sizeof(double), cudaMemcpyDeviceToHost, N->stream) != cudaSuccess ||
       cudaStreamSynchronize(N->stream) != cudaSuccess)
     return HBF_ERR_CUDA;
@@ -924,9 +942,9 @@ int hbf_unet_adam(hbf_unet* N, double lr, double b1, double b2, double eps) {
   for (int k = 0; k < 15; ++k) {
     auto& Ly = N->L[k];
     const long long nw = k < 14 ? (long long)taps(N->d) * Ly.cout * Ly.cin : 16;
-    k_adam<<<grid(nw), kThreads, 0, N->stream>>>(Ly.W, Ly.gW, Ly.mW, Ly.vW, k < 14 ? Ly.Wb : nullptr, nw, (float)lr,
+    launch_kernel(N->stream, dim3(grid(nw)), dim3(kThreads), 0, k_adam, Ly.W, Ly.gW, Ly.mW, Ly.vW, k < 14 ? Ly.Wb : nullptr, nw, (float)lr,
                                                   (float)b1, (float)b2, (float)eps, c1, c2);
-    k_adam<<<grid(Ly.cout), kThreads, 0, N->stream>>>(Ly.b, Ly.gb, Ly.mb, Ly.vb, nullptr, Ly.cout, (float)lr,
+    launch_kernel(N->stream, dim3(grid(Ly.cout)), dim3(kThreads), 0, k_adam, Ly.b, Ly.gb, Ly.mb, Ly.vb, nullptr, Ly.cout, (float)lr,
                                                        (float)b1, (float)b2, (float)eps, c1, c2);
   }
   // (the first layer's padded input channels have zero gradient and stay zero)

@@ -67,6 +67,7 @@ template <int D, int NTB>
 __global__ void __launch_bounds__(128) k_conv_fwd(const bf16* __restrict__ in, int Cin, const bf16* __restrict__ W,
                                                   const float* __restrict__ bias, int Cout, bf16* __restrict__ out,
                                                   int out_stride, int out_off, int relu, Box box) {
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, t4 = lane & 3;
   const long long P = (long long)box.X * box.Y * box.Z;
@@ -146,6 +147,7 @@ __device__ __forceinline__ void ldsm4t(uint32_t* r, uint32_t a) {
 template <int D>
 __global__ void __launch_bounds__(128) k_conv_wgrad(const bf16* __restrict__ x, int Cin, const bf16* __restrict__ gz,
                                                     int Cout, float* __restrict__ gW, Box box, int chunk) {
+  pdl_wait();
   __shared__ __align__(16) unsigned char sm[2][2][kWgPts * kWgRow];  // [buffer][gz, x]
   __shared__ float part[4][kWgTile * kWgTile];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;

@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(kTcThreads) k_conv_fwd_tc(const bf16* __restri
                                                             const float* __restrict__ bias, int Cout, int nt,
                                                             bf16* __restrict__ out, int out_stride, int out_off,
                                                             int relu, Box box, int tcols, int* __restrict__ err) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[3];  // one per stage, and one for the last MMA
   __shared__ uint32_t tmem_slot;
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(kTcHaloThreads) k_conv_fwd_tc_halo(const bf16*
                                                            bf16* __restrict__ out, int out_stride, int out_off,
                                                            int relu, Box box, int nbuf, int tcols,
                                                            int* __restrict__ err) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_slot;
