@@ -551,8 +551,8 @@ int hbf_batch_get_tiling(const hbf_batch* b, int* tile, int* blocks_per_sm, int6
 /* Multigrid levels on which every cavity has at most max_cells cells (and
  * all coarser levels) run as one launch per V-cycle, one thread-block cluster
  * per cavity, with barriers between colour sweeps; the arithmetic and its
- * order are those of the level-by-level launches.  0 disables it; default
- * 4096. */
+ * order are those of the level-by-level launches.  0 disables it; by default
+ * 4096, and in HBF_MIXED batches up to 16384 when they have few cavities. */
 int hbf_batch_set_tail(hbf_batch* b, int max_cells);
 /* Time a representative launch sequence (explicit stages and one viscous
  * V-cycle of every cavity; no cavity state changes) for each tiling

@@ -526,6 +526,17 @@ static bool plan_tail_kind(hbf_batch* B, int lf, int& nblk, size_t& smem) {
   return smem <= kTailSmem;
 }
 
+// Cells of the largest level a tail takes by default: 64^2 whatever the number
+// of cavities, and in FP32 as many as leave 2048 to each block of a cavity's
+// cluster, up to the single cavity's 16384 (16 cavities of 64^2 to 256^2, 8
+// blocks each: a colour sweep of all 128^2 levels takes 6.5 us as a launch, 2
+// us as a phase of the tail).  FP64 phases are bound by their operations.
+static int default_tail_cells(const hbf_batch* B) {
+  int nblk = 16;
+  while (nblk > 1 && nblk * B->ncav > 152) nblk >>= 1;
+  return B->precision == HBF_MIXED ? std::max(4096, std::min(16384, 2048 * nblk)) : 4096;
+}
+
 template <int D, typename T>
 static void plan_tail(hbf_batch* B, Inst& I) {
   const int lf = B->tail_level;
@@ -1346,11 +1357,12 @@ int prepare(hbf_batch* B) {
     ensure_dense(x, 2, 0.0);
   }
   B->tail_level = B->maxlev;
-  if (B->tail_cells > 0)
+  const int tail_cells = B->tail_cells < 0 ? default_tail_cells(B) : B->tail_cells;
+  if (tail_cells > 0)
     for (int l = 0; l < B->maxlev; ++l) {
       bool small = true;
       for (int c = 0; c < B->ncav && small; ++c)
-        if (l < B->nlev[c]) small = B->cav[c]->lv[l].g.ncell <= B->tail_cells;
+        if (l < B->nlev[c]) small = B->cav[c]->lv[l].g.ncell <= tail_cells;
       if (small) {
         B->tail_level = l;
         break;

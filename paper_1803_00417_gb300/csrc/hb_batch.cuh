@@ -61,6 +61,20 @@ __host__ __device__ inline double node_weight(const Geom& g, int dim, int t) {
   return w;
 }
 
+// the lane's elements of a tile in order: load(t), eight in flight, then use
+template <typename L, typename U>
+__device__ __forceinline__ void red_tile(const Tile& T0, int lane, L&& load, U&& use) {
+  int t = T0.begin + lane;
+  for (; t + 7 * 32 < T0.end; t += 8 * 32) {
+    decltype(load(0)) v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = load(t + 32 * q);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) use(v[q]);
+  }
+  for (; t < T0.end; t += 32) use(load(t));
+}
+
 // One warp per tile: lanes stride over the tile's elements, then a fixed
 // xor-shuffle tree; no block barriers, so short tiles stay cheap.
 template <typename T>
@@ -75,22 +89,28 @@ __global__ void __launch_bounds__(256) k_batch_reduce(const RedArg<T>* __restric
     const Tile T0 = tiles[ti];
     double acc = 0.0;
     if (!mask || mask[T0.cav]) {
-      const RedArg<T> a = args[T0.cav];
+      const RedArg<T>& a = args[T0.cav];
+      const T* __restrict__ x = a.x;
       // max and dot accumulate in T over the lane's share of the tile (at
-      // most tile/32 elements), then in FP64 across lanes and tiles
+      // most tile/32 elements), then in FP64 across lanes and tiles.  Loads are
+      // grouped eight at a time: one by one their latency was the kernel's time.
       if (mode == 0) {
         T m = T(0);
-        for (int t = T0.begin + lane; t < T0.end; t += 32) {
-          T v = a.x[t] < T(0) ? -a.x[t] : a.x[t];
-          if (!isfinite(v)) v = T(INFINITY);
-          m = v > m ? v : m;
-        }
+        red_tile(T0, lane, [&](int t) { return x[t] < T(0) ? -x[t] : x[t]; },
+                 [&](T v) {
+                   if (!isfinite(v)) v = T(INFINITY);
+                   m = v > m ? v : m;
+                 });
         acc = (double)m;
       } else if (mode == 1) {
-        for (int t = T0.begin + lane; t < T0.end; t += 32) acc += (double)a.x[t];
+        red_tile(T0, lane, [&](int t) { return x[t]; }, [&](T v) { acc += (double)v; });
       } else if (mode == 2) {
+        const T* __restrict__ y = a.y;
         T d = T(0);
-        for (int t = T0.begin + lane; t < T0.end; t += 32) d += a.x[t] * a.y[t];
+        struct Pair {
+          T x, y;
+        };
+        red_tile(T0, lane, [&](int t) { return Pair{x[t], y[t]}; }, [&](Pair v) { d += v.x * v.y; });
         acc = (double)d;
       } else {
         for (int t = T0.begin + lane; t < T0.end; t += 32) acc += node_weight(a.g, a.dim, t) * (double)a.x[t];

@@ -1,8 +1,8 @@
 """Multigrid solves at the sizes where their paths change: grids that are their
 own coarsest level, with exact (at most 128 unknowns) and swept bottoms; small
 FP32 finest levels with stored faces that run wholly inside the V-cycle tail,
-against the same solves level by level and in the general layout; and the first
-grid above that range.
+against the same solves level by level and in the general layout; the first
+grids above that range; and a batch's tails likewise.
 
 Tolerances: the oracle's steps to 1e-10 (each side stops its solves at 1e-10 of
 the right-hand side and the steps scale that down); solver routes of the mixed
@@ -77,3 +77,31 @@ def test_mixed_routes_agree(n):
         sim.close()
     for other in outs[1:]:
         assert np.max(np.abs(other - outs[0])) <= 1e-8 * np.max(np.abs(outs[0]))
+
+
+# the last level sizes that a batch's default tail takes in mixed precision, and the first above
+@pytest.mark.parametrize("sizes", [((128, 128), (96, 64)), ((160, 128), (64, 64), (256, 256))])
+def test_batch_default_tail_matches_level_by_level(sizes):
+    from paper_1803_00417_gb300.hbflow import MIXED, Batch
+
+    cfgs = [cavity(n, Re=100.0, Bi=10.0, Pa=1e4, nexp=1.2) for n in sizes]
+    outs = []
+    for tail in (None, 0):
+        B = Batch([c["n"] for c in cfgs], [c["h"] for c in cfgs], [c["wall_u"] for c in cfgs], precision=MIXED)
+        if tail is not None:
+            B.set_tail(tail)
+        for i, c in enumerate(cfgs):
+            v = B.cavity(i)
+            v.set_rheology(c["K"], c["nexp"], c["tau_y"], c["m"])
+            u, p = random_state(c["n"], seed=sum(c["n"]))
+            v.set_velocity(u)
+            v.set_pressure(p)
+        B.set_dt([c["dt"] for c in cfgs])
+        for _ in range(2):
+            st = B.step()
+            assert all(s[k]["converged"] for s in st for k in ("mac", "visc", "nodal")), st
+        outs.append([np.concatenate([B.cavity(i).get_field("U"), B.cavity(i).get_field("P")])
+                     for i in range(len(cfgs))])
+        B.close()
+    for a, b in zip(*outs):
+        assert np.max(np.abs(b - a)) <= 1e-8 * np.max(np.abs(a))
