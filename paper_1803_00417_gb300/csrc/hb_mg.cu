@@ -3,7 +3,7 @@
 // V(nu1, nu2) cycle, as stated for the three solves of Sec. III A:
 //   nu1 smoothing sweeps; r = b - A x; restrict r to the next level's b;
 //   x_coarse = 0; recurse; x += P x_coarse; nu2 sweeps.
-//   coarsest level: nu_bottom sweeps in a single thread block.
+//   coarsest level: an exact inverse (at most 128 unknowns) or nu_bottom sweeps.
 //   stop when ||b - A x||_inf <= rtol ||b||_inf.
 // Singular problems (MAC and nodal potentials) remove the (weighted) mean of
 // the right-hand side and pin the mean of the iterate after each cycle and the
@@ -862,8 +862,8 @@ static void bottom_fp64(Problem<T>& P, int l, double* xd, double* bd, void (*run
 
 // ---------------------------------------------------------------------------
 // fused tail of the V-cycle (k_vcycle_tail): from the first level with at
-// most c->tail_cells cells (hbf_set_tail) down to the exact bottom solve and
-// back in one launch of one block, instead of about twenty launches per level
+// most c->tail_cells cells (hbf_set_tail) down to the bottom solve and
+// back in one launch of one cluster, instead of about twenty launches per level
 // ---------------------------------------------------------------------------
 
 // the exact bottom solve of problem kind: at most kDenseMax unknowns on the
@@ -1008,6 +1008,22 @@ static bool run_tail(hbf_ctx* c, int l, double beta, T* x0, const T* b0) {
 
 static bool staged_op(hbf_ctx* c, int slot, const float* u, const float* b, float* out, const float* eta,
                       const Geom& g, float beta, int hm);
+
+// r = b - L x on the nodes of a level
+template <int D, typename T>
+static void nodal_resid(hbf_ctx* c, int slot, const T* x, const T* b, T* r, const Geom& g) {
+  if constexpr (D == 3 && std::is_same<T, double>::value)
+    if (nodal_march_level(g)) {
+      const int chunk = nodal_march_chunk(g);
+      launch3(c, slot, any_per(g) ? k_nodal_resid_z<true> : k_nodal_resid_z<false>, nodal_march_grid(g, chunk),
+              dim3(kThreads), x, b, r, g, chunk);
+      return;
+    }
+  if (any_per(g))
+    launch(c, slot, k_nodal_resid<D, T, true>, grid_for(g.nnode), kThreads, x, b, r, g);
+  else
+    launch(c, slot, k_nodal_resid<D, T, false>, grid_for(g.nnode), kThreads, x, b, r, g);
+}
 
 // u - beta L u of a small FP32 finest level (faces0)
 template <int D>
@@ -1462,15 +1478,7 @@ struct NodalProblem : Problem<T> {
       }
   }
   void resid(int l) override {
-    Level& L = c->lv[l];
-    {
-      if (any_per(c->g))
-        launch(c, l == 0 ? kSlotNodalResid : kSlotCoarse, k_nodal_resid<D, T, true>, grid_for(L.g.nnode), kThreads, x(l), b(l),
-           r(l), L.g);
-      else
-        launch(c, l == 0 ? kSlotNodalResid : kSlotCoarse, k_nodal_resid<D, T, false>, grid_for(L.g.nnode), kThreads, x(l), b(l),
-           r(l), L.g);
-    }
+    nodal_resid<D, T>(c, l == 0 ? kSlotNodalResid : kSlotCoarse, x(l), b(l), r(l), c->lv[l].g);
   }
   void restrict_to(int l) override {
     Level &F = c->lv[l], &C = c->lv[l + 1];
@@ -2017,17 +2025,10 @@ int solve_nodal(hbf_ctx* c, const double* rhs, double* phi, hbf_solve_stats* s) 
 }
 
 int nodal_residual(hbf_ctx* c, const double* b, const double* x, double* r) {
-  if (c->dim == 2) {
-    if (any_per(c->g))
-      launch(c, kSlotNodalResid, k_nodal_resid<2, double, true>, grid_for(c->g.nnode), kThreads, x, b, r, c->g);
-    else
-      launch(c, kSlotNodalResid, k_nodal_resid<2, double, false>, grid_for(c->g.nnode), kThreads, x, b, r, c->g);
-  } else {
-    if (any_per(c->g))
-      launch(c, kSlotNodalResid, k_nodal_resid<3, double, true>, grid_for(c->g.nnode), kThreads, x, b, r, c->g);
-    else
-      launch(c, kSlotNodalResid, k_nodal_resid<3, double, false>, grid_for(c->g.nnode), kThreads, x, b, r, c->g);
-  }
+  if (c->dim == 2)
+    nodal_resid<2, double>(c, kSlotNodalResid, x, b, r, c->g);
+  else
+    nodal_resid<3, double>(c, kSlotNodalResid, x, b, r, c->g);
   return cuda_check(c, cudaGetLastError(), "nodal residual");
 }
 
