@@ -966,7 +966,8 @@ __global__ void k_nodal_resid(const T* __restrict__ x, const T* __restrict__ b, 
 // The 3D FP64 residual of large levels, a thread marching up a column of nodes:
 // each plane's sums of the four neighbours and the four diagonal ones serve
 // three nodes, 13 FP64 operations a node instead of 22 (which bound both forms:
-// 55 -> 49 us averaged over the two finest levels at 128^3).  The terms and their order are k_nodal_resid's.
+// the nodal residuals of a 128^3 FP64 step took 1.42 ms, 1.00 now).  The terms
+// and their order are k_nodal_resid's.
 // Threads take the e0 e1 columns in order, blockIdx.y the chunks of planes.
 template <bool PER>
 __global__ void __launch_bounds__(256) k_nodal_resid_z(const double* __restrict__ x, const double* __restrict__ b,
