@@ -480,6 +480,31 @@ __host__ __device__ inline int rb_count(const Geom& g) {
   return ((g.n[0] + 1) / 2) * g.n[1] * (D == 3 ? g.n[2] : 1);
 }
 
+// A periodic axis of an odd number of cells (only a coarsest level has one: the
+// finest level's are even, and a level with an odd axis is not coarsened) makes
+// cells 0 and n - 1 of a row neighbours of one colour.  Such a level takes each
+// colour in two parts with a barrier between them: a cell is in part 1 when it
+// is the last one on an odd number of those axes, so a neighbour through a wrap
+// is always in the other part.
+__host__ __device__ __forceinline__ bool odd_wrap(const Geom& g, int a) { return g.per[a] && (g.n[a] & 1); }
+__host__ __device__ __forceinline__ int rb_parts(const Geom& g) {
+  return odd_wrap(g, 0) || odd_wrap(g, 1) || odd_wrap(g, 2) ? 2 : 1;
+}
+__host__ __device__ __forceinline__ int rb_part(const Geom& g, const int* p) {
+  int part = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) part ^= odd_wrap(g, a) && p[a] == g.n[a] - 1;
+  return part;
+}
+// passes of one component's sweep in order (colour, part), and thread t -> cell
+// of pass q
+__host__ __device__ __forceinline__ int rb_passes(const Geom& g) { return 2 * rb_parts(g); }
+template <int D>
+__host__ __device__ inline bool rb_pass_cell(const Geom& g, int t, int q, int* p) {
+  const int two = rb_parts(g) - 1;
+  return rb_cell<D>(g, t, q >> two, p) && (!two || rb_part(g, p) == (q & 1));
+}
+
 // Gauss-Seidel update of component C at cell p of the current colour
 template <int D, typename T, int C, bool PER = true, typename EF>
 __host__ __device__ __forceinline__ void visc_smooth_cell(T* __restrict__ u, const T* __restrict__ b, const EF& ef,
@@ -717,13 +742,13 @@ __global__ void k_visc_bottom(T* __restrict__ u, const T* __restrict__ b, const 
                               const T* ef2, const __grid_constant__ Geom g, T beta, int nsweep, int hom) {
   pdl_wait();
   const T* ef[3] = {ef0, ef1, ef2};
-  int nt = rb_count<D>(g);
+  const int nt = rb_count<D>(g), np = rb_passes(g);
   for (int sw = 0; sw < nsweep; ++sw)
     for (int c = 0; c < D; ++c)
-      for (int col = 0; col < 2; ++col) {
+      for (int q = 0; q < np; ++q) {
         for (int t = threadIdx.x; t < nt; t += blockDim.x) {
           int p[3];
-          if (!rb_cell<D>(g, t, col, p)) continue;
+          if (!rb_pass_cell<D>(g, t, q, p)) continue;
           T v = visc_gs_point<D, T>(u, b, FaceEta<T>{ef}, g, c, p, beta, hom != 0);
           u[(size_t)c * g.ncell + cidx<D>(g, p[0], p[1], p[2])] = v;
         }
@@ -832,12 +857,12 @@ __global__ void k_cell_resid(const T* __restrict__ x, const T* __restrict__ b, T
 template <int D, typename T>
 __global__ void k_cell_bottom(T* __restrict__ x, const T* __restrict__ b, const __grid_constant__ Geom g, int nsweep) {
   pdl_wait();
-  int nt = rb_count<D>(g);
+  const int nt = rb_count<D>(g), np = rb_passes(g);
   for (int sw = 0; sw < nsweep; ++sw)
-    for (int col = 0; col < 2; ++col) {
+    for (int q = 0; q < np; ++q) {
       for (int t = threadIdx.x; t < nt; t += blockDim.x) {
         int p[3];
-        if (!rb_cell<D>(g, t, col, p)) continue;
+        if (!rb_pass_cell<D>(g, t, q, p)) continue;
         x[cidx<D>(g, p[0], p[1], p[2])] = cell_gs_point<D, T>(x, b, g, p);
       }
       __syncthreads();
@@ -919,6 +944,57 @@ __host__ __device__ inline int mc_count(const Geom& g, int col) {
   int c = 1;
   for (int a = 0; a < D; ++a) c *= (e[a] - ((col >> a) & 1) + 1) / 2;
   return c;
+}
+
+// The passes of a nodal sweep: one class of positions per axis, the even and
+// the odd ones; on a periodic axis of an odd number of cells (see rb_parts)
+// nodes 0 and n - 1, both even, are neighbours through the wrap, and node n is
+// node 0: three classes, the even ones below n - 1 with node n, the odd ones
+// below n, and node n - 1.  Class c of axis a has nd_count positions, the i-th
+// is nd_pos; without such an axis pass and colour (mc_node) are the same.
+__host__ __device__ __forceinline__ int nd_count(const Geom& g, int a, int c) {
+  return odd_wrap(g, a) ? (c == 2 ? 1 : (g.n[a] + 1) / 2 - c) : (g.n[a] + 2 - c) / 2;
+}
+__host__ __device__ __forceinline__ int nd_pos(const Geom& g, int a, int c, int i) {
+  const int n = g.n[a], q = 2 * i + c;
+  if (!odd_wrap(g, a)) return q;
+  return c == 2 ? n - 1 : (q == n - 1 ? n : q);
+}
+template <int D>
+__host__ __device__ __forceinline__ int nd_passes(const Geom& g) {
+  int m = 1;
+#pragma unroll
+  for (int a = 0; a < D; ++a) m *= odd_wrap(g, a) ? 3 : 2;
+  return m;
+}
+template <int D>
+__host__ __device__ __forceinline__ void nd_classes(const Geom& g, int pass, int* c) {
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const int r = odd_wrap(g, a) ? pass / 3 : pass >> 1;
+    c[a] = pass - r * (odd_wrap(g, a) ? 3 : 2);
+    pass = r;
+  }
+}
+template <int D>
+__host__ __device__ inline int nd_pass_count(const Geom& g, int pass) {
+  int c[3], n = 1;
+  nd_classes<D>(g, pass, c);
+  for (int a = 0; a < D; ++a) n *= nd_count(g, a, c[a]);
+  return n;
+}
+// thread t of a pass of nd_pass_count nodes -> node
+template <int D>
+__host__ __device__ inline void nd_pass_node(const Geom& g, int t, int pass, int* p) {
+  int c[3];
+  nd_classes<D>(g, pass, c);
+  p[2] = 0;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const int n = nd_count(g, a, c[a]), r = t / n;
+    p[a] = nd_pos(g, a, c[a], t - r * n);
+    t = r;
+  }
 }
 
 template <int D, typename T, bool PER = true>
@@ -1017,13 +1093,13 @@ __global__ void k_nodal_bottom(T* __restrict__ x, const T* __restrict__ b, const
   pdl_wait();
   const T hh = g_hh<T>(g);
   const T is0 = T(-3.0 / 8.0);
-  const int ncol = 1 << D;
+  const int np = nd_passes<D>(g);
   for (int sw = 0; sw < nsweep; ++sw)
-    for (int col = 0; col < ncol; ++col) {
-      int nt = mc_count<D>(g, col);
+    for (int q = 0; q < np; ++q) {
+      const int nt = nd_pass_count<D>(g, q);
       for (int t = threadIdx.x; t < nt; t += blockDim.x) {
         int p[3];
-        if (!mc_node<D>(g, t, col, p)) continue;
+        nd_pass_node<D>(g, t, q, p);
         int id = nidx(g, p[0], p[1], p[2]);
         T s = nodal_lap_point<D, T>(x, g, p, true);
         x[id] = (hh * b[id] - s) * is0;

@@ -327,7 +327,7 @@ struct SlabNbr {
 
 // neighbour offsets of node p of the slab
 template <int D, bool PER>
-__device__ __forceinline__ void slab_node_offsets(const Geom& g, int ps, const int* p, int* om, int* op) {
+__host__ __device__ __forceinline__ void slab_node_offsets(const Geom& g, int ps, const int* p, int* om, int* op) {
   node_offsets(p[0], g.n[0], 1, PER && g.per[0], om[0], op[0]);
   if (D == 3) node_offsets(p[1], g.n[1], g.n[0] + 1, PER && g.per[1], om[1], op[1]);
   const bool per = PER && g.per[D - 1];  // a periodic neighbour is in the halo
@@ -335,55 +335,96 @@ __device__ __forceinline__ void slab_node_offsets(const Geom& g, int ps, const i
   op[D - 1] = p[D - 1] == g.n[D - 1] && !per ? -ps : ps;
 }
 
-// passes of one sweep: (component, colour), or the colours
-template <int D, int KIND>
-constexpr int tail_passes() {
-  return KIND == kVisc ? 2 * D : (KIND == kMac ? 2 : 1 << D);
+// passes of one sweep: (component, colour), or the colours.  ODD: the level may
+// be odd along a periodic axis and then has more (rb_parts, nd_classes); only a
+// swept coarsest level may, and in the others the code for it costs 5%.
+template <int D, int KIND, bool ODD>
+__host__ __device__ __forceinline__ int tail_passes(const Geom& g) {
+  if (KIND == kNodal) return ODD ? nd_passes<D>(g) : 1 << D;
+  return (KIND == kVisc ? 2 * D : 2) * (ODD ? rb_parts(g) : 1);
+}
+
+// threads of one pass over this block's points of a level, and the point p of
+// thread t (false: none).  An odd periodic slowest axis of nodes is not cut
+// (such a level is swept by block 0 alone).
+template <int D, typename T, int KIND, bool ODD>
+__host__ __device__ __forceinline__ int tail_pass_count(const TailLevel<T>& w, const Geom& g, int pass) {
+  if (KIND != kNodal) return (g.n[0] + 1) / 2 * (D == 3 ? g.n[1] : 1) * (w.k1 - w.k0);
+  int c[3] = {pass & 1, (pass >> 1) & 1, (pass >> 2) & 1};
+  if (ODD) nd_classes<D>(g, pass, c);
+  int nk;
+  if (ODD && odd_wrap(g, D - 1)) {
+    nk = nd_count(g, D - 1, c[D - 1]);
+  } else {
+    const int kf = w.k0 + ((w.k0 + c[D - 1]) & 1);  // the slab's first plane of the colour
+    nk = kf < w.k1 ? (w.k1 - kf + 1) / 2 : 0;
+  }
+  const int c0 = ODD ? nd_count(g, 0, c[0]) : (g.n[0] + 2 - c[0]) / 2;
+  const int c1 = D == 3 ? (ODD ? nd_count(g, 1, c[1]) : (g.n[1] + 2 - c[1]) / 2) : 1;
+  return c0 * c1 * nk;
+}
+template <int D, typename T, int KIND, bool ODD>
+__host__ __device__ __forceinline__ bool tail_pass_point(const TailLevel<T>& w, const Geom& g, int pass, int t, int* p) {
+  p[1] = p[2] = 0;
+  if constexpr (KIND != kNodal) {
+    const int two = ODD ? rb_parts(g) - 1 : 0, col = (pass >> two) & 1;
+    const int nh = (g.n[0] + 1) / 2;
+    const int r = divm(t, nh, g.m_rb), ih = t - r * nh;
+    const int kl = D == 3 ? divm(r, g.n[1], g.m_n1) : r, j = D == 3 ? r - kl * g.n[1] : 0;
+    const int k = w.k0 + kl;
+    p[0] = 2 * ih + ((j + k + col) & 1);
+    p[1] = j;
+    p[D - 1] = k;
+    if (p[0] >= g.n[0]) return false;
+    return !(ODD && two) || rb_part(g, p) == (pass & 1);
+  } else {
+    int c[3] = {pass & 1, (pass >> 1) & 1, (pass >> 2) & 1};
+    if (ODD && rb_parts(g) == 2) {
+      nd_classes<D>(g, pass, c);
+      const int c0 = nd_count(g, 0, c[0]), c1 = D == 3 ? nd_count(g, 1, c[1]) : 1;
+      const int r = t / c0, kk = r / c1;
+      p[0] = nd_pos(g, 0, c[0], t - r * c0);
+      if (D == 3) p[1] = nd_pos(g, 1, c[1], r - kk * c1);
+      p[D - 1] = odd_wrap(g, D - 1) ? nd_pos(g, D - 1, c[D - 1], kk) : w.k0 + ((w.k0 + c[D - 1]) & 1) + 2 * kk;
+      return true;
+    }
+    const int c0 = (g.n[0] + 2 - c[0]) / 2, c1 = D == 3 ? (g.n[1] + 2 - c[1]) / 2 : 1;
+    const int r = divm(t, c0, g.m_mc0[c[0]]), kk = D == 3 ? divm(r, c1, g.m_mc1[c[1]]) : r;
+    p[0] = 2 * (t - r * c0) + c[0];
+    if (D == 3) p[1] = 2 * (r - kk * c1) + c[1];
+    p[D - 1] = w.k0 + ((w.k0 + c[D - 1]) & 1) + 2 * kk;
+    return true;
+  }
 }
 
 // one pass over this block's points of a level
-template <int D, typename T, int KIND, bool PER>
+template <int D, typename T, int KIND, bool PER, bool ODD>
 __device__ __forceinline__ void tail_pass(char* mem, const TailLevel<T>& w, const Geom& g, T bs, int pass,
                                           unsigned rank) {
   const bool per = PER && g.per[D - 1];
   T* x = (T*)(mem + w.x);
   const T* b = (const T*)(mem + w.b);
-  if constexpr (KIND != kNodal) {
-    const int c = KIND == kVisc ? pass >> 1 : 0, col = KIND == kVisc ? pass & 1 : pass;
-    const int nh = (g.n[0] + 1) / 2, n = nh * (D == 3 ? g.n[1] : 1) * (w.k1 - w.k0);
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      const int r = divm(t, nh, g.m_rb), ih = t - r * nh;
-      const int kl = D == 3 ? divm(r, g.n[1], g.m_n1) : r, j = D == 3 ? r - kl * g.n[1] : 0;
-      const int k = w.k0 + kl, i = 2 * ih + ((j + k + col) & 1);
-      if (i >= g.n[0]) continue;
-      const int p[3] = {i, D == 3 ? j : k, k};
-      const int q = i + g.n[0] * j, o = kl * w.ps + q;
-      T v;
-      if constexpr (KIND == kVisc) {
-        const int oc = c * w.rp * w.ps + o;
-        v = hom_gs<D, T>(tail_hom_cell<D, T, PER>(mem, w, g, c, p), b[oc], ((const T*)(mem + w.inv))[oc], bs);
-      } else {
-        const SlabNbr<D, PER> nb(g, w.ps, p);
-        v = cell_gs_value<D, T>(x + o + w.ps, b[o], g_hh<T>(g), nb.om, nb.op, nb.lo, nb.hi);
-      }
-      tail_put<D, T, KIND, PER>(x, w, per, c, k, q, rank, v);
-    }
-  } else {
-    const int b0 = pass & 1, b1 = (pass >> 1) & 1, bz = D == 3 ? (pass >> 2) & 1 : b1;
-    const int c0 = (g.n[0] + 2 - b0) / 2, c1 = D == 3 ? (g.n[1] + 2 - b1) / 2 : 1;
-    const int kf = w.k0 + ((w.k0 + bz) & 1);  // the slab's first plane of the colour
-    const int nk = kf < w.k1 ? (w.k1 - kf + 1) / 2 : 0, n = c0 * c1 * nk;
-    for (int t = threadIdx.x; t < n; t += blockDim.x) {
-      const int r = divm(t, c0, g.m_mc0[b0]), i = 2 * (t - r * c0) + b0;
-      const int kk = D == 3 ? divm(r, c1, g.m_mc1[b1]) : r, j = D == 3 ? 2 * (r - kk * c1) + b1 : 0;
-      const int k = kf + 2 * kk;
-      const int p[3] = {i, D == 3 ? j : k, k};
-      const int q = i + (g.n[0] + 1) * j, o = (k - w.k0) * w.ps + q;
+  const int n = tail_pass_count<D, T, KIND, ODD>(w, g, pass);
+  for (int t = threadIdx.x; t < n; t += blockDim.x) {
+    int p[3];
+    if (!tail_pass_point<D, T, KIND, ODD>(w, g, pass, t, p)) continue;
+    const int k = p[D - 1], q = p[0] + (KIND == kNodal ? g.n[0] + 1 : g.n[0]) * (D == 3 ? p[1] : 0);
+    const int o = (k - w.k0) * w.ps + q;
+    int c = 0;
+    T v;
+    if constexpr (KIND == kVisc) {
+      c = pass >> (ODD ? rb_parts(g) : 1);
+      const int oc = c * w.rp * w.ps + o;
+      v = hom_gs<D, T>(tail_hom_cell<D, T, PER>(mem, w, g, c, p), b[oc], ((const T*)(mem + w.inv))[oc], bs);
+    } else if constexpr (KIND == kMac) {
+      const SlabNbr<D, PER> nb(g, w.ps, p);
+      v = cell_gs_value<D, T>(x + o + w.ps, b[o], g_hh<T>(g), nb.om, nb.op, nb.lo, nb.hi);
+    } else {
       int om[3], op[3];
       slab_node_offsets<D, PER>(g, w.ps, p, om, op);
-      const T s = nodal_nbr_sum<D, T>(x + o + w.ps, om, op);
-      tail_put<D, T, KIND, PER>(x, w, per, 0, k, q, rank, (g_hh<T>(g) * b[o] - s) * T(-3.0 / 8.0));
+      v = (g_hh<T>(g) * b[o] - nodal_nbr_sum<D, T>(x + o + w.ps, om, op)) * T(-3.0 / 8.0);
     }
+    tail_put<D, T, KIND, PER>(x, w, per, c, k, q, rank, v);
   }
 }
 
@@ -430,16 +471,16 @@ constexpr int tail_slots() {
 
 template <int D, typename T>
 struct TailSlot {
-  int col = -1;       // colour; -1: no point
+  int col = -1;       // pass of its component; -1: no point
   int k, q, o;        // plane, point of the plane, offset in x
   int om[D], op[D];   // neighbours
   unsigned wall = 0;  // bit 2a: no neighbour below on axis a (a wall), bit 2a + 1: above
-  __device__ __forceinline__ unsigned flip(int bit) const { return (wall << (31 - bit)) & 0x80000000u; }
+  __host__ __device__ __forceinline__ unsigned flip(int bit) const { return (wall << (31 - bit)) & 0x80000000u; }
 };
 
 // this thread's slot u of the block's points of the level
-template <int D, typename T, int KIND, bool PER>
-__device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const TailLevel<T>& w, const Geom& g, int u) {
+template <int D, typename T, int KIND, bool PER, bool ODD>
+__host__ __device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const TailLevel<T>& w, const Geom& g, int u) {
   int p[3] = {0, 0, 0};
   s.col = -1;
   s.wall = 0;
@@ -455,7 +496,7 @@ __device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const TailLeve
     if (p[0] >= g.n[0]) return;
     p[1] = j;
     p[D - 1] = s.k;
-    s.col = col;
+    s.col = ODD && rb_parts(g) == 2 ? 2 * col + rb_part(g, p) : col;
     s.q = p[0] + g.n[0] * j;
     const HomAxis x(p[0], g.n[0], 1, PER && g.per[0]);
     s.om[0] = x.om;
@@ -473,18 +514,12 @@ __device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const TailLeve
     s.wall |= ((z.fm >> 31) << (2 * D - 2)) | ((z.fp >> 31) << (2 * D - 1));
   } else {
     int t = u;
-    for (int col = 0; col < (1 << D); ++col) {
-      const int b0 = col & 1, b1 = (col >> 1) & 1, bz = D == 3 ? (col >> 2) & 1 : b1;
-      const int c0 = (g.n[0] + 2 - b0) / 2, c1 = D == 3 ? (g.n[1] + 2 - b1) / 2 : 1;
-      const int kf = w.k0 + ((w.k0 + bz) & 1);
-      const int n = kf < w.k1 ? c0 * c1 * ((w.k1 - kf + 1) / 2) : 0;
+    for (int col = 0; col < tail_passes<D, KIND, ODD>(g); ++col) {
+      const int n = tail_pass_count<D, T, KIND, ODD>(w, g, col);
       if (t < n) {
-        const int r = t / c0, kk = r / c1;
-        s.k = kf + 2 * kk;
-        p[0] = 2 * (t - r * c0) + b0;
-        p[1] = D == 3 ? 2 * (r - kk * c1) + b1 : 0;
-        s.q = p[0] + (g.n[0] + 1) * p[1];
-        p[D - 1] = s.k;
+        tail_pass_point<D, T, KIND, ODD>(w, g, col, t, p);
+        s.k = p[D - 1];
+        s.q = p[0] + (g.n[0] + 1) * (D == 3 ? p[1] : 0);
         s.col = col;
         break;
       }
@@ -506,11 +541,12 @@ __device__ __forceinline__ bool tail_fits_slots(const TailLevel<T>& w, const Geo
 
 // sweeps sweeps of the level, a barrier after each pass; then, when r is not
 // null, the residual into r (the whole level's layout) and a barrier
-template <int D, typename T, int KIND, bool PER, class S>
+template <int D, typename T, int KIND, bool PER, bool ODD, class S>
 __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, const Geom& g, T beta, int sweeps, T* r,
                                            unsigned rank, S sync) {
   const T bs = KIND == kVisc ? rn_mul(beta, g_ihh<T>(g)) : T(0);
   constexpr int NS = tail_slots<D, KIND>();
+  const int np = tail_passes<D, KIND, ODD>(g) / (KIND == kVisc ? D : 1);  // passes per component
   const bool per = PER && g.per[D - 1];
   T* const x = (T*)(mem + w.x);
   const T* const b = (const T*)(mem + w.b);
@@ -518,8 +554,8 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
 #pragma unroll 1
     for (int s = 0; s < sweeps; ++s)
 #pragma unroll 1
-      for (int q = 0; q < tail_passes<D, KIND>(); ++q) {
-        tail_pass<D, T, KIND, PER>(mem, w, g, bs, q, rank);
+      for (int q = 0; q < (KIND == kVisc ? D * np : np); ++q) {
+        tail_pass<D, T, KIND, PER, ODD>(mem, w, g, bs, q, rank);
         sync();
       }
     if (r) {
@@ -530,7 +566,7 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
   }
   TailSlot<D, T> sl[NS];
 #pragma unroll
-  for (int i = 0; i < NS; ++i) tail_slot_init<D, T, KIND, PER>(sl[i], w, g, (int)threadIdx.x + i * kTailThreads);
+  for (int i = 0; i < NS; ++i) tail_slot_init<D, T, KIND, PER, ODD>(sl[i], w, g, (int)threadIdx.x + i * kTailThreads);
   const int bc = w.rp * w.ps;  // component stride of b and the reciprocals
   if constexpr (KIND == kVisc) {
     T e[NS][2 * D], bv[NS][D], iv[NS][D];
@@ -568,7 +604,7 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
 #pragma unroll
       for (int c = 0; c < D; ++c)
 #pragma unroll 1
-        for (int col = 0; col < 2; ++col) {
+        for (int col = 0; col < np; ++col) {
 #pragma unroll
           for (int i = 0; i < NS; ++i)
             if (sl[i].col == col)
@@ -598,7 +634,7 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
 #pragma unroll 1
     for (int s = 0; s < sweeps; ++s)
 #pragma unroll 1
-      for (int col = 0; col < tail_passes<D, KIND>(); ++col) {
+      for (int col = 0; col < np; ++col) {
 #pragma unroll
         for (int i = 0; i < NS; ++i)
           if (sl[i].col == col) {
@@ -861,7 +897,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailTabs tb, in
         const int n = sbw.ps * (sbw.k1 - sbw.k0);
         double *xd = (double*)(mem + sbw.x) + sbw.ps, *bd = (double*)(mem + sbw.b);
         if (KIND != kVisc) bottom_sub_mean<D>(bd, n, KIND, g, sh);
-        tail_visit<D, double, KIND, PER>(mem, sbw, g, bot.beta, bot.sweeps, (double*)nullptr, rank, sync);
+        tail_visit<D, double, KIND, PER, PER>(mem, sbw, g, bot.beta, bot.sweeps, (double*)nullptr, rank, sync);
         if (KIND != kVisc) bottom_sub_mean<D>(xd, n, KIND, g, sh);
         for (int q = 0; q < NC; ++q)
           for (int t = threadIdx.x; t < n; t += blockDim.x)
@@ -878,7 +914,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) k_vcycle_tail(TailTabs tb, in
                                       local ? wc.cs : (KIND == kVisc ? sg[l + 1].ncell : 0), g, sg[l + 1], rank);
         sync();
       }
-      tail_visit<D, T, KIND, PER>(mem, w, g, beta, down ? nu1 : nu2, down ? r : (T*)nullptr, rank, sync);
+      tail_visit<D, T, KIND, PER, false>(mem, w, g, beta, down ? nu1 : nu2, down ? r : (T*)nullptr, rank, sync);
       if (down) {
         const bool cwide = sw[l + 1].np > 1;
         if (cwide || rank == 0) {
