@@ -41,14 +41,17 @@ int launch_predict(hbf_ctx* c, double dt) {
   if (st) return st;
   if ((st = tensor_lu(c, c->u, c->Lu))) return st;
   const StepC k = step_consts(g, c->dim, dt, c->rho, c->theta);
-  if (c->dim == 3 && march_box(g)) {
-    const int chunk = march_chunk(g);
+  if (c->dim == 3 && slopes_march(g)) {
     launch3(c, kSlotExplicit, k_slopes_x, slopes_x_grid(g), dim3(kRowX, kRowY), c->u, c->slopes, g);
     launch3(c, kSlotExplicit, k_slopes_yz, slopes_yz_grid(g), dim3(kPredX, kPredY), c->u, c->slopes, g);
+  } else {
+    HB_DISPATCH(c->dim, k_slopes, grid_for(g.ncell), c->u, c->slopes, g);
+  }
+  if (c->dim == 3 && hats_march(g)) {
+    const int chunk = march_plan(g).chunk;
     launch3(c, kSlotExplicit, k_hats_march, march_grid(g, chunk), dim3(kMarchThreads), c->u, c->slopes, c->Gp, c->Lu,
             fo, c->predictor_visc, c->hats, c->tcom, g, k, chunk);
   } else {
-    HB_DISPATCH(c->dim, k_slopes, grid_for(g.ncell), c->u, c->slopes, g);
     HB_DISPATCH(c->dim, k_hats, grid_for(g.ncell), c->u, c->slopes, c->Gp, c->Lu, fo, c->predictor_visc, c->hats,
                 c->tcom, g, k);
   }

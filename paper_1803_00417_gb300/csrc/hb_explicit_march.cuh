@@ -7,7 +7,8 @@
 // twice.  Here a thread takes the neighbour's from the thread, or its own
 // previous cell, that forms them.  The values, and the operations behind each,
 // are those of the one-cell forms, so the bits are the same.  Slopes at 128^3:
-// 472 us in one launch, 128 (x) + 163 (y and z) here.
+// 472 us in one launch, 128 (x) + 163 (y and z) here.  Small boxes and boxes that
+// leave the tiles half empty keep one thread per cell (slopes_march, hats_march).
 #pragma once
 #include "hb_explicit.cuh"
 
@@ -237,27 +238,40 @@ inline dim3 march_grid(const Geom& g, int chunk) {
 // takes the least time when two blocks run on each of the 152 SMs, in waves of
 // equal blocks whose start costs a third of a plane (128^3: 7 planes, 1216
 // blocks, four full waves; 16 planes leave the second wave a third empty).
-inline int march_chunk(long long tiles, int n2) {
-  long long best = 0;
-  int chunk = 6;
-  for (int q = 6; q <= 24; ++q) {
-    const long long nb = tiles * ((n2 + q - 1) / q), waves = (nb + 303) / 304, cost = waves * (3 * q + 1);
-    if (best == 0 || cost < best) {
-      best = cost;
-      chunk = q;
-    }
-  }
-  return chunk;
-}
-inline int march_chunk(const Geom& g) {
+// cost: that time, in thirds of a plane.
+struct MarchPlan {
+  int chunk;
+  long long cost;
+};
+inline MarchPlan march_plan(const Geom& g) {
   const dim3 t = march_grid(g, g.n[2]);
-  return march_chunk((long long)t.x * t.y, g.n[2]);
+  const long long tiles = (long long)t.x * t.y;
+  MarchPlan p{6, 0};
+  for (int q = 6; q <= 24; ++q) {
+    const long long nb = tiles * ((g.n[2] + q - 1) / q), waves = (nb + 303) / 304, cost = waves * (3 * q + 1);
+    if (p.cost == 0 || cost < p.cost) p = {q, cost};
+  }
+  return p;
 }
-// grids wide enough for the tiles: on smaller ones the few blocks would march
-// serially where one thread per cell fills the SMs (and a launch's y and z
-// extents stay within 65535)
-inline bool march_box(const Geom& g) {
-  return g.n[0] >= 48 && (long long)g.ncell >= 48LL * 48 * 48 && g.n[1] <= 65535 && g.n[2] <= 65535;
+// a launch's y and z extents stay within 65535
+inline bool march_extents(const Geom& g) { return g.n[1] <= 65535 && g.n[2] <= 65535; }
+
+// The slopes by lines from 60^3 cells on: below, the chunks are few and their
+// threads form serially what one thread per cell forms at once (40^3: 6 us
+// slower; 48^3 to 56^3: within 5 us either way; 60^3: 8 us faster, 128 x 64 x
+// 64: 50, 160^3: 370).  Narrower boxes than 48 leave most of a row's block idle.
+inline bool slopes_march(const Geom& g) { return march_extents(g) && g.n[0] >= 48 && g.ncell >= 60 * 60 * 60; }
+
+// The transverse terms by march where its waves take less time than one thread
+// per cell: 0.33 ns a cell there, 6.1 us a third of a plane here, so at most 52
+// thirds per million cells.  Boxes whose rows fill the 64-cell tiles and whose
+// blocks fill a wave gain from 0.4 million cells on (64 x 96 x 64: 48 thirds per
+// million cells, 22 us faster; 128 x 64 x 64: 22 us; 160^3: 253 us); 48^3 (172,
+// 60 us slower), 66 x 64 x 64 (92, 62 us slower), 80^3 (72, 50 us slower) and 96
+// x 64 x 64 (64, 14 us slower) do not, 48 x 128 x 128 (56) and 100^3 (52) are
+// within 4 us.
+inline bool hats_march(const Geom& g) {
+  return march_extents(g) && march_plan(g).cost * 1000000 <= 52LL * g.ncell;
 }
 
 // k_hats marching along z: a thread forms the states of its cell's three upper
