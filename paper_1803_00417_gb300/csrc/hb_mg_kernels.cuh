@@ -1078,8 +1078,10 @@ __global__ void __launch_bounds__(256) k_nodal_resid_z(const double* __restrict_
   }
 }
 
-// levels that leave enough columns and chunks for the SMs
-inline bool nodal_march_level(const Geom& g) { return g.nnode >= 48 * 48 * 48 && g.n[2] >= 16 && g.n[2] <= 500000; }
+// Levels that leave enough columns and chunks for the SMs: from 2e5 nodes on (one
+// thread per node against a column, us a launch: 48^3 12.2 and 15.0, 56^3 14.2 and
+// 15.0, 128 x 96 x 16 15.5 and 14.8, 64^3 18.6 and 15.1, 128^3 96 and 68)
+inline bool nodal_march_level(const Geom& g) { return g.nnode >= 200000 && g.n[2] >= 16 && g.n[2] <= 500000; }
 inline int nodal_march_chunk(const Geom& g) {
   const long long cols = ((long long)(g.n[0] + 1) * (g.n[1] + 1) + 255) / 256;
   return cols * ((g.n[2] + 16) / 16) >= 152 * 8 ? 16 : 8;

@@ -1,6 +1,6 @@
-"""Which boxes the predictor's marching kernels take, built for the host: each
-side of the two rules as it was measured (faster or slower than one thread per
-cell, GB300).  No GPU needed."""
+"""Which boxes the predictor's marching kernels and the marching nodal residual
+take, built for the host: each side of the rules as it was measured (faster or
+slower than one thread per cell or node, GB300).  No GPU needed."""
 
 import os
 import shutil
@@ -16,12 +16,16 @@ SRC = """
 #include <cstring>
 #include "hb_internal.h"
 #include "hb_explicit_march.cuh"
+#include "hb_mg_kernels.cuh"
 int main(int argc, char** argv) {
   hb::Geom g;
   std::memset(&g, 0, sizeof g);
-  g.ncell = 1;
-  for (int a = 0; a < 3; ++a) g.ncell *= g.n[a] = std::atoi(argv[1 + a]);
-  return 10 + (hb::slopes_march(g) ? 1 : 0) + (hb::hats_march(g) ? 2 : 0);
+  g.ncell = g.nnode = 1;
+  for (int a = 0; a < 3; ++a) {
+    g.ncell *= g.n[a] = std::atoi(argv[1 + a]);
+    g.nnode *= g.n[a] + 1;
+  }
+  return 10 + (hb::slopes_march(g) ? 1 : 0) + (hb::hats_march(g) ? 2 : 0) + (hb::nodal_march_level(g) ? 4 : 0);
 }
 """
 
@@ -38,12 +42,14 @@ def harness(tmp_path_factory):
     return str(d / "rule")
 
 
-# (slopes, transverse terms) by march
+# (slopes, transverse terms, nodal residual) by march
 @pytest.mark.parametrize("n,want", [
-    ((40, 40, 40), (0, 0)), ((48, 48, 48), (0, 0)), ((72, 56, 40), (0, 0)), ((56, 56, 56), (0, 0)),
-    ((47, 500, 500), (0, 0)), ((60, 60, 60), (1, 0)), ((66, 64, 64), (1, 0)), ((80, 80, 80), (1, 0)),
-    ((96, 64, 64), (1, 0)), ((130, 60, 60), (1, 0)), ((64, 96, 64), (1, 1)), ((120, 60, 60), (1, 1)),
-    ((128, 64, 64), (1, 1)), ((128, 128, 128), (1, 1)), ((256, 256, 256), (1, 1)), ((64, 70000, 6), (0, 0))])
+    ((40, 40, 40), (0, 0, 0)), ((48, 48, 48), (0, 0, 0)), ((72, 56, 40), (0, 0, 0)), ((56, 56, 56), (0, 0, 0)),
+    ((47, 500, 500), (0, 0, 1)), ((60, 60, 60), (1, 0, 1)), ((66, 64, 64), (1, 0, 1)), ((80, 80, 80), (1, 0, 1)),
+    ((96, 64, 64), (1, 0, 1)), ((130, 60, 60), (1, 0, 1)), ((64, 96, 64), (1, 1, 1)), ((120, 60, 60), (1, 1, 1)),
+    ((128, 64, 64), (1, 1, 1)), ((128, 128, 128), (1, 1, 1)), ((256, 256, 256), (1, 1, 1)),
+    ((64, 70000, 6), (0, 0, 0)), ((128, 64, 16), (0, 0, 0)), ((128, 96, 16), (0, 0, 1)), ((64, 64, 48), (0, 0, 1)),
+    ((256, 512, 15), (1, 1, 0))])
 def test_rule(harness, n, want):
     r = subprocess.run([harness, *map(str, n)], capture_output=True, timeout=60)
-    assert r.returncode - 10 == want[0] + 2 * want[1]
+    assert r.returncode - 10 == want[0] + 2 * want[1] + 4 * want[2]
