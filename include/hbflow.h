@@ -145,17 +145,28 @@ int hbf_set_solver(hbf_ctx* ctx, double rtol, int max_cycles, int nu1, int nu2, 
  * factor (or 40 iterations), then recomputes r in FP64.  Default 1e-3; FP32
  * limits a useful drop to about 1e-6.  HBF_ERR_ARG outside [1e-7, 1). */
 int hbf_set_inner_drop(hbf_ctx* ctx, double drop);
-/* HBF_MIXED viscous solve.  on = 1 (default) lets the library choose the
- * layout of the FP32 finest level: on grids of more than 2^19 cells, 3D with
- * walls on every axis and an even x extent, the colour-split layout (the cells
- * with i + j + k even, then the odd ones, each row-major with n_x / 2 cells per
- * row), so that each red-black sweep reads and writes unit-stride runs of one
- * colour; on smaller grids the natural layout with stored face viscosities, as
- * on the coarse levels.  on = 0 keeps the natural layout with the cell
- * viscosity.  The solve runs to the same tolerance in each.  The TMA-staged
- * and one-launch sweep forms, when enabled, take the natural layout.
- * HBF_ERR_ARG unless on is 0 or 1. */
+/* HBF_MIXED viscous solve, 3D with walls on every axis and an even x extent:
+ * on = 1 keeps the FP32 finest-level vectors of the solve in the colour-split
+ * layout (the cells with i + j + k even, then the odd ones, each row-major with
+ * n_x / 2 cells per row), so that each red-black sweep reads and writes
+ * unit-stride runs of one colour; on = 0 keeps the natural layout.  The sweeps'
+ * and the operator's values are the same bit for bit; only the memory traffic
+ * and the summation order of the Krylov dot products differ.  Without a call
+ * the library chooses: the colour-split layout on grids of more than 2^19 cells
+ * that can have it, and on every grid of at most 2^19 cells (also 2D and
+ * periodic) the natural layout with stored face viscosities, as on the coarse
+ * levels; the solve runs to the same tolerance.  The TMA-staged and one-launch
+ * sweep forms, when enabled, take the natural layout.  HBF_ERR_ARG unless on is
+ * 0 or 1. */
 int hbf_set_split_layout(hbf_ctx* ctx, int on);
+/* The layout that the next mixed viscous solve keeps its FP32 finest level in:
+ * HBF_LAYOUT_NATURAL (cell viscosity), HBF_LAYOUT_SPLIT or HBF_LAYOUT_FACES
+ * (natural, with stored face viscosities).  HBF_ERR_ARG for an HBF_FP64
+ * context, which has no such level. */
+#define HBF_LAYOUT_NATURAL 0
+#define HBF_LAYOUT_SPLIT 1
+#define HBF_LAYOUT_FACES 2
+int hbf_get_finest_layout(hbf_ctx* ctx, int* layout);
 /* The fused tail of the V-cycles (the multigrid scheme of Sec. III B): from
  * the first level with at most max_cells cells (a mixed viscous solve's finest
  * level only in its default layout) down to the coarsest-level solve and back

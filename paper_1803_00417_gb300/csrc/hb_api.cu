@@ -402,6 +402,13 @@ int hbf_set_split_layout(hbf_ctx* c, int on) {
   return HBF_OK;
 }
 
+int hbf_get_finest_layout(hbf_ctx* c, int* layout) {
+  if (!c || !layout) return HBF_ERR_ARG;
+  if (c->precision != HBF_MIXED) return fail(c, HBF_ERR_ARG, "only a mixed context has an FP32 finest level");
+  *layout = finest_layout(c);
+  return HBF_OK;
+}
+
 int hbf_set_periodic(hbf_ctx* c, const int periodic[3]) {
   if (!c || !periodic) return HBF_ERR_ARG;
   int per[3] = {0, 0, 0};

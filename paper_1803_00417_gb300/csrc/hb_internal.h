@@ -127,7 +127,8 @@ struct hbf_ctx {
   double K = 1.0;           // the consistency K as given to hbf_set_rheology
   double theta = 0.5;       // implicit weight of the viscous term (1/2: Crank-Nicolson, Eq. 15)
   double inner_drop = 1e-3; // residual drop of each FP32 BiCGStab pass of the mixed viscous solve
-  int split_layout = 1;     // FP32 finest level of the mixed viscous solve in the colour-split layout where it applies
+  int split_layout = -1;    // FP32 finest level of the mixed viscous solve: 1 colour-split where it applies, 0
+                            // natural, -1 the library's rule (finest_layout)
   int split_last = -1;      // the layout of the last mixed viscous solve (vprev32 is kept in it)
   double t = 0.0;           // time: the sum of the dt of every step taken
   long long nstep = 0;      // steps taken
@@ -271,6 +272,7 @@ double reduce_sum(hbf_ctx* c, const double* x, long long n, int* st);
 double reduce_dot(hbf_ctx* c, const double* a, const double* b, long long n, int* st);
 
 // solves (hb_mg.cu)
+int finest_layout(const hbf_ctx* c);  // HBF_LAYOUT_* of the mixed viscous solve's FP32 finest level
 int solve_mac(hbf_ctx* c, const double* rhs, double* phi, hbf_solve_stats* s);
 int solve_viscous(hbf_ctx* c, double beta, const double* rhs, double* u, hbf_solve_stats* s);
 int solve_nodal(hbf_ctx* c, const double* rhs, double* phi, hbf_solve_stats* s);

@@ -260,30 +260,34 @@ static inline bool aligned8(const void* p) { return ((uintptr_t)p & 7) == 0; }
 // form (with the wraps); walls on every axis take PER = false
 static inline bool any_per(const Geom& g) { return g.per[0] || g.per[1] || g.per[2]; }
 
+// A small FP32 finest level of the mixed viscous solve (no layout set, no opt-in
+// form) is handled like the coarse levels: natural layout, stored face
+// viscosities and reciprocals, the branch-free kernels of hb_visc_hom.cuh, and
+// the fused tail where it starts there.  It is bound by the latency of one
+// sweep's chain, not by bytes: 6 us per split sweep and 8 us per natural one at
+// 32^3 to 96 x 64 x 64, 3 us this way; the split layout, with half the bytes,
+// wins from about 80^3 on.
+constexpr int kFaces0Cells = 1 << 19;
+static bool faces0(const hbf_ctx* c) {
+  return c->precision == HBF_MIXED && c->split_layout < 0 && c->g.ncell <= kFaces0Cells && !c->staged_tx &&
+         !c->staged_op_rows && !c->fused_sweep;
+}
+
 // The FP32 finest level of the mixed viscous solve in the colour-split layout
 // (hb_visc_split.cuh): 3D, walls on every axis, even n0, at least two levels,
 // and none of the opt-in sweep or operator forms that read the natural layout
 // (staged, fused) nor a network on level 0.  Every FP32 level-0 vector of the
 // solve (the BiCGStab vectors, the V-cycle's level-0 arrays, the cell
 // viscosity, the previous increment) is then split; FP64 arrays stay natural.
-// A small FP32 finest level of the mixed viscous solve (in the default layout,
-// no opt-in form) is handled like the coarse levels: natural layout, stored
-// face viscosities and reciprocals, the branch-free kernels of hb_visc_hom.cuh,
-// and the fused tail where it starts there.  It is bound by the latency of one
-// sweep's chain, not by bytes: 6 us per split sweep and 8 us per natural one at
-// 32^3 to 96 x 64 x 64, 3 us this way; the split layout, with half the bytes,
-// wins from about 80^3 on.
-constexpr int kFaces0Cells = 1 << 19;
-static bool faces0(const hbf_ctx* c) {
-  return c->precision == HBF_MIXED && c->split_layout && c->g.ncell <= kFaces0Cells && !c->staged_tx &&
-         !c->staged_op_rows && !c->fused_sweep;
-}
-
 static bool split0(const hbf_ctx* c) {
   const Geom& g = c->g;
   return c->split_layout && !faces0(c) && c->dim == 3 && c->precision == HBF_MIXED && !any_per(g) && g.n[0] % 2 == 0 &&
          g.n[0] >= 4 && g.n[1] >= 3 && g.n[2] >= 3 && c->lv.size() >= 2 && c->lv[0].feta != nullptr &&
          !c->staged_tx && !c->staged_op_rows && !c->fused_sweep && !(c->vnet && c->vnet_level == 0);
+}
+
+int finest_layout(const hbf_ctx* c) {
+  return faces0(c) ? HBF_LAYOUT_FACES : split0(c) ? HBF_LAYOUT_SPLIT : HBF_LAYOUT_NATURAL;
 }
 
 // blocks of a reduction over n elements: 2048 elements each (8 per thread),

@@ -106,6 +106,7 @@ SIGNATURES = {
     "hbf_set_staged_op": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]),
     "hbf_set_inner_drop": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_double]),
     "hbf_set_split_layout": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
+    "hbf_get_finest_layout": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
     "hbf_field_size": (ctypes.c_int64, [ctypes.c_void_p, ctypes.c_int]),
     "hbf_set_field": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]),
     "hbf_get_field": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]),
@@ -339,8 +340,16 @@ class HBFlow:
 
     def set_split_layout(self, on):
         """Colour-split layout of the FP32 finest-level vectors of the mixed
-        viscous solve (1, the default where it applies) or the natural one (0)."""
+        viscous solve (1, where it applies) or the natural one (0); without a
+        call the library chooses by size."""
         self._check(self.lib.hbf_set_split_layout(self.ctx, int(on)))
+
+    def finest_layout(self):
+        """Layout of the mixed viscous solve's FP32 finest level: "natural",
+        "colour-split" or "stored faces"."""
+        q = ctypes.c_int()
+        self._check(self.lib.hbf_get_finest_layout(self.ctx, ctypes.byref(q)))
+        return ("natural", "colour-split", "stored faces")[q.value]
 
     def set_staged_op(self, rows, tile_z=16):
         """TMA-staged finest-level viscous operator (rows 4 or 8; 0 off)."""
