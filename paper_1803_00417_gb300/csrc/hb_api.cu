@@ -154,7 +154,7 @@ static int allocate(hbf_ctx* c) {
       A(L.fvx, (long long)D * gl.ncell);
       A(L.fvb, (long long)D * gl.ncell);
       A(L.fvr, (long long)D * gl.ncell);
-      A(L.fvinv, (long long)D * gl.ncell);
+      if (l > 0 || gl.ncell <= kFaces0Cells) A(L.fvinv, (long long)D * gl.ncell);  // else: ensure_inv0
       A(L.fcx, gl.ncell);
       A(L.fcb, gl.ncell);
       A(L.fcr, gl.ncell);
@@ -179,6 +179,13 @@ static int allocate(hbf_ctx* c) {
   }
 #undef A
   return cuda_check(c, cudaStreamSynchronize(c->stream), "allocation");
+}
+
+// the finest level's FP32 reciprocals above kFaces0Cells, which only a batch reads
+int ensure_inv0(hbf_ctx* c) {
+  Level& L = c->lv[0];
+  if (c->precision != HBF_MIXED || L.fvinv) return HBF_OK;
+  return alloc(c, &L.fvinv, (long long)c->dim * L.g.ncell);
 }
 
 struct FieldView {

@@ -1458,6 +1458,7 @@ int hbf_batch_create(hbf_batch** out, int dim, int ncav, const int64_t* n, const
     st = hbf_init_grid(&x, dim, n + 3 * (size_t)c, h[c], wall_u ? wall_u + 18 * (size_t)c : nullptr, precision,
                        (void*)B->stream);
     if (!st) B->cav.push_back(x);
+    if (!st) st = ensure_inv0(x);
   }
   if (!st) st = dalloc(B, &B->mask_all, ncav);
   if (!st) st = dalloc(B, &B->mask_act, ncav);

@@ -204,6 +204,8 @@ struct hbf_ctx {
 namespace hb {
 
 constexpr int kRedBlocks = 1024;
+// a single context's FP32 finest level of at most this many cells stores its faces (faces0 in hb_mg.cu)
+constexpr int kFaces0Cells = 1 << 19;
 
 // beta = theta dt / rho of the viscous solve; theta = 1/2 is computed as
 // dt / (2 rho), the Crank-Nicolson form of Eq. 15
@@ -272,6 +274,7 @@ double reduce_sum(hbf_ctx* c, const double* x, long long n, int* st);
 double reduce_dot(hbf_ctx* c, const double* a, const double* b, long long n, int* st);
 
 // solves (hb_mg.cu)
+int ensure_inv0(hbf_ctx* c);
 int finest_layout(const hbf_ctx* c);  // HBF_LAYOUT_* of the mixed viscous solve's FP32 finest level
 int solve_mac(hbf_ctx* c, const double* rhs, double* phi, hbf_solve_stats* s);
 int solve_viscous(hbf_ctx* c, double beta, const double* rhs, double* u, hbf_solve_stats* s);

@@ -267,7 +267,6 @@ static inline bool any_per(const Geom& g) { return g.per[0] || g.per[1] || g.per
 // sweep's chain, not by bytes: 6 us per split sweep and 8 us per natural one at
 // 32^3 to 96 x 64 x 64, 3 us this way; the split layout, with half the bytes,
 // wins from about 80^3 on.
-constexpr int kFaces0Cells = 1 << 19;
 static bool faces0(const hbf_ctx* c) {
   return c->precision == HBF_MIXED && c->split_layout < 0 && c->g.ncell <= kFaces0Cells && !c->staged_tx &&
          !c->staged_op_rows && !c->fused_sweep;
