@@ -33,10 +33,11 @@ __device__ __forceinline__ void pdl_wait() {
 #endif
 }
 
-// launches a kernel that begins with pdl_wait()
+// launches a kernel that begins with pdl_wait(); early: with leave to start while
+// the one before it drains
 template <typename... P, typename... Args>
-inline cudaError_t launch_kernel(cudaStream_t stream, dim3 grid, dim3 block, size_t smem, void (*kern)(P...),
-                                 Args... args) {
+inline cudaError_t launch_kernel_if(bool early, cudaStream_t stream, dim3 grid, dim3 block, size_t smem,
+                                    void (*kern)(P...), Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -46,8 +47,26 @@ inline cudaError_t launch_kernel(cudaStream_t stream, dim3 grid, dim3 block, siz
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <typename... P, typename... Args>
+inline cudaError_t launch_kernel(cudaStream_t stream, dim3 grid, dim3 block, size_t smem, void (*kern)(P...),
+                                 Args... args) {
+  return launch_kernel_if(true, stream, grid, block, smem, kern, args...);
+}
+
+// Whether a 3D explicit stage of that many blocks (256 cells each) starts early.
+// Its blocks are long (FP64, up to 508 operations a cell), and blocks placed while
+// the predecessor's still hold their SMs are not spread evenly: where an even
+// spread is one block per SM, or one and a half to four, some SM gets one more and
+// the launch takes that much longer than starting early saves (viscosity and
+// predictor, us with and without: 28^3, 86 blocks, 120 and 110; 40^3 177 and 151;
+// 48^3 244 and 194; 53^3, 582 blocks, 260 and 248).  Otherwise early is faster
+// (26^3, 69 blocks, 86 and 110: both grids fit at once; 36^3, 183 blocks, 146 and
+// 147; 54^3, 616 blocks, 269 and 283; 80^3 631 and 656).
+inline bool stage_early(int blocks) {
+  return 2 * blocks <= 152 || (blocks > 152 && 2 * blocks <= 3 * 152) || blocks > 4 * 152;
 }
 
 struct Geom {

@@ -19,7 +19,7 @@ namespace hb {
     if ((dim) == 2)                                                   \
       launch(c, kSlotExplicit, KERNEL<2>, (GRID), kThreads, __VA_ARGS__); \
     else                                                              \
-      launch(c, kSlotExplicit, KERNEL<3>, (GRID), kThreads, __VA_ARGS__); \
+      launch_if(c, kSlotExplicit, stage_early(GRID), KERNEL<3>, (GRID), kThreads, __VA_ARGS__); \
   } while (0)
 
 int launch_eta(hbf_ctx* c) {

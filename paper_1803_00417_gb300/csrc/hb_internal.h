@@ -227,12 +227,17 @@ struct ProfRegion {
 // every kernel launch of the library goes through here: counts it and, when
 // profiling is on, brackets finest-level launches of a slot with events
 template <typename K, typename... Args>
-inline void launch(hbf_ctx* c, int slot, K kern, int grid, int block, Args... args) {
+inline void launch_if(hbf_ctx* c, int slot, bool early, K kern, int grid, int block, Args... args) {
   const bool rec = prof_wants(c->prof, slot);
   if (rec) prof_mark(c, slot, true);
-  launch_kernel(c->stream, dim3(grid), dim3(block), 0, kern, args...);
+  launch_kernel_if(early, c->stream, dim3(grid), dim3(block), 0, kern, args...);
   if (rec) prof_mark(c, slot, false);
   ++c->nlaunch;
+}
+
+template <typename K, typename... Args>
+inline void launch(hbf_ctx* c, int slot, K kern, int grid, int block, Args... args) {
+  launch_if(c, slot, true, kern, grid, block, args...);
 }
 
 template <typename K, typename... Args>

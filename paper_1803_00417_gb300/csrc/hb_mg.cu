@@ -2117,12 +2117,14 @@ void axmy(hbf_ctx* c, double* out, const double* x, double a, const double* y, l
 
 int tensor_lu(hbf_ctx* c, const double* u, double* out) {
   const Level& L = c->lv[0];
-  if (c->dim == 2)
+  if (c->dim == 2) {
     launch(c, kSlotExplicit, k_tensor_lu<2, double>, grid_for(xi_count<2>(L.g), 152 * 24), kThreads, u, out,
            (const double*)L.ef[0], (const double*)L.ef[1], (const double*)L.ef[2], L.g, 0);
-  else
-    launch(c, kSlotExplicit, k_tensor_lu<3, double>, grid_for(xi_count<3>(L.g), 152 * 24), kThreads, u, out,
-           (const double*)L.ef[0], (const double*)L.ef[1], (const double*)L.ef[2], L.g, 0);
+  } else {
+    const int nb = grid_for(xi_count<3>(L.g), 152 * 24);
+    launch_if(c, kSlotExplicit, stage_early(nb), k_tensor_lu<3, double>, nb, kThreads, u, out,
+              (const double*)L.ef[0], (const double*)L.ef[1], (const double*)L.ef[2], L.g, 0);
+  }
   return cuda_check(c, cudaGetLastError(), "k_tensor_lu");
 }
 

@@ -1,6 +1,7 @@
 """Which boxes the predictor's marching kernels and the marching nodal residual
 take, built for the host: each side of the rules as it was measured (faster or
-slower than one thread per cell or node, GB300).  No GPU needed."""
+slower than one thread per cell or node, GB300); and which launches of the
+explicit stages start while their predecessor drains.  No GPU needed."""
 
 import os
 import shutil
@@ -18,6 +19,7 @@ SRC = """
 #include "hb_explicit_march.cuh"
 #include "hb_mg_kernels.cuh"
 int main(int argc, char** argv) {
+  if (argc == 2) return hb::stage_early(std::atoi(argv[1])) ? 11 : 10;
   hb::Geom g;
   std::memset(&g, 0, sizeof g);
   g.ncell = g.nnode = 1;
@@ -53,3 +55,10 @@ def harness(tmp_path_factory):
 def test_rule(harness, n, want):
     r = subprocess.run([harness, *map(str, n)], capture_output=True, timeout=60)
     assert r.returncode - 10 == want[0] + 2 * want[1] + 4 * want[2]
+
+
+# blocks of 256 cells of the cubes 26, 28, 32, 36, 40, 48, 53, 54 and 128
+@pytest.mark.parametrize("blocks,early", [(69, 1), (86, 0), (128, 0), (183, 1), (250, 0), (432, 0), (582, 0), (616, 1),
+                                          (2432, 1)])
+def test_early_start(harness, blocks, early):
+    assert subprocess.run([harness, str(blocks)], timeout=60).returncode - 10 == early
