@@ -170,11 +170,12 @@ int hbf_get_finest_layout(hbf_ctx* ctx, int* layout);
 /* The fused tail of the V-cycles (the multigrid scheme of Sec. III B): from
  * the first level with at most max_cells cells (a mixed viscous solve's finest
  * level only in its default layout) down to the coarsest-level solve and back
- * runs as one launch of one thread-block
- * cluster, with barriers between the colour sweeps; the arithmetic and its
- * order are those of the level-by-level launches.  0 disables it; without a
- * call the library chooses the level by size, dimension and precision.
- * HBF_ERR_ARG for a negative count. */
+ * runs as one launch of one thread-block cluster, with barriers between the
+ * colour sweeps; the arithmetic and its order are those of the level-by-level
+ * launches.  It starts lower where the cluster's shared memory (16 x 200 KB)
+ * does not hold the level.  0 disables it; without a call the library chooses
+ * the level by size, dimension and precision.  HBF_ERR_ARG for a negative
+ * count. */
 int hbf_set_tail(hbf_ctx* ctx, int max_cells);
 /* The 3D FP32 finest-level viscous smoothing of HBF_MIXED contexts: 1 runs
  * each component's red-black Gauss-Seidel sweep (Sec. III A's tensor solve,
@@ -563,7 +564,11 @@ int hbf_batch_get_tiling(const hbf_batch* b, int* tile, int* blocks_per_sm, int6
  * all coarser levels) run as one launch per V-cycle, one thread-block cluster
  * per cavity, with barriers between colour sweeps; the arithmetic and its
  * order are those of the level-by-level launches.  0 disables it; by default
- * 4096, and in HBF_MIXED batches up to 16384 when they have few cavities. */
+ * 4096, and in HBF_MIXED batches up to 16384 when they have few cavities.  A
+ * cluster has the blocks that leave every cavity one on the GPU's 152 SMs (16
+ * at most, one from 77 cavities on), and whatever the count the tail starts at
+ * the first level whose arrays fit their shared memory (200 KB each): 64 x 64
+ * cells need two blocks, so from 77 cavities on such levels are launched. */
 int hbf_batch_set_tail(hbf_batch* b, int max_cells);
 /* Time a representative launch sequence (explicit stages and one viscous
  * V-cycle of every cavity; no cavity state changes) for each tiling

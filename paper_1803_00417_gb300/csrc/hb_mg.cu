@@ -1764,9 +1764,9 @@ static int solve_viscous_mixed(hbf_ctx* c, double beta, const double* b_in, doub
     P.resid(0);
     return reduce_max_abs(c, r, n, &st);
   };
-  // the V-cycle reads q as its level-0 right-hand side in place (the fused
-  // tail starts on level 1 or below, so its argument records never hold level
-  // 0's array)
+  // the V-cycle reads q as its level-0 right-hand side and z as its iterate in
+  // place (a tail that starts on level 0 takes both from its launch, not from
+  // its records)
   auto precond = [&](const float* q, float* z) {
     ViscProblem<D, float> Pz(c, z, beta, true);  // z is 0
     Pz.b0 = q;

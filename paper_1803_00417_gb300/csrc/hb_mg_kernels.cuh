@@ -519,6 +519,8 @@ __host__ __device__ __forceinline__ void visc_smooth_cell(T* __restrict__ u, con
   u[(size_t)C * g.ncell + cidx<D>(g, p[0], p[1], p[2])] = v;
 }
 
+// one thread of that sweep with stored faces (the host checks' reference for
+// hb_visc_hom.cuh, whose form the library runs)
 template <int D, typename T, int C, bool PER = true>
 __host__ __device__ __forceinline__ void k_visc_smooth_c_at(T* __restrict__ u, const T* __restrict__ b, const T* ef0,
                                                            const T* ef1, const T* ef2, const Geom& g, int col, T beta,
