@@ -530,7 +530,11 @@ static bool plan_tail_kind(hbf_batch* B, int lf, int& nblk, size_t& smem) {
 // of cavities, and in FP32 as many as leave 2048 to each block of a cavity's
 // cluster, up to the single cavity's 16384 (16 cavities of 64^2 to 256^2, 8
 // blocks each: a colour sweep of all 128^2 levels takes 6.5 us as a launch, 2
-// us as a phase of the tail).  FP64 phases are bound by their operations.
+// us as a phase of the tail).  FP64 phases are bound by their operations.  From
+// 77 cavities on a cluster is one block, whose shared memory a 64^2 level does not
+// fit (211 KB in FP32, 421 in FP64): the tail then starts below it (a batch of 96
+// takes 17.6 ms a step in mixed precision and 25.0 in FP64; one-block tails from
+// 64^2 on that went through L2, with every launch waiting, took 23.9 and 43.1).
 static int default_tail_cells(const hbf_batch* B) {
   int nblk = 16;
   while (nblk > 1 && nblk * B->ncav > 152) nblk >>= 1;
