@@ -172,7 +172,8 @@ int hbf_get_finest_layout(hbf_ctx* ctx, int* layout);
  * level only in its default layout) down to the coarsest-level solve and back
  * runs as one launch of one thread-block cluster, with barriers between the
  * colour sweeps; the arithmetic and its order are those of the level-by-level
- * launches.  It starts lower where the cluster's shared memory (16 x 200 KB)
+ * launches (but for a swept coarsest level that is odd along a periodic axis,
+ * whose cells next to the wrap are ordered differently).  It starts lower where the cluster's shared memory (16 x 200 KB)
  * does not hold the level.  0 disables it; without a call the library chooses
  * the level by size, dimension and precision.  HBF_ERR_ARG for a negative
  * count. */

@@ -485,7 +485,8 @@ __host__ __device__ inline int rb_count(const Geom& g) {
 // cells 0 and n - 1 of a row neighbours of one colour.  Such a level takes each
 // colour in two parts with a barrier between them: a cell is in part 1 when it
 // is the last one on an odd number of those axes, so a neighbour through a wrap
-// is always in the other part.
+// is always in the other part.  (The tail's register slots keep one pass per
+// colour and store its values behind a barrier: tail_slot_pass.)
 __host__ __device__ __forceinline__ bool odd_wrap(const Geom& g, int a) { return g.per[a] && (g.n[a] & 1); }
 __host__ __device__ __forceinline__ int rb_parts(const Geom& g) {
   return odd_wrap(g, 0) || odd_wrap(g, 1) || odd_wrap(g, 2) ? 2 : 1;

@@ -471,7 +471,7 @@ constexpr int tail_slots() {
 
 template <int D, typename T>
 struct TailSlot {
-  int col = -1;       // pass of its component; -1: no point
+  int col = -1;       // colour; -1: no point
   int k, q, o;        // plane, point of the plane, offset in x
   int om[D], op[D];   // neighbours
   unsigned wall = 0;  // bit 2a: no neighbour below on axis a (a wall), bit 2a + 1: above
@@ -496,7 +496,7 @@ __host__ __device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const
     if (p[0] >= g.n[0]) return;
     p[1] = j;
     p[D - 1] = s.k;
-    s.col = ODD && rb_parts(g) == 2 ? 2 * col + rb_part(g, p) : col;
+    s.col = col;
     s.q = p[0] + g.n[0] * j;
     const HomAxis x(p[0], g.n[0], 1, PER && g.per[0]);
     s.om[0] = x.om;
@@ -521,6 +521,11 @@ __host__ __device__ __forceinline__ void tail_slot_init(TailSlot<D, T>& s, const
         s.k = p[D - 1];
         s.q = p[0] + (g.n[0] + 1) * (D == 3 ? p[1] : 0);
         s.col = col;
+        if (ODD && rb_parts(g) == 2) {  // node n - 1 with the even ones
+          int c[3] = {0, 0, 0};
+          nd_classes<D>(g, col, c);
+          s.col = (c[0] & 1) | ((c[1] & 1) << 1) | ((c[2] & 1) << 2);
+        }
         break;
       }
       t -= n;
@@ -539,6 +544,31 @@ __device__ __forceinline__ bool tail_fits_slots(const TailLevel<T>& w, const Geo
   return n <= tail_slots<D, KIND>() * kTailThreads;
 }
 
+// One colour of the slots: value(i) of each slot i of the colour, put(i, v), a
+// barrier.  On a level that is odd along a periodic axis (wrap) some points of a
+// colour are neighbours through the wrap: every value is formed before any is
+// stored, with a barrier between, so that both read the other's old value.  A
+// barrier costs less than the second pass that the indexed form and the one-block
+// kernels take there (rb_parts: a pass of these small levels is one chain long).
+template <bool ODD, typename T, int NS, class SL, class V, class P, class S>
+__device__ __forceinline__ void tail_slot_pass(const SL* sl, int col, bool wrap, V value, P put, S sync) {
+  if constexpr (ODD) {
+    T v[NS];
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+      if (sl[i].col == col) v[i] = value(i);
+    if (wrap) sync();
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+      if (sl[i].col == col) put(i, v[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < NS; ++i)
+      if (sl[i].col == col) put(i, value(i));
+  }
+  sync();
+}
+
 // sweeps sweeps of the level, a barrier after each pass; then, when r is not
 // null, the residual into r (the whole level's layout) and a barrier
 template <int D, typename T, int KIND, bool PER, bool ODD, class S>
@@ -546,15 +576,15 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
                                            unsigned rank, S sync) {
   const T bs = KIND == kVisc ? rn_mul(beta, g_ihh<T>(g)) : T(0);
   constexpr int NS = tail_slots<D, KIND>();
-  const int np = tail_passes<D, KIND, ODD>(g) / (KIND == kVisc ? D : 1);  // passes per component
   const bool per = PER && g.per[D - 1];
   T* const x = (T*)(mem + w.x);
   const T* const b = (const T*)(mem + w.b);
   if (!tail_fits_slots<D, KIND>(w, g)) {
+    const int np = tail_passes<D, KIND, ODD>(g);
 #pragma unroll 1
     for (int s = 0; s < sweeps; ++s)
 #pragma unroll 1
-      for (int q = 0; q < (KIND == kVisc ? D * np : np); ++q) {
+      for (int q = 0; q < np; ++q) {
         tail_pass<D, T, KIND, PER, ODD>(mem, w, g, bs, q, rank);
         sync();
       }
@@ -564,6 +594,7 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
     }
     return;
   }
+  const bool wrap = ODD && rb_parts(g) == 2;
   TailSlot<D, T> sl[NS];
 #pragma unroll
   for (int i = 0; i < NS; ++i) tail_slot_init<D, T, KIND, PER, ODD>(sl[i], w, g, (int)threadIdx.x + i * kTailThreads);
@@ -604,13 +635,10 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
 #pragma unroll
       for (int c = 0; c < D; ++c)
 #pragma unroll 1
-        for (int col = 0; col < np; ++col) {
-#pragma unroll
-          for (int i = 0; i < NS; ++i)
-            if (sl[i].col == col)
-              tail_put<D, T, KIND, PER>(x, w, per, c, sl[i].k, sl[i].q, rank, hom_gs<D, T>(cell(i, c), bv[i][c], iv[i][c], bs));
-          sync();
-        }
+        for (int col = 0; col < 2; ++col)
+          tail_slot_pass<ODD, T, NS>(
+              sl, col, wrap, [&](int i) { return hom_gs<D, T>(cell(i, c), bv[i][c], iv[i][c], bs); },
+              [&](int i, T v) { tail_put<D, T, KIND, PER>(x, w, per, c, sl[i].k, sl[i].q, rank, v); }, sync);
     if (r) {
 #pragma unroll
       for (int c = 0; c < D; ++c)
@@ -634,23 +662,20 @@ __device__ __forceinline__ void tail_visit(char* mem, const TailLevel<T>& w, con
 #pragma unroll 1
     for (int s = 0; s < sweeps; ++s)
 #pragma unroll 1
-      for (int col = 0; col < np; ++col) {
-#pragma unroll
-        for (int i = 0; i < NS; ++i)
-          if (sl[i].col == col) {
-            const T* q = x + sl[i].o;
-            T v;
-            if constexpr (KIND == kMac) {
-              bool lo[D], hi[D];
-              flags(i, lo, hi);
-              v = cell_gs_value<D, T>(q, bv[i], g_hh<T>(g), sl[i].om, sl[i].op, lo, hi);
-            } else {
-              v = (g_hh<T>(g) * bv[i] - nodal_nbr_sum<D, T>(q, sl[i].om, sl[i].op)) * T(-3.0 / 8.0);
-            }
-            tail_put<D, T, KIND, PER>(x, w, per, 0, sl[i].k, sl[i].q, rank, v);
-          }
-        sync();
-      }
+      for (int col = 0; col < (KIND == kMac ? 2 : 1 << D); ++col)
+        tail_slot_pass<ODD, T, NS>(
+            sl, col, wrap,
+            [&](int i) {
+              const T* q = x + sl[i].o;
+              if constexpr (KIND == kMac) {
+                bool lo[D], hi[D];
+                flags(i, lo, hi);
+                return cell_gs_value<D, T>(q, bv[i], g_hh<T>(g), sl[i].om, sl[i].op, lo, hi);
+              } else {
+                return (g_hh<T>(g) * bv[i] - nodal_nbr_sum<D, T>(q, sl[i].om, sl[i].op)) * T(-3.0 / 8.0);
+              }
+            },
+            [&](int i, T v) { tail_put<D, T, KIND, PER>(x, w, per, 0, sl[i].k, sl[i].q, rank, v); }, sync);
     if (r) {
 #pragma unroll
       for (int i = 0; i < NS; ++i)

@@ -1,9 +1,10 @@
 """The order of a coarsest level's sweeps, built for the host: on walls and on
 periodic axes of even and odd cell counts (a periodic 40 coarsens to 5 cells,
-whose first and last have one colour and are neighbours through the wrap) no
-two points of one pass are neighbours, and every sweep visits every point once;
-for the one-block kernels and for both forms of the fused tail.  No GPU
-needed."""
+whose first and last have one colour and are neighbours through the wrap) every
+sweep visits every point once, and no two points of one pass are neighbours; for
+the one-block kernels and for both forms of the fused tail (whose slot form
+stores a pass's values behind a barrier on such levels and may hold the
+neighbours that the wrap makes).  No GPU needed."""
 
 import os
 import shutil
